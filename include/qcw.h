@@ -90,7 +90,15 @@ QCW_API qcw_status qcw_set_mode(qcw_ctx *ctx, int mode, int fuse_k);
  *     the row and column bits of the same qubits; each pass evolves the tiles on one side of
  *     the diagonal and writes the others as their conjugate transposes (half the arithmetic).
  *     A non-Hermitian matrix loaded with qcw_set_state is not preserved.  One CTA per tile.
- *   HERM_WS (and AUTO, the default): the same Hermitian pass on persistent CTAs whose
+ *   AUTO (the default): from 3 qubits up the state is kept as its 4^n real Pauli coefficients
+ *     v_P = Tr[P rho] between readouts (a second buffer of 4 * 4^n bytes beside rho, allocated on
+ *     first use; without room for it, and for work too short to win back the two changes of
+ *     basis, passes run as HERM_WS): half the bytes of rho per pass, real one-qubit maps of 12
+ *     multiply-adds per four coefficients, CNOT and CZ as signed permutations.  Every readout but
+ *     the ones of the whole matrix has a form on v; the library changes back to rho whenever
+ *     the matrix itself is read (qcw_get_state, qcw_get_device_state, qcw_sync, plain-mode work).
+ *     A non-Hermitian matrix loaded with qcw_set_state is not preserved.
+ *   HERM_WS (and AUTO below 3 qubits): the same Hermitian pass as HERM on persistent CTAs whose
  *     producer warps load and store tiles while consumer warps evolve them, so memory traffic
  *     and arithmetic overlap; each pass reads and writes only the lower triangle r >= c of rho
  *     (a third less memory traffic), and the library completes the matrix whenever it is read
@@ -131,8 +139,8 @@ QCW_API qcw_status qcw_set_fused_wait_limit(qcw_ctx *ctx, unsigned polls, int st
 QCW_API qcw_status qcw_set_validation(qcw_ctx *ctx, int on);
 
 /* Device pointer of rho and the context's stream (borrowed; valid until destroy).  Flushes
- * queued work and completes the matrix first (the HERM_WS pass keeps only the lower triangle
- * r >= c current between readouts): the buffer holds all of rho for work ordered on the
+ * queued work and completes the matrix first (AUTO keeps the state elsewhere, the HERM_WS pass
+ * only the lower triangle r >= c current between readouts): the buffer holds all of rho for work ordered on the
  * returned stream until the next evolution call. */
 QCW_API qcw_status qcw_get_device_state(qcw_ctx *ctx, void **dev_rho, void **cuda_stream);
 

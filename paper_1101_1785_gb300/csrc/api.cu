@@ -8,6 +8,7 @@
 #include <string>
 
 #include "hermitian.h"
+#include "pauli_run.h"
 #include "qcw_internal.h"
 #include "tile.h"
 
@@ -318,12 +319,47 @@ qcw_status plain_super(qcw_ctx *c, const std::vector<c128> &s, const int *qs, in
     return QCW_OK;
 }
 
+bool pauli_allowed(qcw_ctx *c)
+{
+    if (c->fused_kernel != QCW_FUSED_KERNEL_AUTO || c->n < kPMinDigits || c->pauli_off) return false;
+    if (c->pv) return true;
+    if (cudaMalloc(&c->pv, sizeof(float) << (2 * c->n)) != cudaSuccess) {
+        cudaGetLastError();
+        c->pv = nullptr;
+        c->pauli_off = true;  // no room beside rho: the passes on rho itself need none
+        return false;
+    }
+    return true;
+}
+
+qcw_status pauli_settle(qcw_ctx *c)
+{
+    if (!c->pzero) return QCW_OK;
+    CK(launch_pauli_zero(c->pv, c->n, c->nsm, c->stream));
+    c->launches++;
+    c->pzero = false;
+    return QCW_OK;
+}
+
 // Half storage: the warp-specialised pass keeps only the lower triangle current; everything
 // that reads the other triangle (plain kernels, the other fused kernels, state downloads, direct
 // device access) completes the matrix first.  The readouts (trace, probabilities, purity, Pauli
 // expectations, partial trace) and the measurement projection work on the lower triangle as it is.
+// Pauli storage is changed back to rho at the same points, but for the readouts, which have their
+// own form on the Pauli coefficients (qcw_partial_trace of more than six qubits excepted).
 qcw_status ensure_full(qcw_ctx *c)
 {
+    if (c->in_pauli) {
+        if (c->pzero) {
+            launch_zero_state(c->rho, c->n, false, c->nsm, c->stream);
+            CKLAUNCH(c, 1);
+        } else {
+            CK(launch_pauli_to_rho(c->pv, c->rho, c->n, c->stream));
+            c->launches += pauli_convert_launches(c->n);
+        }
+        c->in_pauli = c->pzero = c->half = false;
+        return QCW_OK;
+    }
     if (!c->half) return QCW_OK;
     launch_symmetrize(c->rho, c->n, c->nsm, c->stream);
     CKLAUNCH(c, 1);
@@ -391,6 +427,7 @@ static void ctx_free(qcw_ctx *c)
     if (c->d_result) cudaFree(c->d_result);
     if (c->h_result) cudaFreeHost(c->h_result);
     if (c->d_staging) cudaFree(c->d_staging);
+    if (c->pv) cudaFree(c->pv);
     if (c->d_kacc) cudaFree(c->d_kacc);
     if (c->d_ktmp) cudaFree(c->d_ktmp);
     if (c->d_ckpt) cudaFree(c->d_ckpt);
@@ -544,7 +581,7 @@ extern "C" qcw_status qcw_set_fused_wait_limit(qcw_ctx *ctx, unsigned polls, int
 qcw_status qcw::begin_state_replace(qcw_ctx *c)
 {
     c->queue.clear();
-    c->half = false;
+    c->half = c->in_pauli = c->pzero = false;
     c->state_ver++;
     return clear_error_word(c);
 }
@@ -553,6 +590,12 @@ extern "C" qcw_status qcw_reset(qcw_ctx *ctx)
 {
     CHECK_CTX(ctx);
     ctx->queue.clear();
+    ctx->in_pauli = ctx->pzero = ctx->mode == QCW_MODE_FUSED && pauli_allowed(ctx);
+    if (ctx->in_pauli) {  // the first pass starts from |0..0><0..0| without reading it
+        ctx->half = false;
+        ctx->state_ver++;
+        return clear_error_word(ctx);
+    }
     // In fused mode with the warp-specialised kernel (6 qubits and up) the next passes keep only
     // the lower triangle current anyway: write that half of |0..0><0..0| and start in half storage.
     ctx->half = ctx->mode == QCW_MODE_FUSED && ctx->n >= 6 &&
@@ -589,7 +632,7 @@ extern "C" qcw_status qcw_set_state(qcw_ctx *ctx, const double *rho_c128)
     qcw_status st = ensure_staging(ctx);
     if (st) return st;
     ctx->queue.clear();
-    ctx->half = false;
+    ctx->half = ctx->in_pauli = ctx->pzero = false;
     ctx->state_ver++;
     st = clear_error_word(ctx);
     if (st) return st;
@@ -612,7 +655,7 @@ extern "C" qcw_status qcw_set_state_c64(qcw_ctx *ctx, const float *rho_c64)
     if (ctx->validate && !is_density(rho_c64, ctx->n))
         return set_error(QCW_EINVAL, "state is not Hermitian with unit trace (validation)");
     ctx->queue.clear();
-    ctx->half = false;
+    ctx->half = ctx->in_pauli = ctx->pzero = false;
     ctx->state_ver++;
     qcw_status st = clear_error_word(ctx);
     if (st) return st;
@@ -811,13 +854,49 @@ static qcw_status fetch_results(qcw_ctx *c)
     memcpy(&w, c->h_result + kErrSlot, sizeof w);
     return check_error_word(c, w);
 }
+// The readouts of the current state into device memory: trace (2 values) and P(q = 1) for q < n;
+// purity.  All on whichever form the state is in.
+static qcw_status enqueue_diag(qcw_ctx *c, double *out)
+{
+    if (c->in_pauli) {
+        qcw_status st = pauli_settle(c);
+        if (st) return st;
+        launch_pauli_diag(c->pv, c->n, out, c->stream);
+        CKLAUNCH(c, 1);
+        return QCW_OK;
+    }
+    launch_diag_reduce(c->rho, c->n, c->d_partials, out, c->red_blocks, c->stream);
+    CKLAUNCH(c, launches_per_reduce());
+    return QCW_OK;
+}
+
+static qcw_status enqueue_purity(qcw_ctx *c, double *out)
+{
+    const double *part = nullptr;
+    int nb = 0;
+    if (fused_purity_partials(c, &part, &nb)) {
+        launch_fold(part, nb, out, c->stream);  // summed by the last pass as it wrote the state
+        CKLAUNCH(c, 1);
+        return QCW_OK;
+    }
+    if (c->in_pauli) {
+        qcw_status st = pauli_settle(c);
+        if (st) return st;
+        launch_pauli_purity(c->pv, c->n, c->d_partials, out, c->red_blocks, c->stream);
+    } else if (c->half) {
+        launch_purity_lower(c->rho, c->n, c->d_partials, out, c->red_blocks, c->stream);
+    } else {
+        launch_purity(c->rho, c->n, c->d_partials, out, c->red_blocks, c->stream);
+    }
+    CKLAUNCH(c, launches_per_reduce());
+    return QCW_OK;
+}
+
 static qcw_status diag_readout(qcw_ctx *c)
 {
     qcw_status st = fused_flush(c);
-    if (st) return st;
-    launch_diag_reduce(c->rho, c->n, c->d_partials, c->d_result, c->red_blocks, c->stream);
-    CKLAUNCH(c, launches_per_reduce());
-    return fetch_results(c);
+    if (!st) st = enqueue_diag(c, c->d_result);
+    return st ? st : fetch_results(c);
 }
 
 extern "C" qcw_status qcw_trace(qcw_ctx *ctx, double *re, double *im)
@@ -846,16 +925,8 @@ extern "C" qcw_status qcw_purity(qcw_ctx *ctx, double *out)
     if (!out) return set_error(QCW_EINVAL, "null output");
     qcw_status st = fused_flush(ctx);
     if (st) return st;
-    const double *part = nullptr;
-    int nb = 0;
-    if (fused_purity_partials(ctx, &part, &nb)) {
-        launch_fold(part, nb, ctx->d_result, ctx->stream);  // summed by the last pass as it wrote rho
-        CKLAUNCH(ctx, 1);
-    } else {
-        if (ctx->half) launch_purity_lower(ctx->rho, ctx->n, ctx->d_partials, ctx->d_result, ctx->red_blocks, ctx->stream);
-        else launch_purity(ctx->rho, ctx->n, ctx->d_partials, ctx->d_result, ctx->red_blocks, ctx->stream);
-        CKLAUNCH(ctx, launches_per_reduce());
-    }
+    st = enqueue_purity(ctx, ctx->d_result);
+    if (st) return st;
     st = fetch_results(ctx);
     if (st) return st;
     *out = ctx->h_result[0];
@@ -876,6 +947,13 @@ static qcw_status pauli_readout(qcw_ctx *c, const PauliTerms &T)
 {
     qcw_status st = fused_flush(c);
     if (st) return st;
+    if (c->in_pauli) {
+        st = pauli_settle(c);
+        if (st) return st;
+        launch_pauli_terms(c->pv, T, c->d_result, c->stream);
+        CKLAUNCH(c, 1);
+        return fetch_results(c);
+    }
     launch_pauli_expect(c->rho, c->n, T, c->d_partials, c->red_blocks * (QCW_MAX_QUBITS + 2), c->d_result, c->stream);
     CKLAUNCH(c, 2);
     return fetch_results(c);
@@ -1011,18 +1089,9 @@ extern "C" qcw_status qcw_checkpoint(qcw_ctx *ctx, long long *ticket)
     double *d = ctx->d_ckpt + (size_t)slot * kCkptVals;
     double *h = ctx->h_ckpt + (size_t)slot * kCkptVals;
     const int n = ctx->n;
-    launch_diag_reduce(ctx->rho, n, ctx->d_partials, d, ctx->red_blocks, ctx->stream);
-    CKLAUNCH(ctx, launches_per_reduce());
-    const double *part = nullptr;
-    int nb = 0;
-    if (fused_purity_partials(ctx, &part, &nb)) {
-        launch_fold(part, nb, d + 2 + n, ctx->stream);
-        CKLAUNCH(ctx, 1);
-    } else {
-        if (ctx->half) launch_purity_lower(ctx->rho, n, ctx->d_partials, d + 2 + n, ctx->red_blocks, ctx->stream);
-        else launch_purity(ctx->rho, n, ctx->d_partials, d + 2 + n, ctx->red_blocks, ctx->stream);
-        CKLAUNCH(ctx, launches_per_reduce());
-    }
+    st = enqueue_diag(ctx, d);
+    if (!st) st = enqueue_purity(ctx, d + 2 + n);
+    if (st) return st;
     CK(cudaMemcpyAsync(h, d, sizeof(double) * (size_t)(n + 3), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaMemcpyAsync(h + kCkptVals - 1, device_error_word(ctx), sizeof(double), cudaMemcpyDeviceToHost,
                        ctx->stream));
@@ -1065,7 +1134,8 @@ extern "C" qcw_status qcw_measure(qcw_ctx *ctx, int qubit, int forced, double u,
     if (prob) *prob = pm;
     if (!(pm >= 1e-12)) return set_error(QCW_EZEROPROB, "outcome probability below 1e-12");
     ctx->state_ver++;
-    launch_project(ctx->rho, ctx->n, qubit, m, (float)(1.0 / pm), ctx->half, ctx->nsm, ctx->stream);
+    if (ctx->in_pauli) launch_pauli_project(ctx->pv, ctx->n, qubit, m, 1.0 / pm, ctx->nsm, ctx->stream);
+    else launch_project(ctx->rho, ctx->n, qubit, m, (float)(1.0 / pm), ctx->half, ctx->nsm, ctx->stream);
     CKLAUNCH(ctx, 1);
     return QCW_OK;
 }
@@ -1080,6 +1150,9 @@ extern "C" qcw_status qcw_partial_trace(qcw_ctx *ctx, const int *keep, int nkeep
         if (j && keep[j] <= keep[j - 1]) return set_error(QCW_EINVAL, "kept qubits must ascend");
     }
     qcw_status st = fused_flush(ctx);
+    if (st) return st;
+    const bool from_pauli = ctx->in_pauli && nkeep <= kPauliPtMax;
+    st = from_pauli ? pauli_settle(ctx) : ctx->in_pauli ? ensure_full(ctx) : QCW_OK;
     if (st) return st;
     PTParams p{};
     p.n = n;
@@ -1102,7 +1175,8 @@ extern "C" qcw_status qcw_partial_trace(qcw_ctx *ctx, const int *keep, int nkeep
             return set_error(QCW_ENOMEM, "partial trace output");
         }
     }
-    launch_partial_trace(ctx->rho, p, d_out, ctx->nsm, ctx->stream);
+    if (from_pauli) launch_pauli_ptrace(ctx->pv, p, d_out, ctx->stream);
+    else launch_partial_trace(ctx->rho, p, d_out, ctx->nsm, ctx->stream);
     ctx->launches += 1;
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(out_c128, d_out, nout * sizeof(double2), cudaMemcpyDeviceToHost, ctx->stream);

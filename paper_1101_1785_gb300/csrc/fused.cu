@@ -16,6 +16,7 @@
 #include <mutex>
 #include <tuple>
 
+#include "pauli_run.h"
 #include "planner.h"
 #include "qcw_internal.h"
 #include "tc.cuh"
@@ -106,8 +107,19 @@ struct KTune {
     size_t nops = 0;
 };
 
+struct CachedPauli {
+    uint64_t hash = 0;
+    int k = 0;
+    bool beam = false;
+    std::vector<QOp> ops;  // exact copy for verification
+    std::vector<PauliBlob> passes;
+    int nnode = 0;
+    long long last_use = 0;
+};
+
 struct FusedRuntime {
     std::vector<CachedPlan> cache;
+    std::vector<CachedPauli> pcache;
     long long tick = 0;
     unsigned ws_grid = 0;  // CTAs of the warp-specialised kernel (resident per SM x SMs)
     unsigned tc_grid = 0;  // the same for its tensor-core variant
@@ -818,10 +830,117 @@ static int auto_k(const std::vector<QOp> &ops, size_t b, size_t e, int n, bool h
     return best;
 }
 
+// Per-CTA (or per-team) purity partials of a pass.
+static qcw_status purity_scratch(FusedRuntime *rt, int need)
+{
+    if (rt->ppart_cap < need) {
+        if (rt->d_ppart) cudaFree(rt->d_ppart);
+        rt->d_ppart = nullptr;
+        rt->ppart_cap = 0;
+        if (cudaMalloc(&rt->d_ppart, sizeof(double) * (size_t)need) != cudaSuccess) {
+            cudaGetLastError();
+            return set_error(QCW_ENOMEM, "purity partials");
+        }
+        rt->ppart_cap = need;
+    }
+    rt->ppart_nb = need;
+    return QCW_OK;
+}
+
+// Events around a pass when timing is on (qcw_enable_pass_timing).
+static cudaEvent_t pass_event(qcw_ctx *c, FusedRuntime *rt)
+{
+    cudaEvent_t e = nullptr;
+    if (!c->timing) return e;
+    if (!rt->ev_free.empty()) {
+        e = rt->ev_free.back();
+        rt->ev_free.pop_back();
+    } else {
+        cudaEventCreate(&e);
+    }
+    cudaEventRecord(e, c->stream);
+    rt->ev_pending.push_back(e);
+    return e;
+}
+
 static const size_t kMaxCached = 64;
 // Registers from this size up get beam-searched plans for segments that are replayed (a pass
 // there costs at least ~10 us, so the planning time pays back over a few replays).
 constexpr int kBeamMinQubits = 10;
+
+// Whether a state held as rho is changed to Pauli storage for a plan.  The two changes of basis cost
+// 2.6 ms at 14 qubits, a pass on rho 1.1 ms and the completion of its upper triangle 0.35 ms, and a
+// Pauli pass does the work of about 1.4 passes on rho in 0.6 ms: from two Pauli passes on the
+// change is about even or better, a single one does not win it back.
+static bool pauli_pays(const CachedPauli &p) { return p.passes.size() > 1; }
+
+// The segment in the Pauli basis; *done = false: it is better run on rho.
+static qcw_status run_pauli_segment(qcw_ctx *c, size_t b, size_t e, bool last, bool *done)
+{
+    FusedRuntime *rt = c->fused;
+    *done = false;
+    const uint64_t h = hash_ops(c->queue, b, e, c->n, c->fuse_k, 0);
+    CachedPauli *hit = nullptr;
+    for (CachedPauli &p : rt->pcache)
+        if (p.hash == h && p.k == c->fuse_k && same_ops(p.ops, c->queue, b, e)) {
+            hit = &p;
+            break;
+        }
+    auto plan_into = [&](CachedPauli &p, bool beam) {
+        const PauliPlan plan = plan_pauli(c->queue, b, e, c->n, c->fuse_k, beam);
+        p.beam = beam;
+        p.passes.clear();
+        for (const PPass &ps : plan.passes) p.passes.push_back(pauli_blob(ps));
+    };
+    if (!hit) {
+        if (rt->pcache.size() >= kMaxCached) {  // evict least recently used
+            size_t victim = 0;
+            for (size_t i = 1; i < rt->pcache.size(); i++)
+                if (rt->pcache[i].last_use < rt->pcache[victim].last_use) victim = i;
+            rt->pcache.erase(rt->pcache.begin() + victim);
+        }
+        CachedPauli p;
+        p.hash = h;
+        p.k = c->fuse_k;
+        p.ops.assign(c->queue.begin() + b, c->queue.begin() + e);
+        plan_into(p, false);
+        rt->pcache.push_back(std::move(p));
+        hit = &rt->pcache.back();
+    } else if (!hit->beam && c->n >= kBeamMinQubits) {
+        plan_into(*hit, true);  // the segment is replayed: plan it once with the beam search
+    }
+    hit->last_use = ++rt->tick;
+    if (!c->in_pauli) {
+        if (!pauli_pays(*hit)) return QCW_OK;
+        cudaError_t er = launch_rho_to_pauli(c->rho, c->pv, c->n, c->stream);
+        if (er != cudaSuccess) return cuda_error(er, "change to Pauli storage");
+        c->launches += pauli_convert_launches(c->n);
+        c->in_pauli = true;
+        c->half = false;  // (the change reads the lower triangle only, so half storage needed no completion)
+    }
+    *done = true;
+    for (size_t p = 0; p < hit->passes.size(); p++) {
+        const PauliBlob &B = hit->passes[p];
+        double *ppart = nullptr;
+        const bool lastp = last && p + 1 == hit->passes.size();
+        if (lastp) {
+            qcw_status st = purity_scratch(rt, 2 * (int)pauli_grid(B.h, c->nsm));
+            if (st) return st;
+            ppart = rt->d_ppart;
+        }
+        pass_event(c, rt);
+        c->state_ver++;
+        cudaError_t er = launch_pauli_pass(B, c->pv, c->n, c->nsm, c->pzero, device_error_word(c), c->wait_limit,
+                                           c->stall_tile, ppart, c->stream);
+        pass_event(c, rt);
+        if (er != cudaSuccess) return cuda_error(er, "Pauli pass launch");
+        c->pzero = false;
+        c->launches++;
+        c->passes++;
+        if (lastp) c->purity_ver = c->state_ver;
+    }
+    return QCW_OK;
+}
 
 // last: nothing follows this segment in the flush, so its last pass (if warp-specialised) also
 // leaves the purity partials of the resulting rho.
@@ -829,6 +948,15 @@ static qcw_status run_segment(qcw_ctx *c, size_t b, size_t e, bool last)
 {
     FusedRuntime *rt = c->fused;
     const int n = c->n;
+    if (pauli_allowed(c)) {
+        bool done = false;
+        qcw_status ps = run_pauli_segment(c, b, e, last, &done);
+        if (ps || done) return ps;
+    }
+    if (c->in_pauli) {
+        qcw_status fs = ensure_full(c);
+        if (fs) return fs;
+    }
     const bool herm0 = herm_kernel(c);
     KTune &tn = rt->tune;
     bool trial = false;
@@ -953,17 +1081,7 @@ static qcw_status run_segment(qcw_ctx *c, size_t b, size_t e, bool last)
     const FPhase *dph = reinterpret_cast<const FPhase *>(hit->dbuf + hit->phase_off);
     const float2 *dco = reinterpret_cast<const float2 *>(hit->dbuf + hit->coef_off);
     for (size_t p = 0; p < hit->hpass.size(); p++) {
-        cudaEvent_t e0 = nullptr, e1 = nullptr;
-        if (c->timing) {
-            if (rt->ev_free.size() >= 2) {
-                e1 = rt->ev_free.back(); rt->ev_free.pop_back();
-                e0 = rt->ev_free.back(); rt->ev_free.pop_back();
-            } else {
-                cudaEventCreate(&e0);
-                cudaEventCreate(&e1);
-            }
-            cudaEventRecord(e0, c->stream);
-        }
+        pass_event(c, rt);
         if (!ws_pass(c, hit->hpass[p])) {
             qcw_status fs = ensure_full(c);  // the other kernels read both triangles
             if (fs) return fs;
@@ -974,19 +1092,9 @@ static qcw_status run_segment(qcw_ctx *c, size_t b, size_t e, bool last)
             const unsigned npairs = (unsigned)hit->grid[p];
             double *ppart = nullptr;
             if (last && p + 1 == hit->hpass.size()) {
-                const int need = (int)std::min(npairs, wgrid);
-                if (rt->ppart_cap < need) {
-                    if (rt->d_ppart) cudaFree(rt->d_ppart);
-                    rt->d_ppart = nullptr;
-                    rt->ppart_cap = 0;
-                    if (cudaMalloc(&rt->d_ppart, sizeof(double) * (size_t)need) != cudaSuccess) {
-                        cudaGetLastError();
-                        return set_error(QCW_ENOMEM, "purity partials");
-                    }
-                    rt->ppart_cap = need;
-                }
+                qcw_status ps = purity_scratch(rt, (int)std::min(npairs, wgrid));
+                if (ps) return ps;
                 ppart = rt->d_ppart;
-                rt->ppart_nb = need;
             }
             const unsigned wl = c->wait_limit ? c->wait_limit : kWsWaitLimit;
             auto kern = tc ? (ppart ? k_fused_herm_tc<true> : k_fused_herm_tc<false>)
@@ -1001,11 +1109,7 @@ static qcw_status run_segment(qcw_ctx *c, size_t b, size_t e, bool last)
         }
         c->launches++;
         c->passes++;
-        if (c->timing) {
-            cudaEventRecord(e1, c->stream);
-            rt->ev_pending.push_back(e0);
-            rt->ev_pending.push_back(e1);
-        }
+        pass_event(c, rt);
         cudaError_t er = cudaGetLastError();
         if (er != cudaSuccess) return cuda_error(er, "fused pass launch");
         if (last && p + 1 == hit->hpass.size() && ws_pass(c, hit->hpass[p])) c->purity_ver = c->state_ver;

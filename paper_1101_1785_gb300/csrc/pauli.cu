@@ -1,0 +1,666 @@
+// Pauli-basis path (see pauli.h): the pass kernel, the changes of basis to and from rho, and the
+// readouts, all on the real vector v_P = Tr[P rho].
+#include <algorithm>
+#include <cstddef>
+#include <cstring>
+
+#include "pauli.cuh"
+#include "pauli_run.h"
+#include "qcw_internal.h"
+
+namespace qcw {
+
+// ------------------------------------------------------------------ pass kernel
+// Persistent, one CTA per SM: two teams of 256 threads work on alternate tiles of the CTA's list
+// out of three tile buffers, so one buffer's loads (cp.async, released through an mbarrier) are in
+// flight while the two teams evolve theirs.  Each buffer has one mbarrier per team: a buffer's tiles
+// go to the two teams in turn, and a team that waited on the other's phases by parity could take an
+// earlier one for its own.  A thread stores and reloads the same chunks of a
+// buffer, so the write-back of tile i and the load of tile i + 3 need no barrier between them.
+// Traffic: one read and one write of v, 8 * 4^n bytes.  Measured at n = 14 (2.15 GB): 0.62 ms per
+// pass of four rounds and seven operations (k_fused_herm_ws, on rho: 1.10 ms per pass, and a third
+// more passes), 0.55 ms with the operations left out, 0.34 ms (6.2 TB/s) with the rounds left out:
+// the rounds' trips through shared memory are what it waits for.  Each wait is bounded: the team that gives
+// up sets the error word and stops, the other runs out of tiles or gives up in turn.
+constexpr int kPBuf = 3;
+constexpr int kPThreads = 512;
+constexpr unsigned kPWaitLimit = 1u << 21;
+
+template <int BYTES>
+struct PauliParams {
+    PauliHdr h;
+    int pad[1];
+    unsigned blob[BYTES / 4];  // PRound[nround], POp[nop], coefficient pairs float2[ncoef]
+};
+static_assert(offsetof(PauliParams<16>, blob) % 16 == 0, "vector loads from the parameter block");
+
+// offsets in the blob (4-byte units)
+__host__ __device__ inline int pb_ops(const PauliHdr &h) { return (int)(sizeof(PRound) / 4) * h.nround; }
+__host__ __device__ inline int pb_coef(const PauliHdr &h) { return pb_ops(h) + ((h.nop + 3) & ~3); }
+
+size_t pauli_pass_smem(const PauliHdr &h, bool dense)
+{
+    const size_t prog = dense ? 4 * (size_t)pb_coef(h) + sizeof(float2) * (size_t)h.ncoef : sizeof(PRound) * (size_t)h.nround;
+    return (size_t)kPBuf * (sizeof(float) << (2 * h.t)) + prog + 16 * sizeof(double) + 2 * kPBuf * sizeof(uint64_t);
+}
+
+template <int BYTES, bool DENSE, bool PUR>
+__global__ void __launch_bounds__(kPThreads, 1)
+    k_pauli_pass(float *__restrict__ v, unsigned ntiles, int init, unsigned long long *__restrict__ err,
+                 unsigned wait_limit, int stall_tile, double *__restrict__ ppart, double pscale,
+                 const __grid_constant__ PauliParams<BYTES> prm)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const PauliHdr &H = prm.h;
+    const int t = H.t;
+    const unsigned nchunk = 1u << (2 * (t - 1));
+    const size_t tbytes = sizeof(float) << (2 * t);
+    unsigned char *p = smem + kPBuf * tbytes;
+    PRound *rounds = reinterpret_cast<PRound *>(p);
+    const int nword = DENSE ? pb_coef(H) + 2 * H.ncoef : pb_ops(H);  // of the program kept in shared memory
+    double *red = reinterpret_cast<double *>(reinterpret_cast<unsigned *>(rounds) + nword);
+    uint64_t *full = reinterpret_cast<uint64_t *>(red + 16);
+    const unsigned tid = threadIdx.x & 255u, team = threadIdx.x >> 8;
+    for (int i = threadIdx.x; i < nword; i += kPThreads) reinterpret_cast<unsigned *>(rounds)[i] = prm.blob[i];
+    if (threadIdx.x < 2 * kPBuf) mbar_init(&full[threadIdx.x], 256);
+    __syncthreads();
+    // this thread's chunks are tid + 256 i: offsets split into a part of tid (tile digits 1..4) and
+    // a part of i (digits 5, 6)
+    uint64_t glo = 0;
+    for (int d = 1; d < t && d < 5; d++) glo += (uint64_t)((tid >> (2 * (d - 1))) & 3u) << (2 * H.td[d]);
+    const int s5 = t > 5 ? 2 * H.td[5] : 0, s6 = t > 6 ? 2 * H.td[6] : 0;
+    const unsigned plo = pauli_swz(tid);
+    const unsigned mine = tid < nchunk ? (nchunk + 255u) >> 8 : 0u;  // chunks of this thread
+    const unsigned ntile = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+    auto base_of = [&](unsigned i) {
+        const unsigned tile = blockIdx.x + i * gridDim.x;
+        uint64_t b = glo;
+        for (int d = 0; d < H.nod; d++) b += (uint64_t)((tile >> (2 * d)) & 3u) << (2 * H.od[d]);
+        return b;
+    };
+    auto goff = [&](unsigned i) { return ((uint64_t)(i & 3u) << s5) + ((uint64_t)(i >> 2) << s6); };
+    const uint64_t step5 = 1ull << s5, jump6 = (1ull << s6) - 3 * step5;  // full tiles: k walks digit 5, then 6
+    auto load = [&](unsigned i) {
+        if (blockIdx.x == 0 && (int)i == stall_tile) return;
+        const unsigned b = i % kPBuf;
+        float4 *buf = reinterpret_cast<float4 *>(smem + b * tbytes);
+        uint64_t *bar = &full[2 * b + (i & 1u)];
+        if (init) {  // |0..0><0..0|: 1 on every string of I and Z
+            const bool zt = ((blockIdx.x + i * gridDim.x) & 0xAAAAAAAAu) == 0;
+            for (unsigned k = 0; k < mine; k++)
+                buf[plo ^ pauli_swz(256u * k)] = zt && ((tid + 256u * k) & 0xAAAu) == 0 ? make_float4(1.f, 1.f, 0.f, 0.f)
+                                                                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+            mbar_arrive(bar);
+        } else {
+            const float *src = v + base_of(i);
+            if (t == kPTile) {
+#pragma unroll
+                for (unsigned k = 0; k < 16; k++) {
+                    cp_async16(buf + (plo ^ pauli_swz(256u * k)), src);
+                    src += (k & 3u) == 3u ? jump6 : step5;
+                }
+            } else {
+                for (unsigned k = 0; k < mine; k++) cp_async16(buf + (plo ^ pauli_swz(256u * k)), src + goff(k));
+            }
+            cp_async_mbar_arrive(bar);
+        }
+    };
+    if (team == 0) {
+        if (ntile > 0) load(0);
+        if (ntile > 2) load(2);
+    } else if (ntile > 1) {
+        load(1);
+    }
+    double pacc = 0.0;
+    for (unsigned i = team; i < ntile; i += 2) {
+        const unsigned b = i % kPBuf;
+        const bool ok = bar_and(1 + team, 256, mbar_wait(&full[2 * b + team], (i / (2 * kPBuf)) & 1u, wait_limit));
+        if (!ok) {
+            if (tid == 0) atomicOr(err, 1ull);
+            break;
+        }
+        if constexpr (DENSE) {
+            const unsigned *w = reinterpret_cast<const unsigned *>(rounds);
+            const ProgShared prog{rounds, reinterpret_cast<const POp *>(w + pb_ops(H)), smem_u32(w + pb_coef(H))};
+            pauli_rounds<true>(smem_u32(smem) + (unsigned)(b * tbytes), rounds, H.nround, prog, tid, 1 + team);
+        } else {
+            const ProgParam prog{prm.blob, pb_ops(H), pb_coef(H)};
+            pauli_rounds<false>(smem_u32(smem) + (unsigned)(b * tbytes), rounds, H.nround, prog, tid, 1 + team);
+        }
+        float *dst = v + base_of(i);
+        const unsigned ba = smem_u32(smem) + (unsigned)(b * tbytes);
+        float ps = 0.f;
+        auto put = [&](unsigned k, float *to) {
+            const float4 x = p_lds4(ba + 16u * (plo ^ pauli_swz(256u * k)));
+            *reinterpret_cast<float4 *>(to) = x;
+            if (PUR) ps = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, ps))));
+        };
+        if (t == kPTile) {
+#pragma unroll
+            for (unsigned k = 0; k < 16; k++) {
+                put(k, dst);
+                dst += (k & 3u) == 3u ? jump6 : step5;
+            }
+        } else {
+            for (unsigned k = 0; k < mine; k++) put(k, dst + goff(k));
+        }
+        if (PUR) pacc += (double)ps;
+        if (i + kPBuf < ntile) load(i + kPBuf);
+    }
+    cp_async_wait_all();
+    if (PUR) {  // one partial per team, fixed order: shuffle tree per warp, then the warps in turn
+        pacc = warp_sum(pacc);
+        if ((threadIdx.x & 31u) == 0) red[threadIdx.x >> 5] = pacc;
+        bar_sync(1 + team, 256);
+        if (tid == 0) {
+            double s = 0;
+            for (int w = 0; w < 8; w++) s += red[8 * team + w];
+            ppart[2 * blockIdx.x + team] = s * pscale;
+        }
+    }
+}
+
+template <int BYTES, bool DENSE>
+static cudaError_t launch_pass(const PauliBlob &B, float *v, unsigned ntiles, unsigned grid, bool init,
+                               unsigned long long *err, unsigned wait_limit, int stall_tile, double *ppart, double pscale,
+                               cudaStream_t s)
+{
+    PauliParams<BYTES> prm;
+    prm.h = B.h;
+    memcpy(prm.blob, B.words.data(), 4 * B.words.size());
+    auto kern = ppart ? k_pauli_pass<BYTES, DENSE, true> : k_pauli_pass<BYTES, DENSE, false>;
+    const size_t sm = pauli_pass_smem(B.h, DENSE);
+    if (ensure_smem_attr(reinterpret_cast<const void *>(kern), sm)) return cudaErrorInvalidValue;
+    kern<<<grid, kPThreads, sm, s>>>(v, ntiles, init ? 1 : 0, err, wait_limit ? wait_limit : kPWaitLimit, stall_tile, ppart,
+                                     pscale, prm);
+    return cudaGetLastError();
+}
+
+PauliBlob pauli_blob(const PPass &p)
+{
+    PauliBlob B;
+    PauliHdr &h = B.h;
+    memset(&h, 0, sizeof h);
+    h.t = p.t;
+    h.nod = (int)p.od.size();
+    h.nround = (int)p.rounds.size();
+    h.nop = (int)p.ops.size();
+    h.ncoef = (int)p.coefs.size();
+    for (size_t i = 0; i < p.td.size(); i++) h.td[i] = (int8_t)p.td[i];
+    for (size_t i = 0; i < p.od.size(); i++) h.od[i] = (int8_t)p.od[i];
+    static_assert(sizeof(PRound) == 96 && sizeof(POp) == 4, "blob layout");
+    B.words.assign((size_t)pb_coef(h) + 2 * h.ncoef, 0u);
+    memcpy(B.words.data(), p.rounds.data(), sizeof(PRound) * p.rounds.size());
+    for (const POp &o : p.ops) B.dense |= o.kind >= PO_TWO && o.kind < PO_TWO + 3;
+    if (h.nop) memcpy(B.words.data() + pb_ops(h), p.ops.data(), sizeof(POp) * p.ops.size());
+    for (size_t i = 0; i < p.coefs.size(); i++)
+        for (int j = 0; j < 2; j++) memcpy(B.words.data() + pb_coef(h) + 2 * i + j, &p.coefs[i], sizeof(float));
+    return B;
+}
+
+// A launch copies its whole parameter block, so the usual pass (no dense two-qubit map, a few
+// rounds) has a small one.
+cudaError_t launch_pauli_pass(const PauliBlob &B, float *v, int nd, int nsm, bool init, unsigned long long *err,
+                              unsigned wait_limit, int stall_tile, double *ppart, cudaStream_t s)
+{
+    const unsigned ntiles = 1u << (2 * B.h.nod), grid = pauli_grid(B.h, nsm);
+    double pscale = 1.0;
+    for (int i = 0; i < nd; i++) pscale *= 0.5;
+    constexpr int kSmall = 3840;
+    constexpr int kLarge = 8 * kPMaxCoef + (int)sizeof(PRound) * kPMaxRounds + 4 * kPMaxOps;
+    if (!B.dense && 4 * B.words.size() <= kSmall)
+        return launch_pass<kSmall, false>(B, v, ntiles, grid, init, err, wait_limit, stall_tile, ppart, pscale, s);
+    return launch_pass<kLarge, true>(B, v, ntiles, grid, init, err, wait_limit, stall_tile, ppart, pscale, s);
+}
+
+unsigned pauli_grid(const PauliHdr &h, int nsm)
+{
+    return std::min(1u << (2 * h.nod), (unsigned)nsm);
+}
+
+// ------------------------------------------------------------------ change of basis
+// rho[r][c], c = r ^ x: 2^-n sum_z (-1)^{z.r} (-i)^{|x & z|} v_{x,z}.  With the signs u = s v
+// (s = -1 where |x & z| mod 4 is 1 or 2) the terms with even |x & z| are real, the odd ones
+// imaginary, and since flipping r by x changes the sign of exactly the odd ones, one real
+// Walsh-Hadamard transform W_{x,r} = sum_z (-1)^{z.r} u_{x,z} holds both parts:
+//   2^n rho[r][r ^ x] = (W_{x,r} + W_{x,r^x}) / 2 + i (W_{x,r} - W_{x,r^x}) / 2.
+// Conversely W = 2^n (Re + Im) rho[r][r ^ x] and v = s 2^-n WHT(W).  The transform is separable over
+// the qubits: k_pauli_high runs it in place over the z bits of all but the seven lowest qubits,
+// k_pauli_emit / k_pauli_absorb over those and between v and rho, in 16 KiB tiles: everything is
+// real and each stage reads and writes its data once.
+// Applied to a chunk (labels I, Z, X, Y of the lowest qubit, idx a multiple of 4): Y adds one.
+template <typename V>
+__device__ __forceinline__ void p_signs4(V &a, uint64_t idx)
+{
+    const int k = __popcll(idx & (idx >> 1) & 0x5555555555555555ull);
+    if ((k + 1) & 2) a.x = -a.x, a.y = -a.y, a.z = -a.z;
+    if ((k + 2) & 2) a.w = -a.w;
+}
+
+// Bits of v to the even positions.
+__device__ __forceinline__ uint64_t p_spread(unsigned v)
+{
+    uint64_t x = v;
+    x = (x | (x << 16)) & 0x0000FFFF0000FFFFull;
+    x = (x | (x << 8)) & 0x00FF00FF00FF00FFull;
+    x = (x | (x << 4)) & 0x0F0F0F0F0F0F0F0Full;
+    x = (x | (x << 2)) & 0x3333333333333333ull;
+    x = (x | (x << 1)) & 0x5555555555555555ull;
+    return x;
+}
+
+template <int NB, typename T, typename F, typename G>
+__device__ __forceinline__ void p_wht(F ld, G st)
+{
+    T e[1 << NB];
+#pragma unroll
+    for (int j = 0; j < (1 << NB); j++) e[j] = ld(j);
+#pragma unroll
+    for (int b = 0; b < NB; b++)
+#pragma unroll
+        for (int j = 0; j < (1 << NB); j++)
+            if (!(j & (1 << b))) {
+                const T a = e[j], c = e[j | (1 << b)];
+                e[j] = a + c;
+                e[j | (1 << b)] = a - c;
+            }
+#pragma unroll
+    for (int j = 0; j < (1 << NB); j++) st(j, e[j]);
+}
+
+struct alignas(16) F4 {
+    float x, y, z, w;
+};
+__device__ __forceinline__ F4 operator+(F4 a, F4 b) { return F4{a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w}; }
+__device__ __forceinline__ F4 operator-(F4 a, F4 b) { return F4{a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w}; }
+
+constexpr int kCvThreads = 256;
+constexpr int kCvLow = 7;  // qubits transformed by the emit / absorb stage
+
+// In place over the z bits of the `hi` high qubits: a CTA owns one x of them and a run of 4 * 2^rb
+// low elements (2^hi rows of that run in shared memory).  sign_in: apply s first, sign_out: last.
+__global__ void __launch_bounds__(kCvThreads) k_pauli_high(float *__restrict__ v, int hi, int low, int rb, int sign_in,
+                                                           int sign_out)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    F4 *sm = reinterpret_cast<F4 *>(smem);
+    const unsigned nrun = 1u << (2 * low - 2 - rb);  // runs of a row
+    const unsigned run = blockIdx.x % nrun, xa = blockIdx.x / nrun;
+    const uint64_t xo = p_spread(xa) << (2 * low + 1);
+    const unsigned rows = 1u << hi, nv = rows << rb, rmask = (1u << rb) - 1u;
+    auto at = [&](unsigned e) {
+        return xo + (p_spread(e >> rb) << (2 * low)) + 4ull * (((uint64_t)run << rb) + (e & rmask));
+    };
+    for (unsigned e = threadIdx.x; e < nv; e += kCvThreads) {
+        const uint64_t g = at(e);
+        F4 a = *reinterpret_cast<const F4 *>(v + g);
+        if (sign_in) p_signs4(a, g);
+        sm[e] = a;
+    }
+    __syncthreads();
+    for (int b = 0; b < hi; b += 3) {
+        const int nb = hi - b < 3 ? hi - b : 3;
+        const int sh = b + rb;
+        for (unsigned i = threadIdx.x; i < (nv >> nb); i += kCvThreads) {
+            const unsigned lo = i & ((1u << sh) - 1u), base = ((i >> sh) << (sh + nb)) | lo;
+            auto ld = [&](int j) { return sm[base + ((unsigned)j << sh)]; };
+            auto st = [&](int j, F4 x) { sm[base + ((unsigned)j << sh)] = x; };
+            if (nb == 3) p_wht<3, F4>(ld, st);
+            else if (nb == 2) p_wht<2, F4>(ld, st);
+            else p_wht<1, F4>(ld, st);
+        }
+        __syncthreads();
+    }
+    for (unsigned e = threadIdx.x; e < nv; e += kCvThreads) {
+        const uint64_t g = at(e);
+        F4 a = sm[e];
+        if (sign_out) p_signs4(a, g);
+        *reinterpret_cast<F4 *>(v + g) = a;
+    }
+}
+
+// Tile of the low stage: high qubits' labels (ra, ca) with ca <= ra (x = ra ^ ca), one value xh of
+// the x bits of low qubits above the four lowest; it holds, for the two rows ra and ca of the
+// transform, W over all z / r bits of the m low qubits and all x bits of the ml lowest.
+constexpr int kCvPitch = 17;                       // floats per r_L (16 x values + 1)
+constexpr int kCvArray = (1 << kCvLow) * kCvPitch;  // one of the two arrays
+
+struct CvTile {
+    unsigned ra, ca, xh;
+    int m, ml, mh, narr;
+    uint64_t off[2];  // element offset of the arrays' low part in v
+};
+
+__device__ __forceinline__ CvTile cv_tile(int n, unsigned blk)
+{
+    CvTile T;
+    T.m = n < kCvLow ? n : kCvLow;
+    T.ml = T.m < 4 ? T.m : 4;
+    T.mh = T.m - T.ml;
+    T.xh = blk & ((1u << T.mh) - 1u);
+    const unsigned long long p = blk >> T.mh;
+    unsigned long long c = (unsigned long long)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);
+    while ((c + 1) * (c + 2) / 2 <= p) c++;
+    while (c * (c + 1) / 2 > p) c--;
+    T.ra = (unsigned)c;
+    T.ca = (unsigned)(p - c * (c + 1) / 2);
+    T.narr = T.ra == T.ca ? 1 : 2;
+    const uint64_t x = p_spread(T.ra ^ T.ca) << 1;
+    T.off[0] = (x | p_spread(T.ra)) << (2 * T.m);
+    T.off[1] = (x | p_spread(T.ca)) << (2 * T.m);
+    return T;
+}
+
+// WHT over the z bits of the low qubits, both arrays.
+__device__ __forceinline__ void cv_transform(const CvTile &T, float *sm)
+{
+    for (int b = 0; b < T.m; b += 4) {
+        const int nb = T.m - b < 4 ? T.m - b : 4;
+        const unsigned per = 1u << (T.m - nb + T.ml);
+        for (unsigned i = threadIdx.x; i < per * (unsigned)T.narr; i += kCvThreads) {
+            const unsigned a = i >= per ? 1u : 0u, k = i - a * per;
+            const unsigned xl = k & ((1u << T.ml) - 1u), q = k >> T.ml;
+            const unsigned z0 = ((q >> b) << (b + nb)) | (q & ((1u << b) - 1u));
+            float *p = sm + a * kCvArray + z0 * kCvPitch + xl;
+            const unsigned stp = (unsigned)kCvPitch << b;
+            auto ld = [&](int j) { return p[j * stp]; };
+            auto st = [&](int j, float x) { p[j * stp] = x; };
+            if (nb == 4) p_wht<4, float>(ld, st);
+            else if (nb == 3) p_wht<3, float>(ld, st);
+            else if (nb == 2) p_wht<2, float>(ld, st);
+            else p_wht<1, float>(ld, st);
+        }
+        __syncthreads();
+    }
+}
+
+// Position in an array, and element offset in v's low part, of chunk k (4 elements: the labels of
+// the lowest qubit) of the tile's 2^mh runs of 4^ml elements.
+__device__ __forceinline__ void cv_chunk(const CvTile &T, unsigned k, unsigned &pos, uint64_t &off)
+{
+    const unsigned lowc = k & ((1u << (2 * T.ml - 2)) - 1u), zh = k >> (2 * T.ml - 2);
+    off = ((p_spread(zh) | (p_spread(T.xh) << 1)) << (2 * T.ml)) + 4u * lowc;
+    unsigned z = 0, x = 0;
+    for (int d = 0; d < T.ml - 1; d++) {
+        z |= ((lowc >> (2 * d)) & 1u) << (d + 1);
+        x |= ((lowc >> (2 * d + 1)) & 1u) << (d + 1);
+    }
+    pos = ((zh << T.ml) | z) * kCvPitch + x;  // labels (I, Z, X, Y): + (0, pitch, 1, pitch + 1)
+}
+
+__global__ void __launch_bounds__(kCvThreads) k_pauli_emit(const float *__restrict__ v, float2 *__restrict__ rho, int n,
+                                                           float scale, int sign)
+{
+    __shared__ float sm[2 * kCvArray];
+    const CvTile T = cv_tile(n, blockIdx.x);
+    const unsigned nch = 1u << (T.mh + 2 * T.ml - 2);
+    for (unsigned i = threadIdx.x; i < nch * (unsigned)T.narr; i += kCvThreads) {
+        const unsigned a = i >= nch ? 1u : 0u;
+        unsigned pos;
+        uint64_t off;
+        cv_chunk(T, i - a * nch, pos, off);
+        off += T.off[a];
+        float4 x = *reinterpret_cast<const float4 *>(v + off);
+        if (sign) p_signs4(x, off);
+        float *p = sm + a * kCvArray + pos;
+        p[0] = x.x, p[kCvPitch] = x.y, p[1] = x.z, p[kCvPitch + 1] = x.w;
+    }
+    __syncthreads();
+    cv_transform(T, sm);
+    const float *wa = sm, *wb = T.narr == 2 ? sm + kCvArray : sm;
+    const float h = 0.5f * scale;
+    const unsigned lmask = (1u << T.ml) - 1u, cols = 1u << T.ml, half = cols >> 1;
+    const uint64_t dim = 1ull << n;
+    // block (ra, ca), then its mirror (ca, ra): rows in turn, two columns per thread
+    for (int blkm = 0; blkm < T.narr; blkm++) {
+        const uint64_t rowb = (uint64_t)(blkm ? T.ca : T.ra) << T.m, colb = (uint64_t)(blkm ? T.ra : T.ca) << T.m;
+        for (unsigned i = threadIdx.x; i < (half << T.m); i += kCvThreads) {
+            const unsigned row = i / half, c0 = 2 * (i % half);
+            const unsigned colh = ((row >> T.ml) ^ T.xh) << T.ml;
+            float o[4];
+#pragma unroll
+            for (int j = 0; j < 2; j++) {
+                const unsigned col = colh | (c0 + j), xl = (row ^ col) & lmask;
+                const unsigned r = blkm ? col : row, c = blkm ? row : col;
+                const float A = wa[r * kCvPitch + xl], B = wb[c * kCvPitch + xl];
+                o[2 * j] = h * (A + B);
+                o[2 * j + 1] = blkm ? h * (B - A) : h * (A - B);
+            }
+            *reinterpret_cast<float4 *>(rho + (rowb + row) * dim + colb + colh + c0) = make_float4(o[0], o[1], o[2], o[3]);
+        }
+    }
+}
+
+// The lower triangle of rho (r >= c; the diagonal's real part) -> W, transformed over the low qubits.
+__global__ void __launch_bounds__(kCvThreads) k_pauli_absorb(const float2 *__restrict__ rho, float *__restrict__ v, int n,
+                                                             int sign)
+{
+    __shared__ float sm[2 * kCvArray];
+    const CvTile T = cv_tile(n, blockIdx.x);
+    const unsigned lmask = (1u << T.ml) - 1u, cols = 1u << T.ml, half = cols >> 1;
+    const uint64_t dim = 1ull << n;
+    const uint64_t rowb = (uint64_t)T.ra << T.m, colb = (uint64_t)T.ca << T.m;
+    float *wa = sm, *wb = T.narr == 2 ? sm + kCvArray : sm;
+    for (unsigned i = threadIdx.x; i < (half << T.m); i += kCvThreads) {
+        const unsigned row = i / half, c0 = 2 * (i % half);
+        const unsigned colh = ((row >> T.ml) ^ T.xh) << T.ml;
+        if (T.narr == 1 && row < (colh | c0)) continue;
+        const float4 x = *reinterpret_cast<const float4 *>(rho + (rowb + row) * dim + colb + colh + c0);
+#pragma unroll
+        for (int j = 0; j < 2; j++) {
+            const unsigned col = colh | (c0 + j), xl = (row ^ col) & lmask;
+            const float re = j ? x.z : x.x, im = j ? x.w : x.y;
+            if (T.narr == 1 && row < col) continue;
+            if (T.narr == 1 && row == col) {
+                wa[row * kCvPitch + xl] = re;
+            } else {
+                wa[row * kCvPitch + xl] = re + im;
+                wb[col * kCvPitch + xl] = re - im;
+            }
+        }
+    }
+    __syncthreads();
+    cv_transform(T, sm);
+    const unsigned nch = 1u << (T.mh + 2 * T.ml - 2);
+    for (unsigned i = threadIdx.x; i < nch * (unsigned)T.narr; i += kCvThreads) {
+        const unsigned a = i >= nch ? 1u : 0u;
+        unsigned pos;
+        uint64_t off;
+        cv_chunk(T, i - a * nch, pos, off);
+        off += T.off[a];
+        const float *p = sm + a * kCvArray + pos;
+        float4 x = make_float4(p[0], p[kCvPitch], p[1], p[kCvPitch + 1]);
+        if (sign) p_signs4(x, off);
+        *reinterpret_cast<float4 *>(v + off) = x;
+    }
+}
+
+static cudaError_t launch_high(float *v, int n, int sign_in, int sign_out, cudaStream_t s)
+{
+    const int hi = n - kCvLow, low = kCvLow;
+    const int rb = std::max(2, std::min(4, 11 - hi));  // runs of 64 floats, 16 for the widest registers
+    const size_t sm = sizeof(F4) << (hi + rb);
+    if (ensure_smem_attr(reinterpret_cast<const void *>(k_pauli_high), sm)) return cudaErrorInvalidValue;
+    const unsigned blocks = 1u << (hi + 2 * low - 2 - rb);
+    k_pauli_high<<<blocks, kCvThreads, sm, s>>>(v, hi, low, rb, sign_in, sign_out);
+    return cudaGetLastError();
+}
+
+static unsigned cv_blocks(int n)
+{
+    const int m = std::min(n, kCvLow), mh = m - std::min(m, 4);
+    const unsigned long long M = 1ull << (n - m);
+    return (unsigned)((M * (M + 1) / 2) << mh);
+}
+
+int pauli_convert_launches(int n) { return n > kCvLow ? 2 : 1; }
+
+// rho <- v (v is used up: the high stage works in place).  n >= 3.
+cudaError_t launch_pauli_to_rho(float *v, float2 *rho, int n, cudaStream_t s)
+{
+    if (n > kCvLow) {
+        const cudaError_t e = launch_high(v, n, 1, 0, s);
+        if (e != cudaSuccess) return e;
+    }
+    float scale = 1.f;
+    for (int i = 0; i < n; i++) scale *= 0.5f;
+    k_pauli_emit<<<cv_blocks(n), kCvThreads, 0, s>>>(v, rho, n, scale, n > kCvLow ? 0 : 1);
+    return cudaGetLastError();
+}
+
+// v <- rho, from its lower triangle.
+cudaError_t launch_rho_to_pauli(const float2 *rho, float *v, int n, cudaStream_t s)
+{
+    k_pauli_absorb<<<cv_blocks(n), kCvThreads, 0, s>>>(rho, v, n, n > kCvLow ? 0 : 1);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || n <= kCvLow) return e;
+    return launch_high(v, n, 0, 1, s);
+}
+
+// ------------------------------------------------------------------ readouts
+__global__ void k_pauli_zero(float4 *__restrict__ v, uint64_t nchunk)
+{
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < nchunk; i += (uint64_t)gridDim.x * blockDim.x)
+        v[i] = (i & 0xAAAAAAAAAAAAAAAAull) == 0 ? make_float4(1.f, 1.f, 0.f, 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+cudaError_t launch_pauli_zero(float *v, int n, int nsm, cudaStream_t s)
+{
+    const uint64_t nchunk = 1ull << (2 * n - 2);
+    const uint64_t g = (nchunk + 255) / 256, cap = (uint64_t)nsm * 32;
+    k_pauli_zero<<<(unsigned)(g < cap ? g : cap), 256, 0, s>>>(reinterpret_cast<float4 *>(v), nchunk);
+    return cudaGetLastError();
+}
+
+// out[0], out[1] = trace; out[2 + q] = P(qubit q = 1) = (v_I - v_{Z_q}) / 2.
+__global__ void k_pauli_diag(const float *__restrict__ v, int n, double *__restrict__ out)
+{
+    const int q = threadIdx.x;
+    const double v0 = v[0];
+    if (q == 0) out[0] = v0, out[1] = 0.0;
+    if (q < n) out[2 + q] = 0.5 * (v0 - (double)v[1ull << (2 * (n - 1 - q))]);
+}
+
+void launch_pauli_diag(const float *v, int n, double *out, cudaStream_t s) { k_pauli_diag<<<1, 32, 0, s>>>(v, n, out); }
+
+// out[s] = Tr[P_s rho]: the string's own coefficient.
+__global__ void k_pauli_terms(const float *__restrict__ v, const __grid_constant__ PauliTerms T, double *__restrict__ out)
+{
+    const int s = threadIdx.x;
+    if (s < T.count) out[s] = v[(p_spread(T.flip[s]) << 1) | p_spread(T.ym[s] | T.zm[s])];
+}
+
+void launch_pauli_terms(const float *v, const PauliTerms &T, double *out, cudaStream_t s)
+{
+    k_pauli_terms<<<1, 64, 0, s>>>(v, T, out);
+}
+
+// Projection on outcome m of a qubit, times scale: (I, Z, X, Y) -> ((I + s Z) / 2, s (I + s Z) / 2, 0, 0).
+__global__ void k_pauli_project(float *__restrict__ v, uint64_t items, int d, float sgn, float h)
+{
+    float4 *v4 = reinterpret_cast<float4 *>(v);
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < items; i += (uint64_t)gridDim.x * blockDim.x) {
+        if (d == 0) {
+            const float4 x = v4[i];
+            const float a = h * fmaf(sgn, x.y, x.x);
+            v4[i] = make_float4(a, sgn * a, 0.f, 0.f);
+        } else {
+            const int sh = 2 * (d - 1);
+            const uint64_t b = ((i >> sh) << (sh + 2)) | (i & ((1ull << sh) - 1)), st = 1ull << sh;
+            const float4 x = v4[b], z = v4[b + st];
+            const float4 a = make_float4(h * fmaf(sgn, z.x, x.x), h * fmaf(sgn, z.y, x.y), h * fmaf(sgn, z.z, x.z),
+                                         h * fmaf(sgn, z.w, x.w));
+            v4[b] = a;
+            v4[b + st] = make_float4(sgn * a.x, sgn * a.y, sgn * a.z, sgn * a.w);
+            v4[b + 2 * st] = zero;
+            v4[b + 3 * st] = zero;
+        }
+    }
+}
+
+void launch_pauli_project(float *v, int n, int qubit, int m, double scale, int nsm, cudaStream_t s)
+{
+    const int d = n - 1 - qubit;
+    const uint64_t items = d == 0 ? 1ull << (2 * n - 2) : 1ull << (2 * n - 4);
+    const uint64_t g = (items + 255) / 256, cap = (uint64_t)nsm * 32;
+    k_pauli_project<<<(unsigned)(g < cap ? g : cap), 256, 0, s>>>(v, items, d, m ? -1.f : 1.f, (float)(0.5 * scale));
+}
+
+// Purity 2^-n sum v^2: squares in FP32 over 16 elements, totals in FP64, fixed tree.
+constexpr int kPpThreads = 256;
+__global__ void __launch_bounds__(kPpThreads) k_pauli_purity(const float4 *__restrict__ v, uint64_t n4, double scale,
+                                                             double *__restrict__ part)
+{
+    double acc = 0;
+    const uint64_t stride = (uint64_t)gridDim.x * kPpThreads;
+    for (uint64_t i = blockIdx.x * (uint64_t)kPpThreads + threadIdx.x; i < n4; i += 4 * stride) {
+        float s = 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (i + u * stride < n4) {
+                const float4 a = v[i + u * stride];
+                s = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(a.z, a.z, fmaf(a.w, a.w, s))));
+            }
+        acc += (double)s;
+    }
+    __shared__ double sh[kPpThreads / 32];
+    acc = warp_sum(acc);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0;
+        for (int w = 0; w < kPpThreads / 32; w++) t += sh[w];
+        part[blockIdx.x] = t * scale;
+    }
+}
+
+void launch_pauli_purity(const float *v, int n, double *partials, double *out, int nblocks, cudaStream_t s)
+{
+    const uint64_t n4 = 1ull << (2 * n - 2), need = (n4 + 4 * kPpThreads - 1) / (4 * kPpThreads);
+    const int nb = (int)(need < (uint64_t)nblocks ? need : (uint64_t)nblocks);
+    double scale = 1.0;
+    for (int i = 0; i < n; i++) scale *= 0.5;
+    k_pauli_purity<<<nb, kPpThreads, 0, s>>>(reinterpret_cast<const float4 *>(v), n4, scale, partials);
+    launch_fold(partials, nb, out, s);
+}
+
+// Reduced state of the kept qubits (k <= 6): their strings' coefficients, changed to rho_A in FP64.
+__global__ void __launch_bounds__(256) k_pauli_ptrace(const float *__restrict__ v, PTParams p, double2 *__restrict__ out)
+{
+    __shared__ double w[4096];
+    const int k = p.nkeep;
+    const unsigned N = 1u << (2 * k), dim = 1u << k;
+    for (unsigned e = threadIdx.x; e < N; e += 256) {  // e = x * dim + z
+        const unsigned x = e >> k, z = e & (dim - 1);
+        uint64_t idx = 0;
+        for (int j = 0; j < k; j++)
+            idx |= ((uint64_t)((x >> (k - 1 - j)) & 1u) << (2 * p.kpos[j] + 1)) |
+                   ((uint64_t)((z >> (k - 1 - j)) & 1u) << (2 * p.kpos[j]));
+        const int c = __popc(x & z);
+        w[e] = ((c + 1) & 2) ? -(double)v[idx] : (double)v[idx];
+    }
+    __syncthreads();
+    for (int b = 0; b < k; b++) {
+        for (unsigned i = threadIdx.x; i < N / 2; i += 256) {
+            const unsigned e = ((i >> b) << (b + 1)) | (i & ((1u << b) - 1u));
+            const double a = w[e], c = w[e | (1u << b)];
+            w[e] = a + c;
+            w[e | (1u << b)] = a - c;
+        }
+        __syncthreads();
+    }
+    const double h = 0.5 / (double)dim;
+    for (unsigned e = threadIdx.x; e < N; e += 256) {
+        const unsigned r = e >> k, c = e & (dim - 1), x = r ^ c;
+        const double a = w[x * dim + r], b = w[x * dim + c];
+        out[e] = make_double2(h * (a + b), h * (a - b));
+    }
+}
+
+void launch_pauli_ptrace(const float *v, const PTParams &p, double2 *out, cudaStream_t s)
+{
+    k_pauli_ptrace<<<1, 256, 0, s>>>(v, p, out);
+}
+
+}  // namespace qcw

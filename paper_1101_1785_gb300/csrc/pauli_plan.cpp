@@ -1,0 +1,515 @@
+// Planner of the Pauli-basis path: operations -> merged nodes -> passes -> rounds.
+//
+// Nodes.  Every one-qubit operation is multiplied into the map that follows the last two-qubit
+// operation on its qubit (they commute past everything else), so between two two-qubit operations
+// a qubit has exactly one real 4 x 4 map.  CNOT and CZ nodes carry the maps of their two qubits
+// that follow; any other two-qubit operation is a dense 16 x 16 node into which such maps, and a
+// directly following two-qubit operation on the same pair, are multiplied.
+#include "pauli.h"
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
+#include "tile.h"
+
+namespace qcw {
+
+namespace {
+
+// label of member index 2 r + c of pauli_transfer's basis (I, X, Y, Z)
+const int kLab[4] = {0, 2, 3, 1};
+
+struct M4 {
+    double m[16];
+    bool id;
+};
+
+M4 m4_identity()
+{
+    M4 r{};
+    for (int i = 0; i < 4; i++) r.m[5 * i] = 1.0;
+    r.id = true;
+    return r;
+}
+
+// a <- b a
+void m4_lmul(M4 &a, const M4 &b)
+{
+    if (b.id) return;
+    if (a.id) {
+        a = b;
+        return;
+    }
+    M4 r;
+    for (int i = 0; i < 4; i++)
+        for (int j = 0; j < 4; j++) {
+            double s = 0;
+            for (int k = 0; k < 4; k++) s += b.m[4 * i + k] * a.m[4 * k + j];
+            r.m[4 * i + j] = s;
+        }
+    r.id = false;
+    a = r;
+}
+
+bool m4_tp(const M4 &a)  // first row (1, 0, 0, 0): keeps the trace
+{
+    return std::fabs(a.m[0] - 1.0) < 1e-12 && std::fabs(a.m[1]) < 1e-13 && std::fabs(a.m[2]) < 1e-13 &&
+           std::fabs(a.m[3]) < 1e-13;
+}
+
+M4 one_map(const QOp &op)
+{
+    c128 S[16];
+    if (op.kind != 0) {
+        for (int i = 0; i < 16; i++) S[i] = op.m[i];
+    } else {
+        const c128 *u = op.m.data();
+        for (int r2 = 0; r2 < 2; r2++)
+            for (int c2 = 0; c2 < 2; c2++)
+                for (int r = 0; r < 2; r++)
+                    for (int c = 0; c < 2; c++)
+                        S[(2 * r2 + c2) * 4 + 2 * r + c] = u[2 * r2 + r] * std::conj(u[2 * c2 + c]);
+    }
+    double R[4][4];
+    pauli_transfer1(S, R);
+    M4 t;
+    t.id = false;
+    for (int i = 0; i < 4; i++)
+        for (int j = 0; j < 4; j++) t.m[4 * kLab[i] + kLab[j]] = 2.0 * R[i][j];
+    return t;
+}
+
+// Real 16 x 16 map of a two-qubit operation, index 4 p_first + p_second.
+void two_map(const QOp &op, double *T)
+{
+    std::vector<c128> S(256);
+    if (op.kind != 0) {
+        for (int i = 0; i < 256; i++) S[i] = op.m[i];
+    } else {
+        const c128 *u = op.m.data();
+        for (int r2 = 0; r2 < 4; r2++)
+            for (int c2 = 0; c2 < 4; c2++)
+                for (int r = 0; r < 4; r++)
+                    for (int c = 0; c < 4; c++)
+                        S[(size_t)(r2 * 4 + c2) * 16 + r * 4 + c] = u[r2 * 4 + r] * std::conj(u[c2 * 4 + c]);
+    }
+    double R[16][16];
+    pauli_transfer(S, R);
+    auto lab = [](int e) {  // member 8 r_a + 4 r_b + 2 c_a + c_b
+        const int a = 2 * ((e >> 3) & 1) + ((e >> 1) & 1), b = 2 * ((e >> 2) & 1) + (e & 1);
+        return 4 * kLab[a] + kLab[b];
+    };
+    // pauli_transfer's basis has D = -i Y per qubit with i where their number is odd, so its
+    // member with two D is -(Y Y)
+    auto sg = [](int e) { return (e & 12) == 12 && (e & 3) == 0 ? -1.0 : 1.0; };
+    for (int i = 0; i < 16; i++)
+        for (int j = 0; j < 16; j++) T[16 * lab(i) + lab(j)] = 4.0 * R[i][j] * sg(i) * sg(j);
+}
+
+struct Node {
+    int kind;   // PO_ONE, PO_CX, PO_CZ, PO_TWO
+    int a, b;   // qubits (b = -1 for PO_ONE); PO_CX: a controls
+    M4 A, B;    // maps that follow on a and b (PO_ONE: A is the map)
+    std::vector<double> T;  // PO_TWO
+};
+
+// Image of label pair (pa, pb) under the conjugation by CNOT (a controls) or CZ, and its sign.
+int conj_label(bool cz, int e, double *sgn)
+{
+    int xa = (e >> 3) & 1, za = (e >> 2) & 1, xb = (e >> 1) & 1, zb = e & 1;
+    if (!cz) {
+        *sgn = (xa & zb & (xb ^ za ^ 1)) ? -1.0 : 1.0;
+        xb ^= xa;
+        za ^= zb;
+    } else {
+        *sgn = (xa & xb & (za ^ zb)) ? -1.0 : 1.0;
+        za ^= xb;
+        zb ^= xa;
+    }
+    return 8 * xa + 4 * za + 2 * xb + zb;
+}
+
+// T <- (A (x) B) T
+void kron_lmul(std::vector<double> &T, const M4 &A, const M4 &B)
+{
+    if (A.id && B.id) return;
+    std::vector<double> R(256, 0.0);
+    for (int ia = 0; ia < 4; ia++)
+        for (int ib = 0; ib < 4; ib++)
+            for (int ka = 0; ka < 4; ka++)
+                for (int kb = 0; kb < 4; kb++) {
+                    const double w = A.m[4 * ia + ka] * B.m[4 * ib + kb];
+                    if (w == 0) continue;
+                    for (int j = 0; j < 16; j++) R[16 * (4 * ia + ib) + j] += w * T[16 * (4 * ka + kb) + j];
+                }
+    T.swap(R);
+}
+
+std::vector<double> node_matrix(const Node &nd)  // its two-qubit operation and following maps
+{
+    std::vector<double> T(256, 0.0);
+    if (nd.kind == PO_TWO) T = nd.T;
+    else
+        for (int e = 0; e < 16; e++) {
+            double s;
+            const int f = conj_label(nd.kind == PO_CZ, e, &s);
+            T[16 * e + f] = s;
+        }
+    kron_lmul(T, nd.A, nd.B);
+    return T;
+}
+
+// The same map with the two qubits exchanged.
+std::vector<double> exchanged(const std::vector<double> &T)
+{
+    std::vector<double> R(256);
+    auto x = [](int e) { return 4 * (e & 3) + (e >> 2); };
+    for (int i = 0; i < 16; i++)
+        for (int j = 0; j < 16; j++) R[16 * x(i) + x(j)] = T[16 * i + j];
+    return R;
+}
+
+std::vector<double> matmul16(const std::vector<double> &A, const std::vector<double> &B)
+{
+    std::vector<double> R(256, 0.0);
+    for (int i = 0; i < 16; i++)
+        for (int k = 0; k < 16; k++) {
+            const double w = A[16 * i + k];
+            if (w == 0) continue;
+            for (int j = 0; j < 16; j++) R[16 * i + j] += w * B[16 * k + j];
+        }
+    return R;
+}
+
+// Exactly CNOT (*a, *b in order control, target) or CZ.
+int classify(const QOp &op, int *a, int *b)
+{
+    *a = op.qubits[0];
+    *b = op.qubits[1];
+    if (op.kind != 0) return PO_TWO;
+    const c128 *u = op.m.data();
+    auto is = [&](const int *col, const double *val) {
+        for (int i = 0; i < 4; i++)
+            for (int j = 0; j < 4; j++)
+                if (u[4 * i + j] != (j == col[i] ? c128(val[i], 0) : c128(0, 0))) return false;
+        return true;
+    };
+    const double one[4] = {1, 1, 1, 1}, cz[4] = {1, 1, 1, -1};
+    const int id[4] = {0, 1, 2, 3}, cx[4] = {0, 1, 3, 2}, xc[4] = {0, 3, 2, 1};
+    if (is(cx, one)) return PO_CX;
+    if (is(xc, one)) {
+        std::swap(*a, *b);
+        return PO_CX;
+    }
+    return is(id, cz) ? PO_CZ : PO_TWO;
+}
+
+// FP32 rounding of a map's coefficients with feedback.  A channel repeated after every gate (a
+// depolarising factor 1 - 4 p / 3, say) rounds the same way each time, so the coefficients it
+// shrinks would drift by up to 3e-8 per application, all in one direction.  c: the scale error the
+// qubit's maps have collected so far; the next map's linear part is scaled by 1 - c before it is
+// rounded, and c becomes what its own rounding adds, so the sum stays within one rounding.
+void round_map(M4 &a, double &c)
+{
+    if (a.id) return;
+    double num = 0, den = 0;
+    for (int i = 1; i < 4; i++)
+        for (int j = 1; j < 4; j++) {
+            double &x = a.m[4 * i + j];
+            const double f = (double)(float)(x * (1.0 - c));
+            num += f * x;
+            den += x * x;
+            x = f;
+        }
+    if (den > 0) c += num / den - 1.0;
+}
+
+std::vector<Node> make_nodes(const std::vector<QOp> &ops, size_t begin, size_t end, int n)
+{
+    std::vector<Node> out;
+    std::vector<int> last(n, -1);
+    std::vector<M4> pre(n, m4_identity());
+    for (size_t i = begin; i < end; i++) {
+        const QOp &op = ops[i];
+        if (op.k == 1) {
+            const int q = op.qubits[0];
+            const M4 m = one_map(op);
+            if (last[q] < 0) m4_lmul(pre[q], m);
+            else m4_lmul(out[last[q]].a == q ? out[last[q]].A : out[last[q]].B, m);
+            continue;
+        }
+        int a, b;
+        const int kind = classify(op, &a, &b);
+        const bool same = last[a] >= 0 && last[a] == last[b];
+        if (same && (kind == PO_TWO || out[last[a]].kind == PO_TWO)) {  // one dense map for both
+            Node &nd = out[last[a]];
+            Node nw{kind, a, b, m4_identity(), m4_identity(), {}};
+            if (kind == PO_TWO) {
+                nw.T.resize(256);
+                two_map(op, nw.T.data());
+            }
+            std::vector<double> T2 = node_matrix(nw);
+            if (nd.a != a) T2 = exchanged(T2);
+            nd.T = matmul16(T2, node_matrix(nd));
+            nd.kind = PO_TWO;
+            nd.A = nd.B = m4_identity();
+            continue;
+        }
+        Node nd{kind, a, b, m4_identity(), m4_identity(), {}};
+        if (kind == PO_TWO) {
+            nd.T.resize(256);
+            two_map(op, nd.T.data());
+            if (!pre[a].id || !pre[b].id) {
+                std::vector<double> P(256, 0.0);
+                for (int e = 0; e < 16; e++) P[17 * e] = 1.0;
+                kron_lmul(P, pre[a], pre[b]);
+                nd.T = matmul16(nd.T, P);
+            }
+        } else {
+            for (int q : {a, b})
+                if (!pre[q].id) out.push_back(Node{PO_ONE, q, -1, pre[q], m4_identity(), {}});
+        }
+        pre[a] = pre[b] = m4_identity();
+        last[a] = last[b] = (int)out.size();
+        out.push_back(std::move(nd));
+    }
+    std::vector<Node> fin;
+    for (int q = 0; q < n; q++)
+        if (!pre[q].id) fin.push_back(Node{PO_ONE, q, -1, pre[q], m4_identity(), {}});
+    for (Node &nd : out) {
+        if (nd.kind == PO_TWO) {
+            nd.T = node_matrix(nd);
+            nd.A = nd.B = m4_identity();
+            fin.push_back(std::move(nd));
+        } else if (nd.kind == PO_ONE) {
+            fin.push_back(std::move(nd));
+        } else {
+            // maps that do not keep the trace follow as general one-qubit maps
+            const Node g = nd;
+            if (!m4_tp(nd.A)) nd.A = m4_identity();
+            if (!m4_tp(nd.B)) nd.B = m4_identity();
+            fin.push_back(std::move(nd));
+            if (!m4_tp(g.A)) fin.push_back(Node{PO_ONE, g.a, -1, g.A, m4_identity(), {}});
+            if (!m4_tp(g.B)) fin.push_back(Node{PO_ONE, g.b, -1, g.B, m4_identity(), {}});
+        }
+    }
+    std::vector<double> err(n, 0.0);
+    for (Node &nd : fin) {
+        if (nd.kind == PO_TWO) continue;
+        round_map(nd.A, err[nd.a]);
+        if (nd.b >= 0) round_map(nd.B, err[nd.b]);
+    }
+    return fin;
+}
+
+std::vector<unsigned> pass_candidates(int nd, int t, int kmax)
+{
+    std::vector<unsigned> out;
+    const unsigned all = (1u << nd) - 1u;
+    const int k = kmax ? std::min(kmax, t) : t;
+    const unsigned low = 3u;  // the two lowest digits are in every tile
+    for (unsigned s = 0; s <= all; s++) {
+        if (__builtin_popcount(s) != k) continue;
+        if (!kmax && (s & low) != low) continue;
+        if (kmax && __builtin_popcount(s | low) > t) continue;
+        out.push_back(s);
+    }
+    return out;
+}
+
+// Positions of the round: the group-index bits go to the chunk-index bits outside digits db and dc,
+// the first three to bits with independent contributions to the bank position (see pauli_swz).
+void round_positions(int t, PRound &r)
+{
+    std::vector<int> order;
+    bool taken[12] = {};
+    unsigned basis[3];
+    int nb = 0;
+    auto inside = [&](int bit) { return bit / 2 + 1 == r.db || bit / 2 + 1 == r.dc; };
+    for (int bit = 0; bit < 2 * (t - 1) && nb < 3; bit++) {
+        if (inside(bit)) continue;
+        unsigned v = pauli_swz(1u << bit) & 7u;
+        for (int i = 0; i < nb; i++) v = std::min(v, v ^ basis[i]);
+        if (!v) continue;
+        basis[nb++] = v;
+        order.push_back(bit);
+        taken[bit] = true;
+    }
+    for (int bit = 0; bit < 2 * (t - 1); bit++)
+        if (!inside(bit) && !taken[bit]) order.push_back(bit);
+    r.nob = (uint8_t)order.size();
+    auto at = [&](int bit) { return (uint16_t)(16u * pauli_swz(1u << bit)); };
+    for (unsigned g = 0; g < 16; g++)
+        for (int i = 0; i < 4; i++) {
+            if (!((g >> i) & 1u)) continue;
+            if (i < (int)order.size()) r.lo[g] ^= at(order[i]);
+            if (4 + i < (int)order.size()) r.hi[g] ^= at(order[4 + i]);
+        }
+    uint16_t *m = r.st;
+    m[0] = at(2 * (r.db - 1)), m[1] = at(2 * (r.db - 1) + 1);
+    m[2] = at(2 * (r.dc - 1)), m[3] = at(2 * (r.dc - 1) + 1);
+    for (int i = 0; i < 4; i++) r.ld[i] = m[i];
+    // the label pair that moves to (p_b, p_c): x_t ^= x_c, z_c ^= z_t (CNOT); z ^= the other x (CZ)
+    if (r.perm == PP_CX_BC) r.ld[1] ^= m[3], r.ld[2] ^= m[0];
+    if (r.perm == PP_CX_CB) r.ld[3] ^= m[1], r.ld[0] ^= m[2];
+    if (r.perm == PP_CZ) r.ld[1] ^= m[2], r.ld[3] ^= m[0];
+}
+
+void push_tp(std::vector<float> &c, const M4 &m)  // rows 1..3
+{
+    for (int i = 4; i < 16; i++) c.push_back((float)m.m[i]);
+}
+
+int node_coefs(const Node &nd) { return nd.kind == PO_TWO ? 256 : nd.kind == PO_ONE ? 16 : 24; }
+
+// Append node nd to a pass; dig(q) = 0, 1, 2: the register digit of its qubits.  maps_only: its
+// permutation is the round's own.
+template <typename F>
+void emit(PPass &ps, const Node &nd, bool maps_only, F dig)
+{
+    POp op{};
+    op.coef = (uint16_t)(ps.coefs.size() / 4);
+    const int da = dig(nd.a), db = nd.b >= 0 ? dig(nd.b) : -1;
+    if (maps_only) {
+        op.kind = PO_MM;
+        push_tp(ps.coefs, da == 1 ? nd.A : nd.B);
+        push_tp(ps.coefs, da == 1 ? nd.B : nd.A);
+    } else if (nd.kind == PO_ONE) {
+        op.kind = (uint16_t)(PO_ONE + da);
+        for (int i = 0; i < 16; i++) ps.coefs.push_back((float)nd.A.m[i]);
+    } else if (nd.kind == PO_CX) {
+        op.kind = (uint16_t)(PO_CX + 2 * da + (db > da ? db - 1 : db));
+        push_tp(ps.coefs, nd.A);
+        push_tp(ps.coefs, nd.B);
+    } else if (nd.kind == PO_CZ) {
+        const int lo = std::min(da, db), hi = std::max(da, db);
+        op.kind = (uint16_t)(PO_CZ + lo + hi - 1);  // (0,1) (0,2) (1,2)
+        push_tp(ps.coefs, da < db ? nd.A : nd.B);
+        push_tp(ps.coefs, da < db ? nd.B : nd.A);
+    } else {
+        const int lo = std::min(da, db), hi = std::max(da, db);
+        op.kind = (uint16_t)(PO_TWO + lo + hi - 1);  // (1,0) (2,0) (2,1)
+        const std::vector<double> T = da > db ? nd.T : exchanged(nd.T);
+        for (double x : T) ps.coefs.push_back((float)x);
+    }
+    ps.ops.push_back(op);
+}
+
+}  // namespace
+
+PauliPlan plan_pauli(const std::vector<QOp> &ops, size_t begin, size_t end, int n, int kmax, bool beam)
+{
+    PauliPlan plan;
+    plan.n = n;
+    plan.nd = std::max(n, kPMinDigits);
+    const int nd = plan.nd, t = std::min(nd, kPTile);
+    std::vector<Node> nodes = make_nodes(ops, begin, end, n);
+    auto digit = [&](int q) { return n - 1 - q; };
+    std::vector<unsigned> mask(nodes.size());
+    for (size_t i = 0; i < nodes.size(); i++) {
+        mask[i] = 1u << digit(nodes[i].a);
+        if (nodes[i].b >= 0) mask[i] |= 1u << digit(nodes[i].b), plan.nnode2++;
+    }
+    const bool whole = nd <= t && !kmax;
+    std::vector<unsigned> cand;
+    if (whole) cand.push_back((1u << nd) - 1u);
+    else cand = pass_candidates(nd, t, kmax);
+    std::vector<unsigned> seq;
+    if (beam && cand.size() > 1) seq = beam_pass_sets(mask, cand);
+    std::vector<size_t> rem(nodes.size());
+    for (size_t i = 0; i < rem.size(); i++) rem[i] = i;
+    size_t nseq = 0;
+    while (!rem.empty()) {
+        std::vector<unsigned> rm;
+        for (size_t i : rem) rm.push_back(mask[i]);
+        unsigned Q = 0;
+        if (nseq < seq.size()) {
+            Q = seq[nseq++];
+        } else {
+            size_t best = 0;
+            for (unsigned C : cand) {
+                const size_t a = cand.size() == 1 ? 1 : absorbable(rm, C);
+                if (a > best) best = a, Q = C;
+            }
+        }
+        // the tile: Q, the two lowest digits, then the lowest others
+        unsigned T = Q | 3u;
+        for (int d = 0; d < nd && __builtin_popcount(T) < t; d++) T |= 1u << d;
+        PPass ps;
+        ps.t = t;
+        int tile_of[32];
+        for (int d = 0; d < nd; d++) {
+            tile_of[d] = -1;
+            if (T & (1u << d)) tile_of[d] = (int)ps.td.size(), ps.td.push_back(d);
+            else ps.od.push_back(d);
+        }
+        std::vector<size_t> chosen, rest;
+        unsigned blocked = 0;
+        size_t ncoef = 0;
+        for (size_t j = 0; j < rem.size(); j++) {
+            const int nc = node_coefs(nodes[rem[j]]);
+            if ((rm[j] & ~Q) || (rm[j] & blocked) || ncoef + nc > (size_t)kPMaxCoef || (int)chosen.size() >= kPMaxRounds) {
+                rest.push_back(rem[j]);
+                blocked |= rm[j];
+            } else {
+                chosen.push_back(rem[j]);
+                ncoef += nc;
+            }
+        }
+        // rounds: of all pairs of tile digits beside digit 0, the one that takes most of what is left
+        auto tmask = [&](size_t i) {
+            unsigned m = 1u << tile_of[digit(nodes[i].a)];
+            if (nodes[i].b >= 0) m |= 1u << tile_of[digit(nodes[i].b)];
+            return m;
+        };
+        while (!chosen.empty()) {
+            std::vector<unsigned> cm;
+            for (size_t i : chosen) cm.push_back(tmask(i));
+            PRound r{};
+            size_t best = 0;
+            for (int b = 1; b < t; b++)
+                for (int c = b + 1; c < t; c++) {
+                    const size_t a = absorbable(cm, 1u | (1u << b) | (1u << c));
+                    if (a > best) best = a, r.db = (uint8_t)b, r.dc = (uint8_t)c;
+                }
+            const unsigned R = 1u | (1u << r.db) | (1u << r.dc);
+            r.op0 = (uint16_t)ps.ops.size();
+            std::vector<size_t> left, take;
+            unsigned bl = 0;
+            for (size_t j = 0; j < chosen.size(); j++) {
+                if ((cm[j] & ~R) || (cm[j] & bl)) {
+                    left.push_back(chosen[j]);
+                    bl |= cm[j];
+                } else {
+                    take.push_back(chosen[j]);
+                }
+            }
+            // a CNOT / CZ of db and dc that nothing but digit-0 maps precede starts the round
+            for (size_t j = 0; j < take.size(); j++) {
+                const Node &nd2 = nodes[take[j]];
+                const unsigned m = tmask(take[j]);
+                if (m == 1u) continue;
+                if (!(m & 1u) && (nd2.kind == PO_CX || nd2.kind == PO_CZ)) {
+                    r.perm = nd2.kind == PO_CZ ? PP_CZ : tile_of[digit(nd2.a)] == r.db ? PP_CX_BC : PP_CX_CB;
+                    std::rotate(take.begin(), take.begin() + j, take.begin() + j + 1);
+                }
+                break;
+            }
+            round_positions(t, r);
+            for (size_t j = 0; j < take.size(); j++)
+                emit(ps, nodes[take[j]], j == 0 && r.perm, [&](int q) {
+                    const int d = tile_of[digit(q)];
+                    return d == 0 ? 0 : d == r.db ? 1 : 2;
+                });
+            r.nop = (uint8_t)(ps.ops.size() - r.op0);
+            ps.rounds.push_back(r);
+            chosen.swap(left);
+        }
+        plan.passes.push_back(std::move(ps));
+        rem.swap(rest);
+    }
+    return plan;
+}
+
+}  // namespace qcw

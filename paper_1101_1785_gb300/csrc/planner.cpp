@@ -166,7 +166,7 @@ static std::vector<unsigned> subsets_of_size(int n, int k)
 
 // Operations of rem a pass on qubit set Q can take: an operation joins when its qubits lie in Q
 // and no skipped earlier operation shares a qubit with it (they commute past the skipped ones).
-static size_t absorbable(const std::vector<unsigned> &masks, unsigned Q)
+size_t absorbable(const std::vector<unsigned> &masks, unsigned Q)
 {
     unsigned blocked = 0;
     size_t taken = 0;
@@ -184,7 +184,7 @@ static size_t absorbable(const std::vector<unsigned> &masks, unsigned Q)
 constexpr int kBeamWidth = 64;
 constexpr int kBeamBranch = 12;
 
-static std::vector<unsigned> beam_pass_sets(const std::vector<unsigned> &masks, const std::vector<unsigned> &cand)
+std::vector<unsigned> beam_pass_sets(const std::vector<unsigned> &masks, const std::vector<unsigned> &cand)
 {
     struct Node {
         std::vector<unsigned> rem;

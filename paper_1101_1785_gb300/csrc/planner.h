@@ -39,4 +39,9 @@ enum class PassSearch { ORDER, BEST, BEAM };
 std::vector<PassPlan> plan_passes(const std::vector<QOp> &ops, size_t begin, size_t end, int n, int kmax,
                                   bool count_only = false, PassSearch search = PassSearch::ORDER);
 
+// Operations of rem (their qubit masks, in order) that a pass on the qubit set Q can take.
+size_t absorbable(const std::vector<unsigned> &masks, unsigned Q);
+// The pass sets the beam search finds for operations with these masks, out of cand.
+std::vector<unsigned> beam_pass_sets(const std::vector<unsigned> &masks, const std::vector<unsigned> &cand);
+
 }  // namespace qcw

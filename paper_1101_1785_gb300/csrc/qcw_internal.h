@@ -157,6 +157,13 @@ struct qcw_ctx {
     // half storage: only the lower triangle (r >= c) of rho is current (the warp-specialised
     // pass leaves it so); ensure_full completes the matrix before anything else reads it
     bool half = false;
+    // Pauli storage (pauli.h): pv holds v_P = Tr[P rho] and rho is stale while in_pauli; pzero: the
+    // state is |0..0><0..0| and neither buffer has been written yet (the first pass starts from it).
+    // pv is allocated on first use and kept; pauli_off: it could not be allocated.
+    float *pv = nullptr;
+    bool in_pauli = false;
+    bool pzero = false;
+    bool pauli_off = false;
     // Version of rho: bumped by everything that changes it.  The last fused pass of a flush
     // also sums |rho_rc|^2 over what it writes (per-CTA partials in the fused runtime);
     // purity_ver records the version those partials describe.
@@ -194,6 +201,10 @@ void fused_destroy(qcw_ctx *ctx);
 void fused_collect_timing(qcw_ctx *ctx);
 qcw_status plain_apply(qcw_ctx *c, const QOp &op);
 qcw_status ensure_full(qcw_ctx *c);
+// Whether fused work of this context runs in the Pauli basis (allocates pv on first use).
+bool pauli_allowed(qcw_ctx *c);
+// in_pauli: make pv hold the state (a pending |0..0><0..0| is written).
+qcw_status pauli_settle(qcw_ctx *c);
 // rho is about to be overwritten from outside the queue: drop queued work, mark the storage
 // full, bump the state version and clear the error word.
 qcw_status begin_state_replace(qcw_ctx *c);

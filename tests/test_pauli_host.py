@@ -1,0 +1,114 @@
+"""CPU tests of the Pauli-basis planner: its passes, replayed on the Pauli coefficients of a
+random state the way the kernel walks them (tiles, rounds, swizzled positions), must give the
+coefficients of the oracle's state after the original operations."""
+
+import ctypes
+import itertools
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import oracle
+import workloads as wl
+from tests._helpers import haar_unitary, random_rho
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1101_1785_gb300", "csrc")
+PAULI = [np.eye(2), np.diag([1, -1]), np.array([[0, 1], [1, 0]]), np.array([[0, -1j], [1j, 0]])]  # label 2 x + z
+
+
+@pytest.fixture(scope="module")
+def shim(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("pauli") / "libpauli_shim.so")
+    src = [os.path.join(CSRC, f) for f in ("planner.cpp", "tile.cpp", "pauli_plan.cpp")]
+    src.append(os.path.join(os.path.dirname(os.path.abspath(__file__)), "cpp", "pauli_shim.cpp"))
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, "-I", os.path.join(ROOT, "include"),
+                    "-I", "/usr/local/cuda/include", "-o", out, *src], check=True)
+    return ctypes.CDLL(out)
+
+
+def coefficients(rho):
+    """Tr[P rho] for every string, index = base-4 digits with qubit n - 1 lowest (flattened)."""
+    n = rho.shape[0].bit_length() - 1
+    t = rho.reshape([2] * (2 * n))
+    for q in range(n):  # row axis of the first qubit left is 0, its column axis n - q; labels go last
+        t = np.moveaxis(t, [0, n - q], [0, 1])
+        t = np.stack([np.einsum("cr,rc...->...", p, t) for p in PAULI], axis=-1)
+    return np.ascontiguousarray(t.real.reshape(-1))
+
+
+def test_coefficient_helper():
+    rho = random_rho(np.random.default_rng(0), 3)
+    v = coefficients(rho)
+    for i, lab in enumerate(itertools.product(range(4), repeat=3)):
+        p = np.kron(np.kron(PAULI[lab[0]], PAULI[lab[1]]), PAULI[lab[2]])
+        assert abs(np.trace(p @ rho) - v[i]) < 1e-12
+
+
+def _replay(shim, n, ops, v, kmax, beam):
+    kind, k, qs, mats, off = [], [], [], [], []
+    pos = 0
+    for op in ops:
+        if op.kind == "gate":
+            m = op.mats[0]
+        else:
+            m = sum(np.kron(a, a.conj()) for a in op.mats)
+        kind.append(0 if op.kind == "gate" else 1)
+        k.append(len(op.qubits))
+        qs += (list(op.qubits) + [0])[:2]
+        off.append(pos)
+        mats.append(np.ascontiguousarray(m, dtype=np.complex128).ravel())
+        pos += mats[-1].size
+    I = lambda a: np.asarray(a, dtype=np.int32)
+    kind, k, qs, off = I(kind), I(k), I(qs), np.asarray(off, dtype=np.int64)
+    mats = np.concatenate(mats)
+    nr, bad = ctypes.c_int(), ctypes.c_int()
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    npass = shim.pauli_replay(n, kmax, int(beam), len(ops), p(kind), p(k), p(qs), p(mats), p(off), p(v),
+                              ctypes.byref(nr), ctypes.byref(bad))
+    assert npass > 0 and bad.value == 0
+    return npass
+
+
+def _two_qubit_ops(rng, n, count):
+    ops = []
+    for i in range(count):
+        a, b = (int(x) for x in rng.permutation(n)[:2])
+        kind = i % 5
+        if kind == 0:
+            ops.append(wl.Op("gate", (a, b), haar_unitary(rng, 4)[None]))
+        elif kind == 1:
+            ops.append(wl.Op("kraus", (a, b), np.stack([np.sqrt(w) * haar_unitary(rng, 4) for w in (0.6, 0.3)])))
+        elif kind == 2:
+            ops.append(wl.Op("gate", (a, b), wl.gate_matrix("CNOT")[None]))
+        elif kind == 3:
+            ops.append(wl.Op("gate", (a, b), wl.gate_matrix("CZ")[None]))
+        else:  # target before control in the list
+            x = wl.gate_matrix("CNOT")
+            s = wl.gate_matrix("SWAP")
+            ops.append(wl.Op("gate", (a, b), (s @ x @ s)[None]))
+        q = int(rng.integers(n))
+        ops.append(wl.Op("kraus", (q,), np.stack([np.sqrt(0.5) * haar_unitary(rng, 2), 0.4 * haar_unitary(rng, 2)])))
+        ops.append(wl.Op("gate", (q,), haar_unitary(rng, 2)[None]))
+    return ops
+
+
+@pytest.mark.parametrize("n,kmax,beam", [(3, 0, 0), (4, 2, 0), (5, 0, 0), (6, 5, 0), (7, 0, 0), (8, 0, 0), (8, 3, 1), (9, 0, 1)])
+@pytest.mark.parametrize("what", ["mixed", "haar70", "two"])
+def test_plan_replays_the_circuit(shim, n, kmax, beam, what):
+    rng = np.random.default_rng(100 * n + kmax)
+    if what == "two":
+        ops = _two_qubit_ops(rng, n, 25)
+    else:
+        ops = wl.random_circuit(n, 60, 17 * n + kmax, what, "adpd" if what == "mixed" else "dep").ops
+    rho = random_rho(rng, n)
+    v = coefficients(rho)
+    want = rho.copy()
+    for op in ops:
+        oracle.apply_op(want, op)
+    _replay(shim, n, ops, v, kmax, beam)
+    # FP32 coefficients of the composed maps: 2^-24 relative each, at most a few per operation kept
+    scale = np.linalg.norm(coefficients(want))
+    assert np.linalg.norm(v - coefficients(want)) <= len(ops) * 2.0 ** -24 * scale
