@@ -185,8 +185,9 @@ QCW_API qcw_status qcw_apply_gate(qcw_ctx *ctx, const double *u, const int *qubi
  * Sec. 5.2.2, Eq. rhoE2) for nkraus (1..QCW_MAX_KRAUS) operators of k (1..QCW_MAX_GATE_QUBITS) qubits,
  * stored one after another (nkraus * 2 * 4^k doubles).  Trace-decreasing sets are accepted as
  * given.  One- and two-qubit channels act as composed superoperators (and join fused passes);
- * wider ones run term by term on the plain path with two scratch copies of rho, allocated on
- * first use and kept until the context is destroyed. */
+ * wider ones run as one pass over rho (all operators at once, on the plain path); many operators
+ * on a small register, or more than a launch carries (48, 12, 3 for k = 3, 4, 5), use scratch
+ * copies of rho, allocated on first use and kept until the context is destroyed. */
 QCW_API qcw_status qcw_apply_kraus(qcw_ctx *ctx, const double *kraus, int nkraus, const int *qubits,
                            int k);
 

@@ -254,8 +254,10 @@ qcw_status plain_gate2(qcw_ctx *c, const c128 *u, int q1, int q2, const int *ctr
     return QCW_OK;
 }
 
-// k-qubit dense gate as two passes: U on the row labels, then conj(U) on the column labels.
-qcw_status plain_gatek(qcw_ctx *c, const c128 *u, const int *qs, int k, float2 *target = nullptr)
+// Dense gate on three or four qubits as two passes: U on the row labels, then conj(U) on the column
+// labels.  Both are near the HBM bound (12 qubits: 2 x 36 us and 2 x 53 us); the one-pass kernel of
+// wide.cu, bound by its shared-memory trips, takes longer for a single operator up to k = 4.
+qcw_status plain_gatek(qcw_ctx *c, const c128 *u, const int *qs, int k)
 {
     const int n = c->n, m = 1 << k;
     for (int side = 0; side < 2; side++) {
@@ -263,7 +265,7 @@ qcw_status plain_gatek(qcw_ctx *c, const c128 *u, const int *qs, int k, float2 *
         p.k = k;
         int base = side == 0 ? 2 * n - 1 : n - 1;  // row bits, then column bits
         for (int i = 0; i < m * m; i++) p.u[i] = f2(side == 0 ? u[i] : std::conj(u[i]));
-        int v[5];
+        int v[4];
         for (int j = 0; j < k; j++) v[j] = base - qs[j];
         for (int i = 0; i < m; i++) {
             uint64_t o = 0;
@@ -275,7 +277,7 @@ qcw_status plain_gatek(qcw_ctx *c, const c128 *u, const int *qs, int k, float2 *
             for (int b = a + 1; b < k; b++)
                 if (v[b] < v[a]) { int t = v[a]; v[a] = v[b]; v[b] = t; }
         for (int j = 0; j < k; j++) p.pos[j] = v[j];
-        launch_gatek_side(p, target ? target : c->rho, n, c->nsm, c->stream);
+        launch_gatek_side(p, c->rho, n, c->nsm, c->stream);
         CKLAUNCH(c, 1);
     }
     return QCW_OK;
@@ -367,29 +369,68 @@ qcw_status ensure_full(qcw_ctx *c)
     return QCW_OK;
 }
 
-// Kraus channel on k >= 3 qubits (Eq. rhoE2 term by term): acc = sum_j K_j rho K_j^dagger, each
-// term on a copy of rho with the dense k-qubit side passes (K_j on the rows, conj(K_j) on the
-// columns), then rho = acc.  Two scratch copies of rho stay allocated for later channels.
-static qcw_status plain_kraus_list(qcw_ctx *c, const QOp &op)
+// The operators of op as FP32 in device memory, ordered on the context's stream.
+static qcw_status upload_operators(qcw_ctx *c, const QOp &op, const float2 **dev)
 {
-    const size_t bytes = sizeof(float2) << (2 * c->n);
-    for (float2 **b : {&c->d_kacc, &c->d_ktmp})
-        if (!*b && cudaMalloc(b, bytes) != cudaSuccess) {
+    const size_t cnt = op.m.size();
+    if (c->kops_cap < cnt) {
+        float2 *d = nullptr, *h = nullptr;
+        if (!c->kops_ev && cudaEventCreateWithFlags(&c->kops_ev, cudaEventDisableTiming) != cudaSuccess) {
             cudaGetLastError();
-            *b = nullptr;
+            return set_error(QCW_ENOMEM, "operator upload event");
+        }
+        if (cudaMalloc(&d, sizeof(float2) * cnt) != cudaSuccess || cudaMallocHost(&h, sizeof(float2) * cnt) != cudaSuccess) {
+            cudaGetLastError();
+            if (d) cudaFree(d);
+            return set_error(QCW_ENOMEM, "operator upload");
+        }
+        CK(cudaStreamSynchronize(c->stream));  // the old buffers may be in use
+        if (c->d_kops) cudaFree(c->d_kops);
+        if (c->h_kops) cudaFreeHost(c->h_kops);
+        c->d_kops = d;
+        c->h_kops = h;
+        c->kops_cap = cnt;
+    }
+    CK(cudaEventSynchronize(c->kops_ev));  // the last upload has left the pinned copy
+    for (size_t i = 0; i < cnt; i++) c->h_kops[i] = f2(op.m[i]);
+    CK(cudaMemcpyAsync(c->d_kops, c->h_kops, sizeof(float2) * cnt, cudaMemcpyHostToDevice, c->stream));
+    CK(cudaEventRecord(c->kops_ev, c->stream));
+    *dev = c->d_kops;
+    return QCW_OK;
+}
+
+// Kraus channels on k >= 3 qubits (Eq. rhoE2) and five-qubit gates: the whole sum of K_j rho K_j^dagger in one
+// pass (wide.cu).  The scratch copies of rho that a channel of many operators needs stay allocated.
+static qcw_status plain_wide(qcw_ctx *c, const QOp &op)
+{
+    WideOp w{op.m.data(), (int)(op.m.size() >> (2 * op.k)), op.k, op.qubits, nullptr};
+    const int copies = wide_scratch(c->n, w.k, w.nk, c->nsm);
+    if (copies > c->kacc_copies) {
+        float2 *b = nullptr;
+        if (cudaMalloc(&b, (size_t)copies * (sizeof(float2) << (2 * c->n))) != cudaSuccess) {
+            cudaGetLastError();
             return set_error(QCW_ENOMEM, "Kraus scratch");
         }
-    const size_t msz = (size_t)1 << (2 * op.k);
-    const size_t nk = op.m.size() / msz;
-    CK(cudaMemsetAsync(c->d_kacc, 0, bytes, c->stream));
-    for (size_t j = 0; j < nk; j++) {
-        CK(cudaMemcpyAsync(c->d_ktmp, c->rho, bytes, cudaMemcpyDeviceToDevice, c->stream));
-        qcw_status st = plain_gatek(c, op.m.data() + j * msz, op.qubits, op.k, c->d_ktmp);
-        if (st) return st;
-        launch_accumulate(c->d_kacc, c->d_ktmp, c->n, c->nsm, c->stream);
-        CKLAUNCH(c, 1);
+        if (c->d_kacc) cudaFree(c->d_kacc);  // waits for the work that uses it
+        c->d_kacc = b;
+        c->kacc_copies = copies;
     }
-    CK(cudaMemcpyAsync(c->rho, c->d_kacc, bytes, cudaMemcpyDeviceToDevice, c->stream));
+    if (wide_splits(c->n, w.k, w.nk, c->nsm)) {
+        // one launch for all operators, from an uploaded copy (not while the stream is captured: a
+        // graph has to carry the operators itself)
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+            cudaGetLastError();  // the legacy stream while another one is captured
+            cap = cudaStreamCaptureStatusActive;
+        }
+        if (cap == cudaStreamCaptureStatusNone) {
+            qcw_status st = upload_operators(c, op, &w.dev);
+            if (st) return st;
+        }
+    }
+    int nl = 0;
+    CK(launch_wide(w, c->rho, c->d_kacc, c->n, c->nsm, c->stream, &nl));
+    c->launches += nl;
     return QCW_OK;
 }
 
@@ -398,11 +439,11 @@ qcw_status plain_apply(qcw_ctx *c, const QOp &op)
     c->state_ver++;
     qcw_status fs = ensure_full(c);
     if (fs) return fs;
-    if (op.kind == 2) return plain_kraus_list(c, op);
+    if (op.k > 2 && (op.kind == 2 || op.k == 5)) return plain_wide(c, op);
+    if (op.k > 2) return plain_gatek(c, op.m.data(), op.qubits, op.k);
     if (op.kind == 1) return plain_super(c, op.m, op.qubits, op.k);
     if (op.k == 1) return plain_gate1(c, op.m.data(), op.qubits[0], op.controls, op.ncontrols);
-    if (op.k == 2) return plain_gate2(c, op.m.data(), op.qubits[0], op.qubits[1], op.controls, op.ncontrols);
-    return plain_gatek(c, op.m.data(), op.qubits, op.k);
+    return plain_gate2(c, op.m.data(), op.qubits[0], op.qubits[1], op.controls, op.ncontrols);
 }
 
 }  // namespace qcw
@@ -429,7 +470,9 @@ static void ctx_free(qcw_ctx *c)
     if (c->d_staging) cudaFree(c->d_staging);
     if (c->pv) cudaFree(c->pv);
     if (c->d_kacc) cudaFree(c->d_kacc);
-    if (c->d_ktmp) cudaFree(c->d_ktmp);
+    if (c->d_kops) cudaFree(c->d_kops);
+    if (c->h_kops) cudaFreeHost(c->h_kops);
+    if (c->kops_ev) cudaEventDestroy(c->kops_ev);
     if (c->d_ckpt) cudaFree(c->d_ckpt);
     if (c->h_ckpt) cudaFreeHost(c->h_ckpt);
     for (cudaEvent_t e : c->ckpt_ev)

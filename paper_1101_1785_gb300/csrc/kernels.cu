@@ -430,29 +430,9 @@ void launch_gatek_side(const GateKParams &p, float2 *rho, int n, int nsm, cudaSt
     const int th = 128;
     unsigned gr = grid_for(ng, th, nsm);
     switch (p.k) {
-    case 1: k_gatek_side<1><<<gr, th, 0, s>>>(rho, ng, p); break;
-    case 2: k_gatek_side<2><<<gr, th, 0, s>>>(rho, ng, p); break;
     case 3: k_gatek_side<3><<<gr, th, 0, s>>>(rho, ng, p); break;
-    case 4: k_gatek_side<4><<<gr, th, 0, s>>>(rho, ng, p); break;
-    default: k_gatek_side<5><<<gr, th, 0, s>>>(rho, ng, p); break;
+    default: k_gatek_side<4><<<gr, th, 0, s>>>(rho, ng, p); break;
     }
-}
-
-// acc += x, element-wise (Kraus sums over more than two qubits).
-__global__ void k_accumulate(float4 *__restrict__ acc, const float4 *__restrict__ x, uint64_t n4)
-{
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < n4;
-         t += (uint64_t)gridDim.x * blockDim.x) {
-        const float4 a = acc[t], b = x[t];
-        acc[t] = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-    }
-}
-
-void launch_accumulate(float2 *acc, const float2 *x, int n, int nsm, cudaStream_t s)
-{
-    const uint64_t n4 = (1ull << (2 * n)) / 2;
-    k_accumulate<<<grid_for(n4, 256, nsm), 256, 0, s>>>(reinterpret_cast<float4 *>(acc),
-                                                        reinterpret_cast<const float4 *>(x), n4);
 }
 
 // --------------------------------------------------------------------- state set-up

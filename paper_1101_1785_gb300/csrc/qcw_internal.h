@@ -52,11 +52,11 @@ struct Mono2Params {   // uncontrolled two-qubit gate with one entry of modulus 
     uint64_t src_r[4], src_c[4];    // offsets of their inputs: off_r[sigma(i)], off_c[sigma(j)]
 };
 
-struct GateKParams {   // one side (rows or columns) of a k-qubit dense gate, k <= 5
-    float2 u[1024];    // U (or conj(U) for the column side), 2^k x 2^k row-major
+struct GateKParams {   // one side (rows or columns) of a k-qubit dense gate, k = 3, 4
+    float2 u[256];     // U (or conj(U) for the column side), 2^k x 2^k row-major
     int k;
-    int pos[5];        // ascending virtual bit positions of the struck bits on this side
-    uint64_t off[32];  // offset of local index i on this side
+    int pos[4];        // ascending virtual bit positions of the struck bits on this side
+    uint64_t off[16];  // offset of local index i on this side
 };
 
 struct PTParams {
@@ -93,7 +93,18 @@ void launch_fold(const double *partials, int nblocks, double *out, cudaStream_t 
 // |psi_v><psi_v|; *err gets bit 0 if a bounded wait ran out.  Returns false if not launched.
 bool launch_ens_density_tc(const float2 *psi, int nvec, int n, const float *w, float2 *rho, unsigned *err, int nsm,
                            cudaStream_t s);
-void launch_accumulate(float2 *acc, const float2 *x, int n, int nsm, cudaStream_t s);
+// Operations on three to five qubits (wide.cu): rho <- sum_j K_j rho K_j^dagger, nk operators of
+// 2^k x 2^k at m.  scratch: wide_scratch copies of rho.
+struct WideOp {
+    const c128 *m;
+    int nk, k;
+    const int *qubits;
+    const float2 *dev;  // the operators in device memory (FP32), or nullptr: they travel with the launches
+};
+bool wide_splits(int n, int k, int nk, int nsm);
+constexpr int kWideEntries = 3072;  // matrix entries one launch carries in its parameter block
+int wide_scratch(int n, int k, int nk, int nsm);
+cudaError_t launch_wide(const WideOp &op, float2 *rho, float2 *scratch, int n, int nsm, cudaStream_t s, int *launches);
 // Pauli-string expectations Tr[P rho] (polarisation vectors, spin correlation tensor): per
 // string the row-label masks of its X-or-Y qubits (flipped), Y qubits and Z qubits.
 constexpr int kMaxPauliTerms = 3 * QCW_MAX_QUBITS;
@@ -167,9 +178,13 @@ struct qcw_ctx {
     // Version of rho: bumped by everything that changes it.  The last fused pass of a flush
     // also sums |rho_rc|^2 over what it writes (per-CTA partials in the fused runtime);
     // purity_ver records the version those partials describe.
-    // scratch copies of rho for Kraus channels on more than two qubits (allocated on first use)
+    // scratch copies of rho for channels on more than two qubits (allocated on first use)
     float2 *d_kacc = nullptr;
-    float2 *d_ktmp = nullptr;
+    int kacc_copies = 0;
+    // operators of a channel on few tiles, uploaded for one launch (pinned source, guarded by an event)
+    float2 *d_kops = nullptr, *h_kops = nullptr;
+    size_t kops_cap = 0;
+    cudaEvent_t kops_ev = nullptr;
     unsigned long long state_ver = 1;
     unsigned long long purity_ver = 0;
     // asynchronous readouts: QCW_CHECKPOINT_SLOTS slots of kCkptVals doubles on the device and
