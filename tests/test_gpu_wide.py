@@ -1,6 +1,6 @@
 """GPU parity of the one-pass kernel for operations on three to five qubits (gates and channels, one
-or several operators per launch, operators spread over blocks or summed over launches) against the
-oracle."""
+or several operators per launch, operators spread over blocks or summed over launches) and of the
+warp-per-output partial trace, against the oracle."""
 
 import numpy as np
 import pytest
@@ -47,4 +47,23 @@ def test_wide_operations(q, n, k, nk):
             oracle.apply_kraus(want, ks, qs)
     assert np.abs(d.get_state() - want).max() <= ATOL
     assert abs(d.trace() - 1) <= 1e-6
+    d.close()
+
+
+@pytest.mark.parametrize("n,ntr", [(5, 5), (7, 5), (8, 6), (9, 7), (10, 8)])
+@pytest.mark.parametrize("half", [False, True])
+def test_partial_trace_shapes(q, n, ntr, half):
+    """One output per thread, warp and block, on the full matrix and on its lower triangle."""
+    rng = np.random.default_rng(10 * n + ntr)
+    c = wl.random_circuit(n, 40, 70 + n, "mixed", "adpd")
+    want = oracle.run_circuit(c)
+    d = q.Density(n)
+    if half and n >= 6:
+        d.set_mode(q.QCW_MODE_FUSED, 4)
+        d.set_fused_kernel(3)
+    for op in c.ops:
+        d.apply_op(op)
+    for _ in range(3):
+        keep = sorted(int(x) for x in rng.permutation(n)[: n - ntr])
+        np.testing.assert_allclose(d.partial_trace(keep), oracle.partial_trace(want, keep), atol=1e-6, rtol=0)
     d.close()
