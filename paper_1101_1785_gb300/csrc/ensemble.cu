@@ -4,6 +4,7 @@
 #include "qcw_device.cuh"
 #include "qcw_internal.h"
 
+#include <algorithm>
 #include <cmath>
 #include <utility>
 #include <vector>
@@ -13,7 +14,15 @@ struct qcw_ensemble {
     float2 *psi = nullptr;  // nvec x 2^n
     int *d_choice = nullptr;
     float *d_w = nullptr;
-    unsigned *d_err = nullptr;  // error word of the tensor-core density (a bounded wait ran out)
+    // pinned copies of the caller's draws and weights on their way to the device, kEnsSlots in turn,
+    // each with the event after its copy; scratch for densities split over the vectors
+    int *h_choice = nullptr;
+    float *h_w = nullptr;
+    cudaEvent_t slot_ev[2][4] = {};
+    int slot_next[2] = {0, 0};
+    cudaEvent_t ready = nullptr, taken = nullptr;  // vectors ready for a density; density done with them
+    float2 *d_part = nullptr;
+    size_t part_elems = 0;
     void *d_stage = nullptr;  // complex128 staging, one vector
     cudaStream_t stream = nullptr;
 };
@@ -22,6 +31,7 @@ namespace qcw {
 
 constexpr int kEnsThreads = 256;
 constexpr int kEnsMaxOmega = 16;
+constexpr int kEnsSlots = 4;
 
 struct EnsGate {
     float2 u[16];    // 2^k x 2^k, k <= 2
@@ -88,23 +98,59 @@ __global__ void k_ens_noise(float2 *__restrict__ psi, int n, uint64_t items, con
     }
 }
 
-// rho[r][c] = sum_v w_v psi_v[r] conj(psi_v[c]); consecutive threads take consecutive c.
-__global__ void k_ens_density(const float2 *__restrict__ psi, int nvec, int n, const float *__restrict__ w,
-                              float2 *__restrict__ rho)
+// Registers below 6 qubits: a block sums its share of the vectors (staged through shared memory, 16
+// at a time) for every element of rho into its own copy; k_ens_sum adds the copies.  (One thread per
+// element over all vectors left the chip idle: 530 us for 2048 vectors of 5 qubits.)
+constexpr int kSmV = 16;
+__global__ void __launch_bounds__(kEnsThreads) k_ens_density_small(const float2 *__restrict__ psi, int nvec, int n,
+                                                                   const float *__restrict__ w, float2 *__restrict__ part)
 {
-    const uint64_t dim = 1ull << n, items = dim * dim;
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < items;
-         t += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t r = t >> n, c = t & (dim - 1);
-        float2 acc = make_float2(0.f, 0.f);
-        for (int v = 0; v < nvec; v++) {
-            const float2 a = psi[((uint64_t)v << n) + r], b = psi[((uint64_t)v << n) + c];
-            float2 ab = make_float2(0.f, 0.f);
-            cfmac(ab, b, a);  // a conj(b)
-            acc.x = fmaf(w[v], ab.x, acc.x);
-            acc.y = fmaf(w[v], ab.y, acc.y);
+    __shared__ float2 a[kSmV][32], b[kSmV][32];
+    const int dim = 1 << n, el = dim * dim;
+    float2 acc[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) acc[k] = make_float2(0.f, 0.f);
+    for (int v0 = blockIdx.x * kSmV; v0 < nvec; v0 += gridDim.x * kSmV) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < (kSmV << n); e += kEnsThreads) {
+            const int v = e >> n, i = e & (dim - 1);
+            const float2 x = v0 + v < nvec ? psi[((uint64_t)(v0 + v) << n) + i] : make_float2(0.f, 0.f);
+            const float wv = v0 + v < nvec ? w[v0 + v] : 0.f;
+            b[v][i] = x;
+            a[v][i] = make_float2(wv * x.x, wv * x.y);
         }
-        rho[t] = acc;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int e = threadIdx.x + k * kEnsThreads;
+            if (e >= el) break;
+            const int r = e >> n, c = e & (dim - 1);
+#pragma unroll
+            for (int v = 0; v < kSmV; v++) cfmac(acc[k], b[v][c], a[v][r]);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int e = threadIdx.x + k * kEnsThreads;
+        if (e < el) part[(uint64_t)blockIdx.x * el + e] = acc[k];
+    }
+}
+
+// rho = the sum of np copies of el elements, one after the other: a warp per element when there are
+// few of them (lanes take copies in turn, fixed shuffle tree), else a thread.  FP64 sums.
+template <bool WARP>
+__global__ void k_ens_sum(const float2 *__restrict__ part, int np, uint64_t el, float2 *__restrict__ rho)
+{
+    const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, nt = (uint64_t)gridDim.x * blockDim.x;
+    const int lane = WARP ? threadIdx.x & 31 : 0;
+    for (uint64_t e = WARP ? t0 >> 5 : t0; e < el; e += WARP ? nt >> 5 : nt) {
+        double x = 0, y = 0;
+        for (int j = lane; j < np; j += WARP ? 32 : 1) {
+            const float2 v = part[(uint64_t)j * el + e];
+            x += v.x, y += v.y;
+        }
+        if (WARP) x = warp_sum(x), y = warp_sum(y);
+        if (lane == 0) rho[e] = make_float2((float)x, (float)y);
     }
 }
 
@@ -118,7 +164,10 @@ __global__ void k_ens_density(const float2 *__restrict__ psi, int nvec, int n, c
 constexpr int kDenT = 64;   // tile edge
 constexpr int kDenV = 16;   // vectors staged per round
 constexpr int kDenThreads = 256;
+constexpr int kEnsSplitMax = 9;  // qubits up to which the vectors are shared out instead of the tiles
 
+// gridDim.y > 1: grid row y takes its share of the vectors and writes its own copy of rho (rho + y *
+// 4^n), for registers with fewer tiles than the chip has SMs.
 // diag_blocks: only the 64 x 64 tiles inside the 128 x 128 blocks on the diagonal (three lower
 // tiles per block; the tensor-core kernel does the rest).
 __global__ void __launch_bounds__(kDenThreads) k_ens_density_tiled(const float2 *__restrict__ psi, int nvec, int n,
@@ -132,6 +181,9 @@ __global__ void __launch_bounds__(kDenThreads) k_ens_density_tiled(const float2 
     float2(*Bs)[kDenT] = reinterpret_cast<float2(*)[kDenT]>(sbuf + kDenV * kDenT);
     float2(*Tt)[kDenT + 1] = reinterpret_cast<float2(*)[kDenT + 1]>(sbuf);
     const uint64_t dim = 1ull << n;
+    const int share = ((nvec + (int)gridDim.y - 1) / (int)gridDim.y + kDenV - 1) / kDenV * kDenV;
+    const int vbeg = (int)blockIdx.y * share, vend = nvec < vbeg + share ? nvec : vbeg + share;
+    rho += (uint64_t)blockIdx.y * dim * dim;
     const unsigned M = (unsigned)(dim / kDenT);
     const unsigned npairs = diag_blocks ? 3 * (M / 2) : M * (M + 1) / 2;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -153,12 +205,12 @@ __global__ void __launch_bounds__(kDenThreads) k_ens_density_tiled(const float2 
         for (int i = 0; i < 4; i++)
 #pragma unroll
             for (int j = 0; j < 4; j++) acc[i][j] = make_float2(0.f, 0.f);
-        for (int v0 = 0; v0 < nvec; v0 += kDenV) {
+        for (int v0 = vbeg; v0 < vend; v0 += kDenV) {
             __syncthreads();  // the previous round's (or tile's) reads of As / Bs are done
             for (int e = tid; e < kDenV * kDenT; e += kDenThreads) {
                 const int v = e / kDenT, i = e % kDenT;
                 float2 a = make_float2(0.f, 0.f), b = a;
-                if (v0 + v < nvec) {
+                if (v0 + v < vend) {
                     const float2 *pv = psi + ((uint64_t)(v0 + v) << n);
                     const float wv = w[v0 + v];
                     a = pv[r0 + i];
@@ -252,11 +304,18 @@ using namespace qcw;
 static void ens_free(qcw_ensemble *e)
 {
     if (!e) return;
-    if (e->stream) cudaStreamSynchronize(e->stream);
+    if (e->stream) cudaStreamSynchronize(e->stream);  // also behind the last density (taken)
+    if (e->h_choice) cudaFreeHost(e->h_choice);
+    if (e->h_w) cudaFreeHost(e->h_w);
+    for (auto &k : e->slot_ev)
+        for (cudaEvent_t ev : k)
+            if (ev) cudaEventDestroy(ev);
+    if (e->ready) cudaEventDestroy(e->ready);
+    if (e->taken) cudaEventDestroy(e->taken);
+    if (e->d_part) cudaFree(e->d_part);
     if (e->psi) cudaFree(e->psi);
     if (e->d_choice) cudaFree(e->d_choice);
     if (e->d_w) cudaFree(e->d_w);
-    if (e->d_err) cudaFree(e->d_err);
     if (e->d_stage) cudaFree(e->d_stage);
     if (e->stream) cudaStreamDestroy(e->stream);
     delete e;
@@ -278,7 +337,13 @@ extern "C" qcw_status qcw_ensemble_create(int nqubits, int nvec, qcw_ensemble **
     if (er == cudaSuccess) er = cudaMalloc(&e->psi, sizeof(float2) * items);
     if (er == cudaSuccess) er = cudaMalloc(&e->d_choice, sizeof(int) * (size_t)nvec);
     if (er == cudaSuccess) er = cudaMalloc(&e->d_w, sizeof(float) * (size_t)nvec);
-    if (er == cudaSuccess) er = cudaMalloc(&e->d_err, sizeof(unsigned));
+    if (er == cudaSuccess) er = cudaMallocHost(&e->h_choice, sizeof(int) * (size_t)nvec * kEnsSlots);
+    if (er == cudaSuccess) er = cudaMallocHost(&e->h_w, sizeof(float) * (size_t)nvec * kEnsSlots);
+    for (auto &k : e->slot_ev)
+        for (cudaEvent_t &ev : k)
+            if (er == cudaSuccess) er = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (er == cudaSuccess) er = cudaEventCreateWithFlags(&e->ready, cudaEventDisableTiming);
+    if (er == cudaSuccess) er = cudaEventCreateWithFlags(&e->taken, cudaEventDisableTiming);
     if (er == cudaSuccess) er = cudaMalloc(&e->d_stage, sizeof(double2) << nqubits);
     if (er != cudaSuccess) {
         cudaGetLastError();
@@ -330,6 +395,13 @@ extern "C" qcw_status qcw_ensemble_get(qcw_ensemble *e, double *psi_c128)
         ENS_CK(cudaStreamSynchronize(e->stream));
     }
     return QCW_OK;
+}
+
+// The next pinned slot of a kind (0 draws, 1 weights), once its last copy has left it.
+static cudaError_t ens_slot(qcw_ensemble *e, int kind, int *slot)
+{
+    *slot = e->slot_next[kind]++ % kEnsSlots;
+    return cudaEventSynchronize(e->slot_ev[kind][*slot]);
 }
 
 static qcw_status ens_gate(qcw_ensemble *e, const double *u, const int *qs, int k)
@@ -387,12 +459,31 @@ extern "C" qcw_status qcw_ensemble_apply_noise1(qcw_ensemble *e, const double *o
     for (int k = 0; k < nomega; k++)
         for (int i = 0; i < 4; i++) p.om[k][i] = to_f2(omegas + 8 * k + 2 * i);
     p.pos = e->n - 1 - target;
-    // the copy is stream-ordered before the kernel; synchronising keeps the caller's array free
-    ENS_CK(cudaMemcpyAsync(e->d_choice, choice, sizeof(int) * (size_t)e->nvec, cudaMemcpyHostToDevice, e->stream));
+    // through a pinned slot: the caller's array is free when the call returns, without a wait
+    int slot = 0;
+    ENS_CK(ens_slot(e, 0, &slot));
+    int *h = e->h_choice + (size_t)slot * e->nvec;
+    std::copy(choice, choice + e->nvec, h);
+    ENS_CK(cudaMemcpyAsync(e->d_choice, h, sizeof(int) * (size_t)e->nvec, cudaMemcpyHostToDevice, e->stream));
+    ENS_CK(cudaEventRecord(e->slot_ev[0][slot], e->stream));
     const uint64_t items = (uint64_t)e->nvec << (e->n - 1);
     k_ens_noise<<<ens_grid(items, e->nsm), kEnsThreads, 0, e->stream>>>(e->psi, e->n, items, e->d_choice, p);
     ENS_CK(cudaGetLastError());
-    ENS_CK(cudaStreamSynchronize(e->stream));
+    return QCW_OK;
+}
+
+// Scratch for np copies of rho.
+static qcw_status ens_scratch(qcw_ensemble *e, size_t elems)
+{
+    if (elems <= e->part_elems) return QCW_OK;
+    float2 *b = nullptr;
+    if (cudaMalloc(&b, sizeof(float2) * elems) != cudaSuccess) {
+        cudaGetLastError();
+        return set_error(QCW_ENOMEM, "ensemble density scratch");
+    }
+    if (e->d_part) cudaFree(e->d_part);  // waits for the work that uses it
+    e->d_part = b;
+    e->part_elems = elems;
     return QCW_OK;
 }
 
@@ -401,15 +492,34 @@ extern "C" qcw_status qcw_ensemble_density(qcw_ensemble *e, const double *weight
     if (!e || !weights || !ctx) return set_error(QCW_EINVAL, "null argument");
     if (qcw_nqubits(ctx) != e->n) return set_error(QCW_EINVAL, "qubit counts differ");
     if (!finite_all(weights, (size_t)e->nvec)) return set_error(QCW_EINVAL, "non-finite weight");
-    std::vector<float> w(e->nvec);
-    for (int v = 0; v < e->nvec; v++) w[v] = (float)weights[v];
-    ENS_CK(cudaMemcpyAsync(e->d_w, w.data(), sizeof(float) * w.size(), cudaMemcpyHostToDevice, e->stream));
-    ENS_CK(cudaStreamSynchronize(e->stream));  // vectors and weights ready; w may go
+    const uint64_t dim = 1ull << e->n, el = dim * dim;
+    // copies of rho, each from a share of the vectors, where the tiles alone leave SMs idle (up to 9
+    // qubits there are 45 tiles or fewer)
+    int split = 1;
+    if (dim < (uint64_t)kDenT) {
+        split = std::min((e->nvec + kSmV - 1) / kSmV, e->nsm);
+    } else if (e->n <= kEnsSplitMax) {
+        const int m = (int)(dim / kDenT), tiles = m * (m + 1) / 2;
+        split = std::max(1, std::min((e->nvec + 2 * kDenV - 1) / (2 * kDenV), 2 * e->nsm / tiles));
+    }
+    if (split > 1) {
+        qcw_status es = ens_scratch(e, (size_t)split * el);
+        if (es) return es;
+    }
+    int slot = 0;
+    ENS_CK(ens_slot(e, 1, &slot));
+    float *h = e->h_w + (size_t)slot * e->nvec;
+    for (int v = 0; v < e->nvec; v++) h[v] = (float)weights[v];
+    ENS_CK(cudaMemcpyAsync(e->d_w, h, sizeof(float) * (size_t)e->nvec, cudaMemcpyHostToDevice, e->stream));
+    ENS_CK(cudaEventRecord(e->slot_ev[1][slot], e->stream));
     qcw_status st = begin_state_replace(ctx);
     if (st) return st;
-    const uint64_t dim = 1ull << e->n;
-    ENS_CK(cudaMemsetAsync(e->d_err, 0, sizeof(unsigned), ctx->stream));
-    if (dim >= 2 * (uint64_t)kDenT && e->n >= 8) {
+    // ctx's stream takes over from the ensemble's, and back: the vectors, weights and scratch are not
+    // touched again before the density is done with them
+    ENS_CK(cudaEventRecord(e->ready, e->stream));
+    ENS_CK(cudaStreamWaitEvent(ctx->stream, e->ready, 0));
+    float2 *out = split > 1 ? e->d_part : ctx->rho;
+    if (e->n > kEnsSplitMax) {
         // tiles strictly below the 128 x 128 diagonal blocks on the tensor cores, the diagonal
         // blocks (trace, probabilities) in FP32
         const uint64_t blocks = dim / (2 * kDenT), pairs = 3 * blocks;
@@ -418,22 +528,25 @@ extern "C" qcw_status qcw_ensemble_density(qcw_ensemble *e, const double *weight
             e->psi, e->nvec, e->n, e->d_w, ctx->rho, 1);
         ENS_CK(cudaGetLastError());
         ctx->launches++;
-        if (!launch_ens_density_tc(e->psi, e->nvec, e->n, e->d_w, ctx->rho, e->d_err, e->nsm, ctx->stream))
+        if (!launch_ens_density_tc(e->psi, e->nvec, e->n, e->d_w, ctx->rho,
+                                   reinterpret_cast<unsigned *>(device_error_word(ctx)), e->nsm, ctx->stream))
             return set_error(QCW_ECUDA, "tensor-core density kernel could not be configured");
     } else if (dim >= (uint64_t)kDenT) {
         const uint64_t m = dim / kDenT, pairs = m * (m + 1) / 2;
-        const uint64_t cap = (uint64_t)e->nsm * 8;  // 8 CTAs of 256 threads resident per SM
-        k_ens_density_tiled<<<(unsigned)(pairs < cap ? pairs : cap), kDenThreads, 0, ctx->stream>>>(
-            e->psi, e->nvec, e->n, e->d_w, ctx->rho, 0);
+        k_ens_density_tiled<<<dim3((unsigned)pairs, split), kDenThreads, 0, ctx->stream>>>(e->psi, e->nvec, e->n, e->d_w,
+                                                                                          out, 0);
     } else {
-        k_ens_density<<<ens_grid(dim * dim, e->nsm), kEnsThreads, 0, ctx->stream>>>(e->psi, e->nvec, e->n, e->d_w,
-                                                                                   ctx->rho);
+        k_ens_density_small<<<split, kEnsThreads, 0, ctx->stream>>>(e->psi, e->nvec, e->n, e->d_w, out);
     }
     ENS_CK(cudaGetLastError());
     ctx->launches++;
-    unsigned herr = 0;
-    ENS_CK(cudaMemcpyAsync(&herr, e->d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
-    ENS_CK(cudaStreamSynchronize(ctx->stream));  // the ensemble may change right after
-    if (herr) return set_error(QCW_ETIMEOUT, "ensemble density: a bounded wait ran out");
+    if (split > 1) {
+        if (el <= 4096) k_ens_sum<true><<<(unsigned)((el * 32 + 255) / 256), 256, 0, ctx->stream>>>(out, split, el, ctx->rho);
+        else k_ens_sum<false><<<(unsigned)((el + 255) / 256), 256, 0, ctx->stream>>>(out, split, el, ctx->rho);
+        ENS_CK(cudaGetLastError());
+        ctx->launches++;
+    }
+    ENS_CK(cudaEventRecord(e->taken, ctx->stream));
+    ENS_CK(cudaStreamWaitEvent(e->stream, e->taken, 0));
     return QCW_OK;
 }

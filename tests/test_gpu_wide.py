@@ -67,3 +67,34 @@ def test_partial_trace_shapes(q, n, ntr, half):
         keep = sorted(int(x) for x in rng.permutation(n)[: n - ntr])
         np.testing.assert_allclose(d.partial_trace(keep), oracle.partial_trace(want, keep), atol=1e-6, rtol=0)
     d.close()
+
+
+@pytest.mark.parametrize("n,nvec", [(1, 3), (3, 2048), (5, 16), (5, 2049), (6, 4096), (7, 700), (8, 515), (9, 600)])
+def test_density_shared_out_over_the_vectors(q, n, nvec):
+    """Registers with few tiles: every block sums a share of the vectors.  A second noise step and
+    density right behind the first (no host wait in between) must not disturb it."""
+    rng = np.random.default_rng(100 * n + nvec)
+    psi = rng.standard_normal((nvec, 1 << n)) + 1j * rng.standard_normal((nvec, 1 << n))
+    psi /= np.linalg.norm(psi, axis=1)[:, None]
+    psi = psi.astype(np.complex64).astype(np.complex128)
+    w = rng.uniform(0.1, 1.0, nvec)
+    w /= w.sum()
+    om = np.stack([wl.gate_matrix("I"), wl.gate_matrix("X"), wl.gate_matrix("Z")])
+    e = q.Ensemble(n, nvec)
+    e.set(psi)
+    ds = [q.Density(n), q.Density(n)]
+    want = []
+    for d in ds:
+        t = int(rng.integers(n))
+        pick = rng.integers(0, 3, nvec).astype(np.int32)
+        e.apply_noise1(om, t, pick)
+        v = psi.reshape(nvec, 1 << t, 2, -1)
+        psi = np.einsum("vij,vajb->vaib", om[pick], v).reshape(nvec, -1)
+        e.density(w, d)
+        want.append((psi * w[:, None]).T @ psi.conj())
+    for d, x in zip(ds, want):
+        # FP32 products and sums of at most a few hundred terms of weight w |psi|^2 per block
+        assert np.abs(d.get_state() - x).max() <= 32 * 2.0 ** -24 * np.abs(x).max()
+        assert abs(d.trace() - 1) <= 1e-6
+        d.close()
+    e.close()
