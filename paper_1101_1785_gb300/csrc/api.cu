@@ -808,8 +808,7 @@ extern "C" qcw_status qcw_apply_kraus(qcw_ctx *ctx, const double *kraus, int nkr
     return submit(ctx, std::move(op));
 }
 
-qcw_status qcw::convert_ops(int n, const qcw_op *ops, int nops, const double *matrices, std::vector<QOp> &out,
-                            bool validate)
+qcw_status qcw::check_ops(int n, const qcw_op *ops, int nops, const double *matrices, bool validate)
 {
     if (nops < 0 || (nops > 0 && (!ops || !matrices))) return set_error(QCW_EINVAL, "bad op list");
     for (int i = 0; i < nops; i++) {  // validate everything first: all or nothing
@@ -836,6 +835,14 @@ qcw_status qcw::convert_ops(int n, const qcw_op *ops, int nops, const double *ma
             return set_error(QCW_EINVAL, "bad op kind");
         }
     }
+    return QCW_OK;
+}
+
+qcw_status qcw::convert_ops(int n, const qcw_op *ops, int nops, const double *matrices, std::vector<QOp> &out,
+                            bool validate)
+{
+    qcw_status st = check_ops(n, ops, nops, matrices, validate);
+    if (st) return st;
     out.reserve(out.size() + nops);
     for (int i = 0; i < nops; i++) {
         const qcw_op &o = ops[i];

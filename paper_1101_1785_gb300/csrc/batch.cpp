@@ -2,7 +2,7 @@
 //
 // The paper's multiverse evaluates independent evolution paths on separate processors
 // (Sec. 5.1, Sec. 5.2.1); here independent circuits share one GPU: every circuit is planned
-// into a tile program (fusion width chosen per circuit by the cost model), the programs'
+// into a Pauli-basis tile program, the programs'
 // work items are listed level by level (pass order inside each circuit, circuits in
 // decreasing modeled cost), and one launch of the engine kernel drains the list.  The launch
 // (counter resets, kernel, readout copies) is captured once into a CUDA graph and replayed.
@@ -25,8 +25,12 @@ struct qcw_batch {
     std::vector<size_t> rho_off;
     std::vector<int> red_first, red_n;
     char *ddesc = nullptr;
-    float2 *arena = nullptr;
+    float *arena = nullptr;
     size_t arena_elems = 0;
+    void *conv = nullptr;  // scratch of qcw_batch_get_state, kept while it is small
+    float2 *hconv = nullptr;
+    size_t conv_bytes = 0;
+    bool dense = false;
     unsigned *counters = nullptr;
     size_t ncounters = 0;
     WItem *ditems = nullptr;
@@ -61,6 +65,8 @@ static void batch_free(qcw_batch *b)
     if (b->done) cudaEventDestroy(b->done);
     cudaFree(b->ddesc);
     cudaFree(b->arena);
+    cudaFree(b->conv);
+    if (b->hconv) cudaFreeHost(b->hconv);
     cudaFree(b->counters);
     cudaFree(b->ditems);
     cudaFree(b->dint);
@@ -90,7 +96,7 @@ static qcw_status batch_capture(qcw_batch *b)
     BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     cudaMemsetAsync(b->counters, 0, sizeof(unsigned) * b->ncounters, b->stream);
     cudaMemsetAsync(b->dint + 1, 0, 2 * sizeof(int), b->stream);
-    engine_launch(L, b->grid, b->smem, b->stream);
+    engine_launch(L, b->dense, b->grid, b->smem, b->stream);
     cudaMemcpyAsync(b->hred, b->dred, sizeof(double) * b->nred, cudaMemcpyDeviceToHost, b->stream);
     cudaMemcpyAsync(b->herr, b->dint + 2, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
     cudaError_t e = cudaStreamEndCapture(b->stream, &b->graph);
@@ -121,14 +127,14 @@ extern "C" qcw_status qcw_batch_create(int ncirc, const int *nqubits, const long
         b->owns_stream = true;
     }
     qcw_status st = QCW_OK;
-    const int tbmax = 13;
-    // plan every circuit (ops are validated against its own register size)
+    // plan every circuit (ops are checked against its own register size)
     for (int j = 0; j < ncirc && !st; j++) {
-        std::vector<QOp> q;
-        st = convert_ops(nqubits[j], ops + op_begin[j], (int)(op_begin[j + 1] - op_begin[j]), matrices, q);
-        for (QOp &o : q)
-            if (!st && o.k > 2) st = set_error(QCW_ENOTSUP, "batched circuits take 1- and 2-qubit operations");
-        if (!st) b->progs.push_back(make_program(q, nqubits[j], fuse_k, tbmax));
+        const qcw_op *o = ops + op_begin[j];
+        const int cnt = (int)(op_begin[j + 1] - op_begin[j]);
+        st = check_ops(nqubits[j], o, cnt, matrices);
+        for (int i = 0; i < cnt && !st; i++)
+            if (o[i].k > 2) st = set_error(QCW_ENOTSUP, "batched circuits take 1- and 2-qubit operations");
+        if (!st) b->progs.push_back(make_program(o, cnt, matrices, nqubits[j], fuse_k));
     }
     if (st) {
         batch_free(b);
@@ -151,22 +157,27 @@ extern "C" qcw_status qcw_batch_create(int ncirc, const int *nqubits, const long
         doff[j] = dbytes;
         dbytes += program_desc_bytes(p);
         b->rho_off[j] = aelems;
-        aelems += std::max<size_t>((size_t)1 << (2 * p.n), 32);  // 256-byte granularity
+        aelems += program_elems(p.n);  // a multiple of 256 bytes
         coff[j] = b->ncounters;
-        b->ncounters += p.tp.passes.size();
-        unsigned long long rows = reduce_rows(p.n);
-        int chunks = p.whole ? 1 : (int)(((1ull << p.n) + rows - 1) / rows);
+        b->ncounters += p.tiles.size();
+        const int chunks = program_chunks(p);
         b->red_first[j] = (int)b->nred / kRedVals;
         b->red_n[j] = chunks;
         b->nred += (size_t)chunks * kRedVals;
-        b->npass += (long long)p.tp.passes.size();
-        b->nphase += (long long)p.tp.phases.size();
+        b->npass += (long long)p.tiles.size();
+        b->nphase += p.rounds;
+        b->dense |= p.dense;
         b->modeled += p.cost;
     }
     std::vector<char> hdesc(dbytes);
-    for (int j = 0; j < ncirc; j++) program_write_desc(b->progs[j], hdesc.data(), doff[j]);
+    for (int j = 0; j < ncirc; j++) {
+        Program &p = b->progs[j];
+        memcpy(hdesc.data() + doff[j], p.desc.data(), p.desc.size());
+        p.off = doff[j];
+        std::vector<char>().swap(p.desc);
+    }
     b->arena_elems = aelems;
-    if (cudaMalloc(&b->ddesc, dbytes) != cudaSuccess || cudaMalloc(&b->arena, aelems * sizeof(float2)) != cudaSuccess ||
+    if (cudaMalloc(&b->ddesc, dbytes) != cudaSuccess || cudaMalloc(&b->arena, aelems * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&b->counters, sizeof(unsigned) * (b->ncounters + 1)) != cudaSuccess ||
         cudaMalloc(&b->dint, 4 * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&b->dred, sizeof(double) * b->nred) != cudaSuccess ||
@@ -185,16 +196,15 @@ extern "C" qcw_status qcw_batch_create(int ncirc, const int *nqubits, const long
         const Program &p = b->progs[j];
         int nch = 0;
         program_items(p, b->arena + b->rho_off[j], b->ddesc, b->counters + coff[j],
-                      b->dred + (size_t)b->red_first[j] * kRedVals, 0, (int)p.tp.passes.size(), true, true, levels,
+                      b->dred + (size_t)b->red_first[j] * kRedVals, 0, (int)p.tiles.size(), true, true, levels,
                       &nch);
     }
     for (auto &lv : levels) b->items.insert(b->items.end(), lv.begin(), lv.end());
     int nitems = (int)b->items.size();
     size_t smem = 0;
-    for (const Program &p : b->progs)
-        for (size_t s : p.tp.smem) smem = std::max(smem, s);
+    for (const Program &p : b->progs) smem = std::max(smem, p.smem);
     b->smem = smem;
-    st = engine_prepare(b->dev, smem, &b->grid);
+    st = engine_prepare(b->dev, b->dense, smem, &b->grid);
     if (!st && cudaMalloc(&b->ditems, sizeof(WItem) * std::max(nitems, 1)) != cudaSuccess) {
         cudaGetLastError();
         st = set_error(QCW_ENOMEM, "batch items");
@@ -266,12 +276,33 @@ extern "C" qcw_status qcw_batch_get_state(qcw_batch *b, int circuit, double *rho
     if (!b || !rho_c128 || circuit < 0 || circuit >= (int)b->progs.size()) return set_error(QCW_EINVAL, "bad argument");
     qcw_status st = qcw_batch_wait(b, -1);
     if (st) return st;
-    size_t cnt = (size_t)1 << (2 * b->progs[circuit].n);
-    std::vector<float2> tmp(cnt);
-    BCK(cudaMemcpy(tmp.data(), b->arena + b->rho_off[circuit], cnt * sizeof(float2), cudaMemcpyDeviceToHost));
+    const int n = b->progs[circuit].n;
+    const size_t cnt = (size_t)1 << (2 * n), need = program_scratch(n), kKeep = (size_t)64 << 20;
+    if (need > b->conv_bytes) {
+        BCK(cudaFree(b->conv));
+        if (b->hconv) BCK(cudaFreeHost(b->hconv));
+        b->conv = nullptr;
+        b->hconv = nullptr;
+        b->conv_bytes = 0;
+        if (cudaMalloc(&b->conv, need) != cudaSuccess || cudaMallocHost(&b->hconv, program_elems(n) * sizeof(float2)) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(b->conv);
+            b->conv = nullptr;
+            return set_error(QCW_ENOMEM, "batch state download");
+        }
+        b->conv_bytes = need;
+    }
+    BCK(program_rho(b->arena + b->rho_off[circuit], n, b->conv, b->hconv, b->stream));
     for (size_t i = 0; i < cnt; i++) {
-        rho_c128[2 * i] = tmp[i].x;
-        rho_c128[2 * i + 1] = tmp[i].y;
+        rho_c128[2 * i] = b->hconv[i].x;
+        rho_c128[2 * i + 1] = b->hconv[i].y;
+    }
+    if (b->conv_bytes > kKeep) {
+        BCK(cudaFree(b->conv));
+        BCK(cudaFreeHost(b->hconv));
+        b->conv = nullptr;
+        b->hconv = nullptr;
+        b->conv_bytes = 0;
     }
     return QCW_OK;
 }

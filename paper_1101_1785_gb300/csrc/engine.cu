@@ -5,19 +5,26 @@
 // order where an item's dependency (the previous pass of the same circuit) always comes
 // earlier in the list, so a CTA only ever waits for items that running CTAs already hold;
 // every wait is bounded (spin_limit polls) and a wait that runs out sets *err instead of
-// hanging.  A circuit whose rho fits one tile (2n <= tile bits) is one item: its state is
-// built in shared memory, evolved through every phase and read out there, then written once.
-// Larger circuits are split into one item per tile and pass, chained by per-pass counters,
-// followed by readout chunks.  Each circuit is processed by a fixed item decomposition with
-// a fixed thread-to-data mapping, so its result does not depend on what else is in the batch.
+// hanging.  States are kept as Pauli coefficients (pauli.h) from |0..0> to the readouts, which are
+// coefficients themselves (trace, probabilities) or their sum of squares (purity).  A circuit
+// whose state fits one tile (up to seven qubits) is one item: it starts, runs through every round
+// and is read out in shared memory.  Larger circuits are split into one item per tile and pass,
+// chained by per-pass counters, followed by readout chunks.  Each circuit is processed by a fixed
+// item decomposition with a fixed thread-to-data mapping, so its result does not depend on what
+// else is in the batch.
+//
+// Two CTAs per SM (64 KiB tile and the pass's program each) overlap one's loads with the other's
+// rounds.  64 circuits of 4 to 10 qubits: on complex tiles without symmetry 1.01 ms per launch.
 #include <algorithm>
 #include <cstring>
 
 #include "engine.h"
+#include "pauli.cuh"
 #include "qcw_internal.h"
-#include "tile.cuh"
 
 namespace qcw {
+
+constexpr int kEngThreads = 256;
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
 {
@@ -26,7 +33,7 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
     return v;
 }
 
-using RedShared = double[kTileThreads / 32][kRedVals];
+using RedShared = double[kEngThreads / 32][kRedVals];
 
 // Fold per-thread accumulators (first nv used) into out[0..nv) with a fixed tree.
 __device__ __forceinline__ void red_store(double (&acc)[kRedVals], int nv, double *out, RedShared &sh)
@@ -42,72 +49,155 @@ __device__ __forceinline__ void red_store(double (&acc)[kRedVals], int nv, doubl
     __syncthreads();
     if ((int)threadIdx.x < nv) {
         double t = 0;
-        for (int j = 0; j < kTileThreads / 32; j++) t += sh[j][threadIdx.x];
+        for (int j = 0; j < kEngThreads / 32; j++) t += sh[j][threadIdx.x];
         out[threadIdx.x] = t;
     }
     __syncthreads();
 }
 
-// Readouts of rows [row0, row0 + rows) of an n-qubit rho stored at `src` with row stride 2^n:
-// trace (re, im) and p1[q] from the diagonal, purity from every element of those rows.
-__device__ __forceinline__ void readout_rows(const float2 *__restrict__ src, int n, unsigned long long row0,
-                                             unsigned long long rows, double *out, RedShared &sh)
+// Shared memory of an item: the tile, then the pass's program (rounds, operations, coefficient pairs).
+struct EngSmem {
+    unsigned char *base;
+    __device__ __forceinline__ float4 *tile() const { return reinterpret_cast<float4 *>(base); }
+    __device__ __forceinline__ unsigned *prog(int t) const { return reinterpret_cast<unsigned *>(base + (sizeof(float) << (2 * t))); }
+};
+
+// Bring a pass's program to shared memory.
+__device__ __forceinline__ ProgShared eng_stage(const PassDesc &D, const EngSmem &sm)
+{
+    const int nr = D.h.nround * (int)(sizeof(PRound) / 4), no = (D.h.nop + 3) & ~3;
+    const unsigned *src = reinterpret_cast<const unsigned *>(&D + 1);
+    unsigned *dst = sm.prog(D.h.t);
+    for (int i = threadIdx.x; i < nr + no; i += kEngThreads) dst[i] = src[i];
+    for (int i = threadIdx.x; i < D.h.ncoef; i += kEngThreads) dst[nr + no + 2 * i] = dst[nr + no + 2 * i + 1] = src[nr + no + i];
+    const PRound *r = reinterpret_cast<const PRound *>(dst);
+    return ProgShared{r, reinterpret_cast<const POp *>(dst + nr), smem_u32(dst + nr + no)};
+}
+
+__device__ __forceinline__ void eng_init(const EngSmem &sm, int t, unsigned tile)
+{
+    const bool zt = (tile & 0xAAAAAAAAu) == 0;
+    for (unsigned k = threadIdx.x; k < (1u << (2 * (t - 1))); k += kEngThreads)
+        sm.tile()[pauli_swz(k)] = zt && (k & 0xAAAu) == 0 ? make_float4(1.f, 1.f, 0.f, 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+__device__ __forceinline__ uint64_t eng_base(const PauliHdr &h, unsigned tile)
+{
+    uint64_t b = 0;
+    for (int d = 0; d < h.nod; d++) b += (uint64_t)((tile >> (2 * d)) & 3u) << (2 * h.od[d]);
+    return b;
+}
+
+__device__ __forceinline__ uint64_t eng_chunk(const PauliHdr &h, unsigned k)
+{
+    uint64_t b = 0;
+    for (int d = 1; d < h.t; d++) b += (uint64_t)((k >> (2 * (d - 1))) & 3u) << (2 * h.td[d]);
+    return b;
+}
+
+// Out of line: the rounds need nearly all 128 registers, so nothing of the item loop lives across them.
+template <bool DENSE>
+__device__ __noinline__ void eng_rounds(unsigned tile, const PRound *rounds, int nround, const POp *ops, unsigned coef)
+{
+    const ProgShared prog{rounds, ops, coef};
+    pauli_rounds<DENSE>(tile, rounds, nround, prog, threadIdx.x, 0);
+}
+
+template <bool DENSE>
+__device__ void run_tile(const WItem &W, const EngSmem &sm)
+{
+    const PassDesc &D = *reinterpret_cast<const PassDesc *>(W.pass);
+    const unsigned nch = 1u << (2 * (D.h.t - 1));
+    float *g = W.v + eng_base(D.h, W.tile);
+    if (W.flags & WF_INIT) {
+        eng_init(sm, D.h.t, W.tile);
+    } else {
+        for (unsigned k = threadIdx.x; k < nch; k += kEngThreads) cp_async16(sm.tile() + pauli_swz(k), g + eng_chunk(D.h, k));
+    }
+    const ProgShared prog = eng_stage(D, sm);
+    cp_async_wait_all();
+    __syncthreads();
+    eng_rounds<DENSE>(smem_u32(sm.base), prog.rounds, D.h.nround, prog.ops, prog.coef);
+    for (unsigned k = threadIdx.x; k < nch; k += kEngThreads)
+        *reinterpret_cast<float4 *>(g + eng_chunk(D.h, k)) = p_lds4(smem_u32(sm.base) + 16u * pauli_swz(k));
+}
+
+// Trace (2 values), purity and P(q = 1): v0 and vz(q), the strings I..I and Z_q, by thread; s the
+// thread's share of the sum of squares.
+template <typename F>
+__device__ __forceinline__ void eng_readout(double s, bool first, int n, float v0, F vz, double *out, RedShared &sh)
 {
     double acc[kRedVals];
 #pragma unroll
-    for (int v = 0; v < kRedVals; v++) acc[v] = 0;
-    const unsigned long long dim = 1ull << n;
-    for (unsigned long long r = row0 + threadIdx.x; r < row0 + rows; r += kTileThreads) {
-        float2 d = src[r * dim + r];
-        acc[0] += d.x;
-        acc[1] += d.y;
+    for (int i = 0; i < kRedVals; i++) acc[i] = 0;
+    const int nd = n < kPMinDigits ? kPMinDigits : n;
+    double scale = 1.0;
+    for (int i = 0; i < nd; i++) scale *= 0.5;
+    acc[2] = s * scale;
+    if (first) {
+        if (threadIdx.x == 0) acc[0] = v0;
 #pragma unroll
         for (int q = 0; q < QCW_MAX_QUBITS; q++)
-            if (q < n && ((r >> (n - 1 - q)) & 1)) acc[3 + q] += d.x;
-    }
-    const float4 *s4 = reinterpret_cast<const float4 *>(src + row0 * dim);
-    const unsigned long long n4 = rows * dim / 2;
-    for (unsigned long long i = threadIdx.x; i < n4; i += 4 * kTileThreads) {
-        float s = 0.f;
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            unsigned long long j = i + (unsigned long long)u * kTileThreads;
-            if (j < n4) {
-                float4 a = s4[j];
-                s = fmaf(a.x, a.x, s); s = fmaf(a.y, a.y, s); s = fmaf(a.z, a.z, s); s = fmaf(a.w, a.w, s);
-            }
-        }
-        acc[2] += (double)s;
+            if (q < n && (int)threadIdx.x == q) acc[3 + q] = 0.5 * ((double)v0 - (double)vz(q));
     }
     red_store(acc, n + 3, out, sh);
 }
 
-__device__ void run_tiles(const WItem &W, unsigned char *smem)
+__device__ __forceinline__ float sq4(float4 a, float s)
 {
-    const FPass &P = *W.pass;
-    const TileSmem sm = tile_smem(smem, P.TB, P.L);
-    tile_hoff(P, sm.hoff);
-    __syncthreads();
-    for (unsigned t = W.tile0; t < W.tile0 + W.ntile; t++) {
-        tile_process(W.rho, P, t, W.phases, W.coefs, sm, (W.flags & WF_INIT) != 0);
+    return fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(a.z, a.z, fmaf(a.w, a.w, s))));
+}
+
+template <bool DENSE>
+__device__ void run_whole(const WItem &W, const EngSmem &sm, RedShared &sh)
+{
+    const PauliHdr &h = reinterpret_cast<const PassDesc *>(W.pass)->h;
+    const int t = h.t;
+    const unsigned nch = 1u << (2 * (t - 1));
+    eng_init(sm, t, 0);
+    const char *p = W.pass;
+    for (int i = 0; i < W.npass; i++) {
+        const PassDesc &D = *reinterpret_cast<const PassDesc *>(p);
+        const ProgShared prog = eng_stage(D, sm);
         __syncthreads();
+        eng_rounds<DENSE>(smem_u32(sm.base), prog.rounds, D.h.nround, prog.ops, prog.coef);
+        __syncthreads();
+        p += D.bytes;
+    }
+    double acc = 0;
+    const float4 *tile = sm.tile();
+    for (unsigned k = threadIdx.x; k < nch; k += kEngThreads) {
+        const float4 x = tile[pauli_swz(k)];
+        acc += (double)sq4(x, 0.f);
+        *reinterpret_cast<float4 *>(W.v + 4 * (size_t)k) = x;
+    }
+    if (W.red) {
+        auto vz = [&](int q) {
+            const unsigned e = 1u << (2 * (W.n - 1 - q));
+            return reinterpret_cast<const float *>(tile)[4 * pauli_swz(e >> 2) + (e & 3u)];
+        };
+        eng_readout(acc, true, W.n, reinterpret_cast<const float *>(tile)[0], vz, W.red, sh);
     }
 }
 
-__device__ void run_whole(const WItem &W, unsigned char *smem, RedShared &sh)
+__device__ void run_reduce(const WItem &W, RedShared &sh)
 {
-    const FPass &P0 = W.pass[0];
-    const TileSmem sm = tile_smem(smem, P0.TB, P0.L);
-    tile_hoff(P0, sm.hoff);
-    __syncthreads();
-    tile_load(W.rho, P0, 0, sm, (W.flags & WF_INIT) != 0);
-    for (int p = 0; p < W.npass; p++) tile_phases(W.pass[p], W.phases, W.coefs, sm);
-    // the tile is the whole matrix in flat order (tile bits 0..2n-1)
-    if (W.red) readout_rows(sm.tile, W.n, 0, 1ull << W.n, W.red, sh);
-    tile_store(W.rho, P0, 0, sm);
+    double acc = 0;
+    const float4 *v4 = reinterpret_cast<const float4 *>(W.v + W.e0);
+    const unsigned long long n4 = W.ecount / 4;
+    for (unsigned long long i = threadIdx.x; i < n4; i += 4 * kEngThreads) {
+        float s = 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (i + u * kEngThreads < n4) s = sq4(__ldcg(v4 + i + u * kEngThreads), s);
+        acc += (double)s;
+    }
+    auto vz = [&](int q) { return __ldcg(W.v + (1ull << (2 * (W.n - 1 - q)))); };
+    eng_readout(acc, W.e0 == 0, W.n, __ldcg(W.v), vz, W.red, sh);
 }
 
-__global__ void __launch_bounds__(kTileThreads, 2) k_engine(EngineLaunch L)
+template <bool DENSE>
+__global__ void __launch_bounds__(kEngThreads, 2) k_engine(EngineLaunch L)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_item;
@@ -133,9 +223,10 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_engine(EngineLaunch L)
             }
             __syncthreads();
         }
-        if (W.kind == WI_TILES) run_tiles(W, smem);
-        else if (W.kind == WI_WHOLE) run_whole(W, smem, s_red);
-        else readout_rows(W.rho, W.n, W.red_row0, W.red_rows, W.red, s_red);
+        const EngSmem sm{smem};
+        if (W.kind == WI_TILES) run_tile<DENSE>(W, sm);
+        else if (W.kind == WI_WHOLE) run_whole<DENSE>(W, sm, s_red);
+        else run_reduce(W, s_red);
         __syncthreads();
         if (W.done && threadIdx.x == 0) {
             __threadfence();
@@ -144,17 +235,19 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_engine(EngineLaunch L)
     }
 }
 
-void engine_launch(const EngineLaunch &L, int grid, size_t smem, cudaStream_t s)
+void engine_launch(const EngineLaunch &L, bool dense, int grid, size_t smem, cudaStream_t s)
 {
-    k_engine<<<grid, kTileThreads, smem, s>>>(L);
+    if (dense) k_engine<true><<<grid, kEngThreads, smem, s>>>(L);
+    else k_engine<false><<<grid, kEngThreads, smem, s>>>(L);
 }
 
-qcw_status engine_prepare(int dev, size_t smem, int *grid)
+qcw_status engine_prepare(int dev, bool dense, size_t smem, int *grid)
 {
-    qcw_status st = ensure_smem_attr(reinterpret_cast<const void *>(k_engine), smem);
+    const void *k = dense ? reinterpret_cast<const void *>(k_engine<true>) : reinterpret_cast<const void *>(k_engine<false>);
+    qcw_status st = ensure_smem_attr(k, smem);
     if (st) return st;
     int occ = 0, nsm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_engine, kTileThreads, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kEngThreads, smem);
     if (e != cudaSuccess) return cuda_error(e, "engine occupancy");
     e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return cuda_error(e, "SM count");
@@ -164,90 +257,58 @@ qcw_status engine_prepare(int dev, size_t smem, int *grid)
 }
 
 // ------------------------------------------------------------------ host: programs
-// Cost model (SM-seconds per element of rho), from GB300 measurements of k_fused_pass: one
-// pass moves 16 bytes per element at ~44 GB/s per SM (6.67 TB/s / 152); a two-qubit phase
-// costs ~0.54 ns per element per SM (64 FP32 FMA at the measured issue efficiency), a
-// one-qubit phase about a quarter of that.
-static const double kCostPass = 16.0 / 44e9;
-static const double kCostPhase2 = 0.54e-9;
-static const double kCostPhase1 = 0.15e-9;
+// Cost model (SM-seconds per coefficient), from the pass kernel at 14 qubits: 344 us for a pass's one
+// read and one write of 2^28 coefficients on 152 SMs, 68 us per round with its operations.
+static const double kCostPass = 0.195e-9;
+static const double kCostRound = 0.038e-9;
 
-double model_cost(const TilePlan &tp, int n)
+static size_t pass_smem(int t, int nround, int nop, int ncoef)
 {
-    double el = (double)(1ull << (2 * n));
-    double c = 0;
-    for (const FPass &p : tp.passes) c += kCostPass * el;
-    for (const FPhase &f : tp.phases)
-        c += (f.nq == PH_TWO ? kCostPhase2 : f.nq == PH_PRODUCT ? 2 * kCostPhase1 : kCostPhase1) * el;
-    return c;
+    return (sizeof(float) << (2 * t)) + sizeof(PRound) * nround + 4 * (size_t)((nop + 3) & ~3) + sizeof(float2) * ncoef;
 }
 
-int choose_fuse_k(const std::vector<QOp> &ops, size_t b, size_t e, int n, int tbmax)
-{
-    int best = n < 5 ? n : 5;
-    double bc = -1;
-    for (int k = 2; k <= 5 && k <= n; k++) {
-        TilePlan tp;
-        append_tile_plan(plan_passes(ops, b, e, n, k, true), n, tbmax, tp);
-        double c = model_cost(tp, n);
-        if (bc < 0 || c < bc) {
-            bc = c;
-            best = k;
-        }
-    }
-    return best;
-}
+size_t engine_max_smem() { return pass_smem(kPTile, kPMaxRounds, kPMaxOps, kPMaxCoef); }
 
-Program make_program(const std::vector<QOp> &ops, int n, int fuse_k, int tbmax)
+Program make_program(const qcw_op *ops, int nops, const double *matrices, int n, int fuse_k)
 {
     Program p;
+    PauliPlan plan = plan_pauli_list(ops, nops, matrices, n, fuse_k);
     p.n = n;
-    p.tbmax = tbmax;
-    p.whole = 2 * n <= tbmax;
-    std::vector<PassPlan> plan;
-    if (p.whole) {
-        p.k = n;
-        plan = plan_passes(ops, 0, ops.size(), n, n);
-        if (plan.empty()) plan.emplace_back();
-        plan.resize(1);  // with k = n every op joins the first pass
-        plan[0].Q.clear();
-        for (int q = 0; q < n; q++) plan[0].Q.push_back(q);
-    } else {
-        p.k = fuse_k ? std::min(fuse_k, n) : choose_fuse_k(ops, 0, ops.size(), n, tbmax);
-        plan = plan_passes(ops, 0, ops.size(), n, p.k);
-        if (plan.empty()) plan.emplace_back();  // an empty pass still writes the initial state
+    p.nd = plan.nd;
+    p.whole = p.nd <= kPTile;
+    if (plan.passes.empty()) {  // an empty pass still writes the initial state
+        PPass ps;
+        ps.t = std::min(p.nd, kPTile);
+        for (int d = 0; d < p.nd; d++) (d < ps.t ? ps.td : ps.od).push_back(d);
+        plan.passes.push_back(ps);
     }
-    append_tile_plan(plan, n, tbmax, p.tp);
-    p.cost = model_cost(p.tp, n);
+    for (const PPass &ps : plan.passes) {
+        PassDesc D;
+        D.h = pauli_header(ps);
+        const size_t nr = sizeof(PRound) * ps.rounds.size(), no = 4 * (size_t)((ps.ops.size() + 3) & ~(size_t)3);
+        const size_t nc = sizeof(float) * ((ps.coefs.size() + 3) & ~(size_t)3);
+        D.bytes = (int)(sizeof D + nr + no + nc);
+        const size_t at = p.desc.size();
+        p.pass_off.push_back(at);
+        p.desc.resize(at + D.bytes, 0);
+        char *w = p.desc.data() + at;
+        memcpy(w, &D, sizeof D);
+        if (nr) memcpy(w + sizeof D, ps.rounds.data(), nr);
+        if (!ps.ops.empty()) memcpy(w + sizeof D + nr, ps.ops.data(), sizeof(POp) * ps.ops.size());
+        if (!ps.coefs.empty()) memcpy(w + sizeof D + nr + no, ps.coefs.data(), sizeof(float) * ps.coefs.size());
+        p.tiles.push_back(1u << (2 * ps.od.size()));
+        p.smem = std::max(p.smem, pass_smem(ps.t, (int)ps.rounds.size(), (int)ps.ops.size(), (int)ps.coefs.size()));
+        p.dense |= pass_dense(ps);
+        p.rounds += (long long)ps.rounds.size();
+        p.cost += (double)program_elems(n) * (kCostPass + kCostRound * (double)ps.rounds.size());
+    }
     return p;
 }
 
-static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
-
-size_t program_desc_bytes(const Program &p)
-{
-    return al256(sizeof(FPass) * p.tp.passes.size()) + al256(sizeof(FPhase) * p.tp.phases.size()) +
-           al256(sizeof(float2) * p.tp.coefs.size());
-}
-
-void program_write_desc(Program &p, char *host, size_t off)
-{
-    p.off_pass = off;
-    memcpy(host + off, p.tp.passes.data(), sizeof(FPass) * p.tp.passes.size());
-    off += al256(sizeof(FPass) * p.tp.passes.size());
-    p.off_phase = off;
-    if (!p.tp.phases.empty()) memcpy(host + off, p.tp.phases.data(), sizeof(FPhase) * p.tp.phases.size());
-    off += al256(sizeof(FPhase) * p.tp.phases.size());
-    p.off_coef = off;
-    if (!p.tp.coefs.empty()) memcpy(host + off, p.tp.coefs.data(), sizeof(float2) * p.tp.coefs.size());
-}
-
-void program_items(const Program &p, float2 *rho, const char *desc, unsigned *counters, double *red, int pass_begin,
+void program_items(const Program &p, float *v, const char *desc, unsigned *counters, double *red, int pass_begin,
                    int pass_end, bool init, bool readout, std::vector<std::vector<WItem>> &levels, int *nchunks)
 {
-    const FPass *dpass = reinterpret_cast<const FPass *>(desc + p.off_pass);
-    const FPhase *dph = reinterpret_cast<const FPhase *>(desc + p.off_phase);
-    const float2 *dco = reinterpret_cast<const float2 *>(desc + p.off_coef);
+    const char *base = desc + p.off;
     *nchunks = 0;
     auto level = [&](size_t l) -> std::vector<WItem> & {
         if (levels.size() <= l) levels.resize(l + 1);
@@ -255,13 +316,10 @@ void program_items(const Program &p, float2 *rho, const char *desc, unsigned *co
     };
     if (p.whole) {
         WItem w{};
-        w.rho = rho;
-        w.pass = dpass;
-        w.phases = dph;
-        w.coefs = dco;
-        w.npass = (int)p.tp.passes.size();
+        w.v = v;
+        w.pass = base;
+        w.npass = (int)p.tiles.size();
         w.kind = WI_WHOLE;
-        w.flags = init ? WF_INIT : 0;
         w.n = p.n;
         w.red = readout ? red : nullptr;
         level(0).push_back(w);
@@ -269,45 +327,58 @@ void program_items(const Program &p, float2 *rho, const char *desc, unsigned *co
         return;
     }
     for (int ps = pass_begin; ps < pass_end; ps++) {
-        unsigned nt = program_tiles(p, ps);
-        for (unsigned t = 0; t < nt; t++) {
+        for (unsigned t = 0; t < p.tiles[ps]; t++) {
             WItem w{};
-            w.rho = rho;
-            w.pass = dpass + ps;
-            w.phases = dph;
-            w.coefs = dco;
-            w.tile0 = t;
-            w.ntile = 1;
+            w.v = v;
+            w.pass = base + p.pass_off[ps];
+            w.tile = t;
+            w.npass = 1;
             w.kind = WI_TILES;
             w.flags = (init && ps == 0) ? WF_INIT : 0;
             w.n = p.n;
             if (ps > pass_begin) {
                 w.dep = counters + (ps - 1 - pass_begin);
-                w.dep_target = program_tiles(p, ps - 1);
+                w.dep_target = p.tiles[ps - 1];
             }
             w.done = counters + (ps - pass_begin);
             level(ps - pass_begin).push_back(w);
         }
     }
-    if (readout && pass_end == (int)p.tp.passes.size()) {
-        unsigned long long rows = reduce_rows(p.n), dim = 1ull << p.n;
+    if (readout && pass_end == (int)p.tiles.size()) {
+        const unsigned long long total = program_elems(p.n);
         int c = 0;
-        for (unsigned long long r0 = 0; r0 < dim; r0 += rows, c++) {
+        for (unsigned long long e0 = 0; e0 < total; e0 += kReduceElems, c++) {
             WItem w{};
-            w.rho = rho;
+            w.v = v;
             w.kind = WI_REDUCE;
             w.n = p.n;
             w.red = red + (size_t)c * kRedVals;
-            w.red_row0 = r0;
-            w.red_rows = rows;
+            w.e0 = e0;
+            w.ecount = std::min(kReduceElems, total - e0);
             if (pass_end > pass_begin) {
                 w.dep = counters + (pass_end - 1 - pass_begin);
-                w.dep_target = program_tiles(p, pass_end - 1);
+                w.dep_target = p.tiles[pass_end - 1];
             }
             level(pass_end - pass_begin).push_back(w);
         }
         *nchunks = c;
     }
+}
+
+size_t program_scratch(int n) { return program_elems(n) * (sizeof(float) + sizeof(float2)); }
+
+cudaError_t program_rho(const float *v, int n, void *scratch, float2 *host, cudaStream_t s)
+{
+    const size_t el = program_elems(n);
+    const int nd = std::max(n, kPMinDigits);
+    float2 *rho = static_cast<float2 *>(scratch);
+    float *w = reinterpret_cast<float *>(rho + el);
+    cudaError_t e = cudaMemcpyAsync(w, v, sizeof(float) * el, cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess) e = launch_pauli_to_rho(w, rho, nd, s);
+    // a padded register's own qubits are the lowest: its rho is the corner where the others are |0>
+    const size_t row = sizeof(float2) << n;
+    if (e == cudaSuccess) e = cudaMemcpy2DAsync(host, row, rho, sizeof(float2) << nd, row, (size_t)1 << n, cudaMemcpyDeviceToHost, s);
+    return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
 }
 
 }  // namespace qcw

@@ -6,35 +6,40 @@
 
 #include <vector>
 
-#include "tile.h"
+#include "pauli_run.h"
 
 namespace qcw {
 
 // Kinds of work item.
 enum : int {
-    WI_TILES = 0,   // tiles [tile0, tile0 + ntile) of one pass of a multi-tile program
-    WI_REDUCE = 1,  // FP64 readouts over rows [red_row0, red_row0 + red_rows) of rho
-    WI_WHOLE = 2,   // a whole program whose rho fits one tile: load once, all passes, readouts, store
+    WI_TILES = 0,   // one tile of one pass of a multi-tile program
+    WI_REDUCE = 1,  // FP64 readouts over a run of elements (trace and P(q = 1) with the first)
+    WI_WHOLE = 2,   // a whole program whose state fits one tile: all passes, readouts, store
 };
 enum : int { WF_INIT = 1 };  // the item's tiles start as |0..0><0..0| instead of being loaded
 
 struct WItem {
-    float2 *rho;
-    const FPass *pass;       // first pass of the item
-    const FPhase *phases;    // phase array of the program
-    const float2 *coefs;     // coefficient array of the program
+    float *v;                // the state's Pauli coefficients
+    const char *pass;        // description of the (first) pass
     unsigned *dep;           // wait until *dep >= dep_target (nullptr: no dependency)
     unsigned *done;          // incremented once the item's stores are complete (nullptr: none)
     double *red;             // readout output (kinds 1, 2): trace re, trace im, purity, p1[n]
-    unsigned long long red_row0, red_rows;
+    unsigned long long e0, ecount;  // kind 1: elements [e0, e0 + ecount)
     unsigned dep_target;
-    unsigned tile0, ntile;
+    unsigned tile;
     int npass;
     int kind;
     int flags;
     int n;
-    int pad;
 };
+
+// A pass in a descriptor buffer: this header, then PRound[nround], POp[nop] (padded to 16 bytes) and
+// float[ncoef] (padded); `bytes` from one pass to the next.
+struct PassDesc {
+    PauliHdr h;
+    int bytes;
+};
+static_assert(sizeof(PassDesc) % 16 == 0, "16-byte sections");
 
 constexpr int kRedVals = 3 + QCW_MAX_QUBITS;  // values per readout block
 
@@ -47,48 +52,53 @@ struct EngineLaunch {
     long long spin_limit;
 };
 
-void engine_launch(const EngineLaunch &L, int grid, size_t smem, cudaStream_t s);
-qcw_status engine_prepare(int dev, size_t smem, int *grid);
+// dense: some pass has dense two-qubit maps.
+void engine_launch(const EngineLaunch &L, bool dense, int grid, size_t smem, cudaStream_t s);
+qcw_status engine_prepare(int dev, bool dense, size_t smem, int *grid);
 
-// A circuit turned into device-ready descriptors.
+// A circuit turned into device-ready descriptors.  Registers below kPMinDigits qubits are padded with
+// qubits in |0> above them: nd digits.
 struct Program {
-    int n = 0, k = 0, tbmax = 13;
-    bool whole = false;      // rho fits one tile: one WI_WHOLE item
-    TilePlan tp;
+    int n = 0, nd = 0;
+    bool whole = false;      // the state fits one tile: one WI_WHOLE item
+    bool dense = false;
+    std::vector<char> desc;  // the passes, PassDesc after PassDesc
+    std::vector<size_t> pass_off;
+    std::vector<unsigned> tiles;  // per pass
+    size_t smem = 0;         // largest need of a pass
+    long long rounds = 0;
     double cost = 0;         // modeled SM-seconds
-    size_t off_pass = 0, off_phase = 0, off_coef = 0;  // offsets inside a descriptor buffer
+    size_t off = 0;          // offset inside a descriptor buffer
 };
 
-// Plan ops for an n-qubit register; fuse_k = 0 lets the cost model choose the width.
-Program make_program(const std::vector<QOp> &ops, int n, int fuse_k, int tbmax);
+// Plan a checked op list for an n-qubit register; fuse_k (0: no bound) bounds the qubits of a pass.
+Program make_program(const qcw_op *ops, int nops, const double *matrices, int n, int fuse_k);
 
-// Modeled cost (SM-seconds) of running a plan; used to choose the fusion width.
-double model_cost(const TilePlan &tp, int n);
-int choose_fuse_k(const std::vector<QOp> &ops, size_t b, size_t e, int n, int tbmax);
+// Elements of an n-qubit program's state.
+inline size_t program_elems(int n) { return (size_t)1 << (2 * (n < kPMinDigits ? kPMinDigits : n)); }
+// Bytes of a program's descriptors in a descriptor buffer.
+inline size_t program_desc_bytes(const Program &p) { return (p.desc.size() + 255) & ~(size_t)255; }
 
-// Bytes a program's descriptors occupy in a descriptor buffer (256-byte aligned sections).
-size_t program_desc_bytes(const Program &p);
-// Copy a program's descriptors to host staging at `base + off` and record the offsets.
-void program_write_desc(Program &p, char *host, size_t off);
-
-// Number of tiles of pass p of a program.
-inline unsigned program_tiles(const Program &p, size_t pass) { return 1u << p.tp.passes[pass].nother; }
-
-// Readout chunks of a multi-tile program (rows per chunk chosen for ~2^17 elements).
-inline unsigned long long reduce_rows(int n)
+// Readout chunks of a multi-tile program: 2^17 elements each.
+constexpr unsigned long long kReduceElems = 1ull << 17;
+inline int program_chunks(const Program &p)
 {
-    unsigned long long rows = (1ull << 17) >> n;
-    if (rows < 1) rows = 1;
-    if (rows > (1ull << n)) rows = 1ull << n;
-    return rows;
+    return p.whole ? 1 : (int)((program_elems(p.n) + kReduceElems - 1) / kReduceElems);
 }
+
+// Shared memory of the engine kernel for any pass a planner can produce.
+size_t engine_max_smem();
 
 // Items of passes [pass_begin, pass_end) of one program.  Appends to `levels[l]` (level = pass
 // index - pass_begin; readouts on the level after the last pass).  desc: device base of the
 // descriptor buffer holding the program; counters: (pass_end - pass_begin) zeroed device
 // counters, one per pass of the range; red: its readout blocks (chunk count in *nchunks).
-void program_items(const Program &p, float2 *rho, const char *desc, unsigned *counters, double *red,
-                   int pass_begin, int pass_end, bool init, bool readout, std::vector<std::vector<WItem>> &levels,
-                   int *nchunks);
+void program_items(const Program &p, float *v, const char *desc, unsigned *counters, double *red, int pass_begin,
+                   int pass_end, bool init, bool readout, std::vector<std::vector<WItem>> &levels, int *nchunks);
+
+// rho of a program's state (2^n x 2^n, complex64) into scratch (program_scratch bytes, device) and from
+// there to the host; v is left as it is.
+size_t program_scratch(int n);
+cudaError_t program_rho(const float *v, int n, void *scratch, float2 *host, cudaStream_t s);
 
 }  // namespace qcw

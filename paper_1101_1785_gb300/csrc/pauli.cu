@@ -176,10 +176,16 @@ static cudaError_t launch_pass(const PauliBlob &B, float *v, unsigned ntiles, un
     return cudaGetLastError();
 }
 
-PauliBlob pauli_blob(const PPass &p)
+bool pass_dense(const PPass &p)
 {
-    PauliBlob B;
-    PauliHdr &h = B.h;
+    for (const POp &o : p.ops)
+        if (o.kind >= PO_TWO && o.kind < PO_TWO + 3) return true;
+    return false;
+}
+
+PauliHdr pauli_header(const PPass &p)
+{
+    PauliHdr h;
     memset(&h, 0, sizeof h);
     h.t = p.t;
     h.nod = (int)p.od.size();
@@ -188,10 +194,18 @@ PauliBlob pauli_blob(const PPass &p)
     h.ncoef = (int)p.coefs.size();
     for (size_t i = 0; i < p.td.size(); i++) h.td[i] = (int8_t)p.td[i];
     for (size_t i = 0; i < p.od.size(); i++) h.od[i] = (int8_t)p.od[i];
+    return h;
+}
+
+PauliBlob pauli_blob(const PPass &p)
+{
+    PauliBlob B;
+    B.h = pauli_header(p);
+    B.dense = pass_dense(p);
+    const PauliHdr &h = B.h;
     static_assert(sizeof(PRound) == 96 && sizeof(POp) == 4, "blob layout");
     B.words.assign((size_t)pb_coef(h) + 2 * h.ncoef, 0u);
     memcpy(B.words.data(), p.rounds.data(), sizeof(PRound) * p.rounds.size());
-    for (const POp &o : p.ops) B.dense |= o.kind >= PO_TWO && o.kind < PO_TWO + 3;
     if (h.nop) memcpy(B.words.data() + pb_ops(h), p.ops.data(), sizeof(POp) * p.ops.size());
     for (size_t i = 0; i < p.coefs.size(); i++)
         for (int j = 0; j < 2; j++) memcpy(B.words.data() + pb_coef(h) + 2 * i + j, &p.coefs[i], sizeof(float));

@@ -83,6 +83,9 @@ struct PauliPlan {
 // every qubit of its tile; else on at most kmax qubits.  beam: pass sets by the beam search.
 PauliPlan plan_pauli(const std::vector<QOp> &ops, size_t begin, size_t end, int n, int kmax, bool beam);
 
+// The same for a caller's checked operation list (gates and channels on one and two qubits).
+PauliPlan plan_pauli_list(const qcw_op *ops, int nops, const double *matrices, int n, int kmax);
+
 // Position of 16-byte chunk c of a tile in shared memory: bits 0..2 (which 16 of 128 bytes) are
 // mixed with the bits above so that digits 1..6 of the tile each contribute a different plane of
 // GF(2)^3 there; any two digits then reach all eight positions, and a quarter-warp whose lanes

@@ -58,36 +58,60 @@ bool m4_tp(const M4 &a)  // first row (1, 0, 0, 0): keeps the trace
            std::fabs(a.m[3]) < 1e-13;
 }
 
-M4 one_map(const QOp &op)
+// Real map of a one-qubit superoperator S (S[2 r' + c'][2 r + c]) on the labels:
+// T_ij = Tr[P_i S(P_j)] / 2, with P = I, Z, X, Y read off rows and columns of S directly.
+// Entries below 1e-14 are rounding residue of exact zeros.
+M4 super_map(const c128 *S)
 {
-    c128 S[16];
-    if (op.kind != 0) {
-        for (int i = 0; i < 16; i++) S[i] = op.m[i];
-    } else {
-        const c128 *u = op.m.data();
-        for (int r2 = 0; r2 < 2; r2++)
-            for (int c2 = 0; c2 < 2; c2++)
-                for (int r = 0; r < 2; r++)
-                    for (int c = 0; c < 2; c++)
-                        S[(2 * r2 + c2) * 4 + 2 * r + c] = u[2 * r2 + r] * std::conj(u[2 * c2 + c]);
+    double cr[4][4], ci[4][4];  // S applied to P_j, element e (for Y: to Y / -i)
+    for (int e = 0; e < 4; e++) {
+        const c128 *r = S + 4 * e;
+        cr[e][0] = r[0].real() + r[3].real(), ci[e][0] = r[0].imag() + r[3].imag();
+        cr[e][1] = r[0].real() - r[3].real(), ci[e][1] = r[0].imag() - r[3].imag();
+        cr[e][2] = r[1].real() + r[2].real(), ci[e][2] = r[1].imag() + r[2].imag();
+        // Y = -i (b01 - b10): real part of -i z is Im z, imaginary part -Re z
+        cr[e][3] = r[1].imag() - r[2].imag(), ci[e][3] = r[2].real() - r[1].real();
     }
-    double R[4][4];
-    pauli_transfer1(S, R);
     M4 t;
     t.id = false;
-    for (int i = 0; i < 4; i++)
-        for (int j = 0; j < 4; j++) t.m[4 * kLab[i] + kLab[j]] = 2.0 * R[i][j];
+    for (int j = 0; j < 4; j++) {
+        t.m[j] = 0.5 * (cr[0][j] + cr[3][j]);
+        t.m[4 + j] = 0.5 * (cr[0][j] - cr[3][j]);
+        t.m[8 + j] = 0.5 * (cr[1][j] + cr[2][j]);
+        t.m[12 + j] = 0.5 * (ci[2][j] - ci[1][j]);  // Re of i (s01 - s10)
+    }
+    for (double &x : t.m)
+        if (std::fabs(x) < 1e-14) x = 0.0;
     return t;
 }
 
+// A queued operation or one of a caller's list: kind 0 with U, 1 with its superoperator.
+struct OpView {
+    int kind, k;
+    const int *qubits;
+    const c128 *m;
+};
+
+M4 one_map(const OpView &op)
+{
+    if (op.kind != 0) return super_map(op.m);
+    c128 S[16];
+    const c128 *u = op.m;
+    for (int r2 = 0; r2 < 2; r2++)
+        for (int c2 = 0; c2 < 2; c2++)
+            for (int r = 0; r < 2; r++)
+                for (int c = 0; c < 2; c++) S[(2 * r2 + c2) * 4 + 2 * r + c] = u[2 * r2 + r] * std::conj(u[2 * c2 + c]);
+    return super_map(S);
+}
+
 // Real 16 x 16 map of a two-qubit operation, index 4 p_first + p_second.
-void two_map(const QOp &op, double *T)
+void two_map(const OpView &op, double *T)
 {
     std::vector<c128> S(256);
     if (op.kind != 0) {
         for (int i = 0; i < 256; i++) S[i] = op.m[i];
     } else {
-        const c128 *u = op.m.data();
+        const c128 *u = op.m;
         for (int r2 = 0; r2 < 4; r2++)
             for (int c2 = 0; c2 < 4; c2++)
                 for (int r = 0; r < 4; r++)
@@ -183,12 +207,12 @@ std::vector<double> matmul16(const std::vector<double> &A, const std::vector<dou
 }
 
 // Exactly CNOT (*a, *b in order control, target) or CZ.
-int classify(const QOp &op, int *a, int *b)
+int classify(const OpView &op, int *a, int *b)
 {
     *a = op.qubits[0];
     *b = op.qubits[1];
     if (op.kind != 0) return PO_TWO;
-    const c128 *u = op.m.data();
+    const c128 *u = op.m;
     auto is = [&](const int *col, const double *val) {
         for (int i = 0; i < 4; i++)
             for (int j = 0; j < 4; j++)
@@ -225,19 +249,28 @@ void round_map(M4 &a, double &c)
     if (den > 0) c += num / den - 1.0;
 }
 
-std::vector<Node> make_nodes(const std::vector<QOp> &ops, size_t begin, size_t end, int n)
-{
+class NodeBuilder {
+  public:
+    explicit NodeBuilder(int n) : n(n), last(n, -1), pre(n, m4_identity()) {}
+    void add(const OpView &op);
+    std::vector<Node> finish();
+
+  private:
+    int n;
     std::vector<Node> out;
-    std::vector<int> last(n, -1);
-    std::vector<M4> pre(n, m4_identity());
-    for (size_t i = begin; i < end; i++) {
-        const QOp &op = ops[i];
+    std::vector<int> last;
+    std::vector<M4> pre;
+};
+
+void NodeBuilder::add(const OpView &op)
+{
+    {
         if (op.k == 1) {
             const int q = op.qubits[0];
             const M4 m = one_map(op);
             if (last[q] < 0) m4_lmul(pre[q], m);
             else m4_lmul(out[last[q]].a == q ? out[last[q]].A : out[last[q]].B, m);
-            continue;
+            return;
         }
         int a, b;
         const int kind = classify(op, &a, &b);
@@ -254,7 +287,7 @@ std::vector<Node> make_nodes(const std::vector<QOp> &ops, size_t begin, size_t e
             nd.T = matmul16(T2, node_matrix(nd));
             nd.kind = PO_TWO;
             nd.A = nd.B = m4_identity();
-            continue;
+            return;
         }
         Node nd{kind, a, b, m4_identity(), m4_identity(), {}};
         if (kind == PO_TWO) {
@@ -274,6 +307,10 @@ std::vector<Node> make_nodes(const std::vector<QOp> &ops, size_t begin, size_t e
         last[a] = last[b] = (int)out.size();
         out.push_back(std::move(nd));
     }
+}
+
+std::vector<Node> NodeBuilder::finish()
+{
     std::vector<Node> fin;
     for (int q = 0; q < n; q++)
         if (!pre[q].id) fin.push_back(Node{PO_ONE, q, -1, pre[q], m4_identity(), {}});
@@ -398,13 +435,12 @@ void emit(PPass &ps, const Node &nd, bool maps_only, F dig)
 
 }  // namespace
 
-PauliPlan plan_pauli(const std::vector<QOp> &ops, size_t begin, size_t end, int n, int kmax, bool beam)
+static PauliPlan plan_nodes(std::vector<Node> nodes, int n, int kmax, bool beam)
 {
     PauliPlan plan;
     plan.n = n;
     plan.nd = std::max(n, kPMinDigits);
     const int nd = plan.nd, t = std::min(nd, kPTile);
-    std::vector<Node> nodes = make_nodes(ops, begin, end, n);
     auto digit = [&](int q) { return n - 1 - q; };
     std::vector<unsigned> mask(nodes.size());
     for (size_t i = 0; i < nodes.size(); i++) {
@@ -510,6 +546,43 @@ PauliPlan plan_pauli(const std::vector<QOp> &ops, size_t begin, size_t end, int 
         rem.swap(rest);
     }
     return plan;
+}
+
+PauliPlan plan_pauli(const std::vector<QOp> &ops, size_t begin, size_t end, int n, int kmax, bool beam)
+{
+    NodeBuilder nb(n);
+    for (size_t i = begin; i < end; i++) nb.add(OpView{ops[i].kind, ops[i].k, ops[i].qubits, ops[i].m.data()});
+    return plan_nodes(nb.finish(), n, kmax, beam);
+}
+
+PauliPlan plan_pauli_list(const qcw_op *ops, int nops, const double *matrices, int n, int kmax)
+{
+    NodeBuilder nb(n);
+    c128 S[256];
+    for (int i = 0; i < nops; i++) {
+        const qcw_op &o = ops[i];
+        const c128 *m = reinterpret_cast<const c128 *>(matrices + o.offset);
+        if (o.kind != QCW_OP_KRAUS) {
+            nb.add(OpView{0, o.k, o.qubits, m});
+            continue;
+        }
+        const int d = 1 << o.k, D = d * d;  // sum_j K_j (x) conj K_j
+        for (int e = 0; e < D * D; e++) S[e] = 0;
+        for (int j = 0; j < o.nkraus; j++, m += D)
+            for (int r2 = 0; r2 < d; r2++)
+                for (int c2 = 0; c2 < d; c2++)
+                    for (int r = 0; r < d; r++) {
+                        const double a = m[r2 * d + r].real(), b = m[r2 * d + r].imag();
+                        if (a == 0 && b == 0) continue;
+                        c128 *row = S + (r2 * d + c2) * D + r * d;
+                        for (int c = 0; c < d; c++) {
+                            const double x = m[c2 * d + c].real(), y = m[c2 * d + c].imag();
+                            row[c] += c128(a * x + b * y, b * x - a * y);
+                        }
+                    }
+        nb.add(OpView{1, o.k, o.qubits, S});
+    }
+    return plan_nodes(nb.finish(), n, kmax, false);
 }
 
 }  // namespace qcw

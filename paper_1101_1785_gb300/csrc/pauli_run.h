@@ -19,6 +19,8 @@ struct PauliBlob {
     std::vector<unsigned> words;
 };
 PauliBlob pauli_blob(const PPass &p);
+PauliHdr pauli_header(const PPass &p);
+bool pass_dense(const PPass &p);  // has dense two-qubit maps
 unsigned pauli_grid(const PauliHdr &h, int nsm);
 
 // One pass over v (nd digits).  init: v is |0..0><0..0| and not read.  ppart (2 pauli_grid values):

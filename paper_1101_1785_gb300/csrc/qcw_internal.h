@@ -223,6 +223,8 @@ qcw_status pauli_settle(qcw_ctx *c);
 // rho is about to be overwritten from outside the queue: drop queued work, mark the storage
 // full, bump the state version and clear the error word.
 qcw_status begin_state_replace(qcw_ctx *c);
+// The checks of an op list against an n-qubit register alone.
+qcw_status check_ops(int n, const qcw_op *ops, int nops, const double *matrices, bool validate = false);
 // Validate an op list against an n-qubit register and convert it to queued operations
 // (Kraus sets become superoperators); nothing is appended on error.
 qcw_status convert_ops(int n, const qcw_op *ops, int nops, const double *matrices, std::vector<QOp> &out,

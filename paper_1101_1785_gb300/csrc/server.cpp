@@ -81,8 +81,7 @@ int floor_log2(size_t x)
 struct Request {
     long long id = 0;
     int n = 0;
-    Program prog;
-    std::vector<char> hdesc;  // host copy of the descriptors (kept until the upload completes)
+    Program prog;  // its descriptors are kept until the upload completes
     size_t rho_off = 0, desc_off = 0, red_off = 0;
     int rho_order = 0, desc_order = 0, red_order = 0;
     int next_pass = 0;
@@ -108,7 +107,7 @@ struct qcw_server {
     long long spin_limit = 20000000;
     double wait_limit_s = 30.0;
     // device pools
-    float2 *arena = nullptr;
+    float *arena = nullptr;
     char *desc = nullptr;
     double *red = nullptr, *hred = nullptr;
     Buddy arena_alloc, desc_alloc, red_alloc;
@@ -168,8 +167,8 @@ extern "C" qcw_status qcw_server_create(size_t budget_bytes, int max_live, int p
     s->budget = budget_bytes;
     s->max_live = max_live;
     s->passes_per_step = passes_per_step;
-    // rho storage is 8 * 4^n bytes against a 16 * 4^n footprint: the arena is half the budget
-    int arena_order = floor_log2(budget_bytes / 2);
+    // a state is 4 * 4^n bytes of Pauli coefficients against a 16 * 4^n footprint: a quarter of the budget
+    int arena_order = floor_log2(budget_bytes / 4);
     s->arena_alloc.init(8, arena_order);
     int desc_order = 26;  // 64 MiB of plan descriptors
     s->desc_alloc.init(8, desc_order);
@@ -178,7 +177,7 @@ extern "C" qcw_status qcw_server_create(size_t budget_bytes, int max_live, int p
     s->red_alloc.init(8, red_order);
     s->max_items = 1 << 20;
     s->max_counters = 1 << 20;
-    s->smem = tile_smem_bytes(13, 3);
+    s->smem = engine_max_smem();
     qcw_status st = QCW_OK;
     cudaError_t e = cudaGetDevice(&s->dev);
     if (e != cudaSuccess) st = cuda_error(e, "cudaGetDevice");
@@ -194,7 +193,8 @@ extern "C" qcw_status qcw_server_create(size_t budget_bytes, int max_live, int p
         cudaGetLastError();
         st = set_error(QCW_ENOMEM, "server buffers");
     }
-    if (!st) st = engine_prepare(s->dev, s->smem, &s->grid);
+    if (!st) st = engine_prepare(s->dev, true, s->smem, &s->grid);
+    if (!st) st = engine_prepare(s->dev, false, s->smem, &s->grid);
     if (!st) {
         e = cudaEventCreateWithFlags(&s->done, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaMemset(s->counters + s->max_counters, 0, sizeof(unsigned));
@@ -214,16 +214,13 @@ extern "C" qcw_status qcw_server_submit(qcw_server *s, int nqubits, const qcw_op
     if (!s) return set_error(QCW_EINVAL, "null server");
     if (nqubits < 1 || nqubits > 13) return set_error(QCW_EINVAL, "served requests take 1..13 qubits");
     if (((size_t)16 << (2 * nqubits)) > s->budget) return set_error(QCW_EINVAL, "request larger than the budget");
-    std::vector<QOp> q;
-    qcw_status st = convert_ops(nqubits, ops, nops, matrices, q);
+    qcw_status st = check_ops(nqubits, ops, nops, matrices);
     if (st) return st;
-    for (QOp &o : q)
-        if (o.k > 2) return set_error(QCW_ENOTSUP, "served circuits take 1- and 2-qubit operations");
+    for (int i = 0; i < nops; i++)
+        if (ops[i].k > 2) return set_error(QCW_ENOTSUP, "served circuits take 1- and 2-qubit operations");
     Request *r = new Request();
     r->n = nqubits;
-    r->prog = make_program(q, nqubits, 0, 13);
-    r->hdesc.assign(program_desc_bytes(r->prog), 0);
-    program_write_desc(r->prog, r->hdesc.data(), 0);
+    r->prog = make_program(ops, nops, matrices, nqubits, 0);
     r->t_submit = now_s();
     std::lock_guard<std::mutex> lk(s->mu);
     r->id = s->next_id++;
@@ -297,13 +294,13 @@ extern "C" qcw_status qcw_server_step(qcw_server *s, int *launched_items)
             Request *r = s->waiting.front();
             size_t fp = (size_t)16 << (2 * r->n);
             if (s->used + fp > s->budget) break;
-            size_t rho_bytes = std::max<size_t>((size_t)8 << (2 * r->n), 256);
+            size_t rho_bytes = sizeof(float) * program_elems(r->n);
             if (!s->arena_alloc.alloc(rho_bytes, &r->rho_off, &r->rho_order)) break;
-            if (!s->desc_alloc.alloc(r->hdesc.size(), &r->desc_off, &r->desc_order)) {
+            if (!s->desc_alloc.alloc(program_desc_bytes(r->prog), &r->desc_off, &r->desc_order)) {
                 s->arena_alloc.release(r->rho_off, r->rho_order);
                 break;
             }
-            int chunks = r->prog.whole ? 1 : (int)(((1ull << r->n) + reduce_rows(r->n) - 1) / reduce_rows(r->n));
+            const int chunks = program_chunks(r->prog);
             if (!s->red_alloc.alloc(sizeof(double) * kRedVals * chunks, &r->red_off, &r->red_order)) {
                 s->arena_alloc.release(r->rho_off, r->rho_order);
                 s->desc_alloc.release(r->desc_off, r->desc_order);
@@ -313,7 +310,7 @@ extern "C" qcw_status qcw_server_step(qcw_server *s, int *launched_items)
             s->used += fp;
             s->waiting.pop_front();
             r->t_admit = now_s();
-            cudaError_t e = cudaMemcpyAsync(s->desc + r->desc_off, r->hdesc.data(), r->hdesc.size(),
+            cudaError_t e = cudaMemcpyAsync(s->desc + r->desc_off, r->prog.desc.data(), r->prog.desc.size(),
                                             cudaMemcpyHostToDevice, s->stream);
             s->live.push_back(r);
             if (e != cudaSuccess) return cuda_error(e, "descriptor upload");
@@ -325,12 +322,12 @@ extern "C" qcw_status qcw_server_step(qcw_server *s, int *launched_items)
     size_t ncount = 0;
     for (Request *r : s->live) {
         const Program &p = r->prog;
-        const int np = (int)p.tp.passes.size();
+        const int np = (int)p.tiles.size();
         const int p0 = r->next_pass, p1 = p.whole ? np : std::min(np, p0 + s->passes_per_step);
         const bool readout = p.whole || p1 == np;
         if (!p.whole && ncount + np > s->max_counters) continue;  // waits for the next step
         int nch = 0;
-        program_items(p, s->arena + r->rho_off / sizeof(float2), s->desc + r->desc_off, s->counters + ncount,
+        program_items(p, s->arena + r->rho_off / sizeof(float), s->desc + r->desc_off, s->counters + ncount,
                       s->red + r->red_off / sizeof(double), p0, p1, p0 == 0, readout, levels, &nch);
         if (!p.whole) ncount += (size_t)(p1 - p0);
         r->finishing = readout;
@@ -359,7 +356,9 @@ extern "C" qcw_status qcw_server_step(qcw_server *s, int *launched_items)
     if (e == cudaSuccess) e = cudaMemsetAsync(s->dint + 1, 0, 2 * sizeof(int), s->stream);
     if (e == cudaSuccess && ncount) e = cudaMemsetAsync(s->counters, 0, sizeof(unsigned) * ncount, s->stream);
     if (e != cudaSuccess) return cuda_error(e, "step upload");
-    engine_launch(L, s->grid, s->smem, s->stream);
+    bool dense = false;
+    for (const Request *r : s->live) dense |= r->prog.dense;
+    engine_launch(L, dense, s->grid, s->smem, s->stream);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "engine launch");
     for (Request *r : s->live)
