@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cstddef>
 #include <cstring>
+#include <type_traits>
 
 #include "pauli.cuh"
 #include "pauli_run.h"
@@ -288,34 +289,80 @@ struct alignas(16) F4 {
 __device__ __forceinline__ F4 operator+(F4 a, F4 b) { return F4{a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w}; }
 __device__ __forceinline__ F4 operator-(F4 a, F4 b) { return F4{a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w}; }
 
-constexpr int kCvThreads = 256;
 constexpr int kCvLow = 7;  // qubits transformed by the emit / absorb stage
 
-// In place over the z bits of the `hi` high qubits: a CTA owns one x of them and a run of 4 * 2^rb
-// low elements (2^hi rows of that run in shared memory).  sign_in: apply s first, sign_out: last.
-__global__ void __launch_bounds__(kCvThreads) k_pauli_high(float *__restrict__ v, int hi, int low, int rb, int sign_in,
+// In place over the z bits of the `hi` high qubits.  A CTA owns one x of them and a run of 4 * 2^rb
+// low elements: 2^hi rows of that run, 2048 chunks (4096 at hi = 10) in shared memory.  A thread
+// loads 16 chunks and transforms them in registers (the top row bits), then the rest takes one trip
+// through shared memory (two from hi = 8 up).  Bound by HBM if the integer work per chunk is small,
+// hence the offsets split into a thread's and a chunk number's part: n = 14 (2.15 GB) 0.57 ms with
+// the general index arithmetic for every chunk and radix-8 steps all through shared memory.
+constexpr int kHiThreads = 128;
+__global__ void __launch_bounds__(kHiThreads) k_pauli_high(float *__restrict__ v, int hi, int low, int rb, int sign_in,
                                                            int sign_out)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     F4 *sm = reinterpret_cast<F4 *>(smem);
     const unsigned nrun = 1u << (2 * low - 2 - rb);  // runs of a row
-    const unsigned run = blockIdx.x % nrun, xa = blockIdx.x / nrun;
+    const unsigned run = blockIdx.x % nrun, xa = blockIdx.x / nrun, rmask = (1u << rb) - 1u;
+    const int ebits = hi + rb;                       // chunk index e: row above rb bits of the run
     const uint64_t xo = p_spread(xa) << (2 * low + 1);
-    const unsigned rows = 1u << hi, nv = rows << rb, rmask = (1u << rb) - 1u;
     auto at = [&](unsigned e) {
         return xo + (p_spread(e >> rb) << (2 * low)) + 4ull * (((uint64_t)run << rb) + (e & rmask));
     };
-    for (unsigned e = threadIdx.x; e < nv; e += kCvThreads) {
-        const uint64_t g = at(e);
-        F4 a = *reinterpret_cast<const F4 *>(v + g);
-        if (sign_in) p_signs4(a, g);
-        sm[e] = a;
+    auto low_count = [&](unsigned e) {  // |x & z| of the low qubits
+        const unsigned l = 4u * ((run << rb) + (e & rmask));
+        return __popc(l & (l >> 1) & 0x55555555u);
+    };
+    auto signs = [&](F4 &a, unsigned k) {
+        if ((k + 1) & 2) a.x = -a.x, a.y = -a.y, a.z = -a.z;
+        if ((k + 2) & 2) a.w = -a.w;
+    };
+    const int top = hi < 4 ? hi : 4;  // row bits among the four highest bits of e
+    for (unsigned b0 = 0; b0 < (1u << (ebits - 11)); b0++) {
+        // chunks e = u 2^(ebits - 4) + b0 128 + tid
+        const unsigned e0 = b0 * kHiThreads + threadIdx.x;
+        const int us = ebits - 4 - rb;  // u shifts the row by this (hi >= 4), else the run and the row
+        const uint64_t g0 = at(e0);
+        const unsigned k0 = low_count(e0) + __popc(xa & (e0 >> rb));
+        F4 a[16];
+        if (hi >= 4) {
+            const uint64_t step = 1ull << (2 * us + 2 * low);
+#pragma unroll
+            for (int u = 0; u < 16; u++)
+                a[u] = *reinterpret_cast<const F4 *>(v + g0 + ((u & 1) + 4 * ((u >> 1) & 1) + 16 * ((u >> 2) & 1) + 64 * (u >> 3)) * step);
+            if (sign_in) {
+                const unsigned xu = xa >> us;
+#pragma unroll
+                for (int u = 0; u < 16; u++) signs(a[u], k0 + __popc(xu & u));
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < 16; u++) {
+                const unsigned e = ((unsigned)u << (ebits - 4)) + e0;
+                a[u] = *reinterpret_cast<const F4 *>(v + at(e));
+                if (sign_in) signs(a[u], low_count(e) + __popc(xa & (e >> rb)));
+            }
+        }
+#pragma unroll
+        for (int b = 3; b >= 0; b--)
+            if (3 - b < top)
+#pragma unroll
+                for (int u = 0; u < 16; u++)
+                    if (!(u & (1 << b))) {
+                        const F4 x = a[u], y = a[u | (1 << b)];
+                        a[u] = x + y;
+                        a[u | (1 << b)] = x - y;
+                    }
+#pragma unroll
+        for (int u = 0; u < 16; u++) sm[((unsigned)u << (ebits - 4)) + e0] = a[u];
     }
     __syncthreads();
-    for (int b = 0; b < hi; b += 3) {
-        const int nb = hi - b < 3 ? hi - b : 3;
-        const int sh = b + rb;
-        for (unsigned i = threadIdx.x; i < (nv >> nb); i += kCvThreads) {
+    // the lower row bits: three at a time, the last three on the way out
+    int rem = hi - top;
+    for (; rem > 3; rem -= rem - 3 < 3 ? rem - 3 : 3) {
+        const int nb = rem - 3 < 3 ? rem - 3 : 3, sh = rb + rem - nb;
+        for (unsigned i = threadIdx.x; i < (1u << (ebits - nb)); i += kHiThreads) {
             const unsigned lo = i & ((1u << sh) - 1u), base = ((i >> sh) << (sh + nb)) | lo;
             auto ld = [&](int j) { return sm[base + ((unsigned)j << sh)]; };
             auto st = [&](int j, F4 x) { sm[base + ((unsigned)j << sh)] = x; };
@@ -325,178 +372,215 @@ __global__ void __launch_bounds__(kCvThreads) k_pauli_high(float *__restrict__ v
         }
         __syncthreads();
     }
-    for (unsigned e = threadIdx.x; e < nv; e += kCvThreads) {
-        const uint64_t g = at(e);
-        F4 a = sm[e];
-        if (sign_out) p_signs4(a, g);
-        *reinterpret_cast<F4 *>(v + g) = a;
-    }
+    auto out = [&](auto nbc) {
+        constexpr int NB = decltype(nbc)::value;
+        for (unsigned i = threadIdx.x; i < (1u << (ebits - NB)); i += kHiThreads) {
+            const unsigned e0 = ((i >> rb) << (rb + NB)) | (i & rmask);
+            const uint64_t g0 = at(e0);
+            const unsigned k0 = sign_out ? low_count(e0) + __popc(xa & (e0 >> rb)) : 0u;
+            auto ld = [&](int j) { return sm[e0 + ((unsigned)j << rb)]; };
+            auto st = [&](int j, F4 x) {
+                if (sign_out) signs(x, k0 + __popc(xa & j));
+                *reinterpret_cast<F4 *>(v + g0 + ((uint64_t)((j & 1) + 4 * ((j >> 1) & 1) + 16 * (j >> 2)) << (2 * low))) = x;
+            };
+            p_wht<NB, F4>(ld, st);
+        }
+    };
+    if (rem == 3) out(std::integral_constant<int, 3>());
+    else if (rem == 2) out(std::integral_constant<int, 2>());
+    else if (rem == 1) out(std::integral_constant<int, 1>());
+    else out(std::integral_constant<int, 0>());
 }
 
-// Tile of the low stage: high qubits' labels (ra, ca) with ca <= ra (x = ra ^ ca), one value xh of
-// the x bits of low qubits above the four lowest; it holds, for the two rows ra and ca of the
-// transform, W over all z / r bits of the m low qubits and all x bits of the ml lowest.
-constexpr int kCvPitch = 17;                       // floats per r_L (16 x values + 1)
-constexpr int kCvArray = (1 << kCvLow) * kCvPitch;  // one of the two arrays
+// The low stage on M = min(n, 7) qubits.  Tile: high qubits' labels (ra, ca) with ca <= ra (x = ra ^
+// ca), one value xh of the x bits of the low qubits above the four lowest; it holds, for the two rows
+// ra and ca of the transform, W over all z / r bits of the low qubits and all x bits of the ML lowest.
+constexpr int kCvThreads = 256;
+constexpr int kCvPitch = 17;  // floats per r_L (16 x values + 1)
 
+template <int M>
 struct CvTile {
+    static constexpr int ML = M < 4 ? M : 4, MH = M - ML;
+    static constexpr int kArray = (1 << M) * kCvPitch;            // floats of one of the two arrays
+    static constexpr int kChunks = 1 << (MH + 2 * ML - 2);        // 4-element chunks of one array
+    static constexpr int kPairs = 1 << (M + ML - 1);              // element pairs of one block of rho
+    static constexpr int U = (kChunks + kCvThreads - 1) / kCvThreads, UP = (kPairs + kCvThreads - 1) / kCvThreads;
     unsigned ra, ca, xh;
-    int m, ml, mh, narr;
+    int narr;
     uint64_t off[2];  // element offset of the arrays' low part in v
+    unsigned pos0;    // this thread's first chunk: position in an array (labels I, Z, X, Y: + 0, pitch, 1, pitch + 1)
+    unsigned loff0;   // and element offset in v's low part; chunk + u 256 adds cpos(u), coff(u)
+
+    __device__ __forceinline__ explicit CvTile(unsigned blk)
+    {
+        xh = blk & ((1u << MH) - 1u);
+        const unsigned long long p = blk >> MH;
+        unsigned long long c = (unsigned long long)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);
+        while ((c + 1) * (c + 2) / 2 <= p) c++;
+        while (c * (c + 1) / 2 > p) c--;
+        ra = (unsigned)c;
+        ca = (unsigned)(p - c * (c + 1) / 2);
+        narr = ra == ca ? 1 : 2;
+        const uint64_t x = p_spread(ra ^ ca) << 1;
+        off[0] = (x | p_spread(ra)) << (2 * M);
+        off[1] = (x | p_spread(ca)) << (2 * M);
+        const unsigned k = threadIdx.x & (kChunks - 1), lowc = k & ((1u << (2 * ML - 2)) - 1u), zh = k >> (2 * ML - 2);
+        loff0 = (((unsigned)p_spread(zh) | ((unsigned)p_spread(xh) << 1)) << (2 * ML)) + 4u * lowc;
+        unsigned z = 0, xx = 0;
+#pragma unroll
+        for (int d = 0; d < ML - 1; d++) {
+            z |= ((lowc >> (2 * d)) & 1u) << (d + 1);
+            xx |= ((lowc >> (2 * d + 1)) & 1u) << (d + 1);
+        }
+        pos0 = ((zh << ML) | z) * kCvPitch + xx;
+    }
+    // u-th chunk of this thread (U = 2: the second half of the z bits above)
+    static __device__ __forceinline__ unsigned cpos(int u) { return u * (((256u >> (2 * ML - 2)) << ML) * kCvPitch); }
+    static __device__ __forceinline__ unsigned coff(int u) { return u * ((16u) << (2 * ML)); }
+    __device__ __forceinline__ bool has(int u) const { return threadIdx.x + u * kCvThreads < kChunks; }
 };
 
-__device__ __forceinline__ CvTile cv_tile(int n, unsigned blk)
-{
-    CvTile T;
-    T.m = n < kCvLow ? n : kCvLow;
-    T.ml = T.m < 4 ? T.m : 4;
-    T.mh = T.m - T.ml;
-    T.xh = blk & ((1u << T.mh) - 1u);
-    const unsigned long long p = blk >> T.mh;
-    unsigned long long c = (unsigned long long)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);
-    while ((c + 1) * (c + 2) / 2 <= p) c++;
-    while (c * (c + 1) / 2 > p) c--;
-    T.ra = (unsigned)c;
-    T.ca = (unsigned)(p - c * (c + 1) / 2);
-    T.narr = T.ra == T.ca ? 1 : 2;
-    const uint64_t x = p_spread(T.ra ^ T.ca) << 1;
-    T.off[0] = (x | p_spread(T.ra)) << (2 * T.m);
-    T.off[1] = (x | p_spread(T.ca)) << (2 * T.m);
-    return T;
-}
-
 // WHT over the z bits of the low qubits, both arrays.
-__device__ __forceinline__ void cv_transform(const CvTile &T, float *sm)
+template <int M>
+__device__ __forceinline__ void cv_transform(const CvTile<M> &T, float *sm)
 {
-    for (int b = 0; b < T.m; b += 4) {
-        const int nb = T.m - b < 4 ? T.m - b : 4;
-        const unsigned per = 1u << (T.m - nb + T.ml);
+    constexpr int ML = CvTile<M>::ML;
+    auto step = [&](auto bc, auto nbc) {
+        constexpr int B = decltype(bc)::value, NB = decltype(nbc)::value;
+        constexpr unsigned per = 1u << (M - NB + ML);
         for (unsigned i = threadIdx.x; i < per * (unsigned)T.narr; i += kCvThreads) {
-            const unsigned a = i >= per ? 1u : 0u, k = i - a * per;
-            const unsigned xl = k & ((1u << T.ml) - 1u), q = k >> T.ml;
-            const unsigned z0 = ((q >> b) << (b + nb)) | (q & ((1u << b) - 1u));
-            float *p = sm + a * kCvArray + z0 * kCvPitch + xl;
-            const unsigned stp = (unsigned)kCvPitch << b;
+            const unsigned a = i / per, k = i % per, xl = k & ((1u << ML) - 1u), q = k >> ML;
+            const unsigned z0 = ((q >> B) << (B + NB)) | (q & ((1u << B) - 1u));
+            float *p = sm + a * CvTile<M>::kArray + z0 * kCvPitch + xl;
+            constexpr unsigned stp = (unsigned)kCvPitch << B;
             auto ld = [&](int j) { return p[j * stp]; };
             auto st = [&](int j, float x) { p[j * stp] = x; };
-            if (nb == 4) p_wht<4, float>(ld, st);
-            else if (nb == 3) p_wht<3, float>(ld, st);
-            else if (nb == 2) p_wht<2, float>(ld, st);
-            else p_wht<1, float>(ld, st);
+            p_wht<NB, float>(ld, st);
         }
         __syncthreads();
-    }
+    };
+    step(std::integral_constant<int, 0>(), std::integral_constant<int, ML>());
+    if constexpr (M > 4) step(std::integral_constant<int, 4>(), std::integral_constant<int, M - 4>());
 }
 
-// Position in an array, and element offset in v's low part, of chunk k (4 elements: the labels of
-// the lowest qubit) of the tile's 2^mh runs of 4^ml elements.
-__device__ __forceinline__ void cv_chunk(const CvTile &T, unsigned k, unsigned &pos, uint64_t &off)
-{
-    const unsigned lowc = k & ((1u << (2 * T.ml - 2)) - 1u), zh = k >> (2 * T.ml - 2);
-    off = ((p_spread(zh) | (p_spread(T.xh) << 1)) << (2 * T.ml)) + 4u * lowc;
-    unsigned z = 0, x = 0;
-    for (int d = 0; d < T.ml - 1; d++) {
-        z |= ((lowc >> (2 * d)) & 1u) << (d + 1);
-        x |= ((lowc >> (2 * d + 1)) & 1u) << (d + 1);
-    }
-    pos = ((zh << T.ml) | z) * kCvPitch + x;  // labels (I, Z, X, Y): + (0, pitch, 1, pitch + 1)
-}
-
+template <int M>
 __global__ void __launch_bounds__(kCvThreads) k_pauli_emit(const float *__restrict__ v, float2 *__restrict__ rho, int n,
                                                            float scale, int sign)
 {
-    __shared__ float sm[2 * kCvArray];
-    const CvTile T = cv_tile(n, blockIdx.x);
-    const unsigned nch = 1u << (T.mh + 2 * T.ml - 2);
-    for (unsigned i = threadIdx.x; i < nch * (unsigned)T.narr; i += kCvThreads) {
-        const unsigned a = i >= nch ? 1u : 0u;
-        unsigned pos;
-        uint64_t off;
-        cv_chunk(T, i - a * nch, pos, off);
-        off += T.off[a];
-        float4 x = *reinterpret_cast<const float4 *>(v + off);
-        if (sign) p_signs4(x, off);
-        float *p = sm + a * kCvArray + pos;
-        p[0] = x.x, p[kCvPitch] = x.y, p[1] = x.z, p[kCvPitch + 1] = x.w;
+    using C = CvTile<M>;
+    constexpr int ML = C::ML;
+    __shared__ float sm[2 * C::kArray];
+    const C T(blockIdx.x);
+    const float h = 0.5f * scale;
+    {
+        float4 x[2][C::U];  // all loads in flight
+#pragma unroll
+        for (int a = 0; a < 2; a++)
+#pragma unroll
+            for (int u = 0; u < C::U; u++)
+                if (a < T.narr && T.has(u)) x[a][u] = *reinterpret_cast<const float4 *>(v + T.off[a] + T.loff0 + C::coff(u));
+#pragma unroll
+        for (int a = 0; a < 2; a++)
+#pragma unroll
+            for (int u = 0; u < C::U; u++)
+                if (a < T.narr && T.has(u)) {
+                    float4 y = x[a][u];
+                    if (sign) p_signs4(y, T.off[a] + T.loff0 + C::coff(u));
+                    float *p = sm + a * C::kArray + T.pos0 + C::cpos(u);
+                    p[0] = h * y.x, p[kCvPitch] = h * y.y, p[1] = h * y.z, p[kCvPitch + 1] = h * y.w;
+                }
     }
     __syncthreads();
-    cv_transform(T, sm);
-    const float *wa = sm, *wb = T.narr == 2 ? sm + kCvArray : sm;
-    const float h = 0.5f * scale;
-    const unsigned lmask = (1u << T.ml) - 1u, cols = 1u << T.ml, half = cols >> 1;
+    cv_transform<M>(T, sm);
+    // block (ra, ca), then its mirror (ca, ra): rows in turn, two columns per thread; the x bits
+    // row ^ column of a thread's elements are the same in all its rows
+    constexpr unsigned half = 1u << (ML - 1), lmask = (1u << ML) - 1u, rstep = kCvThreads / half;
+    const unsigned row0 = threadIdx.x / half, c0 = 2 * (threadIdx.x % half);
+    const unsigned x0 = (row0 & lmask) ^ c0, x1 = x0 ^ 1u;
     const uint64_t dim = 1ull << n;
-    // block (ra, ca), then its mirror (ca, ra): rows in turn, two columns per thread
-    for (int blkm = 0; blkm < T.narr; blkm++) {
-        const uint64_t rowb = (uint64_t)(blkm ? T.ca : T.ra) << T.m, colb = (uint64_t)(blkm ? T.ra : T.ca) << T.m;
-        for (unsigned i = threadIdx.x; i < (half << T.m); i += kCvThreads) {
-            const unsigned row = i / half, c0 = 2 * (i % half);
-            const unsigned colh = ((row >> T.ml) ^ T.xh) << T.ml;
-            float o[4];
 #pragma unroll
-            for (int j = 0; j < 2; j++) {
-                const unsigned col = colh | (c0 + j), xl = (row ^ col) & lmask;
-                const unsigned r = blkm ? col : row, c = blkm ? row : col;
-                const float A = wa[r * kCvPitch + xl], B = wb[c * kCvPitch + xl];
-                o[2 * j] = h * (A + B);
-                o[2 * j + 1] = blkm ? h * (B - A) : h * (A - B);
-            }
-            *reinterpret_cast<float4 *>(rho + (rowb + row) * dim + colb + colh + c0) = make_float4(o[0], o[1], o[2], o[3]);
+    for (int blkm = 0; blkm < 2; blkm++) {
+        if (blkm == T.narr) break;
+        const float *wr = blkm ? sm + C::kArray : sm, *wc = T.narr == 2 && !blkm ? sm + C::kArray : sm;  // by row, by column
+        float2 *dst = rho + (((uint64_t)(blkm ? T.ca : T.ra) << M) + row0) * dim + ((uint64_t)(blkm ? T.ra : T.ca) << M) + c0;
+        wr += row0 * kCvPitch;
+        wc += c0 * kCvPitch;
+#pragma unroll
+        for (int u = 0; u < C::UP; u++) {
+            const unsigned row = row0 + u * rstep;
+            if (row >= (1u << M)) break;
+            const unsigned colh = ((row >> ML) ^ T.xh) << ML;
+            const float A0 = wr[u * rstep * kCvPitch + x0], A1 = wr[u * rstep * kCvPitch + x1];
+            const float B0 = wc[colh * kCvPitch + x0], B1 = wc[(colh + 1) * kCvPitch + x1];
+            // the imaginary part is (W at the row - W at the column) in block and mirror alike
+            *reinterpret_cast<float4 *>(dst + u * rstep * dim + colh) = make_float4(A0 + B0, A0 - B0, A1 + B1, A1 - B1);
         }
     }
 }
 
 // The lower triangle of rho (r >= c; the diagonal's real part) -> W, transformed over the low qubits.
+template <int M>
 __global__ void __launch_bounds__(kCvThreads) k_pauli_absorb(const float2 *__restrict__ rho, float *__restrict__ v, int n,
                                                              int sign)
 {
-    __shared__ float sm[2 * kCvArray];
-    const CvTile T = cv_tile(n, blockIdx.x);
-    const unsigned lmask = (1u << T.ml) - 1u, cols = 1u << T.ml, half = cols >> 1;
+    using C = CvTile<M>;
+    constexpr int ML = C::ML;
+    __shared__ float sm[2 * C::kArray];
+    const C T(blockIdx.x);
+    constexpr unsigned half = 1u << (ML - 1), lmask = (1u << ML) - 1u, rstep = kCvThreads / half;
+    const unsigned row0 = threadIdx.x / half, c0 = 2 * (threadIdx.x % half);
+    const unsigned x0 = (row0 & lmask) ^ c0, x1 = x0 ^ 1u;
     const uint64_t dim = 1ull << n;
-    const uint64_t rowb = (uint64_t)T.ra << T.m, colb = (uint64_t)T.ca << T.m;
-    float *wa = sm, *wb = T.narr == 2 ? sm + kCvArray : sm;
-    for (unsigned i = threadIdx.x; i < (half << T.m); i += kCvThreads) {
-        const unsigned row = i / half, c0 = 2 * (i % half);
-        const unsigned colh = ((row >> T.ml) ^ T.xh) << T.ml;
-        if (T.narr == 1 && row < (colh | c0)) continue;
-        const float4 x = *reinterpret_cast<const float4 *>(rho + (rowb + row) * dim + colb + colh + c0);
+    const float2 *src = rho + (((uint64_t)T.ra << M) + row0) * dim + ((uint64_t)T.ca << M) + c0;
+    const bool two = T.narr == 2;
+    float *wr = sm + row0 * kCvPitch, *wc = (two ? sm + C::kArray : sm) + c0 * kCvPitch;
+    float4 in[C::UP];  // all loads in flight
 #pragma unroll
-        for (int j = 0; j < 2; j++) {
-            const unsigned col = colh | (c0 + j), xl = (row ^ col) & lmask;
-            const float re = j ? x.z : x.x, im = j ? x.w : x.y;
-            if (T.narr == 1 && row < col) continue;
-            if (T.narr == 1 && row == col) {
-                wa[row * kCvPitch + xl] = re;
-            } else {
-                wa[row * kCvPitch + xl] = re + im;
-                wb[col * kCvPitch + xl] = re - im;
-            }
+    for (int u = 0; u < C::UP; u++) {
+        const unsigned row = row0 + u * rstep, colh = ((row >> ML) ^ T.xh) << ML;
+        if (row < (1u << M) && (two || row >= (colh | c0))) in[u] = *reinterpret_cast<const float4 *>(src + u * rstep * dim + colh);
+    }
+#pragma unroll
+    for (int u = 0; u < C::UP; u++) {
+        const unsigned row = row0 + u * rstep, colh = ((row >> ML) ^ T.xh) << ML, col = colh | c0;
+        if (row >= (1u << M) || (!two && row < col)) continue;
+        const float4 x = in[u];
+        if (!two && row == col) {
+            wr[u * rstep * kCvPitch + x0] = x.x;
+            continue;  // column c0 + 1 lies above the diagonal
         }
+        wr[u * rstep * kCvPitch + x0] = x.x + x.y;
+        wc[colh * kCvPitch + x0] = x.x - x.y;
+        if (!two && row == col + 1) {
+            wr[u * rstep * kCvPitch + x1] = x.z;
+            continue;
+        }
+        wr[u * rstep * kCvPitch + x1] = x.z + x.w;
+        wc[(colh + 1) * kCvPitch + x1] = x.z - x.w;
     }
     __syncthreads();
-    cv_transform(T, sm);
-    const unsigned nch = 1u << (T.mh + 2 * T.ml - 2);
-    for (unsigned i = threadIdx.x; i < nch * (unsigned)T.narr; i += kCvThreads) {
-        const unsigned a = i >= nch ? 1u : 0u;
-        unsigned pos;
-        uint64_t off;
-        cv_chunk(T, i - a * nch, pos, off);
-        off += T.off[a];
-        const float *p = sm + a * kCvArray + pos;
-        float4 x = make_float4(p[0], p[kCvPitch], p[1], p[kCvPitch + 1]);
-        if (sign) p_signs4(x, off);
-        *reinterpret_cast<float4 *>(v + off) = x;
-    }
+    cv_transform<M>(T, sm);
+#pragma unroll
+    for (int a = 0; a < 2; a++)
+#pragma unroll
+        for (int u = 0; u < C::U; u++)
+            if (a < T.narr && T.has(u)) {
+                const float *p = sm + a * C::kArray + T.pos0 + C::cpos(u);
+                float4 y = make_float4(p[0], p[kCvPitch], p[1], p[kCvPitch + 1]);
+                const uint64_t o = T.off[a] + T.loff0 + C::coff(u);
+                if (sign) p_signs4(y, o);
+                *reinterpret_cast<float4 *>(v + o) = y;
+            }
 }
 
 static cudaError_t launch_high(float *v, int n, int sign_in, int sign_out, cudaStream_t s)
 {
     const int hi = n - kCvLow, low = kCvLow;
-    const int rb = std::max(2, std::min(4, 11 - hi));  // runs of 64 floats, 16 for the widest registers
+    const int rb = std::max(2, 11 - hi);  // runs of 64 bytes and more
     const size_t sm = sizeof(F4) << (hi + rb);
     if (ensure_smem_attr(reinterpret_cast<const void *>(k_pauli_high), sm)) return cudaErrorInvalidValue;
     const unsigned blocks = 1u << (hi + 2 * low - 2 - rb);
-    k_pauli_high<<<blocks, kCvThreads, sm, s>>>(v, hi, low, rb, sign_in, sign_out);
+    k_pauli_high<<<blocks, kHiThreads, sm, s>>>(v, hi, low, rb, sign_in, sign_out);
     return cudaGetLastError();
 }
 
@@ -505,6 +589,17 @@ static unsigned cv_blocks(int n)
     const int m = std::min(n, kCvLow), mh = m - std::min(m, 4);
     const unsigned long long M = 1ull << (n - m);
     return (unsigned)((M * (M + 1) / 2) << mh);
+}
+
+template <int M>
+static void emit_m(const float *v, float2 *rho, int n, float scale, int sign, cudaStream_t s)
+{
+    k_pauli_emit<M><<<cv_blocks(n), kCvThreads, 0, s>>>(v, rho, n, scale, sign);
+}
+template <int M>
+static void absorb_m(const float2 *rho, float *v, int n, int sign, cudaStream_t s)
+{
+    k_pauli_absorb<M><<<cv_blocks(n), kCvThreads, 0, s>>>(rho, v, n, sign);
 }
 
 int pauli_convert_launches(int n) { return n > kCvLow ? 2 : 1; }
@@ -518,14 +613,28 @@ cudaError_t launch_pauli_to_rho(float *v, float2 *rho, int n, cudaStream_t s)
     }
     float scale = 1.f;
     for (int i = 0; i < n; i++) scale *= 0.5f;
-    k_pauli_emit<<<cv_blocks(n), kCvThreads, 0, s>>>(v, rho, n, scale, n > kCvLow ? 0 : 1);
+    const int sign = n > kCvLow ? 0 : 1;
+    switch (n) {
+    case 3: emit_m<3>(v, rho, n, scale, sign, s); break;
+    case 4: emit_m<4>(v, rho, n, scale, sign, s); break;
+    case 5: emit_m<5>(v, rho, n, scale, sign, s); break;
+    case 6: emit_m<6>(v, rho, n, scale, sign, s); break;
+    default: emit_m<kCvLow>(v, rho, n, scale, sign, s); break;
+    }
     return cudaGetLastError();
 }
 
 // v <- rho, from its lower triangle.
 cudaError_t launch_rho_to_pauli(const float2 *rho, float *v, int n, cudaStream_t s)
 {
-    k_pauli_absorb<<<cv_blocks(n), kCvThreads, 0, s>>>(rho, v, n, n > kCvLow ? 0 : 1);
+    const int sign = n > kCvLow ? 0 : 1;
+    switch (n) {
+    case 3: absorb_m<3>(rho, v, n, sign, s); break;
+    case 4: absorb_m<4>(rho, v, n, sign, s); break;
+    case 5: absorb_m<5>(rho, v, n, sign, s); break;
+    case 6: absorb_m<6>(rho, v, n, sign, s); break;
+    default: absorb_m<kCvLow>(rho, v, n, sign, s); break;
+    }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || n <= kCvLow) return e;
     return launch_high(v, n, 0, 1, s);
