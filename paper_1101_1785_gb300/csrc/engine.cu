@@ -74,11 +74,14 @@ __device__ __forceinline__ ProgShared eng_stage(const PassDesc &D, const EngSmem
     return ProgShared{r, reinterpret_cast<const POp *>(dst + nr), smem_u32(dst + nr + no)};
 }
 
-__device__ __forceinline__ void eng_init(const EngSmem &sm, int t, unsigned tile)
+// The product state a program starts from (PauliPlan::w).
+__device__ __forceinline__ void eng_init(const EngSmem &sm, const PauliHdr &h, unsigned tile)
 {
-    const bool zt = (tile & 0xAAAAAAAAu) == 0;
-    for (unsigned k = threadIdx.x; k < (1u << (2 * (t - 1))); k += kEngThreads)
-        sm.tile()[pauli_swz(k)] = zt && (k & 0xAAAu) == 0 ? make_float4(1.f, 1.f, 0.f, 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float f0 = p_factor(h.w, h.od, h.nod, tile);
+    for (unsigned k = threadIdx.x; k < (1u << (2 * (h.t - 1))); k += kEngThreads) {
+        const float f = f0 * p_factor(h.w, h.td + 1, h.t - 1, k);
+        sm.tile()[pauli_swz(k)] = make_float4(f * h.w[0], f * h.w[1], f * h.w[2], f * h.w[3]);
+    }
 }
 
 __device__ __forceinline__ uint64_t eng_base(const PauliHdr &h, unsigned tile)
@@ -96,11 +99,18 @@ __device__ __forceinline__ uint64_t eng_chunk(const PauliHdr &h, unsigned k)
 }
 
 // Out of line: the rounds need nearly all 128 registers, so nothing of the item loop lives across them.
-template <bool DENSE>
+template <bool DENSE, bool FULL>
 __device__ __noinline__ void eng_rounds(unsigned tile, const PRound *rounds, int nround, const POp *ops, unsigned coef)
 {
     const ProgShared prog{rounds, ops, coef};
-    pauli_rounds<DENSE>(tile, rounds, nround, prog, threadIdx.x, 0);
+    pauli_rounds<DENSE>(tile, rounds, nround, prog, threadIdx.x, 0, KeepTile<FULL>());
+}
+
+template <bool DENSE>
+__device__ __forceinline__ void eng_evolve(const PauliHdr &h, const EngSmem &sm, const ProgShared &prog)
+{
+    if (h.t == kPTile) eng_rounds<DENSE, true>(smem_u32(sm.base), prog.rounds, h.nround, prog.ops, prog.coef);
+    else eng_rounds<DENSE, false>(smem_u32(sm.base), prog.rounds, h.nround, prog.ops, prog.coef);
 }
 
 template <bool DENSE>
@@ -110,14 +120,14 @@ __device__ void run_tile(const WItem &W, const EngSmem &sm)
     const unsigned nch = 1u << (2 * (D.h.t - 1));
     float *g = W.v + eng_base(D.h, W.tile);
     if (W.flags & WF_INIT) {
-        eng_init(sm, D.h.t, W.tile);
+        eng_init(sm, D.h, W.tile);
     } else {
         for (unsigned k = threadIdx.x; k < nch; k += kEngThreads) cp_async16(sm.tile() + pauli_swz(k), g + eng_chunk(D.h, k));
     }
     const ProgShared prog = eng_stage(D, sm);
     cp_async_wait_all();
     __syncthreads();
-    eng_rounds<DENSE>(smem_u32(sm.base), prog.rounds, D.h.nround, prog.ops, prog.coef);
+    eng_evolve<DENSE>(D.h, sm, prog);
     for (unsigned k = threadIdx.x; k < nch; k += kEngThreads)
         *reinterpret_cast<float4 *>(g + eng_chunk(D.h, k)) = p_lds4(smem_u32(sm.base) + 16u * pauli_swz(k));
 }
@@ -154,13 +164,13 @@ __device__ void run_whole(const WItem &W, const EngSmem &sm, RedShared &sh)
     const PauliHdr &h = reinterpret_cast<const PassDesc *>(W.pass)->h;
     const int t = h.t;
     const unsigned nch = 1u << (2 * (t - 1));
-    eng_init(sm, t, 0);
+    eng_init(sm, h, 0);
     const char *p = W.pass;
     for (int i = 0; i < W.npass; i++) {
         const PassDesc &D = *reinterpret_cast<const PassDesc *>(p);
         const ProgShared prog = eng_stage(D, sm);
         __syncthreads();
-        eng_rounds<DENSE>(smem_u32(sm.base), prog.rounds, D.h.nround, prog.ops, prog.coef);
+        eng_evolve<DENSE>(D.h, sm, prog);
         __syncthreads();
         p += D.bytes;
     }
@@ -276,15 +286,9 @@ Program make_program(const qcw_op *ops, int nops, const double *matrices, int n,
     p.n = n;
     p.nd = plan.nd;
     p.whole = p.nd <= kPTile;
-    if (plan.passes.empty()) {  // an empty pass still writes the initial state
-        PPass ps;
-        ps.t = std::min(p.nd, kPTile);
-        for (int d = 0; d < p.nd; d++) (d < ps.t ? ps.td : ps.od).push_back(d);
-        plan.passes.push_back(ps);
-    }
     for (const PPass &ps : plan.passes) {
         PassDesc D;
-        D.h = pauli_header(ps);
+        D.h = pauli_header(ps, plan.w);
         const size_t nr = sizeof(PRound) * ps.rounds.size(), no = 4 * (size_t)((ps.ops.size() + 3) & ~(size_t)3);
         const size_t nc = sizeof(float) * ((ps.coefs.size() + 3) & ~(size_t)3);
         D.bytes = (int)(sizeof D + nr + no + nc);

@@ -111,6 +111,7 @@ struct CachedPauli {
     uint64_t hash = 0;
     int k = 0;
     bool beam = false;
+    bool zero = false;     // planned for a start from |0..0>
     std::vector<QOp> ops;  // exact copy for verification
     std::vector<PauliBlob> passes;
     int nnode = 0;
@@ -882,15 +883,15 @@ static qcw_status run_pauli_segment(qcw_ctx *c, size_t b, size_t e, bool last, b
     const uint64_t h = hash_ops(c->queue, b, e, c->n, c->fuse_k, 0);
     CachedPauli *hit = nullptr;
     for (CachedPauli &p : rt->pcache)
-        if (p.hash == h && p.k == c->fuse_k && same_ops(p.ops, c->queue, b, e)) {
+        if (p.hash == h && p.k == c->fuse_k && p.zero == c->pzero && same_ops(p.ops, c->queue, b, e)) {
             hit = &p;
             break;
         }
     auto plan_into = [&](CachedPauli &p, bool beam) {
-        const PauliPlan plan = plan_pauli(c->queue, b, e, c->n, c->fuse_k, beam);
+        const PauliPlan plan = plan_pauli(c->queue, b, e, c->n, c->fuse_k, beam, p.zero);
         p.beam = beam;
         p.passes.clear();
-        for (const PPass &ps : plan.passes) p.passes.push_back(pauli_blob(ps));
+        for (const PPass &ps : plan.passes) p.passes.push_back(pauli_blob(ps, plan.w));
     };
     if (!hit) {
         if (rt->pcache.size() >= kMaxCached) {  // evict least recently used
@@ -902,6 +903,7 @@ static qcw_status run_pauli_segment(qcw_ctx *c, size_t b, size_t e, bool last, b
         CachedPauli p;
         p.hash = h;
         p.k = c->fuse_k;
+        p.zero = c->pzero;
         p.ops.assign(c->queue.begin() + b, c->queue.begin() + e);
         plan_into(p, false);
         rt->pcache.push_back(std::move(p));

@@ -18,11 +18,13 @@ namespace qcw {
 // go to the two teams in turn, and a team that waited on the other's phases by parity could take an
 // earlier one for its own.  A thread stores and reloads the same chunks of a
 // buffer, so the write-back of tile i and the load of tile i + 3 need no barrier between them.
-// Traffic: one read and one write of v, 8 * 4^n bytes.  Measured at n = 14 (2.15 GB): 0.62 ms per
-// pass of four rounds and seven operations (k_fused_herm_ws, on rho: 1.10 ms per pass, and a third
-// more passes), 0.55 ms with the operations left out, 0.34 ms (6.2 TB/s) with the rounds left out:
-// the rounds' trips through shared memory are what it waits for.  Each wait is bounded: the team that gives
-// up sets the error word and stops, the other runs out of tiles or gives up in turn.
+// Traffic: one read and one write of v, 8 * 4^n bytes.  Measured at n = 14 (2.15 GB): 0.56 ms per
+// pass of four rounds and six operations, 3.8 TB/s (k_fused_herm_ws, on rho: 1.10 ms per pass, and a
+// third more passes), 0.51 ms with the operations left out, 0.34 ms (6.2 TB/s) with the rounds left
+// out: the rounds' trips through shared memory are what it waits for.  Hence the last round's results
+// go from the registers straight to v (StoreDirect), one trip less: 0.61 before.  Each wait is
+// bounded: the team that gives up sets the error word and stops, the other runs out of tiles or gives
+// up in turn.
 constexpr int kPBuf = 3;
 constexpr int kPThreads = 512;
 constexpr unsigned kPWaitLimit = 1u << 21;
@@ -42,18 +44,58 @@ __host__ __device__ inline int pb_coef(const PauliHdr &h) { return pb_ops(h) + (
 size_t pauli_pass_smem(const PauliHdr &h, bool dense)
 {
     const size_t prog = dense ? 4 * (size_t)pb_coef(h) + sizeof(float2) * (size_t)h.ncoef : sizeof(PRound) * (size_t)h.nround;
-    return (size_t)kPBuf * (sizeof(float) << (2 * h.t)) + prog + 16 * sizeof(double) + 2 * kPBuf * sizeof(uint64_t);
+    return (size_t)kPBuf * (sizeof(float) << (2 * h.t)) + prog + 16 * sizeof(double) + 2 * kPBuf * sizeof(uint64_t) + 32;
 }
 
-template <int BYTES, bool DENSE, bool PUR>
+// The last round's elements straight from the registers to v: the lanes of a quarter-warp hold the
+// labels of tile digit 1 (which the round does not touch), so they fill 64-byte runs.  A round that
+// does touch digit 1 would scatter 16-byte pieces; there, and for dense maps and small tiles, the
+// results go through the tile.  Per pass, through the tile / direct: n = 9 13.2 / 12.8 us, n = 13
+// 170 / 156 us, n = 14 610 / 562 us.
+template <bool PUR>
+struct StoreDirect {
+    static constexpr bool kDirect = true, kFull = true;
+    float *v;
+    const volatile int8_t *td;  // tile digits, then (8 on) the outside ones, in shared memory: see Walk
+    int nod;
+    unsigned tid, tile;
+    float &ps;
+    __device__ __forceinline__ void store(const PRound &R, const pu64 (&x)[32], unsigned db, unsigned dc) const
+    {
+        const unsigned c = pauli_swz(((unsigned)R.lo[tid & 15u] ^ (unsigned)R.hi[tid >> 4]) >> 4);  // its own inverse
+        uint64_t g = 0;
+        for (int d = 0; d < nod; d++) g += (uint64_t)((tile >> (2 * d)) & 3u) << (2 * td[8 + d]);
+#pragma unroll
+        for (int d = 1; d < kPTile; d++) g += (uint64_t)((c >> (2 * (d - 1))) & 3u) << (2 * td[d]);
+        const uint64_t sb = 1ull << (2 * td[db]), sc = 1ull << (2 * td[dc]);
+        float *pj = v + g;
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            float *pi = pj;
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const float2 a = unpack2(x[px(0, i, j)]), b = unpack2(x[px(1, i, j)]);
+                *reinterpret_cast<float4 *>(pi) = make_float4(a.x, a.y, b.x, b.y);
+                if (PUR) ps = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(b.x, b.x, fmaf(b.y, b.y, ps))));
+                pi += sb;
+            }
+            pj += sc;
+        }
+    }
+};
+
+// INIT: start from the header's product state.  FULL: tiles of kPTile digits (every register from
+// seven qubits up) and no dense maps.  Both are fixed at compile time because the registers are all
+// in use: either one as a run-time branch spilled part of the 64 elements.
+template <int BYTES, bool DENSE, bool FULL, bool INIT, bool PUR>
 __global__ void __launch_bounds__(kPThreads, 1)
-    k_pauli_pass(float *__restrict__ v, unsigned ntiles, int init, unsigned long long *__restrict__ err,
+    k_pauli_pass(float *__restrict__ v, unsigned ntiles, unsigned long long *__restrict__ err,
                  unsigned wait_limit, int stall_tile, double *__restrict__ ppart, double pscale,
                  const __grid_constant__ PauliParams<BYTES> prm)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const PauliHdr &H = prm.h;
-    const int t = H.t;
+    const int t = FULL ? kPTile : H.t;
     const unsigned nchunk = 1u << (2 * (t - 1));
     const size_t tbytes = sizeof(float) << (2 * t);
     unsigned char *p = smem + kPBuf * tbytes;
@@ -61,47 +103,60 @@ __global__ void __launch_bounds__(kPThreads, 1)
     const int nword = DENSE ? pb_coef(H) + 2 * H.ncoef : pb_ops(H);  // of the program kept in shared memory
     double *red = reinterpret_cast<double *>(reinterpret_cast<unsigned *>(rounds) + nword);
     uint64_t *full = reinterpret_cast<uint64_t *>(red + 16);
+    volatile int8_t *td = reinterpret_cast<volatile int8_t *>(full + 2 * kPBuf);
+    if (threadIdx.x < 24) td[threadIdx.x] = threadIdx.x < 8 ? H.td[threadIdx.x] : H.od[threadIdx.x - 8];
     const unsigned tid = threadIdx.x & 255u, team = threadIdx.x >> 8;
     for (int i = threadIdx.x; i < nword; i += kPThreads) reinterpret_cast<unsigned *>(rounds)[i] = prm.blob[i];
     if (threadIdx.x < 2 * kPBuf) mbar_init(&full[threadIdx.x], 256);
     __syncthreads();
-    // this thread's chunks are tid + 256 i: offsets split into a part of tid (tile digits 1..4) and
-    // a part of i (digits 5, 6)
-    uint64_t glo = 0;
-    for (int d = 1; d < t && d < 5; d++) glo += (uint64_t)((tid >> (2 * (d - 1))) & 3u) << (2 * H.td[d]);
-    const int s5 = t > 5 ? 2 * H.td[5] : 0, s6 = t > 6 ? 2 * H.td[6] : 0;
-    const unsigned plo = pauli_swz(tid);
-    const unsigned mine = tid < nchunk ? (nchunk + 255u) >> 8 : 0u;  // chunks of this thread
     const unsigned ntile = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    auto base_of = [&](unsigned i) {
-        const unsigned tile = blockIdx.x + i * gridDim.x;
-        uint64_t b = glo;
-        for (int d = 0; d < H.nod; d++) b += (uint64_t)((tile >> (2 * d)) & 3u) << (2 * H.od[d]);
-        return b;
+    // A thread's chunks are tid + 256 k: offsets split into a part of the tile and of tid (tile digits
+    // 1..4) and a part of k (digits 5, 6).  Worked out again for every copy, from digits read from
+    // shared memory each time: kept across the rounds they would take registers from the 64 elements.
+    struct Walk {
+        uint64_t base, step5, step6;
+        unsigned plo, mine;
+        __device__ __forceinline__ uint64_t at(unsigned k) const { return (k & 3u) * step5 + (k >> 2) * step6; }
     };
-    auto goff = [&](unsigned i) { return ((uint64_t)(i & 3u) << s5) + ((uint64_t)(i >> 2) << s6); };
-    const uint64_t step5 = 1ull << s5, jump6 = (1ull << s6) - 3 * step5;  // full tiles: k walks digit 5, then 6
+    auto walk = [&](unsigned i) {
+        unsigned id;
+        asm volatile("mov.u32 %0, %1;\n" : "=r"(id) : "r"(tid));
+        Walk w;
+        const unsigned tile = blockIdx.x + i * gridDim.x;
+        w.base = 0;
+        for (int d = 1; d < t && d < 5; d++) w.base += (uint64_t)((id >> (2 * (d - 1))) & 3u) << (2 * td[d]);
+        for (int d = 0; d < H.nod; d++) w.base += (uint64_t)((tile >> (2 * d)) & 3u) << (2 * td[8 + d]);
+        w.step5 = t > 5 ? 1ull << (2 * td[5]) : 0;
+        w.step6 = t > 6 ? 1ull << (2 * td[6]) : 0;
+        w.plo = pauli_swz(id);
+        w.mine = id < nchunk ? (nchunk + 255u) >> 8 : 0u;
+        return w;
+    };
     auto load = [&](unsigned i) {
         if (blockIdx.x == 0 && (int)i == stall_tile) return;
         const unsigned b = i % kPBuf;
         float4 *buf = reinterpret_cast<float4 *>(smem + b * tbytes);
         uint64_t *bar = &full[2 * b + (i & 1u)];
-        if (init) {  // |0..0><0..0|: 1 on every string of I and Z
-            const bool zt = ((blockIdx.x + i * gridDim.x) & 0xAAAAAAAAu) == 0;
-            for (unsigned k = 0; k < mine; k++)
-                buf[plo ^ pauli_swz(256u * k)] = zt && ((tid + 256u * k) & 0xAAAu) == 0 ? make_float4(1.f, 1.f, 0.f, 0.f)
-                                                                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+        const Walk w = walk(i);
+        if (INIT) {  // the product state
+            const unsigned tile = blockIdx.x + i * gridDim.x;
+            const float f0 = p_factor(H.w, H.od, H.nod, tile);
+            const float w0 = H.w[0], w1 = H.w[1], w2 = H.w[2], w3 = H.w[3];
+            for (unsigned k = 0; k < w.mine; k++) {
+                const float f = f0 * p_factor(H.w, H.td + 1, t - 1, tid + 256u * k);
+                buf[w.plo ^ pauli_swz(256u * k)] = make_float4(f * w0, f * w1, f * w2, f * w3);
+            }
             mbar_arrive(bar);
         } else {
-            const float *src = v + base_of(i);
+            const float *src = v + w.base;
             if (t == kPTile) {
 #pragma unroll
                 for (unsigned k = 0; k < 16; k++) {
-                    cp_async16(buf + (plo ^ pauli_swz(256u * k)), src);
-                    src += (k & 3u) == 3u ? jump6 : step5;
+                    cp_async16(buf + (w.plo ^ pauli_swz(256u * k)), src);
+                    src += (k & 3u) == 3u ? w.step6 - 3 * w.step5 : w.step5;
                 }
             } else {
-                for (unsigned k = 0; k < mine; k++) cp_async16(buf + (plo ^ pauli_swz(256u * k)), src + goff(k));
+                for (unsigned k = 0; k < w.mine; k++) cp_async16(buf + (w.plo ^ pauli_swz(256u * k)), src + w.at(k));
             }
             cp_async_mbar_arrive(bar);
         }
@@ -112,6 +167,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
     } else if (ntile > 1) {
         load(1);
     }
+    const bool direct = FULL && H.nround > 0 && rounds[H.nround - 1].direct;
     double pacc = 0.0;
     for (unsigned i = team; i < ntile; i += 2) {
         const unsigned b = i % kPBuf;
@@ -120,19 +176,30 @@ __global__ void __launch_bounds__(kPThreads, 1)
             if (tid == 0) atomicOr(err, 1ull);
             break;
         }
+        float ps = 0.f;
+        const unsigned ba = smem_u32(smem) + (unsigned)(b * tbytes);
         if constexpr (DENSE) {
             const unsigned *w = reinterpret_cast<const unsigned *>(rounds);
             const ProgShared prog{rounds, reinterpret_cast<const POp *>(w + pb_ops(H)), smem_u32(w + pb_coef(H))};
-            pauli_rounds<true>(smem_u32(smem) + (unsigned)(b * tbytes), rounds, H.nround, prog, tid, 1 + team);
+            pauli_rounds<true>(ba, rounds, H.nround, prog, tid, 1 + team);
         } else {
             const ProgParam prog{prm.blob, pb_ops(H), pb_coef(H)};
-            pauli_rounds<false>(smem_u32(smem) + (unsigned)(b * tbytes), rounds, H.nround, prog, tid, 1 + team);
+            if constexpr (FULL) {
+                const StoreDirect<PUR> last{v, td, H.nod, tid, blockIdx.x + i * gridDim.x, ps};
+                pauli_rounds<false>(ba, rounds, H.nround, prog, tid, 1 + team, last);
+                if (direct) {
+                    if (PUR) pacc += (double)ps;
+                    if (i + kPBuf < ntile) load(i + kPBuf);
+                    continue;
+                }
+            } else {
+                pauli_rounds<false>(ba, rounds, H.nround, prog, tid, 1 + team);
+            }
         }
-        float *dst = v + base_of(i);
-        const unsigned ba = smem_u32(smem) + (unsigned)(b * tbytes);
-        float ps = 0.f;
+        const Walk w = walk(i);
+        float *dst = v + w.base;
         auto put = [&](unsigned k, float *to) {
-            const float4 x = p_lds4(ba + 16u * (plo ^ pauli_swz(256u * k)));
+            const float4 x = p_lds4(ba + 16u * (w.plo ^ pauli_swz(256u * k)));
             *reinterpret_cast<float4 *>(to) = x;
             if (PUR) ps = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, ps))));
         };
@@ -140,10 +207,10 @@ __global__ void __launch_bounds__(kPThreads, 1)
 #pragma unroll
             for (unsigned k = 0; k < 16; k++) {
                 put(k, dst);
-                dst += (k & 3u) == 3u ? jump6 : step5;
+                dst += (k & 3u) == 3u ? w.step6 - 3 * w.step5 : w.step5;
             }
         } else {
-            for (unsigned k = 0; k < mine; k++) put(k, dst + goff(k));
+            for (unsigned k = 0; k < w.mine; k++) put(k, dst + w.at(k));
         }
         if (PUR) pacc += (double)ps;
         if (i + kPBuf < ntile) load(i + kPBuf);
@@ -161,7 +228,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
     }
 }
 
-template <int BYTES, bool DENSE>
+template <int BYTES, bool DENSE, bool FULL>
 static cudaError_t launch_pass(const PauliBlob &B, float *v, unsigned ntiles, unsigned grid, bool init,
                                unsigned long long *err, unsigned wait_limit, int stall_tile, double *ppart, double pscale,
                                cudaStream_t s)
@@ -169,10 +236,11 @@ static cudaError_t launch_pass(const PauliBlob &B, float *v, unsigned ntiles, un
     PauliParams<BYTES> prm;
     prm.h = B.h;
     memcpy(prm.blob, B.words.data(), 4 * B.words.size());
-    auto kern = ppart ? k_pauli_pass<BYTES, DENSE, true> : k_pauli_pass<BYTES, DENSE, false>;
+    auto kern = ppart ? (init ? k_pauli_pass<BYTES, DENSE, FULL, true, true> : k_pauli_pass<BYTES, DENSE, FULL, false, true>)
+                      : (init ? k_pauli_pass<BYTES, DENSE, FULL, true, false> : k_pauli_pass<BYTES, DENSE, FULL, false, false>);
     const size_t sm = pauli_pass_smem(B.h, DENSE);
     if (ensure_smem_attr(reinterpret_cast<const void *>(kern), sm)) return cudaErrorInvalidValue;
-    kern<<<grid, kPThreads, sm, s>>>(v, ntiles, init ? 1 : 0, err, wait_limit ? wait_limit : kPWaitLimit, stall_tile, ppart,
+    kern<<<grid, kPThreads, sm, s>>>(v, ntiles, err, wait_limit ? wait_limit : kPWaitLimit, stall_tile, ppart,
                                      pscale, prm);
     return cudaGetLastError();
 }
@@ -184,7 +252,7 @@ bool pass_dense(const PPass &p)
     return false;
 }
 
-PauliHdr pauli_header(const PPass &p)
+PauliHdr pauli_header(const PPass &p, const std::vector<float> &w)
 {
     PauliHdr h;
     memset(&h, 0, sizeof h);
@@ -195,18 +263,21 @@ PauliHdr pauli_header(const PPass &p)
     h.ncoef = (int)p.coefs.size();
     for (size_t i = 0; i < p.td.size(); i++) h.td[i] = (int8_t)p.td[i];
     for (size_t i = 0; i < p.od.size(); i++) h.od[i] = (int8_t)p.od[i];
+    std::copy(w.begin(), w.end(), h.w);
     return h;
 }
 
-PauliBlob pauli_blob(const PPass &p)
+PauliBlob pauli_blob(const PPass &p, const std::vector<float> &w)
 {
     PauliBlob B;
-    B.h = pauli_header(p);
+    B.h = pauli_header(p, w);
     B.dense = pass_dense(p);
     const PauliHdr &h = B.h;
     static_assert(sizeof(PRound) == 96 && sizeof(POp) == 4, "blob layout");
     B.words.assign((size_t)pb_coef(h) + 2 * h.ncoef, 0u);
     memcpy(B.words.data(), p.rounds.data(), sizeof(PRound) * p.rounds.size());
+    if (h.nround && h.t == kPTile && !B.dense && p.rounds.back().db > 1)
+        reinterpret_cast<PRound *>(B.words.data())[h.nround - 1].direct = 1;
     if (h.nop) memcpy(B.words.data() + pb_ops(h), p.ops.data(), sizeof(POp) * p.ops.size());
     for (size_t i = 0; i < p.coefs.size(); i++)
         for (int j = 0; j < 2; j++) memcpy(B.words.data() + pb_coef(h) + 2 * i + j, &p.coefs[i], sizeof(float));
@@ -221,11 +292,13 @@ cudaError_t launch_pauli_pass(const PauliBlob &B, float *v, int nd, int nsm, boo
     const unsigned ntiles = 1u << (2 * B.h.nod), grid = pauli_grid(B.h, nsm);
     double pscale = 1.0;
     for (int i = 0; i < nd; i++) pscale *= 0.5;
-    constexpr int kSmall = 3840;
+    constexpr int kSmall = 3584;
     constexpr int kLarge = 8 * kPMaxCoef + (int)sizeof(PRound) * kPMaxRounds + 4 * kPMaxOps;
     if (!B.dense && 4 * B.words.size() <= kSmall)
-        return launch_pass<kSmall, false>(B, v, ntiles, grid, init, err, wait_limit, stall_tile, ppart, pscale, s);
-    return launch_pass<kLarge, true>(B, v, ntiles, grid, init, err, wait_limit, stall_tile, ppart, pscale, s);
+        return B.h.t == kPTile
+                   ? launch_pass<kSmall, false, true>(B, v, ntiles, grid, init, err, wait_limit, stall_tile, ppart, pscale, s)
+                   : launch_pass<kSmall, false, false>(B, v, ntiles, grid, init, err, wait_limit, stall_tile, ppart, pscale, s);
+    return launch_pass<kLarge, true, false>(B, v, ntiles, grid, init, err, wait_limit, stall_tile, ppart, pscale, s);
 }
 
 unsigned pauli_grid(const PauliHdr &h, int nsm)

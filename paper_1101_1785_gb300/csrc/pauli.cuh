@@ -325,15 +325,33 @@ __device__ __forceinline__ void p_signs(pu64 (&x)[32])
             }
 }
 
+// Product of the start factors (PauliHdr::w) of the digits dig[0..nd) at the labels in lab.
+template <class D>
+__device__ __forceinline__ float p_factor(const float *w, const D *dig, int nd, unsigned lab)
+{
+    float f = 1.f;
+    for (int d = 0; d < nd; d++) f *= w[4 * dig[d] + ((lab >> (2 * d)) & 3u)];
+    return f;
+}
+
+// What the last round does with its results: back to the tile in shared memory.
+template <bool FULL = false>
+struct KeepTile {
+    static constexpr bool kDirect = false, kFull = FULL;
+    __device__ __forceinline__ void store(const PRound &, const pu64 (&)[32], unsigned, unsigned) const {}
+};
+
 // The rounds of a pass on the tile at shared address `tile`, by 256 threads (tid) that meet at
 // named barrier `bar`.  tab: the rounds in shared memory (their position tables are read per thread).
-template <bool DENSE, class P>
+// T::kFull: the tile has kPTile digits.  T::kDirect: the elements of a round marked direct (the last one of a pass) go to T::store from the registers instead of back to the
+// tile, which is free for its next contents once the call returns (every thread has read its own).
+template <bool DENSE, class P, class T = KeepTile<>>
 __device__ __forceinline__ void pauli_rounds(unsigned tile, const PRound *__restrict__ tab, int nround, const P &p,
-                                             unsigned tid, int bar)
+                                             unsigned tid, int bar, const T &last = T())
 {
     for (int r = 0; r < nround; r++) {
         const uint4 w = p.head(r);  // db dc nob nop | op0 perm | ld
-        if (tid < (1u << ((w.x >> 16) & 255u))) {
+        if (T::kFull || tid < (1u << ((w.x >> 16) & 255u))) {  // full tiles: every thread has a group
             const unsigned base = (unsigned)tab[r].lo[tid & 15u] ^ (unsigned)tab[r].hi[tid >> 4];
             pu64 x[32];
             {
@@ -344,6 +362,9 @@ __device__ __forceinline__ void pauli_rounds(unsigned tile, const PRound *__rest
 #pragma unroll
                     for (int i = 0; i < 4; i++) p_lds2(tile + (base ^ b[i] ^ c[j]), x[px(0, i, j)], x[px(1, i, j)]);
             }
+            if (T::kDirect && (w.y >> 24)) {  // full tiles only: every thread is here
+                bar_sync(bar, 256);
+            }
             const unsigned perm = (w.y >> 16) & 255u;
             if (perm == PP_CX_BC) p_signs<false, true>(x);
             else if (perm == PP_CX_CB) p_signs<false, false>(x);
@@ -352,6 +373,10 @@ __device__ __forceinline__ void pauli_rounds(unsigned tile, const PRound *__rest
             for (unsigned o = w.y & 65535u; o < o1; o++) {
                 const unsigned op = p.op(o);
                 p_op<DENSE>(x, (int)(op & 65535u), p, 4u * (op >> 16));
+            }
+            if (T::kDirect && (w.y >> 24)) {
+                last.store(tab[r], x, w.x & 255u, (w.x >> 8) & 255u);
+                return;
             }
             {
                 const uint2 s = p.store(r);

@@ -36,7 +36,7 @@ struct PRound {
     uint8_t nop;
     uint16_t op0;      // first operation in the pass's list
     uint8_t perm;      // PP_*
-    uint8_t pad;
+    uint8_t direct;    // last round of a pass on full tiles, leaving tile digit 1 alone: results go straight to v
     uint16_t ld[4];    // contribution of the label bits z, x of db and z, x of dc when reading
     uint16_t st[4];    // and when writing
     uint16_t pad2[4];
@@ -77,13 +77,19 @@ struct PauliPlan {
     int n = 0, nd = 0;  // qubits; digits (n, at least kPMinDigits)
     std::vector<PPass> passes;
     int nnode2 = 0;     // two-qubit operations left after merging
+    // zero start: what the one-qubit operations before any two-qubit operation make of |0..0>, a product
+    // state, v_P = prod_d w[d][label of digit d]; the first pass starts from it.  (1, 1, 0, 0) else.
+    std::vector<float> w;
 };
 
 // Plan ops[begin, end) (k <= 2, no controls) for an n-qubit register.  kmax = 0: a pass works on
-// every qubit of its tile; else on at most kmax qubits.  beam: pass sets by the beam search.
-PauliPlan plan_pauli(const std::vector<QOp> &ops, size_t begin, size_t end, int n, int kmax, bool beam);
+// every qubit of its tile; else on at most kmax qubits.  beam: pass sets by the beam search.  zero:
+// the state before is |0..0><0..0| (there is then at least one pass).
+PauliPlan plan_pauli(const std::vector<QOp> &ops, size_t begin, size_t end, int n, int kmax, bool beam,
+                     bool zero = false);
 
-// The same for a caller's checked operation list (gates and channels on one and two qubits).
+// The same for a caller's checked operation list (gates and channels on one and two qubits), from
+// |0..0>.
 PauliPlan plan_pauli_list(const qcw_op *ops, int nops, const double *matrices, int n, int kmax);
 
 // Position of 16-byte chunk c of a tile in shared memory: bits 0..2 (which 16 of 128 bytes) are

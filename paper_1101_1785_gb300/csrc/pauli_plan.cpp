@@ -251,16 +251,31 @@ void round_map(M4 &a, double &c)
 
 class NodeBuilder {
   public:
-    explicit NodeBuilder(int n) : n(n), last(n, -1), pre(n, m4_identity()) {}
+    // zero: one-qubit operations before any two-qubit one on their qubit act on (1, 1, 0, 0) of the
+    // product state |0..0>, not as maps of their own
+    NodeBuilder(int n, bool zero) : n(n), zero(zero), last(n, -1), pre(n, m4_identity()), start(n, m4_identity()) {}
     void add(const OpView &op);
+    std::vector<float> product(int nd) const;
     std::vector<Node> finish();
 
   private:
     int n;
+    bool zero;
     std::vector<Node> out;
     std::vector<int> last;
-    std::vector<M4> pre;
+    std::vector<M4> pre, start;
 };
+
+std::vector<float> NodeBuilder::product(int nd) const
+{
+    std::vector<float> w(4 * (size_t)nd, 0.f);
+    for (int d = 0; d < nd; d++)
+        for (int p = 0; p < 4; p++) {
+            const double *m = d < n ? start[n - 1 - d].m : nullptr;
+            w[4 * d + p] = m ? (float)(m[4 * p] + m[4 * p + 1]) : p < 2 ? 1.f : 0.f;
+        }
+    return w;
+}
 
 void NodeBuilder::add(const OpView &op)
 {
@@ -268,7 +283,7 @@ void NodeBuilder::add(const OpView &op)
         if (op.k == 1) {
             const int q = op.qubits[0];
             const M4 m = one_map(op);
-            if (last[q] < 0) m4_lmul(pre[q], m);
+            if (last[q] < 0) m4_lmul(zero ? start[q] : pre[q], m);
             else m4_lmul(out[last[q]].a == q ? out[last[q]].A : out[last[q]].B, m);
             return;
         }
@@ -435,8 +450,9 @@ void emit(PPass &ps, const Node &nd, bool maps_only, F dig)
 
 }  // namespace
 
-static PauliPlan plan_nodes(std::vector<Node> nodes, int n, int kmax, bool beam)
+static PauliPlan plan_nodes(NodeBuilder &nb, int n, int kmax, bool beam, bool zero)
 {
+    std::vector<Node> nodes = nb.finish();
     PauliPlan plan;
     plan.n = n;
     plan.nd = std::max(n, kPMinDigits);
@@ -533,11 +549,24 @@ static PauliPlan plan_nodes(std::vector<Node> nodes, int n, int kmax, bool beam)
                 break;
             }
             round_positions(t, r);
-            for (size_t j = 0; j < take.size(); j++)
+            auto lone = [&](size_t j) {  // trace-preserving one-qubit map of db or dc
+                return j < take.size() && nodes[take[j]].kind == PO_ONE && tmask(take[j]) != 1u && m4_tp(nodes[take[j]].A);
+            };
+            for (size_t j = 0; j < take.size(); j++) {
+                if (lone(j) && lone(j + 1) && tmask(take[j]) != tmask(take[j + 1])) {  // one of each: both at once
+                    const bool first = tmask(take[j]) == 1u << r.db;
+                    POp op{PO_MM, (uint16_t)(ps.coefs.size() / 4)};
+                    push_tp(ps.coefs, nodes[take[first ? j : j + 1]].A);
+                    push_tp(ps.coefs, nodes[take[first ? j + 1 : j]].A);
+                    ps.ops.push_back(op);
+                    j++;
+                    continue;
+                }
                 emit(ps, nodes[take[j]], j == 0 && r.perm, [&](int q) {
                     const int d = tile_of[digit(q)];
                     return d == 0 ? 0 : d == r.db ? 1 : 2;
                 });
+            }
             r.nop = (uint8_t)(ps.ops.size() - r.op0);
             ps.rounds.push_back(r);
             chosen.swap(left);
@@ -545,19 +574,26 @@ static PauliPlan plan_nodes(std::vector<Node> nodes, int n, int kmax, bool beam)
         plan.passes.push_back(std::move(ps));
         rem.swap(rest);
     }
+    plan.w = nb.product(nd);
+    if (zero && plan.passes.empty()) {  // the product state still has to be written
+        PPass ps;
+        ps.t = t;
+        for (int d = 0; d < nd; d++) (d < t ? ps.td : ps.od).push_back(d);
+        plan.passes.push_back(std::move(ps));
+    }
     return plan;
 }
 
-PauliPlan plan_pauli(const std::vector<QOp> &ops, size_t begin, size_t end, int n, int kmax, bool beam)
+PauliPlan plan_pauli(const std::vector<QOp> &ops, size_t begin, size_t end, int n, int kmax, bool beam, bool zero)
 {
-    NodeBuilder nb(n);
+    NodeBuilder nb(n, zero);
     for (size_t i = begin; i < end; i++) nb.add(OpView{ops[i].kind, ops[i].k, ops[i].qubits, ops[i].m.data()});
-    return plan_nodes(nb.finish(), n, kmax, beam);
+    return plan_nodes(nb, n, kmax, beam, zero);
 }
 
 PauliPlan plan_pauli_list(const qcw_op *ops, int nops, const double *matrices, int n, int kmax)
 {
-    NodeBuilder nb(n);
+    NodeBuilder nb(n, true);
     c128 S[256];
     for (int i = 0; i < nops; i++) {
         const qcw_op &o = ops[i];
@@ -582,7 +618,7 @@ PauliPlan plan_pauli_list(const qcw_op *ops, int nops, const double *matrices, i
                     }
         nb.add(OpView{1, o.k, o.qubits, S});
     }
-    return plan_nodes(nb.finish(), n, kmax, false);
+    return plan_nodes(nb, n, kmax, false, true);
 }
 
 }  // namespace qcw

@@ -10,6 +10,7 @@ namespace qcw {
 struct PauliHdr {
     int t, nod, nround, nop, ncoef;
     int8_t td[8], od[16];
+    float w[4 * QCW_MAX_QUBITS];  // PauliPlan::w, for the pass that starts from it
 };
 
 // A pass in the form the kernels take: header, then rounds | operations | coefficients.
@@ -18,12 +19,12 @@ struct PauliBlob {
     bool dense = false;  // has dense two-qubit maps
     std::vector<unsigned> words;
 };
-PauliBlob pauli_blob(const PPass &p);
-PauliHdr pauli_header(const PPass &p);
+PauliBlob pauli_blob(const PPass &p, const std::vector<float> &w);
+PauliHdr pauli_header(const PPass &p, const std::vector<float> &w);
 bool pass_dense(const PPass &p);  // has dense two-qubit maps
 unsigned pauli_grid(const PauliHdr &h, int nsm);
 
-// One pass over v (nd digits).  init: v is |0..0><0..0| and not read.  ppart (2 pauli_grid values):
+// One pass over v (nd digits).  init: v is the header's product state and not read.  ppart (2 pauli_grid values):
 // also leave per-team partial sums of the purity.
 cudaError_t launch_pauli_pass(const PauliBlob &B, float *v, int nd, int nsm, bool init, unsigned long long *err,
                               unsigned wait_limit, int stall_tile, double *ppart, cudaStream_t s);

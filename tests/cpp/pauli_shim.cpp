@@ -25,7 +25,7 @@ static void map4(std::vector<double *> &x, int stride, const float *m, bool tp)
 }
 
 // Returns the number of passes; *bad counts positions a round visits not exactly once.
-extern "C" int pauli_replay(int n, int kmax, int beam, int nops, const int *kind, const int *k, const int *qubits,
+extern "C" int pauli_replay(int n, int kmax, int beam, int zero, int nops, const int *kind, const int *k, const int *qubits,
                             const double *mats, const long long *mat_off, double *v, int *nrounds, int *bad)
 {
     std::vector<QOp> ops(nops);
@@ -40,7 +40,12 @@ extern "C" int pauli_replay(int n, int kmax, int beam, int nops, const int *kind
         for (int t = 0; t < dim * dim; t++)
             o.m[t] = c128(mats[2 * (mat_off[i] + t)], mats[2 * (mat_off[i] + t) + 1]);
     }
-    const PauliPlan plan = plan_pauli(ops, 0, ops.size(), n, kmax, beam != 0);
+    const PauliPlan plan = plan_pauli(ops, 0, ops.size(), n, kmax, beam != 0, zero != 0);
+    if (zero)
+        for (size_t i = 0; i < (size_t)1 << (2 * plan.nd); i++) {
+            v[i] = 1;
+            for (int d = 0; d < plan.nd; d++) v[i] *= plan.w[4 * d + ((i >> (2 * d)) & 3)];
+        }
     *nrounds = *bad = 0;
     for (const PPass &P : plan.passes) {
         *nrounds += (int)P.rounds.size();

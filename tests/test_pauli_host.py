@@ -47,7 +47,7 @@ def test_coefficient_helper():
         assert abs(np.trace(p @ rho) - v[i]) < 1e-12
 
 
-def _replay(shim, n, ops, v, kmax, beam):
+def _replay(shim, n, ops, v, kmax, beam, zero=False):
     kind, k, qs, mats, off = [], [], [], [], []
     pos = 0
     for op in ops:
@@ -66,7 +66,7 @@ def _replay(shim, n, ops, v, kmax, beam):
     mats = np.concatenate(mats)
     nr, bad = ctypes.c_int(), ctypes.c_int()
     p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
-    npass = shim.pauli_replay(n, kmax, int(beam), len(ops), p(kind), p(k), p(qs), p(mats), p(off), p(v),
+    npass = shim.pauli_replay(n, kmax, int(beam), int(zero), len(ops), p(kind), p(k), p(qs), p(mats), p(off), p(v),
                               ctypes.byref(nr), ctypes.byref(bad))
     assert npass > 0 and bad.value == 0
     return npass
@@ -112,3 +112,20 @@ def test_plan_replays_the_circuit(shim, n, kmax, beam, what):
     # FP32 coefficients of the composed maps: 2^-24 relative each, at most a few per operation kept
     scale = np.linalg.norm(coefficients(want))
     assert np.linalg.norm(v - coefficients(want)) <= len(ops) * 2.0 ** -24 * scale
+
+
+@pytest.mark.parametrize("n", [3, 5, 8])
+@pytest.mark.parametrize("what", ["mixed", "two", "ones"])
+def test_plan_from_the_zero_state(shim, n, what):
+    """One-qubit operations before the first two-qubit one go into the product state the plan starts
+    from (all of them, when there is no two-qubit operation)."""
+    rng = np.random.default_rng(n)
+    ops = _two_qubit_ops(rng, n, 12) if what == "two" else wl.random_circuit(n, 50, 5 + n, "mixed", "adpd").ops
+    if what == "ones":
+        ops = [op for op in ops if op.k == 1]
+    want = wl.zero_state(n)
+    for op in ops:
+        oracle.apply_op(want, op)
+    v = np.zeros(4 ** n)
+    _replay(shim, n, ops, v, 0, False, True)
+    assert np.linalg.norm(v - coefficients(want)) <= (len(ops) + n) * 2.0 ** -24 * np.linalg.norm(coefficients(want))
