@@ -54,7 +54,7 @@ typedef enum {
 } qcw_status;
 
 /* Execution modes (qcw_set_mode). */
-#define QCW_MODE_PLAIN 0 /* each apply call launches its own kernel at once */
+#define QCW_MODE_PLAIN 0 /* each apply call launches its own kernels at once (a list call: merged) */
 #define QCW_MODE_FUSED 1 /* apply calls are queued; flush packs them into fused passes */
 
 /* Largest register size: rho of 17 qubits is 128 GiB of complex64. */
@@ -233,9 +233,10 @@ typedef struct {
     long long offset;   /* index, in doubles, of the op's first matrix in `matrices` */
 } qcw_op;
 
-/* Apply nops operations in order, exactly as the matching sequence of qcw_apply_gate /
- * qcw_apply_kraus calls would (gates: one 2^k x 2^k matrix at matrices + offset; Kraus:
- * nkraus matrices one after another).  Every op is checked before any is applied, so on
+/* Apply nops operations in order, as the matching sequence of qcw_apply_gate / qcw_apply_kraus
+ * calls would (gates: one 2^k x 2^k matrix at matrices + offset; Kraus: nkraus matrices one after
+ * another).  In plain mode too the operations of one list share passes over rho where they act on
+ * the same qubits, so the results may differ from the separate calls' by rounding.  Every op is checked before any is applied, so on
  * QCW_EINVAL nothing has changed.  Both arrays may be freed when the call returns. */
 QCW_API qcw_status qcw_apply_ops(qcw_ctx *ctx, const qcw_op *ops, int nops, const double *matrices);
 

@@ -186,7 +186,7 @@ qcw_status plain_gate1(qcw_ctx *c, const c128 *u, int t, const int *ctrl, int nc
     return QCW_OK;
 }
 
-static void quartet_layout(int n, int q1, int q2, int *pos, uint64_t *offr, uint64_t *offc)
+void quartet_layout(int n, int q1, int q2, int *pos, uint64_t *offr, uint64_t *offc)
 {
     int pr1 = 2 * n - 1 - q1, pr2 = 2 * n - 1 - q2, pc1 = n - 1 - q1, pc2 = n - 1 - q2;
     int v[4] = {pc1, pc2, pr1, pr2};
@@ -201,7 +201,7 @@ static void quartet_layout(int n, int q1, int q2, int *pos, uint64_t *offr, uint
 }
 
 // One entry per row, at a distinct column, each exactly 1, -1, i or -i: sigma[i] = its column.
-static bool monomial4(const c128 *u, int *sigma, c128 *val)
+bool monomial4(const c128 *u, int *sigma, c128 *val)
 {
     bool used[4] = {false, false, false, false};
     for (int i = 0; i < 4; i++) {
@@ -867,10 +867,8 @@ extern "C" qcw_status qcw_apply_ops(qcw_ctx *ctx, const qcw_op *ops, int nops, c
     std::vector<QOp> conv;
     qcw_status st = convert_ops(ctx->n, ops, nops, matrices, conv, ctx->validate);
     if (st) return st;
-    for (QOp &op : conv) {
-        st = submit(ctx, std::move(op));
-        if (st) return st;
-    }
+    if (ctx->mode != QCW_MODE_FUSED) return plain_list(ctx, conv);
+    for (QOp &op : conv) ctx->queue.push_back(std::move(op));
     return QCW_OK;
 }
 

@@ -92,6 +92,27 @@ PauliPlan plan_pauli(const std::vector<QOp> &ops, size_t begin, size_t end, int 
 // |0..0>.
 PauliPlan plan_pauli_list(const qcw_op *ops, int nops, const double *matrices, int n, int kmax);
 
+// One pass of the plain path over rho (plain_list.cu): a run of a list's operations that stays on two
+// qubits, as maps of either and permutations; or one dense two-qubit map (T); or a map left over on
+// one qubit (b = -1).
+enum : int {
+    PK_MAP = 0,   // + 0, 1: trace-preserving map of a, of b; 12 coefficients (rows 1..3)
+    PK_GEN = 2,   // + 0, 1: general map, 16
+    PK_CX = 4,    // + 0: a controls; + 1: b controls
+    PK_CZ = 6
+};
+constexpr int kPairMaxOps = 16;  // a longer run is cut: the program travels as a kernel parameter
+struct PairProg {
+    int a = 0, b = -1;
+    std::vector<uint8_t> kind;
+    std::vector<float> coefs;
+    std::vector<double> T;  // index 4 p_a + p_b, labels as everywhere here
+    double one[16];         // b = -1
+};
+
+// Plan ops[begin, end) (k <= 2, no controls) as passes over rho, to be run in order.
+std::vector<PairProg> plan_pairs(const std::vector<QOp> &ops, size_t begin, size_t end, int n);
+
 // Position of 16-byte chunk c of a tile in shared memory: bits 0..2 (which 16 of 128 bytes) are
 // mixed with the bits above so that digits 1..6 of the tile each contribute a different plane of
 // GF(2)^3 there; any two digits then reach all eight positions, and a quarter-warp whose lanes

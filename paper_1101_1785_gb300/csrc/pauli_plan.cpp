@@ -621,4 +621,76 @@ PauliPlan plan_pauli_list(const qcw_op *ops, int nops, const double *matrices, i
     return plan_nodes(nb, n, kmax, false, true);
 }
 
+// Runs on pairs.  A node joins the pass of its qubits while no later pass holds one of them (so the
+// passes can run in the order they were opened); maps of a qubit that is in no open pass wait for its
+// next one, and the qubits left over at the end share passes two by two.
+std::vector<PairProg> plan_pairs(const std::vector<QOp> &ops, size_t begin, size_t end, int n)
+{
+    NodeBuilder nb(n, false);
+    for (size_t i = begin; i < end; i++) nb.add(OpView{ops[i].kind, ops[i].k, ops[i].qubits, ops[i].m.data()});
+    std::vector<PairProg> out;
+    std::vector<int> open(n, -1);
+    std::vector<M4> wait(n, m4_identity());
+    auto map = [&](PairProg &p, int q, const M4 &m) {
+        if (m.id) return;
+        const bool tp = m4_tp(m);
+        p.kind.push_back((uint8_t)((tp ? PK_MAP : PK_GEN) + (q == p.a ? 0 : 1)));
+        for (int i = tp ? 4 : 0; i < 16; i++) p.coefs.push_back((float)m.m[i]);
+    };
+    auto close = [&](int q) {
+        const int j = open[q];
+        if (j >= 0) open[out[j].a] = -1, open[out[j].b] = -1;
+    };
+    auto fresh = [&](int a, int b) -> PairProg & {
+        close(a), close(b);
+        open[a] = open[b] = (int)out.size();
+        PairProg p;
+        p.a = a, p.b = b;
+        for (int q : {a, b}) {
+            map(p, q, wait[q]);
+            wait[q] = m4_identity();
+        }
+        out.push_back(std::move(p));
+        return out.back();
+    };
+    for (const Node &nd : nb.finish()) {
+        if (nd.kind == PO_ONE) {
+            if (open[nd.a] >= 0 && (int)out[open[nd.a]].kind.size() < kPairMaxOps) map(out[open[nd.a]], nd.a, nd.A);
+            else {
+                close(nd.a);
+                m4_lmul(wait[nd.a], nd.A);
+            }
+            continue;
+        }
+        const bool same = open[nd.a] >= 0 && open[nd.a] == open[nd.b];
+        if (nd.kind == PO_TWO) {
+            PairProg &p = fresh(nd.a, nd.b);
+            p.T = nd.T;
+            if (!p.kind.empty()) {  // maps that waited: a pass of their own before
+                PairProg t;
+                t.a = nd.a, t.b = nd.b;
+                t.T.swap(p.T);
+                out.push_back(std::move(t));
+            }
+            open[nd.a] = open[nd.b] = -1;
+            continue;
+        }
+        PairProg &p = same && (int)out[open[nd.a]].kind.size() + 3 <= kPairMaxOps ? out[open[nd.a]] : fresh(nd.a, nd.b);
+        p.kind.push_back((uint8_t)(nd.kind == PO_CZ ? PK_CZ : nd.a == p.a ? PK_CX : PK_CX + 1));
+        map(p, nd.a, nd.A);
+        map(p, nd.b, nd.B);
+    }
+    std::vector<int> left;
+    for (int q = 0; q < n; q++)
+        if (!wait[q].id) left.push_back(q);
+    for (size_t i = 0; i + 1 < left.size(); i += 2) fresh(left[i], left[i + 1]);
+    if (left.size() % 2) {
+        PairProg p;
+        p.a = left.back();
+        std::copy(wait[p.a].m, wait[p.a].m + 16, p.one);
+        out.push_back(std::move(p));
+    }
+    return out;
+}
+
 }  // namespace qcw

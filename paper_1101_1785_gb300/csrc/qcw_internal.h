@@ -215,6 +215,12 @@ qcw_status fused_flush(qcw_ctx *ctx);
 void fused_destroy(qcw_ctx *ctx);
 void fused_collect_timing(qcw_ctx *ctx);
 qcw_status plain_apply(qcw_ctx *c, const QOp &op);
+qcw_status plain_gate2(qcw_ctx *c, const c128 *u, int q1, int q2, const int *ctrl, int nc);
+void quartet_layout(int n, int q1, int q2, int *pos, uint64_t *offr, uint64_t *offc);
+// One entry per row, at a distinct column, each exactly 1, -1, i or -i: sigma[i] = its column.
+bool monomial4(const c128 *u, int *sigma, c128 *val);
+// A whole list in plain mode (plain_list.cu): neighbouring one- and two-qubit operations in fewer passes.
+qcw_status plain_list(qcw_ctx *c, const std::vector<QOp> &ops);
 qcw_status ensure_full(qcw_ctx *c);
 // Whether fused work of this context runs in the Pauli basis (allocates pv on first use).
 bool pauli_allowed(qcw_ctx *c);

@@ -24,9 +24,8 @@ static void map4(std::vector<double *> &x, int stride, const float *m, bool tp)
     }
 }
 
-// Returns the number of passes; *bad counts positions a round visits not exactly once.
-extern "C" int pauli_replay(int n, int kmax, int beam, int zero, int nops, const int *kind, const int *k, const int *qubits,
-                            const double *mats, const long long *mat_off, double *v, int *nrounds, int *bad)
+static std::vector<QOp> op_list(int nops, const int *kind, const int *k, const int *qubits, const double *mats,
+                                const long long *mat_off)
 {
     std::vector<QOp> ops(nops);
     for (int i = 0; i < nops; i++) {
@@ -40,6 +39,14 @@ extern "C" int pauli_replay(int n, int kmax, int beam, int zero, int nops, const
         for (int t = 0; t < dim * dim; t++)
             o.m[t] = c128(mats[2 * (mat_off[i] + t)], mats[2 * (mat_off[i] + t) + 1]);
     }
+    return ops;
+}
+
+// Returns the number of passes; *bad counts positions a round visits not exactly once.
+extern "C" int pauli_replay(int n, int kmax, int beam, int zero, int nops, const int *kind, const int *k, const int *qubits,
+                            const double *mats, const long long *mat_off, double *v, int *nrounds, int *bad)
+{
+    const std::vector<QOp> ops = op_list(nops, kind, k, qubits, mats, mat_off);
     const PauliPlan plan = plan_pauli(ops, 0, ops.size(), n, kmax, beam != 0, zero != 0);
     if (zero)
         for (size_t i = 0; i < (size_t)1 << (2 * plan.nd); i++) {
@@ -147,4 +154,56 @@ extern "C" int pauli_replay(int n, int kmax, int beam, int zero, int nops, const
         }
     }
     return (int)plan.passes.size();
+}
+
+// The plain path's passes over a list, on the coefficients v; returns their number.
+extern "C" int pairs_replay(int n, int nops, const int *kind, const int *k, const int *qubits, const double *mats,
+                            const long long *mat_off, double *v)
+{
+    const std::vector<QOp> ops = op_list(nops, kind, k, qubits, mats, mat_off);
+    const std::vector<PairProg> progs = plan_pairs(ops, 0, ops.size(), n);
+    const size_t N = (size_t)1 << (2 * n);
+    std::vector<double *> x(N);
+    for (size_t i = 0; i < N; i++) x[i] = v + i;
+    for (const PairProg &p : progs) {
+        const int da = n - 1 - p.a, db = n - 1 - p.b;
+        if (p.b < 0) {
+            float m[16];
+            for (int i = 0; i < 16; i++) m[i] = (float)p.one[i];
+            map4(x, 1 << (2 * da), m, false);
+            continue;
+        }
+        if (p.kind.size() > (size_t)kPairMaxOps || (p.T.empty() && p.kind.empty())) return -1;
+        size_t c = 0;
+        for (uint8_t kd : p.kind) {
+            if (kd < PK_CX) {
+                const bool tp = kd < PK_GEN;
+                map4(x, 1 << (2 * ((kd & 1) ? db : da)), &p.coefs[c], tp);
+                c += tp ? 12 : 16;
+                continue;
+            }
+            const std::vector<double> in(v, v + N);
+            for (size_t i = 0; i < N; i++) {
+                const int s = kd == PK_CX + 1 ? db : da, t = kd == PK_CX + 1 ? da : db;  // control, target
+                int pc = (i >> (2 * s)) & 3, pt = (i >> (2 * t)) & 3;
+                const int xa = pc >> 1, za = pc & 1, xb = pt >> 1, zb = pt & 1;
+                const bool cz = kd == PK_CZ;
+                const double sg = (cz ? xa & xb & (za ^ zb) : xa & zb & (xb ^ za ^ 1)) ? -1 : 1;
+                const int fc = cz ? 2 * xa + (za ^ xb) : 2 * xa + (za ^ zb), ft = cz ? 2 * xb + (zb ^ xa) : 2 * (xb ^ xa) + zb;
+                const size_t from = (i & ~(((size_t)3 << (2 * s)) | ((size_t)3 << (2 * t)))) | ((size_t)fc << (2 * s)) | ((size_t)ft << (2 * t));
+                v[i] = sg * in[from];
+            }
+        }
+        if (c != p.coefs.size()) return -2;
+        if (!p.T.empty()) {
+            const std::vector<double> in(v, v + N);
+            for (size_t i = 0; i < N; i++) {
+                const size_t base = i & ~(((size_t)3 << (2 * da)) | ((size_t)3 << (2 * db)));
+                const int e = 4 * ((i >> (2 * da)) & 3) + ((i >> (2 * db)) & 3);
+                v[i] = 0;
+                for (int f = 0; f < 16; f++) v[i] += p.T[16 * e + f] * in[base | ((size_t)(f >> 2) << (2 * da)) | ((size_t)(f & 3) << (2 * db))];
+            }
+        }
+    }
+    return (int)progs.size();
 }

@@ -1,6 +1,7 @@
 """GPU parity of the one-pass kernel for operations on three to five qubits (gates and channels, one
 or several operators per launch, operators spread over blocks or summed over launches) and of the
-warp-per-output partial trace, against the oracle."""
+warp-per-output partial trace, against the oracle; operation lists on the plain path against the same
+operations one by one."""
 
 import numpy as np
 import pytest
@@ -98,3 +99,36 @@ def test_density_shared_out_over_the_vectors(q, n, nvec):
         assert abs(d.trace() - 1) <= 1e-6
         d.close()
     e.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 4, 6, 7, 8])
+@pytest.mark.parametrize("what", ["mixed", "haar70", "all"])
+def test_plain_lists(q, n, what):
+    """A list in plain mode joins its neighbours (all of it in one launch up to six qubits, a pass per
+    pair above); any matrix, not only a Hermitian one."""
+    rng = np.random.default_rng(90 * n)
+    if n == 1:
+        ops = [wl.Op("kraus" if i % 3 == 0 else "gate", (0,), np.stack([0.8 * haar_unitary(rng, 2), 0.6 * haar_unitary(rng, 2)])
+                     if i % 3 == 0 else haar_unitary(rng, 2)[None]) for i in range(12)]
+    else:
+        ops = wl.random_circuit(n, 150 if n < 7 else 60, 31 + n, "haar70" if what == "haar70" else "mixed", "adpd").ops
+    if what == "all" and n > 1:  # dense gates and channels, permutations, wider operations, lost trace
+        for i in range(0, 40, 4):
+            a, b = (int(x) for x in rng.permutation(n)[:2])
+            s = wl.gate_matrix("SWAP")
+            ops.insert(3 * i, wl.Op("gate", (a, b), (s, haar_unitary(rng, 4), s @ wl.gate_matrix("CNOT") @ s)[i % 3][None]))
+            ops.insert(3 * i, wl.Op("kraus", (b, a), np.stack([np.sqrt(0.6) * haar_unitary(rng, 4), 0.6 * haar_unitary(rng, 4)])))
+            ops.insert(3 * i, wl.Op("kraus", (a,), np.stack([np.sqrt(0.6) * haar_unitary(rng, 2), 0.63 * haar_unitary(rng, 2)])))
+            if n > 3:
+                ops.insert(3 * i, wl.Op("gate", tuple(int(x) for x in rng.permutation(n)[:3]), haar_unitary(rng, 8)[None]))
+    z = rng.standard_normal((1 << n, 1 << n)) + 1j * rng.standard_normal((1 << n, 1 << n))
+    z /= np.linalg.norm(z)
+    a, b = q.Density(n), q.Density(n)
+    a.set_state(z), b.set_state(z)
+    a.apply_packed(q.PackedOps(ops))
+    for op in ops:
+        b.apply_op(op)
+    # a handful of FP32 roundings per operation on either side, of elements of norm at most 1
+    assert np.abs(a.get_state() - b.get_state()).max() <= 8 * len(ops) * 2.0 ** -24
+    assert a.stats()["launches"] < b.stats()["launches"]
+    a.close(), b.close()

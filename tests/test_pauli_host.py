@@ -47,7 +47,7 @@ def test_coefficient_helper():
         assert abs(np.trace(p @ rho) - v[i]) < 1e-12
 
 
-def _replay(shim, n, ops, v, kmax, beam, zero=False):
+def _packed(ops):
     kind, k, qs, mats, off = [], [], [], [], []
     pos = 0
     for op in ops:
@@ -64,6 +64,11 @@ def _replay(shim, n, ops, v, kmax, beam, zero=False):
     I = lambda a: np.asarray(a, dtype=np.int32)
     kind, k, qs, off = I(kind), I(k), I(qs), np.asarray(off, dtype=np.int64)
     mats = np.concatenate(mats)
+    return kind, k, qs, mats, off
+
+
+def _replay(shim, n, ops, v, kmax, beam, zero=False):
+    kind, k, qs, mats, off = _packed(ops)
     nr, bad = ctypes.c_int(), ctypes.c_int()
     p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
     npass = shim.pauli_replay(n, kmax, int(beam), int(zero), len(ops), p(kind), p(k), p(qs), p(mats), p(off), p(v),
@@ -129,3 +134,26 @@ def test_plan_from_the_zero_state(shim, n, what):
     v = np.zeros(4 ** n)
     _replay(shim, n, ops, v, 0, False, True)
     assert np.linalg.norm(v - coefficients(want)) <= (len(ops) + n) * 2.0 ** -24 * np.linalg.norm(coefficients(want))
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 6])
+@pytest.mark.parametrize("what", ["mixed", "haar70", "two", "ones"])
+def test_plain_list_passes(shim, n, what):
+    """The plain path's passes over a list (runs on two qubits, dense two-qubit maps, maps left over)."""
+    rng = np.random.default_rng(7 * n)
+    if n == 1 or what == "ones":
+        ops = [wl.Op("gate", (int(rng.integers(n)),), haar_unitary(rng, 2)[None]) for _ in range(9)]
+    elif what == "two":
+        ops = _two_qubit_ops(rng, n, 30)
+    else:
+        ops = wl.random_circuit(n, 80, 9 + n, what, "adpd" if what == "mixed" else "dep").ops
+    rho = random_rho(rng, n)
+    v = coefficients(rho)
+    want = rho.copy()
+    for op in ops:
+        oracle.apply_op(want, op)
+    kind, k, qs, mats, off = _packed(ops)
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    passes = shim.pairs_replay(n, len(ops), p(kind), p(k), p(qs), p(mats), p(off), p(v))
+    assert 0 < passes < len(ops)
+    assert np.linalg.norm(v - coefficients(want)) <= len(ops) * 2.0 ** -24 * np.linalg.norm(coefficients(want))
