@@ -486,12 +486,13 @@ void launch_c64_to_c128(const float2 *src, double2 *dst, size_t count, int nsm, 
 // --------------------------------------------------------------------- FP64 readouts
 // Reductions accumulate per thread, fold each warp with shuffles, each block through
 // shared memory into `partials[block][v]`, and a one-block kernel adds the partials in
-// block order: a fixed tree, so the result does not depend on scheduling.
+// block order: a fixed tree, so the result does not depend on scheduling.  One block writes the
+// result itself: the second launch (3 us with its gap) is most of a small register's readout.  Each
+// launch_* returns its number of launches.
 constexpr int RED_THREADS = 256;
 constexpr int MAXV = QCW_MAX_QUBITS + 2;
 
 int reduce_blocks(int nsm) { return nsm * 4; }
-int launches_per_reduce() { return 2; }
 
 template <int NV>
 __device__ __forceinline__ void block_store(double (&acc)[NV], int nv, double *partials)
@@ -544,14 +545,15 @@ __global__ void __launch_bounds__(RED_THREADS) k_diag(const float2 *__restrict__
     block_store<MAXV>(acc, n + 2, partials);
 }
 
-void launch_diag_reduce(const float2 *rho, int n, double *partials, double *out, int nblocks,
+int launch_diag_reduce(const float2 *rho, int n, double *partials, double *out, int nblocks,
                         cudaStream_t s)
 {
     uint64_t dim = 1ull << n;
     uint64_t need = (dim + RED_THREADS - 1) / RED_THREADS;
     int nb = (int)(need < (uint64_t)nblocks ? need : (uint64_t)nblocks);
-    k_diag<<<nb, RED_THREADS, 0, s>>>(rho, n, partials);
-    k_fold<<<n + 2, 32, 0, s>>>(partials, nb, n + 2, out);
+    k_diag<<<nb, RED_THREADS, 0, s>>>(rho, n, nb == 1 ? out : partials);
+    if (nb > 1) k_fold<<<n + 2, 32, 0, s>>>(partials, nb, n + 2, out);
+    return nb > 1 ? 2 : 1;
 }
 
 // Purity: sum |rho_ij|^2.  Squares and short sums in FP32 (8 elements), totals in FP64.
@@ -578,13 +580,15 @@ __global__ void __launch_bounds__(RED_THREADS) k_purity(const float4 *__restrict
     block_store<1>(acc, 1, partials);
 }
 
-void launch_purity(const float2 *rho, int n, double *partials, double *out, int nblocks, cudaStream_t s)
+int launch_purity(const float2 *rho, int n, double *partials, double *out, int nblocks, cudaStream_t s)
 {
     uint64_t n4 = (1ull << (2 * n)) / 2;
     uint64_t need = (n4 + RED_THREADS - 1) / RED_THREADS;
     int nb = (int)(need < (uint64_t)nblocks ? need : (uint64_t)nblocks);
-    k_purity<<<nb, RED_THREADS, 0, s>>>(reinterpret_cast<const float4 *>(rho), n4, partials);
-    k_fold<<<1, 32, 0, s>>>(partials, nb, 1, out);
+    if (n4 <= 8 * RED_THREADS) nb = 1;  // six qubits: two loads of four per thread
+    k_purity<<<nb, RED_THREADS, 0, s>>>(reinterpret_cast<const float4 *>(rho), n4, nb == 1 ? out : partials);
+    if (nb > 1) k_fold<<<1, 32, 0, s>>>(partials, nb, 1, out);
+    return nb > 1 ? 2 : 1;
 }
 
 // Purity of a Hermitian rho from its lower triangle: sum_r |rho_rr|^2 + 2 sum_{r > c} |rho_rc|^2.
@@ -659,7 +663,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_pauli_expect(const float2 *__re
     }
 }
 
-void launch_pauli_expect(const float2 *rho, int n, const PauliTerms &T, double *partials, int max_partials,
+int launch_pauli_expect(const float2 *rho, int n, const PauliTerms &T, double *partials, int max_partials,
                          double *out, cudaStream_t s)
 {
     const uint64_t dim = 1ull << n;
@@ -667,8 +671,9 @@ void launch_pauli_expect(const float2 *rho, int n, const PauliTerms &T, double *
     uint64_t nb = (uint64_t)max_partials / (uint64_t)T.count;
     if (nb > need) nb = need;
     if (nb < 1) nb = 1;
-    k_pauli_expect<<<dim3((unsigned)nb, T.count), RED_THREADS, 0, s>>>(rho, n, T, partials);
-    k_fold<<<T.count, 32, 0, s>>>(partials, (int)nb, T.count, out);
+    k_pauli_expect<<<dim3((unsigned)nb, T.count), RED_THREADS, 0, s>>>(rho, n, T, nb == 1 ? out : partials);
+    if (nb > 1) k_fold<<<T.count, 32, 0, s>>>(partials, (int)nb, T.count, out);
+    return nb > 1 ? 2 : 1;
 }
 
 // out[0] = the sum of nblocks partials (fixed tree).
@@ -677,12 +682,13 @@ void launch_fold(const double *partials, int nblocks, double *out, cudaStream_t 
     k_fold<<<1, 32, 0, s>>>(partials, nblocks, 1, out);
 }
 
-void launch_purity_lower(const float2 *rho, int n, double *partials, double *out, int nblocks, cudaStream_t s)
+int launch_purity_lower(const float2 *rho, int n, double *partials, double *out, int nblocks, cudaStream_t s)
 {
     const uint64_t dim = 1ull << n;
     int nb = (int)(dim < (uint64_t)nblocks ? dim : (uint64_t)nblocks);
-    k_purity_lower<<<nb, RED_THREADS, 0, s>>>(reinterpret_cast<const float4 *>(rho), n, partials);
-    k_fold<<<1, 32, 0, s>>>(partials, nb, 1, out);
+    k_purity_lower<<<nb, RED_THREADS, 0, s>>>(reinterpret_cast<const float4 *>(rho), n, nb == 1 ? out : partials);
+    if (nb > 1) k_fold<<<1, 32, 0, s>>>(partials, nb, 1, out);
+    return nb > 1 ? 2 : 1;
 }
 
 // Complete rho from its lower triangle: rho[r][c] = conj(rho[c][r]) for r < c.  32 x 32 blocks:

@@ -816,14 +816,15 @@ __global__ void __launch_bounds__(kPpThreads) k_pauli_purity(const float4 *__res
     }
 }
 
-void launch_pauli_purity(const float *v, int n, double *partials, double *out, int nblocks, cudaStream_t s)
+int launch_pauli_purity(const float *v, int n, double *partials, double *out, int nblocks, cudaStream_t s)
 {
     const uint64_t n4 = 1ull << (2 * n - 2), need = (n4 + 4 * kPpThreads - 1) / (4 * kPpThreads);
     const int nb = (int)(need < (uint64_t)nblocks ? need : (uint64_t)nblocks);
     double scale = 1.0;
     for (int i = 0; i < n; i++) scale *= 0.5;
-    k_pauli_purity<<<nb, kPpThreads, 0, s>>>(reinterpret_cast<const float4 *>(v), n4, scale, partials);
-    launch_fold(partials, nb, out, s);
+    k_pauli_purity<<<nb, kPpThreads, 0, s>>>(reinterpret_cast<const float4 *>(v), n4, scale, nb == 1 ? out : partials);
+    if (nb > 1) launch_fold(partials, nb, out, s);
+    return nb > 1 ? 2 : 1;
 }
 
 // Reduced state of the kept qubits (k <= 6): their strings' coefficients, changed to rho_A in FP64.

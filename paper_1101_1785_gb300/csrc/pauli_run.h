@@ -35,7 +35,7 @@ cudaError_t launch_pauli_zero(float *v, int n, int nsm, cudaStream_t s);
 void launch_pauli_diag(const float *v, int n, double *out, cudaStream_t s);
 void launch_pauli_terms(const float *v, const PauliTerms &T, double *out, cudaStream_t s);
 void launch_pauli_project(float *v, int n, int qubit, int m, double scale, int nsm, cudaStream_t s);
-void launch_pauli_purity(const float *v, int n, double *partials, double *out, int nblocks, cudaStream_t s);
+int launch_pauli_purity(const float *v, int n, double *partials, double *out, int nblocks, cudaStream_t s);
 constexpr int kPauliPtMax = 6;  // most kept qubits of launch_pauli_ptrace
 void launch_pauli_ptrace(const float *v, const PTParams &p, double2 *out, cudaStream_t s);
 

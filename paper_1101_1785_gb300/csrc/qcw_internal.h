@@ -79,15 +79,15 @@ void launch_c128_to_c64(const double2 *src, float2 *dst, size_t count, int nsm, 
 void launch_c64_to_c128(const float2 *src, double2 *dst, size_t count, int nsm, cudaStream_t s);
 // Reductions write `nvals` doubles per block into partials, then fold them in block order.
 int reduce_blocks(int nsm);
-void launch_diag_reduce(const float2 *rho, int n, double *partials, double *out, int nblocks,
+int launch_diag_reduce(const float2 *rho, int n, double *partials, double *out, int nblocks,
                         cudaStream_t s);
-void launch_purity(const float2 *rho, int n, double *partials, double *out, int nblocks,
+int launch_purity(const float2 *rho, int n, double *partials, double *out, int nblocks,
                    cudaStream_t s);
 void launch_project(float2 *rho, int n, int qubit, int m, float scale, bool lower, int nsm, cudaStream_t s);
 // Half storage: rho[r][c] = conj(rho[c][r]) for r < c (complete the matrix from its lower
 // triangle), and purity from the lower triangle (2 |rho_rc|^2 below the diagonal).
 void launch_symmetrize(float2 *rho, int n, int nsm, cudaStream_t s);
-void launch_purity_lower(const float2 *rho, int n, double *partials, double *out, int nblocks, cudaStream_t s);
+int launch_purity_lower(const float2 *rho, int n, double *partials, double *out, int nblocks, cudaStream_t s);
 void launch_fold(const double *partials, int nblocks, double *out, cudaStream_t s);
 // Multiverse density on the tensor cores (ensemble_tc.cu) for 2^n >= 128: rho = sum_v w_v
 // |psi_v><psi_v|; *err gets bit 0 if a bounded wait ran out.  Returns false if not launched.
@@ -114,13 +114,12 @@ struct PauliTerms {
     int ny[kMaxPauliTerms];
 };
 // out[s] = Re Tr[P_s rho] for s < T.count (count <= 63), reading only the lower triangle.
-void launch_pauli_expect(const float2 *rho, int n, const PauliTerms &T, double *partials, int max_partials,
+int launch_pauli_expect(const float2 *rho, int n, const PauliTerms &T, double *partials, int max_partials,
                          double *out, cudaStream_t s);
 // The purity partials of the last fused pass, if they describe the current rho.
 bool fused_purity_partials(qcw_ctx *c, const double **partials, int *nblocks);
 void launch_partial_trace(const float2 *rho, const PTParams &p, double2 *out, int nsm,
                           cudaStream_t s);
-int launches_per_reduce();
 
 // ------------------------------------------------------------------ queued operation
 struct QOp {
@@ -153,6 +152,7 @@ struct qcw_ctx {
     // reduction scratch: per-block partials and a small result block (+ pinned mirror)
     double *d_partials = nullptr;
     int red_blocks = 0;
+    double2 *d_pt = nullptr, *h_pt = nullptr;  // partial-trace results (api.cu reduced_buffers)
     double *d_result = nullptr;
     double *h_result = nullptr;  // pinned, 64 doubles
     // staging for complex128 <-> complex64 conversion
