@@ -4,8 +4,8 @@
 Workload (one "step"): a 14-qubit density matrix (16384 x 16384 complex64 on the device)
 starts in |0..0><0..0|; a seeded 1000-gate circuit (kinds uniform over H, X, Z, S, T,
 CNOT, Haar SU(2)) runs with amplitude damping (gamma = 0.01) and phase damping
-(lambda = 0.02) on every touched qubit after each gate, in the fused path (planner +
-Hermitian fused-pass kernel, fusion width chosen per segment by the library's cost model).  After every 100 gates the step reads trace and purity
+(lambda = 0.02) on every touched qubit after each gate, in the fused path (planner + pass kernel on
+the real Pauli coefficients; with ``--fused-kernel`` the kernels on rho).  After every 100 gates the step reads trace and purity
 in FP64; at the end it reads the per-qubit probabilities, measures qubit 0 (u-driven
 projective measurement with renormalisation) and takes the partial trace over qubits 0, 1.
 
@@ -188,16 +188,20 @@ def d2h_bytes_per_step(n):
     return (N_GATES // CHUNK) * (n + 4) * 8 + 2 * 64 * 8 + 16 * (4 ** len(PT_KEEP))
 
 
-def pass_unit_bytes(n):
-    """Algorithmic bytes of one fused pass: one read and one write of rho in complex64."""
-    return 16 * 4 ** n
+def pass_unit_bytes(n, kernel=None):
+    """Algorithmic bytes of one fused pass: one read and one write of rho in complex64, or of its
+    4^n real Pauli coefficients where the pass works on those."""
+    return (8 if kernel == "k_pauli_pass" else 16) * 4 ** n
 
 
 def design_pass_bytes(n, kernel, tile_qubits=6):
     """HBM bytes the timed pass kernel is designed to move.  The warp-specialised kernel reads
     and writes the canonical copy of each tile pair (one tile's worth each way, M (M + 1) / 2
     pairs, M = 2^(n - 6)); the per-tile-pair Hermitian kernel reads a tile and writes it and
-    its mirror; the general kernel reads and writes every element."""
+    its mirror; the general kernel reads and writes every element, the Pauli-basis kernel every
+    coefficient."""
+    if kernel == "k_pauli_pass":
+        return pass_unit_bytes(n, kernel)
     if kernel == "k_fused_pass" or n <= tile_qubits:
         return 16 * 4 ** n
     m = 1 << (n - tile_qubits)
@@ -206,7 +210,7 @@ def design_pass_bytes(n, kernel, tile_qubits=6):
     return tile * 2 * pairs if kernel in ("k_fused_herm_ws", "k_fused_herm_tc") else tile * (pairs + m * m)
 
 
-TIMED_KERNEL = {"auto": "k_fused_herm_ws", "herm_tc": "k_fused_herm_tc", "herm_ws": "k_fused_herm_ws",
+TIMED_KERNEL = {"auto": "k_pauli_pass", "herm_tc": "k_fused_herm_tc", "herm_ws": "k_fused_herm_ws",
                 "herm": "k_fused_herm", "tile": "k_fused_pass"}
 
 
@@ -216,7 +220,8 @@ def kernel_hash():
     import re
 
     h = hashlib.sha256()
-    for f in ("fused.cu", "planner.cpp", "qcw_device.cuh", "tile.cuh", "tile.cpp", "tc.cuh"):
+    for f in ("fused.cu", "planner.cpp", "qcw_device.cuh", "tile.cuh", "tile.cpp", "tc.cuh", "pauli.cu", "pauli.cuh",
+              "pauli_plan.cpp"):
         with open(os.path.join(ROOT, "paper_1101_1785_gb300", "csrc", f)) as fh:
             src = fh.read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
@@ -496,7 +501,7 @@ def run_ours(args):
     e2e_value = replica_rate(N_GATES, args.steps, world, e2e_s)
 
     peaks, peak_kind = load_peaks()
-    per_launch_bytes = pass_unit_bytes(nq)
+    per_launch_bytes = pass_unit_bytes(nq, TIMED_KERNEL[args.fused_kernel])
     avg_ms = st["fused_pass_ms"] / max(1, st["timed_passes"])
     achieved = per_launch_bytes / (avg_ms / 1e3) / 1e9
     hbm = float(peaks["hbm_gbs"])
@@ -527,8 +532,9 @@ def run_ours(args):
                        "l2": f"inputs larger than L2 ({8 * 4 ** nq / 2**20:.0f} MiB rho vs 129 MB L2)"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm, "traffic": traffic,
-                         "achieved_is": "algorithmic bytes (one read and one write of rho, 16 * 4^n) per pass "
-                                        "launch / the launch's event-timed duration",
+                         "achieved_is": "algorithmic bytes (one read and one write of the state: its 4^n real Pauli "
+                                        "coefficients, 8 * 4^n, or rho, 16 * 4^n) per pass launch / the "
+                                        "launch's event-timed duration",
                          "dram_gbs": None if traffic is None else traffic / (avg_ms / 1e3) / 1e9,
                          "peak_kind": peak_kind, "kernel": TIMED_KERNEL[args.fused_kernel],
                          "bytes_per_launch": per_launch_bytes,

@@ -353,9 +353,9 @@ QCW_API qcw_status qcw_partial_trace_static(const void *dev_rho, int nqubits, co
  * separate processors (Sec. 5.1, Sec. 5.2.1); here they share one GPU.  Circuit j has
  * nqubits[j] (1..QCW_MAX_QUBITS) qubits, starts in |0..0><0..0| and applies
  * ops[op_begin[j] .. op_begin[j+1]) (1- and 2-qubit gates and Kraus channels, matrices as in
- * qcw_apply_ops).  fuse_k (0 = chosen per circuit by the cost model, else 2..5) bounds the
- * qubits of a fused pass.  Creation plans every circuit, allocates one device arena for all
- * states and captures the whole run (one persistent kernel) in a CUDA graph on cuda_stream
+ * qcw_apply_ops).  fuse_k (2..5) bounds the qubits of a fused pass; 0: a pass works on every
+ * qubit of its tile.  Creation plans every circuit, allocates one device arena for all
+ * states (kept as 4^n real Pauli coefficients) and captures the whole run (one persistent kernel) in a CUDA graph on cuda_stream
  * (NULL: a non-blocking stream owned by the batch, since the legacy stream cannot be captured).  All arrays are copied; the caller may free them on return. */
 typedef struct qcw_batch qcw_batch;
 QCW_API qcw_status qcw_batch_create(int ncirc, const int *nqubits, const long long *op_begin, const qcw_op *ops,
@@ -370,7 +370,7 @@ QCW_API qcw_status qcw_batch_wait(qcw_batch *b, double timeout_s);
 QCW_API qcw_status qcw_batch_results(qcw_batch *b, double *p1, double *purity, double *trace);
 /* Final rho of one circuit as host complex128 (2 * 4^n doubles). */
 QCW_API qcw_status qcw_batch_get_state(qcw_batch *b, int circuit, double *rho_c128);
-/* Work items, fused passes, phases and modeled SM-seconds of one run. */
+/* Work items, fused passes, rounds of the passes and modeled SM-seconds of one run. */
 QCW_API qcw_status qcw_batch_info(qcw_batch *b, long long *items, long long *passes, long long *phases,
                                   double *modeled_sm_s);
 /* Diagnostics: bound every in-kernel dependency wait to `polls` polls (~128 ns each) and, when

@@ -14,7 +14,9 @@
 // else is in the batch.
 //
 // Two CTAs per SM (64 KiB tile and the pass's program each) overlap one's loads with the other's
-// rounds.  64 circuits of 4 to 10 qubits: on complex tiles without symmetry 1.01 ms per launch.
+// rounds.  64 circuits of 4 to 10 qubits, 50 to 400 gates deep: 0.40 ms per launch (on complex tiles
+// without symmetry 1.01 ms); the passes of the deepest ten-qubit circuit, one after the other, are the
+// longest chain.
 #include <algorithm>
 #include <cstring>
 

@@ -870,9 +870,9 @@ static const size_t kMaxCached = 64;
 constexpr int kBeamMinQubits = 10;
 
 // Whether a state held as rho is changed to Pauli storage for a plan.  The two changes of basis cost
-// 2.6 ms at 14 qubits, a pass on rho 1.1 ms and the completion of its upper triangle 0.35 ms, and a
-// Pauli pass does the work of about 1.4 passes on rho in 0.6 ms: from two Pauli passes on the
-// change is about even or better, a single one does not win it back.
+// 1.7 ms at 14 qubits, a pass on rho 1.1 ms and the completion of its upper triangle 0.35 ms, and a
+// Pauli pass does the work of about 1.4 passes on rho in 0.56 ms: two Pauli passes with the changes
+// take 2.8 ms against 3.4 ms, a single one 2.3 ms against 1.9 ms.
 static bool pauli_pays(const CachedPauli &p) { return p.passes.size() > 1; }
 
 // The segment in the Pauli basis; *done = false: it is better run on rho.

@@ -1,6 +1,5 @@
 // Device side of a fused pass over one tile: cp.async load into shared memory, the pass's
-// phases applied in place, write-back.  Used by k_fused_pass (one tile per CTA) and by the
-// batched persistent kernel (a CTA walks all tiles of all passes of one circuit).
+// phases applied in place, write-back.  Used by k_fused_pass (one tile per CTA).
 //
 // A phase is a composed superoperator on one or two qubits of the pass.  A two-qubit phase
 // gathers 16-element groups (the row quartet x column quartet of Sec. 3.2 for the phase's
@@ -450,26 +449,18 @@ __device__ __forceinline__ uint64_t tile_base(const FPass &P, uint64_t tile)
     return base;
 }
 
-// Bring tile `t` of pass P into shared memory (or, with init, write |0..0><0..0| there: the
-// element of global index 0 is tile index 0 of tile 0).  Expects sm.hoff filled for P.
-__device__ __forceinline__ void tile_load(const float2 *__restrict__ rho, const FPass &P, uint64_t t, const TileSmem &sm,
-                                          bool init)
+// Bring tile `t` of pass P into shared memory.  Expects sm.hoff filled for P.
+__device__ __forceinline__ void tile_load(const float2 *__restrict__ rho, const FPass &P, uint64_t t, const TileSmem &sm)
 {
     const int TB = P.TB, L = P.L;
     const unsigned nvec = 1u << (TB - 1);
-    if (init) {
-        float4 *t4 = reinterpret_cast<float4 *>(sm.tile);
-        for (unsigned v = threadIdx.x; v < nvec; v += kTileThreads)
-            t4[v] = (t == 0 && v == 0) ? make_float4(1.f, 0.f, 0.f, 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
-    } else {
-        const uint64_t base = tile_base(P, t);
-        const unsigned lmask = (1u << L) - 1u;
-        for (unsigned v = threadIdx.x; v < nvec; v += kTileThreads) {
-            unsigned e = 2 * v;
-            cp_async16(&sm.tile[e], rho + base + sm.hoff[e >> L] + (e & lmask));
-        }
-        cp_async_wait_all();
+    const uint64_t base = tile_base(P, t);
+    const unsigned lmask = (1u << L) - 1u;
+    for (unsigned v = threadIdx.x; v < nvec; v += kTileThreads) {
+        unsigned e = 2 * v;
+        cp_async16(&sm.tile[e], rho + base + sm.hoff[e >> L] + (e & lmask));
     }
+    cp_async_wait_all();
     __syncthreads();
 }
 
@@ -520,9 +511,9 @@ __device__ __forceinline__ void tile_store(float2 *__restrict__ rho, const FPass
 // __syncthreads() after that; the caller synchronises before reusing shared memory.
 __device__ __forceinline__ void tile_process(float2 *__restrict__ rho, const FPass &P, uint64_t t,
                                              const FPhase *__restrict__ phases, const float2 *__restrict__ coefs,
-                                             const TileSmem &sm, bool init = false)
+                                             const TileSmem &sm)
 {
-    tile_load(rho, P, t, sm, init);
+    tile_load(rho, P, t, sm);
     tile_phases(P, phases, coefs, sm);
     tile_store(rho, P, t, sm);
 }

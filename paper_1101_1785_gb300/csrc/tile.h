@@ -1,5 +1,5 @@
-// Pass / phase descriptors shared by the fused-pass kernel and the batched persistent
-// kernel, and the host routine that turns planner output into them.
+// Pass / phase descriptors of the fused-pass kernels on rho, and the host routine that turns planner
+// output into them.
 //
 // A pass touches a qubit set Q.  Its tile is the set of 2^TB elements whose flat indices
 // differ only in the "tile bits": the row and column bits of Q plus the lowest column bits
