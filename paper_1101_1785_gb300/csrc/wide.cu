@@ -10,7 +10,7 @@
 // apart and combined once per output, 2 d per element and operator: the arithmetic bounds k = 4
 // and 5 and channels of several operators, HBM a three-qubit gate.  Measured at 12 qubits (rho =
 // 128 MiB) against two side passes and, per operator, a copy and an accumulation: five-qubit gate
-// 395 -> 253 us, channel of three three-qubit operators 570 -> 223 us; the 17-operator channel on all
+// 395 -> 253 us, channel of three three-qubit operators 570 -> 178 us; the 17-operator channel on all
 // of a 5-qubit register (one tile) 420 us -> 25 us with an operator per block.
 #include "qcw_device.cuh"
 #include "qcw_internal.h"
@@ -36,18 +36,30 @@ __host__ __device__ constexpr int wide_ty(int k) { return (1 << k) * wide_py(k) 
 
 // add: also add what it holds at the same places (may be out).  grid.y > 1: block row y runs operator y alone and writes its own
 // copy out + y * 4^n (few tiles: the operators spread over the chip, k_wide_sum adds the copies).
-template <int K, int ENT>
+// ALL: the operators of the launch stay in shared memory (48 of k = 3 take 54 KiB), so that the loop
+// over them has no barriers and a tile's column is read once; else each operator is staged for each
+// tile.  12 qubits, k = 3, staged / ALL: 3 operators 225 / 178 us, 8 540 / 391, 17 906 / 779, 48 2519 /
+// 2405.  For k = 4 the columns kept cost 40 registers more and a quarter of the warps: 2 operators 239 /
+// 258 us, 4 406 / 472; there and for k = 5 each operator is staged.
+template <int K, int ENT, bool ALL>
 __global__ void __launch_bounds__(kWideThreads) k_wide(const float2 *rho, float2 *out, const float2 *add,
                                                        uint64_t ntiles, uint64_t elems, const __grid_constant__ WideParams<ENT> p)
 {
     constexpr int D = 1 << K, TP = 32 / D, PK = D + 1, PY = wide_py(K), RB = K == 5 ? 16 : 8;
     extern __shared__ __align__(16) unsigned char smem[];
     float4 *Ks = reinterpret_cast<float4 *>(smem);                      // (k_r, k_r, k_i, k_i), pitch PK
-    float2 *Ys = reinterpret_cast<float2 *>(Ks + D * PK);               // per warp TP tiles
+    float2 *Ys = reinterpret_cast<float2 *>(Ks + (ALL ? p.nk : 1) * D * PK);  // per warp TP tiles
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = lane & (D - 1), t = lane >> K;
     float2 *Y = Ys + (w * TP + t) * wide_ty(K);
     const int j0 = gridDim.y > 1 ? blockIdx.y : 0, j1 = gridDim.y > 1 ? j0 + 1 : p.nk;
     float2 *dst = out + (gridDim.y > 1 ? blockIdx.y * elems : 0);
+    if constexpr (ALL) {
+        for (int e = threadIdx.x; e < p.nk * D * D; e += kWideThreads) {
+            const float2 m = p.m[e];
+            Ks[(e >> K) * PK + (e & (D - 1))] = make_float4(m.x, m.x, m.y, m.y);
+        }
+        __syncthreads();
+    }
     uint64_t coff = 0;
 #pragma unroll
     for (int b = 0; b < K; b++) coff |= (uint64_t)((c >> b) & 1) << p.cbit[b];
@@ -68,24 +80,31 @@ __global__ void __launch_bounds__(kWideThreads) k_wide(const float2 *rho, float2
         float2 res[D];
 #pragma unroll
         for (int r = 0; r < D; r++) res[r] = make_float2(0.f, 0.f);
-        for (int j = j0; j < j1; j++) {
-            if (first != blockIdx.x * per || j != j0 || j1 - j0 > 1) __syncthreads();  // the last readers of Ks are done
-            if (j1 - j0 > 1 || first == blockIdx.x * per)
-                for (int e = threadIdx.x; e < D * D; e += kWideThreads) {
-                    const float2 m = ENT > 0 ? p.m[j * D * D + e] : p.g[j * D * D + e];
-                    Ks[(e >> K) * PK + (e & (D - 1))] = make_float4(m.x, m.x, m.y, m.y);
-                }
-            float2 x[D];
+        float2 x[D];
+        if constexpr (ALL) {
 #pragma unroll
             for (int r = 0; r < D; r++) x[r] = on ? src[roff(r)] : make_float2(0.f, 0.f);
-            __syncthreads();
+        }
+        for (int j = j0; j < j1; j++) {
+            if constexpr (!ALL) {
+                if (first != blockIdx.x * per || j != j0 || j1 - j0 > 1) __syncthreads();  // the last readers of Ks are done
+                if (j1 - j0 > 1 || first == blockIdx.x * per)
+                    for (int e = threadIdx.x; e < D * D; e += kWideThreads) {
+                        const float2 m = ENT > 0 ? p.m[j * D * D + e] : p.g[j * D * D + e];
+                        Ks[(e >> K) * PK + (e & (D - 1))] = make_float4(m.x, m.x, m.y, m.y);
+                    }
+#pragma unroll
+                for (int r = 0; r < D; r++) x[r] = on ? src[roff(r)] : make_float2(0.f, 0.f);
+                __syncthreads();
+            }
+            const float4 *Kj = Ks + (ALL ? j * D * PK : 0);
             if constexpr (K == 5 || ENT == 0) {  // Y = K T, K broadcast from shared memory
 #pragma unroll 4
                 for (int r = 0; r < D; r++) {
                     unsigned long long a = 0ull, b = 0ull;
 #pragma unroll
                     for (int l = 0; l < D; l++) {
-                        const ulonglong2 k = *reinterpret_cast<const ulonglong2 *>(Ks + r * PK + l);
+                        const ulonglong2 k = *reinterpret_cast<const ulonglong2 *>(Kj + r * PK + l);
                         const unsigned long long xl = pack2(x[l].x, x[l].y);
                         a = ffma2(k.x, xl, a);
                         b = ffma2(k.y, xl, b);
@@ -111,7 +130,7 @@ __global__ void __launch_bounds__(kWideThreads) k_wide(const float2 *rho, float2
                 for (int i = 0; i < RB; i++) a[i] = b[i] = 0ull;
 #pragma unroll 4
                 for (int l = 0; l < D; l++) {
-                    const ulonglong2 k = *reinterpret_cast<const ulonglong2 *>(Ks + c * PK + l);
+                    const ulonglong2 k = *reinterpret_cast<const ulonglong2 *>(Kj + c * PK + l);
 #pragma unroll
                     for (int i = 0; i < RB; i += 2) {
                         const ulonglong2 y = *reinterpret_cast<const ulonglong2 *>(Y + l * PY + rb + i);
@@ -187,8 +206,14 @@ static cudaError_t run_wide(const WideOp &op, int first, int count, const float2
         const c128 z = op.m[(size_t)first * D * D + i];
         p.m[i] = make_float2((float)z.real(), (float)z.imag());
     }
-    auto kern = k_wide<K, ENT>;
-    const size_t sm = sizeof(float4) * D * (D + 1) + sizeof(float2) * (kWideThreads / 32) * TP * wide_ty(K);
+    const size_t ks = sizeof(float4) * D * (D + 1);
+    auto kern = k_wide<K, ENT, false>;
+    bool all = false;
+    if constexpr (K == 3 && ENT == kWideEntries) {
+        all = !split;
+        if (all) kern = k_wide<K, ENT, true>;
+    }
+    const size_t sm = (all ? count : 1) * ks + sizeof(float2) * (kWideThreads / 32) * TP * wide_ty(K);
     if (ensure_smem_attr(reinterpret_cast<const void *>(kern), sm)) return cudaErrorInvalidValue;
     const uint64_t ntiles = 1ull << (2 * (n - K)), per = (uint64_t)(kWideThreads / 32) * TP;
     const uint64_t need = (ntiles + per - 1) / per, cap = (uint64_t)nsm * 16;
