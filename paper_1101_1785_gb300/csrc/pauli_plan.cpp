@@ -233,11 +233,17 @@ int classify(const OpView &op, int *a, int *b)
 // depolarising factor 1 - 4 p / 3, say) rounds the same way each time, so the coefficients it
 // shrinks would drift by up to 3e-8 per application, all in one direction.  c: the scale error the
 // qubit's maps have collected so far; the next map's linear part is scaled by 1 - c before it is
-// rounded, and c becomes what its own rounding adds, so the sum stays within one rounding.
+// rounded, and c becomes what its own rounding adds, so the sum stays within one rounding.  Only where
+// the map's largest entry is well inside FP32's normal range: below it the relative rounding is as
+// large as 1 (a run of channels that takes a qubit's polarisation to nothing, say), above it infinite,
+// and neither says anything about the scale of the maps that follow.
 void round_map(M4 &a, double &c)
 {
     if (a.id) return;
-    double num = 0, den = 0;
+    double big = 0, num = 0, den = 0;
+    for (int i = 1; i < 4; i++)
+        for (int j = 1; j < 4; j++) big = std::max(big, std::fabs(a.m[4 * i + j]));
+    if (!(big >= 1e-30 && big <= 1e30)) return;
     for (int i = 1; i < 4; i++)
         for (int j = 1; j < 4; j++) {
             double &x = a.m[4 * i + j];
@@ -246,7 +252,7 @@ void round_map(M4 &a, double &c)
             den += x * x;
             x = f;
         }
-    if (den > 0) c += num / den - 1.0;
+    c += num / den - 1.0;
 }
 
 class NodeBuilder {

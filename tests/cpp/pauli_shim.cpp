@@ -207,3 +207,32 @@ extern "C" int pairs_replay(int n, int nops, const int *kind, const int *k, cons
     }
     return (int)progs.size();
 }
+
+// The start factors and passes of plan_pauli_list (a caller's list, from |0..0>) against plan_pauli's on
+// the same operations: 0 if alike.
+extern "C" int list_plan_differs(int n, int nops, const int *kind, const int *k, const int *qubits, const double *mats,
+                                 const long long *mat_off, const double *raw, const int *nkraus, const long long *raw_off)
+{
+    const std::vector<QOp> ops = op_list(nops, kind, k, qubits, mats, mat_off);
+    std::vector<qcw_op> list(nops);
+    for (int i = 0; i < nops; i++) {
+        list[i].kind = kind[i] == 0 ? QCW_OP_GATE : QCW_OP_KRAUS;
+        list[i].k = k[i];
+        for (int j = 0; j < k[i]; j++) list[i].qubits[j] = qubits[2 * i + j];
+        list[i].nkraus = nkraus[i];
+        list[i].offset = 2 * raw_off[i];
+    }
+    const PauliPlan a = plan_pauli(ops, 0, ops.size(), n, 0, false, true);
+    const PauliPlan b = plan_pauli_list(list.data(), nops, raw, n, 0);
+    if (a.passes.size() != b.passes.size() || a.w.size() != b.w.size()) return 1;
+    auto differ = [](float x, float y) { return !(x - y <= 1e-6f && y - x <= 1e-6f); };
+    for (size_t i = 0; i < a.w.size(); i++)
+        if (differ(a.w[i], b.w[i])) return 2;
+    for (size_t p = 0; p < a.passes.size(); p++) {
+        const PPass &x = a.passes[p], &y = b.passes[p];
+        if (x.ops.size() != y.ops.size() || x.coefs.size() != y.coefs.size()) return 3;
+        for (size_t i = 0; i < x.coefs.size(); i++)
+            if (differ(x.coefs[i], y.coefs[i])) return 4;
+    }
+    return 0;
+}

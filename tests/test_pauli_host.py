@@ -157,3 +157,45 @@ def test_plain_list_passes(shim, n, what):
     passes = shim.pairs_replay(n, len(ops), p(kind), p(k), p(qs), p(mats), p(off), p(v))
     assert 0 < passes < len(ops)
     assert np.linalg.norm(v - coefficients(want)) <= len(ops) * 2.0 ** -24 * np.linalg.norm(coefficients(want))
+
+
+def _list_differs(shim, n, ops):
+    kind, k, qs, mats, off = _packed(ops)
+    raw = np.concatenate([np.ascontiguousarray(op.mats, dtype=np.complex128).ravel() for op in ops])
+    sizes = [len(op.mats) * 4 ** len(op.qubits) for op in ops]
+    raw_off = np.asarray(np.cumsum([0] + sizes[:-1]), dtype=np.int64)
+    nk = np.asarray([len(op.mats) for op in ops], dtype=np.int32)
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    return shim.list_plan_differs(n, len(ops), p(kind), p(k), p(qs), p(mats), p(off), p(raw), p(nk), p(raw_off))
+
+
+def _depolarising(q, f):
+    """The channel that scales the polarisation of qubit q by f."""
+    w = [(1 + 3 * f) / 4] + [(1 - f) / 4] * 3
+    return wl.Op("kraus", (q,), np.stack([np.sqrt(a) * p for a, p in zip(w, PAULI)]).astype(complex))
+
+
+@pytest.mark.parametrize("count", [1, 60, 140, 185, 195, 210, 300])
+def test_vanishing_maps_leave_later_ones_alone(shim, count):
+    """A long run of depolarising channels (a map whose linear part falls to and below the smallest FP32
+    numbers) on a qubit that is used again afterwards: the maps that follow keep their own scale."""
+    n, f = 3, 0.6
+    c01 = wl.Op("gate", (0, 1), wl.gate_matrix("CNOT")[None])
+    ops = [c01] + [_depolarising(0, f)] * count + [c01, wl.Op("gate", (0,), wl.gate_matrix("H")[None])]
+    want = wl.zero_state(n)
+    for op in ops:
+        oracle.apply_op(want, op)
+    want = coefficients(want)
+    tol = 16 * 2.0 ** -24  # a few roundings of coefficients at most 1
+    v = np.zeros(4 ** n)
+    _replay(shim, n, ops, v, 0, False, True)
+    assert np.abs(v - want).max() <= tol
+    v = coefficients(wl.zero_state(n))
+    _replay(shim, n, ops, v, 0, False)
+    assert np.abs(v - want).max() <= tol
+    v = coefficients(wl.zero_state(n))
+    kind, k, qs, mats, off = _packed(ops)
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    assert shim.pairs_replay(n, len(ops), p(kind), p(k), p(qs), p(mats), p(off), p(v)) > 0
+    assert np.abs(v - want).max() <= tol
+    assert _list_differs(shim, n, ops) == 0
