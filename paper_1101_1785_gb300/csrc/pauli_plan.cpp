@@ -60,7 +60,7 @@ bool m4_tp(const M4 &a)  // first row (1, 0, 0, 0): keeps the trace
 
 // Real map of a one-qubit superoperator S (S[2 r' + c'][2 r + c]) on the labels:
 // T_ij = Tr[P_i S(P_j)] / 2, with P = I, Z, X, Y read off rows and columns of S directly.
-// Entries below 1e-14 are rounding residue of exact zeros.
+// Entries below 1e-14 of the largest are rounding residue of exact zeros.
 M4 super_map(const c128 *S)
 {
     double cr[4][4], ci[4][4];  // S applied to P_j, element e (for Y: to Y / -i)
@@ -80,8 +80,10 @@ M4 super_map(const c128 *S)
         t.m[8 + j] = 0.5 * (cr[1][j] + cr[2][j]);
         t.m[12 + j] = 0.5 * (ci[2][j] - ci[1][j]);  // Re of i (s01 - s10)
     }
+    double big = 0;
+    for (double x : t.m) big = std::max(big, std::fabs(x));
     for (double &x : t.m)
-        if (std::fabs(x) < 1e-14) x = 0.0;
+        if (std::fabs(x) < 1e-14 * big) x = 0.0;
     return t;
 }
 

@@ -199,3 +199,29 @@ def test_vanishing_maps_leave_later_ones_alone(shim, count):
     assert shim.pairs_replay(n, len(ops), p(kind), p(k), p(qs), p(mats), p(off), p(v)) > 0
     assert np.abs(v - want).max() <= tol
     assert _list_differs(shim, n, ops) == 0
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-4, 1e-8, 1e-12, 1e6])
+def test_small_operators_are_kept(shim, scale):
+    """One-qubit operators far from unit norm (an unnormalised branch of a channel): what counts as the
+    residue of an exact zero is measured against the map's own largest entry."""
+    rng = np.random.default_rng(3)
+    n = 3
+    ops = [wl.Op("gate", (0,), scale * haar_unitary(rng, 2)[None]), wl.Op("gate", (0, 2), wl.gate_matrix("CNOT")[None]),
+           wl.Op("kraus", (2,), scale * np.stack([np.sqrt(w) * haar_unitary(rng, 2) for w in (0.7, 0.2)])),
+           wl.Op("gate", (0, 1), wl.gate_matrix("CZ")[None]), wl.Op("gate", (1,), haar_unitary(rng, 2)[None])]
+    want = random_rho(rng, n)
+    v0 = coefficients(want)
+    for op in ops:
+        oracle.apply_op(want, op)
+    want = coefficients(want)
+    tol = 16 * 2.0 ** -24 * np.abs(want).max()
+    v = v0.copy()
+    _replay(shim, n, ops, v, 0, False)
+    assert np.abs(v - want).max() <= tol
+    v = v0.copy()
+    kind, k, qs, mats, off = _packed(ops)
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    assert shim.pairs_replay(n, len(ops), p(kind), p(k), p(qs), p(mats), p(off), p(v)) > 0
+    assert np.abs(v - want).max() <= tol
+    assert _list_differs(shim, n, ops) == 0
