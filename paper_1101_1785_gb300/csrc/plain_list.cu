@@ -4,8 +4,8 @@
 // into one map per qubit, and what stays on two qubits runs in one pass.  12 qubits, 30 gates with
 // depolarising noise: 8 passes of 39 us (269 MB each: 6.8 TB/s, as k_super1 and k_mono2) where there
 // were 69; 2.95 -> 0.61 ms with the readouts.  4 qubits, 40 gates with amplitude and phase damping:
-// one launch of 9 us where there were about 120; 485 -> 126 us.  The errors against 64 bits shrink
-// with the number of roundings (1.4e-6 -> 2.5e-7 and 9.7e-7 -> 8.4e-8 relative).
+// one launch of 9 us where there were about 120; 485 -> 120 us.  The errors against 64 bits shrink
+// with the number of roundings (1.4e-6 -> 2.6e-7 and 9.7e-7 -> 1.3e-7 relative).
 // Lists of one operation, controlled, wider and exactly permuting operations (SWAP, iSWAP) run as they
 // do one by one.
 #include <algorithm>
@@ -18,53 +18,64 @@
 namespace qcw {
 
 // ------------------------------------------------------------------ a run on two qubits
-// 16-member groups as in k_super2 (row and column bits of both qubits), in the Pauli basis of the two
-// qubits between the two sets of butterflies: rho is the complex combination of real coefficient
-// vectors, so every operation is a real map on packed (re, im) pairs, CNOT and CZ rename members.
-// Member of labels (p_a, p_b): x bit of a 8, of b 4; z bit of a 2, of b 1.
-__host__ __device__ constexpr int lx(int pa, int pb) { return 8 * (pa >> 1) + 2 * (pa & 1) + 4 * (pb >> 1) + (pb & 1); }
-
-template <int SR, int SC>
-__device__ __forceinline__ void to_labels(pu64 (&x)[16], int o)
+// 16-member groups as in k_super2: member e = 8 r_a + 4 r_b + 2 c_a + c_b, row and column bits of both
+// qubits.  rho is a complex combination of Hermitian matrices, so every map is real on the Pauli
+// coefficients of its qubit's quartets: as in k_super1 a quartet goes to them, through the map and back.
+// The other qubit's members stay as they are and CNOT and CZ rename them (CZ with signs), so what they
+// hold keeps its own relative precision: a population of 1e-9 beside one of 1 survives operations on
+// other qubits and its own as a control.  (Members kept as coefficients of both qubits across the run
+// need fewer operations, but lose whatever lies below 2^-24 of the group; the 12-qubit circuit takes
+// 698 us with its readouts that way and 702 us this way.)
+__device__ __forceinline__ pu64 padd2(pu64 a, pu64 b)
 {
-    const float2 a = unpack2(x[o]), b = unpack2(x[o + SC]), c = unpack2(x[o + SR]), d = unpack2(x[o + SR + SC]);
-    x[o] = pack2(a.x + d.x, a.y + d.y);            // I
-    x[o + SC] = pack2(a.x - d.x, a.y - d.y);       // Z
-    x[o + SR] = pack2(b.x + c.x, b.y + c.y);       // X
-    x[o + SR + SC] = pack2(c.y - b.y, b.x - c.x);  // Y: i (b - c)
+    pu64 d;
+    asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(d) : "l"(a), "l"(b));
+    return d;
 }
 
-template <int SR, int SC>
-__device__ __forceinline__ void from_labels(pu64 (&x)[16], int o)  // twice the inverse
-{
-    const float2 i = unpack2(x[o]), z = unpack2(x[o + SC]), u = unpack2(x[o + SR]), y = unpack2(x[o + SR + SC]);
-    x[o] = pack2(i.x + z.x, i.y + z.y);
-    x[o + SC] = pack2(u.x + y.y, u.y - y.x);
-    x[o + SR] = pack2(u.x - y.y, u.y + y.x);
-    x[o + SR + SC] = pack2(i.x - z.x, i.y - z.y);
-}
-
+// Map of a (B = false) or b, coefficients halved (from twice the inverse of the change of basis); TP:
+// rows 1..3.  The fence keeps the coefficients from being loaded before the quartets are changed (spills).
 template <bool B, bool TP, int V, class P>
 __device__ __forceinline__ void pair_map(pu64 (&x)[V][16], const P &p, unsigned k)
 {
-    constexpr int N = TP ? 12 : 16;
+    constexpr int N = TP ? 12 : 16, SR = B ? 4 : 8, SC = B ? 1 : 2, O1 = B ? 2 : 1, O2 = B ? 8 : 4;
+#pragma unroll
+    for (int v = 0; v < V; v++)
+#pragma unroll
+        for (int l = 0; l < 4; l++) {  // elements 00, 11, 01, 10 -> I, Z, X, Y = i (e01 - e10)
+            const int o = (l & 1) * O1 + (l >> 1) * O2;
+            const pu64 a = x[v][o], d = x[v][o + SR + SC], s = x[v][o + SC], t = x[v][o + SR];
+            const float2 b = unpack2(s), c = unpack2(t);
+            x[v][o] = padd2(a, d);
+            x[v][o + SR + SC] = padd2(a, fneg2(d));
+            x[v][o + SC] = padd2(s, t);
+            x[v][o + SR] = pack2(c.y - b.y, b.x - c.x);
+        }
+    __syncwarp(__activemask());
     pu64 c[N];
     p_coefs(p, k, c);
 #pragma unroll
     for (int v = 0; v < V; v++)
 #pragma unroll
         for (int l = 0; l < 4; l++) {
-            pu64 in[4];
-#pragma unroll
-            for (int r = 0; r < 4; r++) in[r] = x[v][B ? lx(l, r) : lx(r, l)];
+            const int o = (l & 1) * O1 + (l >> 1) * O2;
+            const pu64 in[4] = {x[v][o], x[v][o + SR + SC], x[v][o + SC], x[v][o + SR]};
+            pu64 out[4];
+            if (TP) out[0] = fmul2(pack2(0.5f, 0.5f), in[0]);
 #pragma unroll
             for (int r = TP ? 1 : 0; r < 4; r++) {
                 const pu64 *w = c + 4 * (TP ? r - 1 : r);
-                x[v][B ? lx(l, r) : lx(r, l)] = ffma2(w[3], in[3], ffma2(w[2], in[2], ffma2(w[1], in[1], fmul2(w[0], in[0]))));
+                out[r] = ffma2(w[3], in[3], ffma2(w[2], in[2], ffma2(w[1], in[1], fmul2(w[0], in[0]))));
             }
+            const float2 u = unpack2(out[2]), y = unpack2(out[3]);
+            x[v][o] = padd2(out[0], out[1]);
+            x[v][o + SR + SC] = padd2(out[0], fneg2(out[1]));
+            x[v][o + SC] = pack2(u.x + y.y, u.y - y.x);
+            x[v][o + SR] = pack2(u.x - y.y, u.y + y.x);
         }
 }
 
+// CNOT (SWAP = false: a controls) or CZ.
 template <bool CZ, bool SWAP, int V>
 __device__ __forceinline__ void pair_perm(pu64 (&x)[V][16])
 {
@@ -73,9 +84,9 @@ __device__ __forceinline__ void pair_perm(pu64 (&x)[V][16])
         pu64 y[16];
 #pragma unroll
         for (int e = 0; e < 16; e++) {
-            const int s = p_src<CZ>(e);
-            const pu64 a = x[v][SWAP ? lx(s & 3, s >> 2) : lx(s >> 2, s & 3)];
-            y[SWAP ? lx(e & 3, e >> 2) : lx(e >> 2, e & 3)] = p_neg<CZ>(e) ? fneg2(a) : a;
+            const int ra = e >> 3, rb = (e >> 2) & 1, ca = (e >> 1) & 1, cb = e & 1;
+            if (CZ) y[e] = (ra & rb) != (ca & cb) ? fneg2(x[v][e]) : x[v][e];
+            else y[e] = x[v][SWAP ? e ^ (8 * rb + 2 * cb) : e ^ (4 * ra + ca)];
         }
 #pragma unroll
         for (int e = 0; e < 16; e++) x[v][e] = y[e];
@@ -86,11 +97,6 @@ __device__ __forceinline__ void pair_perm(pu64 (&x)[V][16])
 template <int V, class P>
 __device__ __forceinline__ void pair_run(pu64 (&x)[V][16], const P &p, unsigned op0, unsigned nop)
 {
-#pragma unroll
-    for (int v = 0; v < V; v++) {
-        to_labels<8, 2>(x[v], 0), to_labels<8, 2>(x[v], 1), to_labels<8, 2>(x[v], 4), to_labels<8, 2>(x[v], 5);
-        to_labels<4, 1>(x[v], 0), to_labels<4, 1>(x[v], 2), to_labels<4, 1>(x[v], 8), to_labels<4, 1>(x[v], 10);
-    }
 #pragma unroll 1
     for (unsigned o = op0; o < op0 + nop; o++) {
         const unsigned w = p.op(o), k = w >> 8;
@@ -103,14 +109,6 @@ __device__ __forceinline__ void pair_run(pu64 (&x)[V][16], const P &p, unsigned 
         case PK_CX + 1: pair_perm<false, true>(x); break;
         case PK_CZ: pair_perm<true, false>(x); break;
         }
-    }
-#pragma unroll
-    for (int v = 0; v < V; v++) {
-        from_labels<4, 1>(x[v], 0), from_labels<4, 1>(x[v], 2), from_labels<4, 1>(x[v], 8), from_labels<4, 1>(x[v], 10);
-        from_labels<8, 2>(x[v], 0), from_labels<8, 2>(x[v], 1), from_labels<8, 2>(x[v], 4), from_labels<8, 2>(x[v], 5);
-        const pu64 q = pack2(0.25f, 0.25f);
-#pragma unroll
-        for (int e = 0; e < 16; e++) x[v][e] = fmul2(x[v][e], q);
     }
 }
 
@@ -136,8 +134,8 @@ __device__ __forceinline__ uint64_t pair_base(uint64_t t, const PairHead &h)
 constexpr int kPairWords = 4 + kPairMaxOps + 2 * 16 * kPairMaxOps;
 constexpr int kPairThreads = 128;
 
-// One read and one write of rho per run.  Bound by HBM: a run of four maps and a CNOT adds about 36
-// issue slots per element, 16 us at 12 qubits where the traffic takes 39.  Two neighbouring groups per
+// One read and one write of rho per run.  Bound by HBM: a run of four maps and a CNOT adds about 50
+// issue slots per element, 22 us at 12 qubits where the traffic takes 39.  Two neighbouring groups per
 // thread (float4) unless column bit 0 is struck; four blocks of 128 threads per SM keep 16 loads in
 // flight each, and the 64 values of two groups with a map's coefficients fit 128 registers.
 template <int V>
@@ -248,9 +246,9 @@ void encode(const PairProg *progs, int cnt, int n, PairParams<W> &prm)
         for (uint8_t kind : p.kind) {
             ops[o++] = kind | (unsigned)k << 8;
             const int m = kind < PK_GEN ? 12 : kind < PK_CX ? 16 : 0;
-            for (int j = 0; j < m; j++, k++) {
-                memcpy(coef + 2 * k, &p.coefs[c], 4), memcpy(coef + 2 * k + 1, &p.coefs[c], 4);
-                c++;
+            for (int j = 0; j < m; j++, k++, c++) {
+                const float half = 0.5f * p.coefs[c];
+                memcpy(coef + 2 * k, &half, 4), memcpy(coef + 2 * k + 1, &half, 4);
             }
         }
     }

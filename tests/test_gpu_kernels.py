@@ -409,3 +409,30 @@ def test_monomial_two_qubit_gates_are_exact_permutations(q):
     oracle.apply_unitary(want, wl.gate_matrix("CNOT"), [1, 3], [4])
     assert np.abs(d.get_state() - want).max() <= 1e-5
     d.close()
+
+
+@pytest.mark.parametrize("n", [3, 4, 6, 7, 10])
+@pytest.mark.parametrize("p", [1e-6, 1e-9])
+def test_lists_keep_small_populations(q, n, p):
+    """A list leaves a population far below the others at its own relative precision while its qubit is
+    only a control or idle, as the operations one by one do."""
+    rng = np.random.default_rng(n)
+    psi = np.zeros(2 ** n, complex)
+    psi[0], psi[2 ** (n - 1)] = np.sqrt(1 - p), np.sqrt(p)
+    start = np.outer(psi, psi)
+    op = lambda m, *qs: wl.Op("gate", qs, np.asarray(m, complex)[None])
+    cx, cz = wl.gate_matrix("CNOT"), wl.gate_matrix("CZ")
+    ops = [op(cx, 0, 1), op(haar_unitary(rng, 2), 1), op(cz, 1, 0), op(haar_unitary(rng, 2), 1), op(cx, 0, n - 1),
+           op(haar_unitary(rng, 2), n - 1), op(cx, 1, 2), op(cz, 0, 2)]
+    want = start.copy()
+    for o in ops:
+        oracle.apply_op(want, o)
+    d = q.Density(n)
+    d.set_state(start)
+    d.apply_packed(q.PackedOps(ops))
+    # sums of elements that went through at most 3 maps (about 5 roundings each) and the trace's own sum
+    tol = 20 * 2.0 ** -24
+    assert abs(d.probabilities()[0] - p) <= tol * p
+    got = d.partial_trace([0])
+    assert abs(got[1, 1] - p) <= tol * p
+    assert np.abs(d.get_state() - want).max() <= tol
