@@ -197,11 +197,10 @@ static uint64_t fnv(uint64_t h, const void *p, size_t n)
     return h;
 }
 
-static uint64_t hash_ops(const std::vector<QOp> &ops, size_t b, size_t e, int n, int k, int tb)
+// Hash of a segment's operations, and with what a plan was made for.
+static uint64_t hash_ops(const std::vector<QOp> &ops, size_t b, size_t e)
 {
     uint64_t h = 1469598103934665603ull;
-    int hdr[3] = {n, k, tb};
-    h = fnv(h, hdr, sizeof(hdr));
     for (size_t i = b; i < e; i++) {
         const QOp &o = ops[i];
         int meta[3] = {o.kind, o.k, o.ncontrols};
@@ -210,6 +209,12 @@ static uint64_t hash_ops(const std::vector<QOp> &ops, size_t b, size_t e, int n,
         h = fnv(h, o.m.data(), sizeof(c128) * o.m.size());
     }
     return h;
+}
+
+static uint64_t hash_with(uint64_t h, int n, int k, int tb)
+{
+    const int hdr[3] = {n, k, tb};
+    return fnv(h, hdr, sizeof(hdr));
 }
 
 static bool same_ops(const std::vector<QOp> &a, const std::vector<QOp> &ops, size_t b, size_t e)
@@ -875,12 +880,33 @@ constexpr int kBeamMinQubits = 10;
 // take 2.8 ms against 3.4 ms, a single one 2.3 ms against 1.9 ms.
 static bool pauli_pays(const CachedPauli &p) { return p.passes.size() > 1; }
 
-// The segment in the Pauli basis; *done = false: it is better run on rho.
-static qcw_status run_pauli_segment(qcw_ctx *c, size_t b, size_t e, bool last, bool *done)
+// What the operations alone say about that, before any is hashed or planned for it.  More qubits than a
+// tile has digits take several passes.  Fewer, with so few two-qubit operations that their maps fit
+// one pass's program even if all are dense, take one; so does nearly every circuit on a register that
+// is one tile (up to seven qubits).  Those stay on rho: hashed and planned for both storages, 200 gates
+// took 439 us where the kernels on rho take 278 us (3 qubits; 756 / 602 us at 7), a single gate on 9
+// qubits 87 / 78 us on its first visit; 8 to 11 qubits with 50 gates and more are 1.5 to 5
+// times faster on the coefficients.
+static bool pauli_may_pay(const qcw_ctx *c, size_t b, size_t e)
+{
+    if (c->n <= kPTile) return false;
+    unsigned used = c->fuse_k ? 0u : 3u << (c->n - 2);  // the two lowest digits are in every tile
+    int two = 0;
+    for (size_t i = b; i < e; i++) {
+        const QOp &op = c->queue[i];
+        for (int j = 0; j < op.k; j++) used |= 1u << op.qubits[j];
+        two += op.k == 2;
+    }
+    const int tile = c->fuse_k ? std::min(c->fuse_k, kPTile) : kPTile;
+    return __builtin_popcount(used) > tile || two >= kPMaxCoef / 256;
+}
+
+// The segment (its operations' hash: ops_hash) in the Pauli basis; *done = false: it is better run on rho.
+static qcw_status run_pauli_segment(qcw_ctx *c, size_t b, size_t e, uint64_t ops_hash, bool last, bool *done)
 {
     FusedRuntime *rt = c->fused;
     *done = false;
-    const uint64_t h = hash_ops(c->queue, b, e, c->n, c->fuse_k, 0);
+    const uint64_t h = hash_with(ops_hash, c->n, c->fuse_k, 0);
     CachedPauli *hit = nullptr;
     for (CachedPauli &p : rt->pcache)
         if (p.hash == h && p.k == c->fuse_k && p.zero == c->pzero && same_ops(p.ops, c->queue, b, e)) {
@@ -950,9 +976,10 @@ static qcw_status run_segment(qcw_ctx *c, size_t b, size_t e, bool last)
 {
     FusedRuntime *rt = c->fused;
     const int n = c->n;
-    if (pauli_allowed(c)) {
+    const uint64_t ops_hash = hash_ops(c->queue, b, e);
+    if ((c->in_pauli || pauli_may_pay(c, b, e)) && pauli_allowed(c)) {
         bool done = false;
-        qcw_status ps = run_pauli_segment(c, b, e, last, &done);
+        qcw_status ps = run_pauli_segment(c, b, e, ops_hash, last, &done);
         if (ps || done) return ps;
     }
     if (c->in_pauli) {
@@ -970,7 +997,7 @@ static qcw_status run_segment(qcw_ctx *c, size_t b, size_t e, bool last)
         k = tn.chosen;
     } else if (n >= 12 && herm0 && e - b >= kTuneMinOps && !tune_poll(tn) && !tn.chosen) {
         // a known segment runs at the width it has not been timed at; a new one alternates
-        const uint64_t key = hash_ops(c->queue, b, e, n, 0, 0);
+        const uint64_t key = hash_with(ops_hash, n, 0, 0);
         int cand = tn.trials & 1;
         bool found = false;
         for (const KTuneSeg &sg : tn.segs)
@@ -994,7 +1021,7 @@ static qcw_status run_segment(qcw_ctx *c, size_t b, size_t e, bool last)
     if (k > n) k = n;
     const bool herm = herm0;
     const int tbmax = herm ? 12 : 13;
-    uint64_t h = hash_ops(c->queue, b, e, n, k, tbmax) ^ (0x9e3779b97f4a7c15ull * (uint64_t)(c->fused_kernel + 1));
+    uint64_t h = hash_with(ops_hash, n, k, tbmax) ^ (0x9e3779b97f4a7c15ull * (uint64_t)(c->fused_kernel + 1));
     CachedPlan *hit = nullptr;
     for (CachedPlan &cp : rt->cache)
         if (cp.hash == h && cp.n == n && cp.k == k && cp.tb == tbmax && same_ops(cp.ops, c->queue, b, e)) {

@@ -597,10 +597,9 @@ __global__ void __launch_bounds__(kCvThreads) k_pauli_emit(const float *__restri
 }
 
 // The lower triangle of rho (r >= c; the diagonal's real part) -> W, transformed over the low qubits.
-template <int M>
-__global__ void __launch_bounds__(kCvThreads) k_pauli_absorb(const float2 *__restrict__ rho, float *__restrict__ v, int n,
-                                                             int sign)
+__global__ void __launch_bounds__(kCvThreads) k_pauli_absorb(const float2 *__restrict__ rho, float *__restrict__ v, int n)
 {
+    constexpr int M = kCvLow;
     using C = CvTile<M>;
     constexpr int ML = C::ML;
     __shared__ float sm[2 * C::kArray];
@@ -644,10 +643,8 @@ __global__ void __launch_bounds__(kCvThreads) k_pauli_absorb(const float2 *__res
         for (int u = 0; u < C::U; u++)
             if (a < T.narr && T.has(u)) {
                 const float *p = sm + a * C::kArray + T.pos0 + C::cpos(u);
-                float4 y = make_float4(p[0], p[kCvPitch], p[1], p[kCvPitch + 1]);
-                const uint64_t o = T.off[a] + T.loff0 + C::coff(u);
-                if (sign) p_signs4(y, o);
-                *reinterpret_cast<float4 *>(v + o) = y;
+                *reinterpret_cast<float4 *>(v + T.off[a] + T.loff0 + C::coff(u)) =
+                    make_float4(p[0], p[kCvPitch], p[1], p[kCvPitch + 1]);
             }
 }
 
@@ -674,11 +671,6 @@ static void emit_m(const float *v, float2 *rho, int n, float scale, int sign, cu
 {
     k_pauli_emit<M><<<cv_blocks(n), kCvThreads, 0, s>>>(v, rho, n, scale, sign);
 }
-template <int M>
-static void absorb_m(const float2 *rho, float *v, int n, int sign, cudaStream_t s)
-{
-    k_pauli_absorb<M><<<cv_blocks(n), kCvThreads, 0, s>>>(rho, v, n, sign);
-}
 
 int pauli_convert_launches(int n) { return n > kCvLow ? 2 : 1; }
 
@@ -702,20 +694,12 @@ cudaError_t launch_pauli_to_rho(float *v, float2 *rho, int n, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// v <- rho, from its lower triangle.
+// v <- rho, from its lower triangle.  n > kCvLow (a state of fewer qubits held as rho stays there).
 cudaError_t launch_rho_to_pauli(const float2 *rho, float *v, int n, cudaStream_t s)
 {
-    const int sign = n > kCvLow ? 0 : 1;
-    switch (n) {
-    case 3: absorb_m<3>(rho, v, n, sign, s); break;
-    case 4: absorb_m<4>(rho, v, n, sign, s); break;
-    case 5: absorb_m<5>(rho, v, n, sign, s); break;
-    case 6: absorb_m<6>(rho, v, n, sign, s); break;
-    default: absorb_m<kCvLow>(rho, v, n, sign, s); break;
-    }
+    k_pauli_absorb<<<cv_blocks(n), kCvThreads, 0, s>>>(rho, v, n);
     const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || n <= kCvLow) return e;
-    return launch_high(v, n, 0, 1, s);
+    return e != cudaSuccess ? e : launch_high(v, n, 0, 1, s);
 }
 
 // ------------------------------------------------------------------ readouts

@@ -189,3 +189,48 @@ def test_wait_that_runs_out_is_reported(q):
     _apply(d, c.ops)
     assert np.abs(d.get_state() - oracle.run_circuit(c)).max() <= ATOL
     d.close()
+
+
+@pytest.mark.parametrize("n", [3, 4, 7])
+@pytest.mark.parametrize("gates", [3, 300])
+def test_small_registers_stay_on_rho(q, n, gates):
+    """A state of up to seven qubits given as a matrix is evolved as one, however long the circuit: a
+    population far below the others keeps its relative precision where nothing acts on its qubit."""
+    rng = np.random.default_rng(n)
+    p = 1e-9
+    psi = np.zeros(2 ** n, complex)
+    psi[0], psi[2 ** (n - 1)] = np.sqrt(1 - p), np.sqrt(p)
+    d = q.Density(n)
+    d.set_mode(q.QCW_MODE_FUSED)
+    d.set_state(np.outer(psi, psi))
+    for i in range(gates):
+        d.apply_gate(haar_unitary(rng, 2), (1 + i % (n - 1),))
+        if n > 2:
+            a, b = (int(x) for x in 1 + rng.permutation(n - 1)[:2])
+            d.apply_gate2(wl.gate_matrix("CNOT"), a, b)
+    # FP32: every operation rounds an element a few times, in either direction
+    assert abs(d.probabilities()[0] - p) <= 2 * gates * 8 * 2.0 ** -24 * p
+    assert d.measure(0, 1)[0] == 1
+
+
+@pytest.mark.parametrize("n,touched,gates", [(8, 7, 11), (8, 8, 40), (9, 2, 1), (9, 2, 60), (10, 7, 70), (11, 11, 20), (9, 4, 5)])
+@pytest.mark.parametrize("k", [0, 3])
+def test_storage_of_a_given_matrix(q, n, touched, gates, k):
+    """Either side of the rule that says when a matrix is changed to Pauli storage."""
+    rng = np.random.default_rng(n + touched)
+    want = random_rho(rng, n, 3)
+    d = q.Density(n)
+    d.set_mode(q.QCW_MODE_FUSED, k)
+    d.set_state(want)
+    where = rng.permutation(n)[:touched]
+    ops = []
+    for i in range(gates):
+        a, b = (int(x) for x in rng.permutation(where)[:2])
+        ops.append(wl.Op("gate", (a, b), (haar_unitary(rng, 4) if i % 3 == 0 else wl.gate_matrix("CNOT"))[None]))
+        ops.append(wl.Op("kraus", (a,), np.stack([np.sqrt(0.7) * haar_unitary(rng, 2), np.sqrt(0.3) * haar_unitary(rng, 2)])))
+    for _ in range(2):
+        _apply(d, ops)
+        for op in ops:
+            oracle.apply_op(want, op)
+        np.testing.assert_allclose(d.probabilities(), oracle.probabilities(want), atol=READ_TOL, rtol=0)
+        assert np.abs(d.get_state() - want).max() <= ATOL
