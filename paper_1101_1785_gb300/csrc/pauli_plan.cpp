@@ -60,7 +60,8 @@ bool m4_tp(const M4 &a)  // first row (1, 0, 0, 0): keeps the trace
 
 // Real map of a one-qubit superoperator S (S[2 r' + c'][2 r + c]) on the labels:
 // T_ij = Tr[P_i S(P_j)] / 2, with P = I, Z, X, Y read off rows and columns of S directly.
-// Entries below 1e-14 of the largest are rounding residue of exact zeros.
+// Entries below 1e-14 of the largest are rounding residue of exact zeros; the largest is T_00, half the
+// trace of what S makes of the identity (|Tr[P S(P')]| <= Tr[S(1)] for S = sum_j K_j . K_j^dagger).
 M4 super_map(const c128 *S)
 {
     double cr[4][4], ci[4][4];  // S applied to P_j, element e (for Y: to Y / -i)
@@ -80,10 +81,9 @@ M4 super_map(const c128 *S)
         t.m[8 + j] = 0.5 * (cr[1][j] + cr[2][j]);
         t.m[12 + j] = 0.5 * (ci[2][j] - ci[1][j]);  // Re of i (s01 - s10)
     }
-    double big = 0;
-    for (double x : t.m) big = std::max(big, std::fabs(x));
+    const double tiny = 1e-14 * t.m[0];
     for (double &x : t.m)
-        if (std::fabs(x) < 1e-14 * big) x = 0.0;
+        if (std::fabs(x) < tiny) x = 0.0;
     return t;
 }
 
@@ -242,18 +242,15 @@ int classify(const OpView &op, int *a, int *b)
 void round_map(M4 &a, double &c)
 {
     if (a.id) return;
-    double big = 0, num = 0, den = 0;
-    for (int i = 1; i < 4; i++)
-        for (int j = 1; j < 4; j++) big = std::max(big, std::fabs(a.m[4 * i + j]));
-    if (!(big >= 1e-30 && big <= 1e30)) return;
-    for (int i = 1; i < 4; i++)
-        for (int j = 1; j < 4; j++) {
-            double &x = a.m[4 * i + j];
-            const double f = (double)(float)(x * (1.0 - c));
-            num += f * x;
-            den += x * x;
-            x = f;
-        }
+    double f[9], num = 0, den = 0;
+    for (int i = 0; i < 9; i++) {
+        const double x = a.m[4 * (i / 3 + 1) + i % 3 + 1];
+        f[i] = (double)(float)(x * (1.0 - c));
+        num += f[i] * x;
+        den += x * x;
+    }
+    if (!(den >= 1e-60 && den <= 1e60)) return;
+    for (int i = 0; i < 9; i++) a.m[4 * (i / 3 + 1) + i % 3 + 1] = f[i];
     c += num / den - 1.0;
 }
 
