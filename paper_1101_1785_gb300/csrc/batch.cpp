@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cstring>
+#include <mutex>
 #include <numeric>
 #include <thread>
 
@@ -27,9 +28,10 @@ struct qcw_batch {
     char *ddesc = nullptr;
     float *arena = nullptr;
     size_t arena_elems = 0;
-    void *conv = nullptr;  // scratch of qcw_batch_get_state, kept while it is small
-    float2 *hconv = nullptr;
-    size_t conv_bytes = 0;
+    // scratch of qcw_batch_get_state for the largest circuit: behind the states in the arena, behind hred
+    float2 *stage = nullptr, *host = nullptr;
+    float *copy = nullptr;
+    std::mutex read_mu;
     bool dense = false;
     unsigned *counters = nullptr;
     size_t ncounters = 0;
@@ -65,8 +67,6 @@ static void batch_free(qcw_batch *b)
     if (b->done) cudaEventDestroy(b->done);
     cudaFree(b->ddesc);
     cudaFree(b->arena);
-    cudaFree(b->conv);
-    if (b->hconv) cudaFreeHost(b->hconv);
     cudaFree(b->counters);
     cudaFree(b->ditems);
     cudaFree(b->dint);
@@ -177,16 +177,22 @@ extern "C" qcw_status qcw_batch_create(int ncirc, const int *nqubits, const long
         std::vector<char>().swap(p.desc);
     }
     b->arena_elems = aelems;
-    if (cudaMalloc(&b->ddesc, dbytes) != cudaSuccess || cudaMalloc(&b->arena, aelems * sizeof(float)) != cudaSuccess ||
+    const int nmax = *std::max_element(nqubits, nqubits + ncirc);
+    const size_t celems = program_copies(nmax) ? program_elems(nmax) : 0;
+    if (cudaMalloc(&b->ddesc, dbytes) != cudaSuccess ||
+        cudaMalloc(&b->arena, (aelems + celems) * sizeof(float) + program_stage(nmax) * sizeof(float2)) != cudaSuccess ||
         cudaMalloc(&b->counters, sizeof(unsigned) * (b->ncounters + 1)) != cudaSuccess ||
         cudaMalloc(&b->dint, 4 * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&b->dred, sizeof(double) * b->nred) != cudaSuccess ||
-        cudaMallocHost(&b->hred, sizeof(double) * b->nred) != cudaSuccess ||
+        cudaMallocHost(&b->hred, sizeof(double) * b->nred + program_pinned(nmax) * sizeof(float2)) != cudaSuccess ||
         cudaMallocHost(&b->herr, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         batch_free(b);
         return set_error(QCW_ENOMEM, "batch buffers");
     }
+    b->copy = b->arena + aelems;
+    b->stage = reinterpret_cast<float2 *>(b->copy + celems);  // (all sizes are multiples of 256 bytes)
+    b->host = reinterpret_cast<float2 *>(b->hred + b->nred);
     // items: circuits in decreasing modeled cost, level by level
     std::vector<int> order(ncirc);
     std::iota(order.begin(), order.end(), 0);
@@ -276,34 +282,8 @@ extern "C" qcw_status qcw_batch_get_state(qcw_batch *b, int circuit, double *rho
     if (!b || !rho_c128 || circuit < 0 || circuit >= (int)b->progs.size()) return set_error(QCW_EINVAL, "bad argument");
     qcw_status st = qcw_batch_wait(b, -1);
     if (st) return st;
-    const int n = b->progs[circuit].n;
-    const size_t cnt = (size_t)1 << (2 * n), need = program_scratch(n), kKeep = (size_t)64 << 20;
-    if (need > b->conv_bytes) {
-        BCK(cudaFree(b->conv));
-        if (b->hconv) BCK(cudaFreeHost(b->hconv));
-        b->conv = nullptr;
-        b->hconv = nullptr;
-        b->conv_bytes = 0;
-        if (cudaMalloc(&b->conv, need) != cudaSuccess || cudaMallocHost(&b->hconv, program_elems(n) * sizeof(float2)) != cudaSuccess) {
-            cudaGetLastError();
-            cudaFree(b->conv);
-            b->conv = nullptr;
-            return set_error(QCW_ENOMEM, "batch state download");
-        }
-        b->conv_bytes = need;
-    }
-    BCK(program_rho(b->arena + b->rho_off[circuit], n, b->conv, b->hconv, b->stream));
-    for (size_t i = 0; i < cnt; i++) {
-        rho_c128[2 * i] = b->hconv[i].x;
-        rho_c128[2 * i + 1] = b->hconv[i].y;
-    }
-    if (b->conv_bytes > kKeep) {
-        BCK(cudaFree(b->conv));
-        BCK(cudaFreeHost(b->hconv));
-        b->conv = nullptr;
-        b->hconv = nullptr;
-        b->conv_bytes = 0;
-    }
+    std::lock_guard<std::mutex> lk(b->read_mu);  // the scratch is shared
+    BCK(program_rho(b->arena + b->rho_off[circuit], b->progs[circuit].n, b->copy, b->stage, b->host, rho_c128, b->stream));
     return QCW_OK;
 }
 

@@ -371,20 +371,57 @@ void program_items(const Program &p, float *v, const char *desc, unsigned *count
     }
 }
 
-size_t program_scratch(int n) { return program_elems(n) * (sizeof(float) + sizeof(float2)); }
-
-cudaError_t program_rho(const float *v, int n, void *scratch, float2 *host, cudaStream_t s)
+// Rows of a piece: 2^17 elements (1 MiB), at least a row block (134 MB at 17 qubits).
+constexpr size_t kPiece = (size_t)1 << 17;
+static int stage_rows(int nd)
 {
-    const size_t el = program_elems(n);
+    return std::max(pauli_row_block(nd), (int)std::min<size_t>((size_t)1 << nd, kPiece >> nd));
+}
+
+size_t program_stage(int n)
+{
     const int nd = std::max(n, kPMinDigits);
-    float2 *rho = static_cast<float2 *>(scratch);
-    float *w = reinterpret_cast<float *>(rho + el);
-    cudaError_t e = cudaMemcpyAsync(w, v, sizeof(float) * el, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = launch_pauli_to_rho(w, rho, nd, s);
-    // a padded register's own qubits are the lowest: its rho is the corner where the others are |0>
-    const size_t row = sizeof(float2) << n;
-    if (e == cudaSuccess) e = cudaMemcpy2DAsync(host, row, rho, sizeof(float2) << nd, row, (size_t)1 << n, cudaMemcpyDeviceToHost, s);
-    return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+    return (size_t)stage_rows(nd) << nd;
+}
+
+size_t program_pinned(int n) { return std::min(program_elems(n), kPiece); }
+
+bool program_copies(int n) { return n > kPTile; }
+
+// Through a pinned buffer of at most 1 MiB, which the conversion to double finds in the cache: 12
+// qubits (134 MB) 20 ms, 13 qubits 78 ms (copied whole to pageable memory 29 and 109 ms; as complex128
+// from the device to the caller's pageable memory 43 and 107 ms).
+cudaError_t program_rho(const float *v, int n, float *copy, float2 *stage, float2 *host, double *out, cudaStream_t s)
+{
+    const int nd = std::max(n, kPMinDigits), rows = stage_rows(nd);
+    cudaError_t e = cudaSuccess;
+    if (program_copies(n)) {
+        e = cudaMemcpyAsync(copy, v, sizeof(float) * program_elems(n), cudaMemcpyDeviceToDevice, s);
+        if (e == cudaSuccess) e = launch_pauli_unfold(copy, nd, s);
+        v = copy;
+    }
+    const size_t dim = (size_t)1 << n, piece = program_pinned(n);
+    for (size_t r = 0; r < dim && e == cudaSuccess; r += rows) {
+        e = launch_pauli_rows(v, stage, nd, (int)r, rows, s);
+        const size_t el = (size_t)rows << nd;
+        for (size_t f = 0; f < el && e == cudaSuccess; f += piece) {
+            const size_t cnt = std::min(piece, el - f);
+            e = cudaMemcpyAsync(host, stage + f, sizeof(float2) * cnt, cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            if (e != cudaSuccess) break;
+            if (n == nd) {
+                double *to = out + 2 * (r * dim + f);
+                for (size_t i = 0; i < cnt; i++) to[2 * i] = host[i].x, to[2 * i + 1] = host[i].y;
+                continue;
+            }
+            // a padded register's own qubits are the lowest: its rho is the corner where the others are |0>
+            for (size_t i = 0; i < dim * dim; i++) {
+                const float2 z = host[((i >> n) << nd) + (i & (dim - 1))];
+                out[2 * i] = z.x, out[2 * i + 1] = z.y;
+            }
+        }
+    }
+    return e;
 }
 
 }  // namespace qcw

@@ -96,9 +96,12 @@ size_t engine_max_smem();
 void program_items(const Program &p, float *v, const char *desc, unsigned *counters, double *red, int pass_begin,
                    int pass_end, bool init, bool readout, std::vector<std::vector<WItem>> &levels, int *nchunks);
 
-// rho of a program's state (2^n x 2^n, complex64) into scratch (program_scratch bytes, device) and from
-// there to the host; v is left as it is.
-size_t program_scratch(int n);
-cudaError_t program_rho(const float *v, int n, void *scratch, float2 *host, cudaStream_t s);
+// rho of a program's state on the host (2^n x 2^n, complex128); v is left as it is.  copy: program_elems(n)
+// floats of device scratch (if program_copies(n)); rho goes in pieces of whole rows through stage
+// (program_stage(n) elements on the device) and from there through host (program_pinned(n), pinned).
+size_t program_stage(int n);
+size_t program_pinned(int n);
+bool program_copies(int n);
+cudaError_t program_rho(const float *v, int n, float *copy, float2 *stage, float2 *host, double *out, cudaStream_t s);
 
 }  // namespace qcw

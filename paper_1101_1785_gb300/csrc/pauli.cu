@@ -489,15 +489,24 @@ struct CvTile {
     unsigned pos0;    // this thread's first chunk: position in an array (labels I, Z, X, Y: + 0, pitch, 1, pitch + 1)
     unsigned loff0;   // and element offset in v's low part; chunk + u 256 adds cpos(u), coff(u)
 
+    // Tile blk of all pairs ca <= ra.
     __device__ __forceinline__ explicit CvTile(unsigned blk)
     {
-        xh = blk & ((1u << MH) - 1u);
         const unsigned long long p = blk >> MH;
         unsigned long long c = (unsigned long long)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);
         while ((c + 1) * (c + 2) / 2 <= p) c++;
         while (c * (c + 1) / 2 > p) c--;
-        ra = (unsigned)c;
-        ca = (unsigned)(p - c * (c + 1) / 2);
+        init((unsigned)c, (unsigned)(p - c * (c + 1) / 2), blk & ((1u << MH) - 1u));
+    }
+    // Tile blk of the pairs that hold row block r.
+    __device__ __forceinline__ CvTile(unsigned blk, unsigned r)
+    {
+        const unsigned c = blk >> MH;
+        init(r > c ? r : c, r > c ? c : r, blk & ((1u << MH) - 1u));
+    }
+    __device__ __forceinline__ void init(unsigned r, unsigned c, unsigned x_high)
+    {
+        ra = r, ca = c, xh = x_high;
         narr = ra == ca ? 1 : 2;
         const uint64_t x = p_spread(ra ^ ca) << 1;
         off[0] = (x | p_spread(ra)) << (2 * M);
@@ -541,14 +550,16 @@ __device__ __forceinline__ void cv_transform(const CvTile<M> &T, float *sm)
     if constexpr (M > 4) step(std::integral_constant<int, 4>(), std::integral_constant<int, M - 4>());
 }
 
-template <int M>
-__global__ void __launch_bounds__(kCvThreads) k_pauli_emit(const float *__restrict__ v, float2 *__restrict__ rho, int n,
-                                                           float scale, int sign)
+// ROWS: only the blocks of row block r0 + blockIdx.y, from rho on; else all of rho.
+template <int M, bool ROWS>
+__global__ void __launch_bounds__(kCvThreads)
+    k_pauli_emit(const float *__restrict__ v, float2 *__restrict__ rho, int n, float scale, int sign, unsigned r0)
 {
     using C = CvTile<M>;
     constexpr int ML = C::ML;
     __shared__ float sm[2 * C::kArray];
-    const C T(blockIdx.x);
+    const unsigned row_block = r0 + blockIdx.y;
+    const C T = ROWS ? C(blockIdx.x, row_block) : C(blockIdx.x);
     const float h = 0.5f * scale;
     {
         float4 x[2][C::U];  // all loads in flight
@@ -579,8 +590,10 @@ __global__ void __launch_bounds__(kCvThreads) k_pauli_emit(const float *__restri
 #pragma unroll
     for (int blkm = 0; blkm < 2; blkm++) {
         if (blkm == T.narr) break;
+        if (ROWS && row_block != (blkm ? T.ca : T.ra)) continue;
         const float *wr = blkm ? sm + C::kArray : sm, *wc = T.narr == 2 && !blkm ? sm + C::kArray : sm;  // by row, by column
-        float2 *dst = rho + (((uint64_t)(blkm ? T.ca : T.ra) << M) + row0) * dim + ((uint64_t)(blkm ? T.ra : T.ca) << M) + c0;
+        const unsigned rb = ROWS ? blockIdx.y : blkm ? T.ca : T.ra;
+        float2 *dst = rho + (((uint64_t)rb << M) + row0) * dim + ((uint64_t)(blkm ? T.ra : T.ca) << M) + c0;
         wr += row0 * kCvPitch;
         wc += c0 * kCvPitch;
 #pragma unroll
@@ -666,32 +679,45 @@ static unsigned cv_blocks(int n)
     return (unsigned)((M * (M + 1) / 2) << mh);
 }
 
-template <int M>
-static void emit_m(const float *v, float2 *rho, int n, float scale, int sign, cudaStream_t s)
+int pauli_convert_launches(int n) { return n > kCvLow ? 2 : 1; }
+
+cudaError_t launch_pauli_unfold(float *v, int n, cudaStream_t s) { return n > kCvLow ? launch_high(v, n, 1, 0, s) : cudaSuccess; }
+
+template <int M, bool ROWS>
+static void emit_m(const float *v, float2 *rho, int n, int r0, int nr, cudaStream_t s)
 {
-    k_pauli_emit<M><<<cv_blocks(n), kCvThreads, 0, s>>>(v, rho, n, scale, sign);
+    float scale = 1.f;
+    for (int i = 0; i < n; i++) scale *= 0.5f;
+    const dim3 grid = ROWS ? dim3(1u << (n - M + CvTile<M>::MH), nr) : dim3(cv_blocks(n));
+    k_pauli_emit<M, ROWS><<<grid, kCvThreads, 0, s>>>(v, rho, n, scale, n > kCvLow ? 0 : 1, (unsigned)r0);
 }
 
-int pauli_convert_launches(int n) { return n > kCvLow ? 2 : 1; }
+template <bool ROWS>
+static cudaError_t emit(const float *v, float2 *rho, int n, int r0, int nr, cudaStream_t s)
+{
+    switch (n) {
+    case 3: emit_m<3, ROWS>(v, rho, n, r0, nr, s); break;
+    case 4: emit_m<4, ROWS>(v, rho, n, r0, nr, s); break;
+    case 5: emit_m<5, ROWS>(v, rho, n, r0, nr, s); break;
+    case 6: emit_m<6, ROWS>(v, rho, n, r0, nr, s); break;
+    default: emit_m<kCvLow, ROWS>(v, rho, n, r0, nr, s); break;
+    }
+    return cudaGetLastError();
+}
 
 // rho <- v (v is used up: the high stage works in place).  n >= 3.
 cudaError_t launch_pauli_to_rho(float *v, float2 *rho, int n, cudaStream_t s)
 {
-    if (n > kCvLow) {
-        const cudaError_t e = launch_high(v, n, 1, 0, s);
-        if (e != cudaSuccess) return e;
-    }
-    float scale = 1.f;
-    for (int i = 0; i < n; i++) scale *= 0.5f;
-    const int sign = n > kCvLow ? 0 : 1;
-    switch (n) {
-    case 3: emit_m<3>(v, rho, n, scale, sign, s); break;
-    case 4: emit_m<4>(v, rho, n, scale, sign, s); break;
-    case 5: emit_m<5>(v, rho, n, scale, sign, s); break;
-    case 6: emit_m<6>(v, rho, n, scale, sign, s); break;
-    default: emit_m<kCvLow>(v, rho, n, scale, sign, s); break;
-    }
-    return cudaGetLastError();
+    const cudaError_t e = launch_pauli_unfold(v, n, s);
+    return e != cudaSuccess ? e : emit<false>(v, rho, n, 0, 0, s);
+}
+
+int pauli_row_block(int n) { return 1 << std::min(n, kCvLow); }
+
+cudaError_t launch_pauli_rows(const float *v, float2 *rows, int n, int row, int count, cudaStream_t s)
+{
+    const int block = pauli_row_block(n);
+    return emit<true>(v, rows, n, row / block, count / block, s);
 }
 
 // v <- rho, from its lower triangle.  n > kCvLow (a state of fewer qubits held as rho stays there).

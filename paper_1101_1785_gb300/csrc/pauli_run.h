@@ -31,6 +31,11 @@ cudaError_t launch_pauli_pass(const PauliBlob &B, float *v, int nd, int nsm, boo
 cudaError_t launch_pauli_to_rho(float *v, float2 *rho, int n, cudaStream_t s);
 cudaError_t launch_rho_to_pauli(const float2 *rho, float *v, int n, cudaStream_t s);
 int pauli_convert_launches(int n);
+// The same in pieces: launch_pauli_unfold once (v is used up; up to seven qubits it is left alone), then
+// rows [row, row + count) of rho, both multiples of pauli_row_block(n).
+cudaError_t launch_pauli_unfold(float *v, int n, cudaStream_t s);
+int pauli_row_block(int n);
+cudaError_t launch_pauli_rows(const float *v, float2 *rows, int n, int row, int count, cudaStream_t s);
 cudaError_t launch_pauli_zero(float *v, int n, int nsm, cudaStream_t s);
 void launch_pauli_diag(const float *v, int n, double *out, cudaStream_t s);
 void launch_pauli_terms(const float *v, const PauliTerms &T, double *out, cudaStream_t s);

@@ -179,3 +179,60 @@ def test_server_bounded_waits(q):
     r = [x for x in res if x["n"] == 5][0]
     assert abs(r["purity"] - oracle.purity(want)) <= RTOL_READ
     srv.close()
+
+
+@pytest.mark.parametrize("sizes", [(1,), (2, 3), (5, 7, 4), (8, 6), (10, 9), (11,)])
+def test_batch_states(q, sizes):
+    """Final states at every piece size of the download (padded, one tile, several row blocks)."""
+    circuits = [wl.random_circuit(n, 30, 70 + n, "mixed", "adpd") for n in sizes]
+    b = q.Batch(circuits)
+    b.run()
+    for j, c in enumerate(circuits):
+        want = wl.zero_state(c.n)
+        for op in c.ops:
+            oracle.apply_op(want, op)
+        got = b.get_state(j)
+        assert np.abs(got - want).max() <= 1e-5
+        assert np.abs(got - got.conj().T).max() == 0.0
+        np.testing.assert_array_equal(b.get_state(j), got)
+
+
+def test_batch_state_without_free_memory(q):
+    """A state can be read when the device has no memory left to give: the batch has what that takes."""
+    import torch
+
+    b = q.Batch([wl.random_circuit(13, 4, 1, "mixed", "adpd")])
+    b.run()
+    want = b.get_state(0)
+    held, left = [], 512 << 20  # reading 13 qubits from scratch of its own would take 805 MB
+    while torch.cuda.mem_get_info()[0] > left + (64 << 20):
+        free = torch.cuda.mem_get_info()[0] - left
+        held.append(torch.empty(min(free, 8 << 30) // (2 << 20) * (2 << 20), dtype=torch.uint8, device="cuda"))
+    try:
+        np.testing.assert_array_equal(b.get_state(0), want)
+    finally:
+        held.clear()
+        torch.cuda.empty_cache()
+
+
+def test_batch_states_read_by_two_threads(q):
+    """Readers of one finished batch share its scratch: large and small states in turn, from two threads."""
+    import threading
+
+    circuits = [wl.random_circuit(n, 10, n, "mixed", "adpd") for n in (12, 9, 5, 11)]
+    b = q.Batch(circuits)
+    b.run()
+    want = [b.get_state(j) for j in range(4)]
+    bad = []
+
+    def read(order):
+        for j in order:
+            if not np.array_equal(b.get_state(j), want[j]):
+                bad.append(j)
+
+    ts = [threading.Thread(target=read, args=(o,)) for o in ((0, 1, 2, 3, 2), (3, 2, 0, 1, 1))]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not bad
