@@ -1,5 +1,6 @@
 // C ABI of the qcw library: argument checks, context lifetime, the plain (one launch per
 // operation) path and the FP64 readouts.  The fused path lives in fused.cu / planner.cpp.
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -400,21 +401,32 @@ static qcw_status upload_operators(qcw_ctx *c, const QOp &op, const float2 **dev
 }
 
 // Kraus channels on k >= 3 qubits (Eq. rhoE2) and five-qubit gates: the whole sum of K_j rho K_j^dagger in one
-// pass (wide.cu).  The scratch copies of rho that a channel of many operators needs stay allocated.
+// pass (wide.cu).  The scratch copies of rho that a channel of many operators needs stay allocated: a
+// captured graph may hold their address.  So a scratch that became too small is kept too, until the
+// context goes, and a new one is at least twice its size (all together at most twice the largest).
+static qcw_status wide_buffer(qcw_ctx *c, int copies)
+{
+    if (copies <= c->kacc_copies) return QCW_OK;
+    const size_t bytes = sizeof(float2) << (2 * c->n);
+    float2 *b = nullptr;
+    for (int want : {std::max(copies, 2 * c->kacc_copies), copies}) {
+        if (cudaMalloc(&b, (size_t)want * bytes) == cudaSuccess) {
+            if (c->d_kacc) c->kacc_old.push_back(c->d_kacc);
+            c->d_kacc = b;
+            c->kacc_copies = want;
+            return QCW_OK;
+        }
+        cudaGetLastError();
+    }
+    return set_error(QCW_ENOMEM, "Kraus scratch");
+}
+
 static qcw_status plain_wide(qcw_ctx *c, const QOp &op)
 {
     WideOp w{op.m.data(), (int)(op.m.size() >> (2 * op.k)), op.k, op.qubits, nullptr};
     const int copies = wide_scratch(c->n, w.k, w.nk, c->nsm);
-    if (copies > c->kacc_copies) {
-        float2 *b = nullptr;
-        if (cudaMalloc(&b, (size_t)copies * (sizeof(float2) << (2 * c->n))) != cudaSuccess) {
-            cudaGetLastError();
-            return set_error(QCW_ENOMEM, "Kraus scratch");
-        }
-        if (c->d_kacc) cudaFree(c->d_kacc);  // waits for the work that uses it
-        c->d_kacc = b;
-        c->kacc_copies = copies;
-    }
+    const qcw_status bs = wide_buffer(c, copies);
+    if (bs) return bs;
     if (wide_splits(c->n, w.k, w.nk, c->nsm)) {
         // one launch for all operators, from an uploaded copy (not while the stream is captured: a
         // graph has to carry the operators itself)
@@ -472,6 +484,7 @@ static void ctx_free(qcw_ctx *c)
     if (c->d_staging) cudaFree(c->d_staging);
     if (c->pv) cudaFree(c->pv);
     if (c->d_kacc) cudaFree(c->d_kacc);
+    for (float2 *b : c->kacc_old) cudaFree(b);
     if (c->d_kops) cudaFree(c->d_kops);
     if (c->h_kops) cudaFreeHost(c->h_kops);
     if (c->kops_ev) cudaEventDestroy(c->kops_ev);

@@ -175,16 +175,17 @@ struct qcw_ctx {
     bool in_pauli = false;
     bool pzero = false;
     bool pauli_off = false;
-    // Version of rho: bumped by everything that changes it.  The last fused pass of a flush
-    // also sums |rho_rc|^2 over what it writes (per-CTA partials in the fused runtime);
-    // purity_ver records the version those partials describe.
     // scratch copies of rho for channels on more than two qubits (allocated on first use)
     float2 *d_kacc = nullptr;
     int kacc_copies = 0;
+    std::vector<float2 *> kacc_old;  // smaller ones from before: captured graphs may still write there
     // operators of a channel on few tiles, uploaded for one launch (pinned source, guarded by an event)
     float2 *d_kops = nullptr, *h_kops = nullptr;
     size_t kops_cap = 0;
     cudaEvent_t kops_ev = nullptr;
+    // Version of rho: bumped by everything that changes it.  The last fused pass of a flush
+    // also sums |rho_rc|^2 over what it writes (per-CTA partials in the fused runtime);
+    // purity_ver records the version those partials describe.
     unsigned long long state_ver = 1;
     unsigned long long purity_ver = 0;
     // asynchronous readouts: QCW_CHECKPOINT_SLOTS slots of kCkptVals doubles on the device and

@@ -132,3 +132,42 @@ def test_plain_lists(q, n, what):
     assert np.abs(a.get_state() - b.get_state()).max() <= 8 * len(ops) * 2.0 ** -24
     assert a.stats()["launches"] < b.stats()["launches"]
     a.close(), b.close()
+
+
+@pytest.mark.parametrize("n,k,nk,more", [(5, 5, 8, 33), (4, 3, 20, 64), (9, 3, 49, 60)])
+def test_captured_channels_keep_their_scratch(q, n, k, nk, more):
+    """A channel of many operators in a captured graph: the graph carries the operators, and a channel
+    of more operators afterwards leaves the scratch it was captured with in place."""
+    import torch
+
+    rng = np.random.default_rng(10 * n + k)
+
+    def channel(count):
+        w = rng.uniform(0.5, 1.5, count)
+        return np.stack([np.sqrt(x) * haar_unitary(rng, 1 << k) for x in w / w.sum()])
+
+    qs = [int(x) for x in rng.permutation(n)[:k]]
+    first, second = channel(nk), channel(more)
+    start = random_rho(rng, n)
+    s = torch.cuda.Stream()
+    rho = torch.zeros(1 << n, 1 << n, dtype=torch.complex64, device="cuda")
+    torch.cuda.synchronize()
+    d = q.Density.from_tensor(rho, s)
+    d.set_state(start)
+    d.apply_kraus(first, qs)  # scratch and kernel attributes are there before the capture
+    d.sync()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        d.apply_kraus(first, qs)
+    d.set_state(start)
+    d.apply_kraus(second, qs)
+    d.sync()
+    held = torch.zeros(1 << 20, device="cuda")  # where memory given back would go
+    with torch.cuda.stream(s):
+        g.replay()
+    want = start.copy()
+    oracle.apply_kraus(want, second, qs)
+    oracle.apply_kraus(want, first, qs)
+    assert np.abs(d.get_state() - want).max() <= ATOL
+    assert float(held.abs().max()) == 0.0
+    d.close()
