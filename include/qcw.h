@@ -117,14 +117,15 @@ QCW_API qcw_status qcw_set_mode(qcw_ctx *ctx, int mode, int fuse_k);
 #define QCW_FUSED_KERNEL_HERM_TC 4
 QCW_API qcw_status qcw_set_fused_kernel(qcw_ctx *ctx, int which);
 
-/* Bounded waits inside the HERM_WS pass kernel.  Producer and consumer warps hand tiles over
- * through shared-memory barriers; each wait gives up after `polls` polls (0 restores the
- * default, about half a second or more), sets the context's error word and ends the kernel.
- * The next qcw_sync or readout then returns QCW_ETIMEOUT, and keeps doing so until qcw_reset or
- * a state load (rho is undefined after such a pass).  stall_tile >= 0 makes the first CTA skip
- * the load of its tile number stall_tile, so that its consumers' wait runs out (a test of the
- * error path without any fault); -1 turns that off.  The paper has no counterpart.
- * Flushes queued work first.  QCW_EINVAL if stall_tile < -1. */
+/* Bounded waits inside the pass kernels that overlap loads with arithmetic (the Pauli-basis pass of
+ * AUTO, HERM_WS, HERM_TC) and inside the tensor-core kernel of qcw_ensemble_density into this context.
+ * Each wait gives up after `polls` polls (0 restores the default, about half a second or more), sets the
+ * context's error word and ends the kernel.  The next qcw_sync, readout or state download (every call
+ * that returns part of the state; qcw_get_device_state too after a density) then returns QCW_ETIMEOUT, and
+ * keeps doing so until qcw_reset or a state load (rho is undefined after such a kernel).  stall_tile >= 0
+ * makes the first CTA skip the load of its tile number stall_tile (in a density: give up its wait for
+ * that tile), so that a wait runs out (a test of the error path without any fault); -1 turns that off.
+ * The paper has no counterpart.  Flushes queued work first.  QCW_EINVAL if stall_tile < -1. */
 QCW_API qcw_status qcw_set_fused_wait_limit(qcw_ctx *ctx, unsigned polls, int stall_tile);
 
 /* Validation mode (off by default; on for every new context when the environment variable
@@ -159,7 +160,8 @@ QCW_API qcw_status qcw_set_state(qcw_ctx *ctx, const double *rho_c128);
 /* Same from host complex64 (2 * 4^n floats), copied without conversion. */
 QCW_API qcw_status qcw_set_state_c64(qcw_ctx *ctx, const float *rho_c64);
 
-/* Host copy of rho as complex128 (2 * 4^n doubles).  Synchronises. */
+/* Host copy of rho as complex128 (2 * 4^n doubles).  Synchronises; QCW_ETIMEOUT after a kernel whose
+ * wait ran out. */
 QCW_API qcw_status qcw_get_state(qcw_ctx *ctx, double *rho_c128_out);
 
 /* ------------------------------------------------------------------- evolution */
@@ -219,7 +221,10 @@ QCW_API qcw_status qcw_ensemble_apply_noise1(qcw_ensemble *e, const double *omeg
                                           const int *choice);
 /* ctx's rho <- sum_v weights[v] |psi_v><psi_v| (weights: host, nvec doubles; FP32 sums of FP32
  * products).  ctx must have the ensemble's qubit count; its queued work is dropped as by
- * qcw_set_state.  Ordered after the ensemble's operations; asynchronous on ctx's stream. */
+ * qcw_set_state.  Ordered after the ensemble's operations; asynchronous on ctx's stream.  From 10
+ * qubits up a kernel with bounded waits takes part: if one runs out, the first call on ctx that reads the
+ * state or hands out its pointer returns QCW_ETIMEOUT (see qcw_set_fused_wait_limit); work ordered on the
+ * stream without such a call in between sees an undefined rho. */
 QCW_API qcw_status qcw_ensemble_density(qcw_ensemble *e, const double *weights, qcw_ctx *ctx);
 
 /* One element of a circuit handed over in a single call (qcw_apply_ops). */
@@ -319,7 +324,8 @@ QCW_API qcw_status qcw_measure(qcw_ctx *ctx, int qubit, int forced, double u, in
 
 /* Reduced density matrix of the kept qubits (strictly ascending, 0 <= nkeep <= n):
  * out[a, a'] = sum_b rho[(a b), (a' b)], where the first kept qubit is the most significant
- * bit of a.  out_c128 receives 2 * 4^nkeep doubles (subsystem states of Sec. 5.2.3). */
+ * bit of a.  out_c128 receives 2 * 4^nkeep doubles (subsystem states of Sec. 5.2.3).  QCW_ETIMEOUT
+ * after a kernel whose wait ran out. */
 QCW_API qcw_status qcw_partial_trace(qcw_ctx *ctx, const int *keep, int nkeep, double *out_c128);
 
 /* Size of the fixed result array used by qcw_partial_trace_static: 4^6 complex128 entries. */
@@ -330,9 +336,10 @@ QCW_API qcw_status qcw_partial_trace(qcw_ctx *ctx, const int *keep, int nkeep, d
  * any thread of the process captures a CUDA graph in global mode, cudaMalloc and cudaFree are
  * not allowed; an application whose allocator already holds the whole device budget has no
  * memory to give; and cudaFree synchronises the device, which a latency-critical loop cannot
- * afford.  qcw_partial_trace takes its device result buffer from cudaMallocAsync; this variant
- * instead writes into one array of QCW_PT_STATIC_MAX_ENTRIES complex128 values (64 KiB) that
- * lives in device memory as part of the library, on every GPU that loads it, until exit.
+ * afford.  qcw_partial_trace of more than 6 qubits takes its device result buffer from
+ * cudaMallocAsync, and a context needs allocations of its own; this variant instead writes into one
+ * array of QCW_PT_STATIC_MAX_ENTRIES complex128 values (64 KiB) that lives in device memory as part
+ * of the library, on every GPU that loads it, until exit.
  *
  * dev_rho: caller's device rho of nqubits (row-major complex64, the layout above); cuda_stream:
  * a cudaStream_t (NULL = legacy default stream) on the current device; keep / nkeep / out_c128

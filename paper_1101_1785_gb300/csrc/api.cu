@@ -370,6 +370,16 @@ qcw_status ensure_full(qcw_ctx *c)
     return QCW_OK;
 }
 
+static bool capturing(qcw_ctx *c)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();  // the legacy stream while another one is captured
+        return true;
+    }
+    return cap != cudaStreamCaptureStatusNone;
+}
+
 // The operators of op as FP32 in device memory, ordered on the context's stream.
 static qcw_status upload_operators(qcw_ctx *c, const QOp &op, const float2 **dev)
 {
@@ -430,12 +440,7 @@ static qcw_status plain_wide(qcw_ctx *c, const QOp &op)
     if (wide_splits(c->n, w.k, w.nk, c->nsm)) {
         // one launch for all operators, from an uploaded copy (not while the stream is captured: a
         // graph has to carry the operators itself)
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
-            cudaGetLastError();  // the legacy stream while another one is captured
-            cap = cudaStreamCaptureStatusActive;
-        }
-        if (cap == cudaStreamCaptureStatusNone) {
+        if (!capturing(c)) {
             qcw_status st = upload_operators(c, op, &w.dev);
             if (st) return st;
         }
@@ -479,8 +484,6 @@ static void ctx_free(qcw_ctx *c)
     if (c->d_partials) cudaFree(c->d_partials);
     if (c->d_result) cudaFree(c->d_result);
     if (c->h_result) cudaFreeHost(c->h_result);
-    if (c->d_pt) cudaFree(c->d_pt);
-    if (c->h_pt) cudaFreeHost(c->h_pt);
     if (c->d_staging) cudaFree(c->d_staging);
     if (c->pv) cudaFree(c->pv);
     if (c->d_kacc) cudaFree(c->d_kacc);
@@ -496,6 +499,15 @@ static void ctx_free(qcw_ctx *c)
     delete c;
 }
 
+// Result block: 64 values (the last one the error word), then the reduced states of up to
+// kSpectralMaxQubits qubits (64 KiB), with a pinned mirror.  An allocation per call, from a pool that
+// gives its memory back at each synchronisation, cost 200 us where the kernel takes 5: eight steps of a
+// five-qubit study with one spectrum each 3.04 -> 1.36 ms, the readouts of a 13-qubit state 1.36 -> 0.94 ms.
+static const int kSpectralMaxQubits = 6;
+constexpr int kReducedAt = 64;
+static_assert(kReducedAt == kErrSlot + 1, "the error word and a reduced state in one copy");
+constexpr size_t kResultBytes = kReducedAt * sizeof(double) + (sizeof(double2) << (2 * kSpectralMaxQubits));
+
 static qcw_status ctx_common(qcw_ctx *c)
 {
     const char *v = getenv("QCW_VALIDATE");
@@ -505,8 +517,8 @@ static qcw_status ctx_common(qcw_ctx *c)
     c->red_blocks = reduce_blocks(c->nsm);
     if (cudaMalloc(&c->d_partials, sizeof(double) * (size_t)c->red_blocks * (QCW_MAX_QUBITS + 2)) != cudaSuccess)
         return set_error(QCW_ENOMEM, "reduction scratch");
-    if (cudaMalloc(&c->d_result, 64 * sizeof(double)) != cudaSuccess) return set_error(QCW_ENOMEM, "result block");
-    if (cudaMallocHost(&c->h_result, 64 * sizeof(double)) != cudaSuccess) return set_error(QCW_ENOMEM, "pinned result");
+    if (cudaMalloc(&c->d_result, kResultBytes) != cudaSuccess) return set_error(QCW_ENOMEM, "result block");
+    if (cudaMallocHost(&c->h_result, kResultBytes) != cudaSuccess) return set_error(QCW_ENOMEM, "pinned result");
     CK(cudaMemset(c->d_result, 0, 64 * sizeof(double)));
     return QCW_OK;
 }
@@ -592,6 +604,8 @@ extern "C" qcw_status qcw_get_device_state(qcw_ctx *ctx, void **dev_rho, void **
     qcw_status st = fused_flush(ctx);
     if (!st) st = ensure_full(ctx);
     if (st) return st;
+    if (ctx->unchecked && !capturing(ctx)) st = wait_error_word(ctx);
+    if (st) return st;
     if (dev_rho) *dev_rho = ctx->rho;
     if (cuda_stream) *cuda_stream = ctx->stream;
     ctx->state_ver++;  // the caller may write rho
@@ -619,10 +633,19 @@ static qcw_status clear_error_word(qcw_ctx *c)
     return QCW_OK;
 }
 
-static qcw_status check_error_word(qcw_ctx *c, unsigned long long word)
+static qcw_status check_error_word(unsigned long long word)
 {
-    if (word) return set_error(QCW_ETIMEOUT, "fused pass: an in-kernel wait ran out; rho is undefined until reset");
+    if (word) return set_error(QCW_ETIMEOUT, "an in-kernel wait ran out (fused pass or ensemble density); rho is undefined until reset");
     return QCW_OK;
+}
+
+// The same from the pinned mirror, once the copy to it is done.
+static qcw_status check_error_word(qcw_ctx *c)
+{
+    unsigned long long w;
+    memcpy(&w, c->h_result + kErrSlot, sizeof w);
+    if (!w) c->unchecked = false;
+    return check_error_word(w);
 }
 
 extern "C" qcw_status qcw_set_fused_wait_limit(qcw_ctx *ctx, unsigned polls, int stall_tile)
@@ -636,10 +659,17 @@ extern "C" qcw_status qcw_set_fused_wait_limit(qcw_ctx *ctx, unsigned polls, int
     return QCW_OK;
 }
 
+qcw_status qcw::wait_error_word(qcw_ctx *c)
+{
+    CK(cudaMemcpyAsync(c->h_result + kErrSlot, device_error_word(c), sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    return check_error_word(c);
+}
+
 qcw_status qcw::begin_state_replace(qcw_ctx *c)
 {
     c->queue.clear();
-    c->half = c->in_pauli = c->pzero = false;
+    c->half = c->in_pauli = c->pzero = c->unchecked = false;
     c->state_ver++;
     return clear_error_word(c);
 }
@@ -648,6 +678,7 @@ extern "C" qcw_status qcw_reset(qcw_ctx *ctx)
 {
     CHECK_CTX(ctx);
     ctx->queue.clear();
+    ctx->unchecked = false;
     ctx->in_pauli = ctx->pzero = ctx->mode == QCW_MODE_FUSED && pauli_allowed(ctx);
     if (ctx->in_pauli) {  // the first pass starts from |0..0><0..0| without reading it
         ctx->half = false;
@@ -690,7 +721,7 @@ extern "C" qcw_status qcw_set_state(qcw_ctx *ctx, const double *rho_c128)
     qcw_status st = ensure_staging(ctx);
     if (st) return st;
     ctx->queue.clear();
-    ctx->half = ctx->in_pauli = ctx->pzero = false;
+    ctx->half = ctx->in_pauli = ctx->pzero = ctx->unchecked = false;
     ctx->state_ver++;
     st = clear_error_word(ctx);
     if (st) return st;
@@ -713,7 +744,7 @@ extern "C" qcw_status qcw_set_state_c64(qcw_ctx *ctx, const float *rho_c64)
     if (ctx->validate && !is_density(rho_c64, ctx->n))
         return set_error(QCW_EINVAL, "state is not Hermitian with unit trace (validation)");
     ctx->queue.clear();
-    ctx->half = ctx->in_pauli = ctx->pzero = false;
+    ctx->half = ctx->in_pauli = ctx->pzero = ctx->unchecked = false;
     ctx->state_ver++;
     qcw_status st = clear_error_word(ctx);
     if (st) return st;
@@ -738,8 +769,7 @@ extern "C" qcw_status qcw_get_state(qcw_ctx *ctx, double *out)
         CKLAUNCH(ctx, 1);
         CK(cudaMemcpyAsync(out + 2 * off, ctx->d_staging, cnt * sizeof(double2), cudaMemcpyDeviceToHost, ctx->stream));
     }
-    CK(cudaStreamSynchronize(ctx->stream));
-    return QCW_OK;
+    return wait_error_word(ctx);
 }
 
 // ------------------------------------------------------------------ evolution
@@ -899,12 +929,7 @@ extern "C" qcw_status qcw_sync(qcw_ctx *ctx)
     qcw_status st = fused_flush(ctx);
     if (!st) st = ensure_full(ctx);
     if (st) return st;
-    CK(cudaMemcpyAsync(ctx->h_result + kErrSlot, device_error_word(ctx), sizeof(double), cudaMemcpyDeviceToHost,
-                       ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    unsigned long long w;
-    memcpy(&w, ctx->h_result + kErrSlot, sizeof w);
-    return check_error_word(ctx, w);
+    return wait_error_word(ctx);
 }
 
 // ------------------------------------------------------------------ readouts
@@ -913,9 +938,7 @@ static qcw_status fetch_results(qcw_ctx *c)
 {
     CK(cudaMemcpyAsync(c->h_result, c->d_result, 64 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    unsigned long long w;
-    memcpy(&w, c->h_result + kErrSlot, sizeof w);
-    return check_error_word(c, w);
+    return check_error_word(c);
 }
 // The readouts of the current state into device memory: trace (2 values) and P(q = 1) for q < n;
 // purity.  All on whichever form the state is in.
@@ -1057,8 +1080,6 @@ extern "C" qcw_status qcw_correlation(qcw_ctx *ctx, int q1, int q2, double *out)
 }
 
 // ------------------------------------------------------------------ entropy and fidelity
-static const int kSpectralMaxQubits = 6;
-
 // Reduced state of `keep` on the host, made exactly Hermitian ((A + A^dagger) / 2).
 static qcw_status reduced_state(qcw_ctx *c, const int *keep, int nkeep, std::vector<c128> &ra)
 {
@@ -1178,7 +1199,7 @@ extern "C" qcw_status qcw_checkpoint_read(qcw_ctx *ctx, long long ticket, double
     const double *h = ctx->h_ckpt + (size_t)slot * kCkptVals;
     unsigned long long w;
     memcpy(&w, h + kCkptVals - 1, sizeof w);
-    qcw_status st = check_error_word(ctx, w);
+    qcw_status st = check_error_word(w);
     if (st) return st;
     memcpy(out, h, sizeof(double) * (size_t)(ctx->n + 3));
     return QCW_OK;
@@ -1203,26 +1224,6 @@ extern "C" qcw_status qcw_measure(qcw_ctx *ctx, int qubit, int forced, double u,
     else launch_project(ctx->rho, ctx->n, qubit, m, (float)(1.0 / pm), ctx->half, ctx->nsm, ctx->stream);
     CKLAUNCH(ctx, 1);
     return QCW_OK;
-}
-
-// Result buffers for reduced states of up to kSpectralMaxQubits qubits (64 KiB on the device, as much
-// pinned), kept in the context.  An allocation on every call, from a pool that gives its memory back at
-// each synchronisation, and a copy into pageable memory cost 200 us where the kernel takes 5: eight
-// steps of a five-qubit study with one spectrum each 3.04 -> 1.36 ms, the readouts of a 13-qubit state
-// 1.36 -> 0.94 ms.  false: no room, the call allocates as it used to (as for more kept qubits).
-static bool reduced_buffers(qcw_ctx *c)
-{
-    if (c->h_pt) return true;
-    const size_t bytes = sizeof(double2) << (2 * kSpectralMaxQubits);
-    double2 *d = nullptr, *h = nullptr;
-    if (cudaMalloc(&d, bytes) != cudaSuccess || cudaMallocHost(&h, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        if (d) cudaFree(d);
-        return false;
-    }
-    c->d_pt = d;
-    c->h_pt = h;
-    return true;
 }
 
 extern "C" qcw_status qcw_partial_trace(qcw_ctx *ctx, const int *keep, int nkeep, double *out_c128)
@@ -1251,34 +1252,30 @@ extern "C" qcw_status qcw_partial_trace(qcw_ctx *ctx, const int *keep, int nkeep
     for (int q = 0; q < n; q++)
         if (!(kept & (1u << q))) p.tpos[p.ntr++] = (int8_t)(n - 1 - q);
     size_t nout = (size_t)1 << (2 * nkeep);
-    double2 *d_out = nullptr;
-    double2 *h_out = nullptr;
-    bool own = false;
-    if (nout * sizeof(double2) <= 64 * sizeof(double)) {
-        d_out = reinterpret_cast<double2 *>(ctx->d_result);
-        h_out = reinterpret_cast<double2 *>(ctx->h_result);
-    } else if (nkeep <= kSpectralMaxQubits && reduced_buffers(ctx)) {
-        d_out = ctx->d_pt;
-        h_out = ctx->h_pt;
-    } else {
-        own = true;
-        if (cudaMallocAsync(&d_out, nout * sizeof(double2), ctx->stream) != cudaSuccess) {
-            cudaGetLastError();
-            return set_error(QCW_ENOMEM, "partial trace output");
-        }
+    double2 *d_out = reinterpret_cast<double2 *>(ctx->d_result + kReducedAt);
+    const bool own = nkeep > kSpectralMaxQubits;
+    if (own && cudaMallocAsync(&d_out, nout * sizeof(double2), ctx->stream) != cudaSuccess) {
+        cudaGetLastError();
+        return set_error(QCW_ENOMEM, "partial trace output");
     }
     if (from_pauli) launch_pauli_ptrace(ctx->pv, p, d_out, ctx->stream);
     else launch_partial_trace(ctx->rho, p, d_out, ctx->nsm, ctx->stream);
     ctx->launches += 1;
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(h_out ? static_cast<void *>(h_out) : out_c128, d_out, nout * sizeof(double2), cudaMemcpyDeviceToHost,
+    // with the error word: right in front of the reduced states
+    double *word = ctx->h_result + kErrSlot;
+    if (e == cudaSuccess && own) {
+        e = cudaMemcpyAsync(out_c128, d_out, nout * sizeof(double2), cudaMemcpyDeviceToHost, ctx->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(word, ctx->d_result + kErrSlot, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
+    } else if (e == cudaSuccess) {
+        e = cudaMemcpyAsync(word, ctx->d_result + kErrSlot, sizeof(double) + nout * sizeof(double2), cudaMemcpyDeviceToHost,
                             ctx->stream);
+    }
     if (own) cudaFreeAsync(d_out, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_error(e, "partial trace");
-    if (h_out) memcpy(out_c128, h_out, nout * sizeof(double2));
-    return QCW_OK;
+    if (!own) memcpy(out_c128, ctx->h_result + kReducedAt, nout * sizeof(double2));
+    return check_error_word(ctx);
 }
 
 // ------------------------------------------------------------------ diagnostics

@@ -63,7 +63,8 @@ __device__ __forceinline__ void ed_split(float x, float &hi, float &lo)
 __global__ void __launch_bounds__(kEdThreads) k_ens_density_tc(const float2 *__restrict__ psi, int nvec, int n,
                                                                const float *__restrict__ w,
                                                                float2 *__restrict__ rho,
-                                                               unsigned *__restrict__ err)
+                                                               unsigned *__restrict__ err, unsigned wait_limit,
+                                                               int stall_tile)
 {
     extern __shared__ __align__(128) unsigned char ed_smem[];
     float *stage = reinterpret_cast<float *>(ed_smem);  // 2 stages x kEdStageFloats
@@ -127,7 +128,7 @@ __global__ void __launch_bounds__(kEdThreads) k_ens_density_tc(const float2 *__r
             const int s = rd & 1;
             const unsigned cms = s ? cm1 : cm0;
             if (cms > 0) {  // the MMAs that last read stage s are done before it is refilled
-                const bool good = tid == 0 ? mbar_wait(&bar[s], (cms - 1) & 1u, kEdWaitLimit) : true;
+                const bool good = tid == 0 ? mbar_wait(&bar[s], (cms - 1) & 1u, wait_limit) : true;
                 ok = bar_and(1, kEdThreads, good);
                 if (!ok) break;
             }
@@ -179,7 +180,8 @@ __global__ void __launch_bounds__(kEdThreads) k_ens_density_tc(const float2 *__r
         {
             const int s = (nround - 1) & 1;
             const unsigned cms = s ? cm1 : cm0;
-            const bool good = tid == 0 ? mbar_wait(&bar[s], (cms - 1) & 1u, kEdWaitLimit) : true;
+            const bool stall = blockIdx.x == 0 && (int)(pr / gridDim.x) == stall_tile;  // a wait given up (tests)
+            const bool good = tid == 0 ? !stall && mbar_wait(&bar[s], (cms - 1) & 1u, wait_limit) : true;
             ok = bar_and(1, kEdThreads, good);
             if (!ok) break;
         }
@@ -236,15 +238,16 @@ size_t ens_density_tc_smem()
 }
 
 // Launches the tensor-core density for 2^n >= 128; returns false (nothing launched) otherwise.
-bool launch_ens_density_tc(const float2 *psi, int nvec, int n, const float *w, float2 *rho, unsigned *err, int nsm,
-                           cudaStream_t s)
+bool launch_ens_density_tc(const float2 *psi, int nvec, int n, const float *w, float2 *rho, unsigned *err,
+                           unsigned wait_limit, int stall_tile, int nsm, cudaStream_t s)
 {
     if (n < 8) return false;  // at least two 128-row blocks: one tile below the diagonal
     const size_t smem = ens_density_tc_smem();
     if (ensure_smem_attr(reinterpret_cast<const void *>(k_ens_density_tc), smem)) return false;
     const uint64_t m = (1ull << n) / kEdT, pairs = m * (m - 1) / 2;
     const uint64_t cap = (uint64_t)nsm * 2;  // two CTAs per SM (256 of the 512 tensor-memory columns each)
-    k_ens_density_tc<<<(unsigned)(pairs < cap ? pairs : cap), kEdThreads, smem, s>>>(psi, nvec, n, w, rho, err);
+    k_ens_density_tc<<<(unsigned)(pairs < cap ? pairs : cap), kEdThreads, smem, s>>>(psi, nvec, n, w, rho, err,
+                                                                                         wait_limit ? wait_limit : kEdWaitLimit, stall_tile);
     return true;
 }
 

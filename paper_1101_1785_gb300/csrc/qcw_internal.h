@@ -90,9 +90,10 @@ void launch_symmetrize(float2 *rho, int n, int nsm, cudaStream_t s);
 int launch_purity_lower(const float2 *rho, int n, double *partials, double *out, int nblocks, cudaStream_t s);
 void launch_fold(const double *partials, int nblocks, double *out, cudaStream_t s);
 // Multiverse density on the tensor cores (ensemble_tc.cu) for 2^n >= 128: rho = sum_v w_v
-// |psi_v><psi_v|; *err gets bit 0 if a bounded wait ran out.  Returns false if not launched.
-bool launch_ens_density_tc(const float2 *psi, int nvec, int n, const float *w, float2 *rho, unsigned *err, int nsm,
-                           cudaStream_t s);
+// |psi_v><psi_v|; *err gets bit 0 if a bounded wait ran out (wait_limit polls, 0: default; the first CTA
+// gives up at its tile stall_tile, -1: never).  Returns false if not launched.
+bool launch_ens_density_tc(const float2 *psi, int nvec, int n, const float *w, float2 *rho, unsigned *err,
+                           unsigned wait_limit, int stall_tile, int nsm, cudaStream_t s);
 // Operations on three to five qubits (wide.cu): rho <- sum_j K_j rho K_j^dagger, nk operators of
 // 2^k x 2^k at m.  scratch: wide_scratch copies of rho.
 struct WideOp {
@@ -149,12 +150,11 @@ struct qcw_ctx {
     bool validate = false;  // qcw_set_validation: check unitarity, Kraus trace, Hermitian states
     int fuse_k = 0;
     int fused_kernel = QCW_FUSED_KERNEL_AUTO;
-    // reduction scratch: per-block partials and a small result block (+ pinned mirror)
+    // reduction scratch: per-block partials and the result block (+ pinned mirror; api.cu kResultBytes)
     double *d_partials = nullptr;
     int red_blocks = 0;
-    double2 *d_pt = nullptr, *h_pt = nullptr;  // partial-trace results (api.cu reduced_buffers)
     double *d_result = nullptr;
-    double *h_result = nullptr;  // pinned, 64 doubles
+    double *h_result = nullptr;  // pinned
     // staging for complex128 <-> complex64 conversion
     void *d_staging = nullptr;
     size_t staging_bytes = 0;
@@ -165,6 +165,9 @@ struct qcw_ctx {
     // tile whose load the first CTA skips (fault injection; -1: none)
     unsigned wait_limit = 0;
     int stall_tile = -1;
+    // an ensemble density with bounded waits was launched into rho and nobody has looked at the error
+    // word since: qcw_get_device_state does then, the readouts always do
+    bool unchecked = false;
     // half storage: only the lower triangle (r >= c) of rho is current (the warp-specialised
     // pass leaves it so); ensure_full completes the matrix before anything else reads it
     bool half = false;
@@ -230,6 +233,8 @@ qcw_status pauli_settle(qcw_ctx *c);
 // rho is about to be overwritten from outside the queue: drop queued work, mark the storage
 // full, bump the state version and clear the error word.
 qcw_status begin_state_replace(qcw_ctx *c);
+// Wait for the context's stream; QCW_ETIMEOUT if a wait in one of its kernels ran out.
+qcw_status wait_error_word(qcw_ctx *c);
 // The checks of an op list against an n-qubit register alone.
 qcw_status check_ops(int n, const qcw_op *ops, int nops, const double *matrices, bool validate = false);
 // Validate an op list against an n-qubit register and convert it to queued operations

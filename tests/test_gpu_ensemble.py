@@ -174,3 +174,47 @@ def test_density_at_the_largest_register(q):
     assert abs(d.trace() - 1) <= 1e-6
     d.close()
     e.close()
+
+
+def test_density_reports_a_wait_that_ran_out(q):
+    """A wait given up in the tensor-core kernel is an error of whatever reads or hands out the matrix, until
+    the state is replaced; the next density is whole again."""
+    n, nvec = 10, 24
+    rng = np.random.default_rng(5)
+    psi = rng.standard_normal((nvec, 1 << n)) + 1j * rng.standard_normal((nvec, 1 << n))
+    psi /= np.linalg.norm(psi, axis=1)[:, None]
+    w = np.full(nvec, 1 / nvec)
+    e, d = q.Ensemble(n, nvec), q.Density(n)
+    e.set(psi)
+    d.set_fused_wait_limit(0, 0)
+    e.density(w, d)
+    for call in (d.device_state, d.get_state, lambda: d.partial_trace([0]), lambda: d.partial_trace(list(range(7))),
+                 lambda: d.eigenvalues([0, 1]), d.trace, d.purity, d.probabilities, d.sync, d.device_state):
+        with pytest.raises(q.QcwError) as err:
+            call()
+        assert err.value.status == q.QCW_ETIMEOUT
+    d.set_fused_wait_limit(0)
+    e.density(w, d)
+    d.device_state()
+    want = (psi * w[:, None]).T @ psi.conj()
+    assert np.abs(d.get_state() - want).max() <= 1e-5
+    d.close()
+    e.close()
+
+
+def test_matrix_readouts_report_a_fused_wait_that_ran_out(q):
+    """The state itself and reduced states fail after such a pass, as the other readouts do."""
+    d = q.Density(8)
+    d.set_mode(q.QCW_MODE_FUSED)
+    d.set_fused_wait_limit(2000, 0)
+    d.reset()
+    for a in range(7):
+        d.apply_gate2(np.eye(4)[[0, 1, 3, 2]], a, a + 1)
+    for call in (d.get_state, lambda: d.partial_trace([0, 1, 2]), lambda: d.entropy([0]), d.purity):
+        with pytest.raises(q.QcwError) as err:
+            call()
+        assert err.value.status == q.QCW_ETIMEOUT
+    d.set_fused_wait_limit(0)
+    d.reset()
+    assert abs(d.get_state()[0, 0] - 1) == 0
+    d.close()
