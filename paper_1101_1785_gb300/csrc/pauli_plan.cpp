@@ -514,6 +514,7 @@ static PauliPlan plan_nodes(NodeBuilder &nb, int n, int kmax, bool beam, bool ze
                 ncoef += nc;
             }
         }
+        if (chosen.empty()) continue;  // a set of the sequence whose operations wait for ones a full pass left
         // rounds: of all pairs of tile digits beside digit 0, the one that takes most of what is left
         auto tmask = [&](size_t i) {
             unsigned m = 1u << tile_of[digit(nodes[i].a)];

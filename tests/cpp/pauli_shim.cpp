@@ -236,3 +236,15 @@ extern "C" int list_plan_differs(int n, int nops, const int *kind, const int *k,
     }
     return 0;
 }
+
+// Passes of a plan that have no operation; *npass: all of them.
+extern "C" int pauli_empty_passes(int n, int kmax, int beam, int nops, const int *kind, const int *k, const int *qubits,
+                                  const double *mats, const long long *mat_off, int *npass)
+{
+    const std::vector<QOp> ops = op_list(nops, kind, k, qubits, mats, mat_off);
+    const PauliPlan plan = plan_pauli(ops, 0, ops.size(), n, kmax, beam != 0, false);
+    int empty = 0;
+    for (const PPass &p : plan.passes) empty += p.ops.empty() ? 1 : 0;
+    *npass = (int)plan.passes.size();
+    return empty;
+}

@@ -225,3 +225,27 @@ def test_small_operators_are_kept(shim, scale):
     assert shim.pairs_replay(n, len(ops), p(kind), p(k), p(qs), p(mats), p(off), p(v)) > 0
     assert np.abs(v - want).max() <= tol
     assert _list_differs(shim, n, ops) == 0
+
+
+@pytest.mark.parametrize("n,kmax", [(8, 0), (9, 0), (10, 0), (8, 3), (10, 5)])
+def test_no_pass_without_operations(shim, n, kmax):
+    """A pass cut at its program's limits leaves operations to later ones; sets of the beam search that
+    find nothing left to do are not run."""
+    for seed in range(12):
+        rng = np.random.default_rng(100 * n + seed)
+        ops = []
+        for i in range(60):  # dense maps on few qubits fill a pass's program, the others wait for them
+            few = rng.permutation(min(n, 4))[:2] if i % 3 else rng.permutation(n)[:2]
+            ops.append(wl.Op("gate", tuple(int(x) for x in few), haar_unitary(rng, 4)[None]))
+        kind, k, qs, mats, off = _packed(ops)
+        p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+        npass = ctypes.c_int()
+        assert shim.pauli_empty_passes(n, kmax, 1, len(ops), p(kind), p(k), p(qs), p(mats), p(off), ctypes.byref(npass)) == 0
+        assert npass.value > 1
+    rho = random_rho(rng, n)
+    v = coefficients(rho)
+    for op in ops:
+        oracle.apply_op(rho, op)
+    _replay(shim, n, ops, v, kmax, True)
+    want = coefficients(rho)
+    assert np.linalg.norm(v - want) <= 2 * len(ops) * 2.0 ** -24 * np.linalg.norm(want)
