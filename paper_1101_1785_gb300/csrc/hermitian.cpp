@@ -13,7 +13,7 @@ using cd = std::complex<double>;
 
 // Eigenvalues only: Householder reduction to a real tridiagonal matrix (Golub and Van Loan, "Matrix
 // Computations", Sec. 8.3: A <- A - v w^H - w v^H with w = p - (beta / 2) (p^H v) v, p = beta A v),
-// then implicit QL steps with Wilkinson's shift on it (Sec. 8.3.5).  O(N^3) once where each sweep
+// then implicit QR steps with Wilkinson's shift on it (Sec. 8.3.3, 8.3.4).  O(N^3) once where each sweep
 // of the Jacobi iteration below costs several times that: 64 x 64 took 6 ms with it.
 static void eigenvalues_only(const cd *A_in, int N, double *w)
 {
@@ -64,37 +64,35 @@ static void eigenvalues_only(const cd *A_in, int N, double *w)
     }
     double scale = 0;
     for (int i = 0; i < N; i++) d[i] = Ar[(size_t)i * N + i], scale = std::max(scale, std::fabs(d[i]) + e[i]);
-    for (int l = 0; l < N; l++) {
-        for (int it = 0; it < 60; it++) {
-            int m = l;
-            while (m + 1 < N && std::fabs(e[m]) > 1e-17 * scale &&
-                   std::fabs(e[m]) > 2.3e-16 * (std::fabs(d[m]) + std::fabs(d[m + 1])))
-                m++;
-            if (m == l) break;
-            const double g0 = (d[l + 1] - d[l]) / (2.0 * e[l]), r0 = std::hypot(g0, 1.0);
-            double g = d[m] - d[l] + e[l] / (g0 + (g0 >= 0 ? r0 : -r0));
-            double s = 1, c = 1, p = 0;
-            int i = m - 1;
-            for (; i >= l; i--) {
-                const double f = s * e[i], b = c * e[i], r = std::hypot(f, g);
-                e[i + 1] = r;
-                if (r == 0) {  // the matrix splits here
-                    d[i + 1] -= p;
-                    e[m] = 0;
-                    break;
-                }
-                s = f / r;
-                c = g / r;
-                g = d[i + 1] - p;
-                const double t = (d[i] - g) * s + 2.0 * c * b;
-                p = s * t;
-                d[i + 1] = g + p;
-                g = c * t - b;
+    // QR steps on the last block lo..hi that does not split: T <- Q^T T Q with Q a product of plane
+    // rotations (c, s) of rows k, k + 1, the first one that of T - mu, the others those that put back the
+    // element (k + 1, k - 1) which the one before it has filled.
+    for (int hi = N - 1, steps = 0; hi > 0;) {
+        int lo = hi;
+        while (lo > 0 && std::fabs(e[lo - 1]) > 1e-17 * scale &&
+               std::fabs(e[lo - 1]) > 2.3e-16 * (std::fabs(d[lo - 1]) + std::fabs(d[lo])))
+            lo--;
+        if (lo == hi || steps == 60) {  // d[hi] is an eigenvalue
+            hi--, steps = 0;
+            continue;
+        }
+        steps++;
+        // mu: of the eigenvalues of the last two rows the one nearer to d[hi]
+        const double half = 0.5 * (d[hi - 1] - d[hi]), root = std::hypot(half, e[hi - 1]);
+        double x = d[lo] - d[hi] + e[hi - 1] * (e[hi - 1] / (half + (half >= 0 ? root : -root))), z = e[lo];
+        for (int k = lo; k < hi; k++) {
+            const double r2 = x * x + z * z, r = r2 > 1e-280 && r2 < 1e280 ? std::sqrt(r2) : std::hypot(x, z);
+            const double c = r > 0 ? x / r : 1.0, s = r > 0 ? z / r : 0.0;
+            if (k > lo) e[k - 1] = r;
+            const double p = c * d[k] + s * e[k], q = c * e[k] + s * d[k + 1];      // rows k and k + 1 rotated
+            const double t = c * e[k] - s * d[k], u = c * d[k + 1] - s * e[k];
+            d[k] = c * p + s * q;  // then the columns
+            d[k + 1] = c * u - s * t;
+            x = e[k] = c * t + s * u;
+            if (k + 1 < hi) {
+                z = s * e[k + 1];
+                e[k + 1] *= c;
             }
-            if (i >= l) continue;
-            d[l] -= p;
-            e[l] = g;
-            e[m] = 0;
         }
     }
     std::sort(d.begin(), d.end());

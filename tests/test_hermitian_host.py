@@ -117,3 +117,41 @@ def test_fidelity_matches_the_matrix_square_root_definition(lib):
         s = v @ np.diag(np.sqrt(np.clip(mu, 0, None))) @ v.conj().T
         want = np.sum(np.sqrt(np.clip(np.linalg.eigvalsh(s @ rho @ s), 0, None)))
         assert abs(_fid(lib, rho, sigma) - want) < 1e-10
+
+
+def _eigvals_only(lib, a):
+    a = np.ascontiguousarray(a, dtype=np.complex128)
+    w = np.zeros(a.shape[0])
+    lib.shim_herm_eig(_p(a), a.shape[0], _p(w), None)
+    return w
+
+
+def _spectra(rng, n):
+    """Matrices whose tridiagonal forms differ in kind: full, low rank, projector, graded, diagonal, clustered,
+    already tridiagonal, zero."""
+    u = haar_unitary(rng, n)
+    yield _random_hermitian(rng, n)
+    yield u[:, :1] @ u[:, :1].conj().T
+    yield u[:, : max(1, n // 2)] @ u[:, : max(1, n // 2)].conj().T
+    yield u @ np.diag(10.0 ** -np.arange(n)) @ u.conj().T
+    yield np.diag(rng.normal(size=n)).astype(complex)
+    yield u @ np.diag(1 + 1e-13 * np.arange(n)) @ u.conj().T
+    yield np.diag(rng.normal(size=n)) + np.diag(np.ones(n - 1), 1) + np.diag(np.ones(n - 1), -1)
+    yield np.zeros((n, n))
+    ghz = np.zeros((n, n))
+    ghz[[0, 0, -1, -1], [0, -1, 0, -1]] = 0.5
+    yield ghz
+    yield np.diag([1.0] + [0.0] * (n - 1)) + 1e-200 * _random_hermitian(rng, n)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 8, 17, 32, 64])
+def test_eigenvalues_without_vectors(lib, n):
+    """The path of the spectra and entropies: no vectors asked for (tridiagonal form and QR steps)."""
+    rng = np.random.default_rng(40 + n)
+    for a in _spectra(rng, n):
+        a = (a + a.conj().T) / 2
+        # backward stable: about n orthogonal steps of a few roundings of the norm each
+        tol = 8 * n * np.finfo(float).eps * max(np.linalg.norm(a, 2), 1e-300)
+        w = _eigvals_only(lib, a)
+        assert np.abs(w - np.linalg.eigvalsh(a)).max() <= tol
+        assert np.abs(w - _eig(lib, a)[0]).max() <= tol
