@@ -669,7 +669,7 @@ qcw_status qcw::wait_error_word(qcw_ctx *c)
 qcw_status qcw::begin_state_replace(qcw_ctx *c)
 {
     c->queue.clear();
-    c->half = c->in_pauli = c->pzero = c->unchecked = false;
+    c->half = c->in_pauli = c->pzero = c->unchecked = c->pauli_off = false;
     c->state_ver++;
     return clear_error_word(c);
 }
@@ -678,7 +678,7 @@ extern "C" qcw_status qcw_reset(qcw_ctx *ctx)
 {
     CHECK_CTX(ctx);
     ctx->queue.clear();
-    ctx->unchecked = false;
+    ctx->unchecked = ctx->pauli_off = false;
     ctx->in_pauli = ctx->pzero = ctx->mode == QCW_MODE_FUSED && pauli_allowed(ctx);
     if (ctx->in_pauli) {  // the first pass starts from |0..0><0..0| without reading it
         ctx->half = false;
@@ -721,7 +721,7 @@ extern "C" qcw_status qcw_set_state(qcw_ctx *ctx, const double *rho_c128)
     qcw_status st = ensure_staging(ctx);
     if (st) return st;
     ctx->queue.clear();
-    ctx->half = ctx->in_pauli = ctx->pzero = ctx->unchecked = false;
+    ctx->half = ctx->in_pauli = ctx->pzero = ctx->unchecked = ctx->pauli_off = false;
     ctx->state_ver++;
     st = clear_error_word(ctx);
     if (st) return st;
@@ -744,7 +744,7 @@ extern "C" qcw_status qcw_set_state_c64(qcw_ctx *ctx, const float *rho_c64)
     if (ctx->validate && !is_density(rho_c64, ctx->n))
         return set_error(QCW_EINVAL, "state is not Hermitian with unit trace (validation)");
     ctx->queue.clear();
-    ctx->half = ctx->in_pauli = ctx->pzero = ctx->unchecked = false;
+    ctx->half = ctx->in_pauli = ctx->pzero = ctx->unchecked = ctx->pauli_off = false;
     ctx->state_ver++;
     qcw_status st = clear_error_word(ctx);
     if (st) return st;

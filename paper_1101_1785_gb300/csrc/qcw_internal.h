@@ -173,7 +173,8 @@ struct qcw_ctx {
     bool half = false;
     // Pauli storage (pauli.h): pv holds v_P = Tr[P rho] and rho is stale while in_pauli; pzero: the
     // state is |0..0><0..0| and neither buffer has been written yet (the first pass starts from it).
-    // pv is allocated on first use and kept; pauli_off: it could not be allocated.
+    // pv is allocated on first use and kept; pauli_off: it could not be allocated (tried again for the
+    // next state).
     float *pv = nullptr;
     bool in_pauli = false;
     bool pzero = false;

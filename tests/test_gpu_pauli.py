@@ -234,3 +234,29 @@ def test_storage_of_a_given_matrix(q, n, touched, gates, k):
             oracle.apply_op(want, op)
         np.testing.assert_allclose(d.probabilities(), oracle.probabilities(want), atol=READ_TOL, rtol=0)
         assert np.abs(d.get_state() - want).max() <= ATOL
+
+
+def test_storage_is_tried_again_for_the_next_state(q):
+    """Without room for the coefficients the passes run on rho; once there is room, the next state takes them."""
+    import torch
+
+    n = 15  # rho 8 GiB, the coefficients 4 GiB
+    d = q.Density(n)
+    d.set_mode(q.QCW_MODE_FUSED)
+    held, left = [], 2 << 30
+    while torch.cuda.mem_get_info()[0] > left + (64 << 20):
+        free = torch.cuda.mem_get_info()[0] - left
+        held.append(torch.empty(min(free, 8 << 30) // (2 << 20) * (2 << 20), dtype=torch.uint8, device="cuda"))
+    d.reset()
+    d.apply_gate1(wl.gate_matrix("H"), 0)
+    d.apply_gate2(wl.gate_matrix("CNOT"), 0, n - 1)
+    assert abs(d.correlation(0, n - 1)[2, 2] - 1) <= READ_TOL
+    held.clear()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    d.reset()
+    d.apply_gate1(wl.gate_matrix("H"), 0)
+    d.apply_gate2(wl.gate_matrix("CNOT"), 0, n - 1)
+    assert abs(d.correlation(0, n - 1)[2, 2] - 1) <= READ_TOL
+    assert before - torch.cuda.mem_get_info()[0] >= 4 << 30
+    d.close()
