@@ -27,7 +27,6 @@ struct qcw_batch {
     std::vector<int> red_first, red_n;
     char *ddesc = nullptr;
     float *arena = nullptr;
-    size_t arena_elems = 0;
     // scratch of qcw_batch_get_state for the largest circuit: behind the states in the arena, behind hred
     float2 *stage = nullptr, *host = nullptr;
     float *copy = nullptr;
@@ -176,7 +175,6 @@ extern "C" qcw_status qcw_batch_create(int ncirc, const int *nqubits, const long
         p.off = doff[j];
         std::vector<char>().swap(p.desc);
     }
-    b->arena_elems = aelems;
     const int nmax = *std::max_element(nqubits, nqubits + ncirc);
     const size_t celems = program_copies(nmax) ? program_elems(nmax) : 0;
     if (cudaMalloc(&b->ddesc, dbytes) != cudaSuccess ||

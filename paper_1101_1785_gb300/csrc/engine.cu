@@ -286,8 +286,7 @@ Program make_program(const qcw_op *ops, int nops, const double *matrices, int n,
     Program p;
     PauliPlan plan = plan_pauli_list(ops, nops, matrices, n, fuse_k);
     p.n = n;
-    p.nd = plan.nd;
-    p.whole = p.nd <= kPTile;
+    p.whole = plan.nd <= kPTile;
     for (const PPass &ps : plan.passes) {
         PassDesc D;
         D.h = pauli_header(ps, plan.w);

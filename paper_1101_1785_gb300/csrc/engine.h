@@ -57,9 +57,9 @@ void engine_launch(const EngineLaunch &L, bool dense, int grid, size_t smem, cud
 qcw_status engine_prepare(int dev, bool dense, size_t smem, int *grid);
 
 // A circuit turned into device-ready descriptors.  Registers below kPMinDigits qubits are padded with
-// qubits in |0> above them: nd digits.
+// qubits in |0> above them.
 struct Program {
-    int n = 0, nd = 0;
+    int n = 0;
     bool whole = false;      // the state fits one tile: one WI_WHOLE item
     bool dense = false;
     std::vector<char> desc;  // the passes, PassDesc after PassDesc

@@ -114,7 +114,6 @@ struct CachedPauli {
     bool zero = false;     // planned for a start from |0..0>
     std::vector<QOp> ops;  // exact copy for verification
     std::vector<PauliBlob> passes;
-    int nnode = 0;
     long long last_use = 0;
 };
 

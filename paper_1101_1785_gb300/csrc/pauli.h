@@ -76,7 +76,6 @@ struct PPass {
 struct PauliPlan {
     int n = 0, nd = 0;  // qubits; digits (n, at least kPMinDigits)
     std::vector<PPass> passes;
-    int nnode2 = 0;     // two-qubit operations left after merging
     // zero start: what the one-qubit operations before any two-qubit operation make of |0..0>, a product
     // state, v_P = prod_d w[d][label of digit d]; the first pass starts from it.  (1, 1, 0, 0) else.
     std::vector<float> w;

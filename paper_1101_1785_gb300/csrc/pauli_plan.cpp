@@ -466,7 +466,7 @@ static PauliPlan plan_nodes(NodeBuilder &nb, int n, int kmax, bool beam, bool ze
     std::vector<unsigned> mask(nodes.size());
     for (size_t i = 0; i < nodes.size(); i++) {
         mask[i] = 1u << digit(nodes[i].a);
-        if (nodes[i].b >= 0) mask[i] |= 1u << digit(nodes[i].b), plan.nnode2++;
+        if (nodes[i].b >= 0) mask[i] |= 1u << digit(nodes[i].b);
     }
     const bool whole = nd <= t && !kmax;
     std::vector<unsigned> cand;
