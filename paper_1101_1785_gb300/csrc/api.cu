@@ -762,6 +762,8 @@ extern "C" qcw_status qcw_get_state(qcw_ctx *ctx, double *out)
     if (st) return st;
     st = ensure_staging(ctx);
     if (st) return st;
+    // ahead of the state: behind it, its own trip would take 7 us of a small state's 27
+    CK(cudaMemcpyAsync(ctx->h_result + kErrSlot, device_error_word(ctx), sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     size_t total = (size_t)1 << (2 * ctx->n);
     for (size_t off = 0; off < total; off += kStageElems) {
         size_t cnt = total - off < kStageElems ? total - off : kStageElems;
@@ -769,7 +771,8 @@ extern "C" qcw_status qcw_get_state(qcw_ctx *ctx, double *out)
         CKLAUNCH(ctx, 1);
         CK(cudaMemcpyAsync(out + 2 * off, ctx->d_staging, cnt * sizeof(double2), cudaMemcpyDeviceToHost, ctx->stream));
     }
-    return wait_error_word(ctx);
+    CK(cudaStreamSynchronize(ctx->stream));
+    return check_error_word(ctx);
 }
 
 // ------------------------------------------------------------------ evolution
