@@ -92,12 +92,16 @@ QCW_API qcw_status qcw_set_mode(qcw_ctx *ctx, int mode, int fuse_k);
  *     A non-Hermitian matrix loaded with qcw_set_state is not preserved.  One CTA per tile.
  *   AUTO (the default): from 3 qubits up the state is kept as its 4^n real Pauli coefficients
  *     v_P = Tr[P rho] between readouts (a second buffer of 4 * 4^n bytes beside rho, allocated on
- *     first use; without room for it, and for work too short to win back the two changes of
- *     basis, passes run as HERM_WS): half the bytes of rho per pass, real one-qubit maps of 12
+ *     first use and kept; without room for it, for a state given as a matrix of up to 7 qubits, and
+ *     for work too short to win back the two changes of basis, passes run as HERM_WS): half the bytes of rho per pass, real one-qubit maps of 12
  *     multiply-adds per four coefficients, CNOT and CZ as signed permutations.  Every readout but
  *     the ones of the whole matrix has a form on v; the library changes back to rho whenever
  *     the matrix itself is read (qcw_get_state, qcw_get_device_state, qcw_sync, plain-mode work).
- *     A non-Hermitian matrix loaded with qcw_set_state is not preserved.
+ *     A non-Hermitian matrix loaded with qcw_set_state is not preserved.  A probability is half the
+ *     difference of two coefficients, so its absolute error is a few 2^-24 of the trace however small
+ *     it is (and it can come out that far below 0).  Operations on rho leave the same error on the
+ *     qubits they act on, but keep smaller populations of the others to relative precision: choose
+ *     HERM_WS where those matter.
  *   HERM_WS (and AUTO below 3 qubits): the same Hermitian pass as HERM on persistent CTAs whose
  *     producer warps load and store tiles while consumer warps evolve them, so memory traffic
  *     and arithmetic overlap; each pass reads and writes only the lower triangle r >= c of rho
@@ -189,7 +193,8 @@ QCW_API qcw_status qcw_apply_gate(qcw_ctx *ctx, const double *u, const int *qubi
  * given.  One- and two-qubit channels act as composed superoperators (and join fused passes);
  * wider ones run as one pass over rho (all operators at once, on the plain path); many operators
  * on a small register, or more than a launch carries (48, 12, 3 for k = 3, 4, 5), use scratch
- * copies of rho, allocated on first use and kept until the context is destroyed. */
+ * copies of rho, allocated on first use and kept until the context is destroyed (also where a later
+ * channel needs more and gets a larger one). */
 QCW_API qcw_status qcw_apply_kraus(qcw_ctx *ctx, const double *kraus, int nkraus, const int *qubits,
                            int k);
 
@@ -257,8 +262,8 @@ QCW_API qcw_status qcw_sync(qcw_ctx *ctx);
 QCW_API qcw_status qcw_trace(qcw_ctx *ctx, double *re, double *im);
 
 /* sum_ij |rho_ij|^2, which equals Tr[rho . rho] (Sec. 5.2.3) for Hermitian rho (FP64).
- * Flushes queued work first.  When the last fused pass of the latest flush was a HERM_WS /
- * HERM_TC pass and nothing has changed rho since, the value comes from sums that pass took
+ * Flushes queued work first.  When the last fused pass of the latest flush was one of AUTO, HERM_WS
+ * or HERM_TC and nothing has changed rho since, the value comes from sums that pass took
  * over its write-back (squares in FP32 within a tile, FP64 above; no extra read of rho);
  * otherwise rho is read.  Either way the summation order is fixed (reproducible bit for bit).
  * Synchronises. */
@@ -281,14 +286,14 @@ QCW_API qcw_status qcw_correlation(qcw_ctx *ctx, int q1, int q2, double *out);
 /* von Neumann entropy S = -Tr[rho_A log2 rho_A] of the reduced state rho_A of the kept qubits
  * (Sec. 5.2; in bits, as S tends to n_q in the classical limit), keep strictly ascending,
  * 1 <= nkeep <= 6.  rho_A is the GPU partial trace (qcw_partial_trace), its eigenvalues come
- * from a host Jacobi eigensolver in FP64 (eigenvalues below 1e-15 count as 0).  Flushes queued
+ * from a host eigensolver in FP64 (eigenvalues below 1e-15 count as 0).  Flushes queued
  * work first; synchronises. */
 QCW_API qcw_status qcw_entropy(qcw_ctx *ctx, const int *keep, int nkeep, double *out);
 
 /* Eigenvalues of the reduced state rho_A of the kept qubits, ascending, into out[2^nkeep]
  * (Sec. 5.2.3: the eigenvalues are monitored as the noise drives rho to the classical form,
  * where they all approach 1 / 2^n_q).  keep strictly ascending, 1 <= nkeep <= 6; the GPU
- * partial trace followed by the host Jacobi eigensolver in FP64, as qcw_entropy.  Flushes
+ * partial trace followed by the host eigensolver in FP64, as qcw_entropy.  Flushes
  * queued work first; synchronises. */
 QCW_API qcw_status qcw_eigenvalues(qcw_ctx *ctx, const int *keep, int nkeep, double *out);
 
@@ -319,7 +324,9 @@ QCW_API qcw_status qcw_checkpoint_read(qcw_ctx *ctx, long long ticket, double *o
  * p_m = sum_{r: q(r) = m} Re rho_rr; the outcome m is `forced` when it is 0 or 1,
  * otherwise m = 0 iff u < p_0 (u: caller's uniform draw in [0, 1)).  Then
  * rho <- P_m rho P_m / p_m with the scale computed in FP64.  *outcome and *prob receive m
- * and p_m.  If p_m < 1e-12 the call returns QCW_EZEROPROB and rho is unchanged. */
+ * and p_m.  If p_m < 1e-12 the call returns QCW_EZEROPROB and rho is unchanged.  (A p_m up to some
+ * 1e-7 of the trace can be rounding alone, see qcw_set_fused_kernel: an outcome that cannot happen is
+ * not always told from one that nearly cannot.) */
 QCW_API qcw_status qcw_measure(qcw_ctx *ctx, int qubit, int forced, double u, int *outcome, double *prob);
 
 /* Reduced density matrix of the kept qubits (strictly ascending, 0 <= nkeep <= n):
@@ -362,7 +369,7 @@ QCW_API qcw_status qcw_partial_trace_static(const void *dev_rho, int nqubits, co
  * ops[op_begin[j] .. op_begin[j+1]) (1- and 2-qubit gates and Kraus channels, matrices as in
  * qcw_apply_ops).  fuse_k (2..5) bounds the qubits of a fused pass; 0: a pass works on every
  * qubit of its tile.  Creation plans every circuit, allocates one device arena for all
- * states (kept as 4^n real Pauli coefficients) and captures the whole run (one persistent kernel) in a CUDA graph on cuda_stream
+ * states (kept as 4^n real Pauli coefficients) and for reading one of them, and captures the whole run (one persistent kernel) in a CUDA graph on cuda_stream
  * (NULL: a non-blocking stream owned by the batch, since the legacy stream cannot be captured).  All arrays are copied; the caller may free them on return. */
 typedef struct qcw_batch qcw_batch;
 QCW_API qcw_status qcw_batch_create(int ncirc, const int *nqubits, const long long *op_begin, const qcw_op *ops,
@@ -375,7 +382,8 @@ QCW_API qcw_status qcw_batch_wait(qcw_batch *b, double timeout_s);
 /* Readouts of the last run (waits): p1 gets sum_j nqubits[j] values (circuit order, per qubit
  * P(q = 1)), purity and trace one value per circuit (FP64).  Any pointer may be NULL. */
 QCW_API qcw_status qcw_batch_results(qcw_batch *b, double *p1, double *purity, double *trace);
-/* Final rho of one circuit as host complex128 (2 * 4^n doubles). */
+/* Final rho of one circuit as host complex128 (2 * 4^n doubles).  Allocates nothing; several threads
+ * may read at once. */
 QCW_API qcw_status qcw_batch_get_state(qcw_batch *b, int circuit, double *rho_c128);
 /* Work items, fused passes, rounds of the passes and modeled SM-seconds of one run. */
 QCW_API qcw_status qcw_batch_info(qcw_batch *b, long long *items, long long *passes, long long *phases,

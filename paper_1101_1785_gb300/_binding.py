@@ -275,14 +275,14 @@ class Density:
         check(lib().qcw_set_validation(self.h, int(bool(on))), "qcw_set_validation")
 
     def set_fused_kernel(self, which: int):
-        """0 = auto (warp-specialised Hermitian from 6 qubits), 1 = one CTA per tile (no symmetry
+        """0 = auto (real Pauli coefficients from 3 qubits, 3 where they do not pay), 1 = one CTA per tile (no symmetry
         assumed), 2 = Hermitian, one CTA per tile pair, 3 = warp-specialised Hermitian (FP32 CUDA
         cores), 4 = 3 with its two-qubit phases on the tensor cores (tcgen05, 3xTF32)."""
         check(lib().qcw_set_fused_kernel(self.h, int(which)), "qcw_set_fused_kernel")
 
     def set_fused_wait_limit(self, polls: int, stall_tile: int = -1):
-        """Poll limit of the fused kernel's in-kernel waits (0 = default) and an optional tile
-        whose load the first CTA skips, so that the wait runs out."""
+        """Poll limit of the in-kernel waits of fused passes and ensemble densities (0 = default) and an
+        optional tile whose load the first CTA skips, so that the wait runs out."""
         check(lib().qcw_set_fused_wait_limit(self.h, int(polls), int(stall_tile)), "qcw_set_fused_wait_limit")
 
     def device_state(self):

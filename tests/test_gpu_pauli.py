@@ -260,3 +260,41 @@ def test_storage_is_tried_again_for_the_next_state(q):
     assert abs(d.correlation(0, n - 1)[2, 2] - 1) <= READ_TOL
     assert before - torch.cuda.mem_get_info()[0] >= 4 << 30
     d.close()
+
+
+@pytest.mark.parametrize("how", ["fused", "list", "batch"])
+@pytest.mark.parametrize("theta", [1e-2, 1e-3, 3e-4, 1e-4, 0.0])
+def test_small_probabilities(q, how, theta):
+    """Probabilities near 0: a weak rotation, and (theta = 0) operations that undo one another.  Absolute
+    error of a few FP32 roundings of numbers at most 1; a forced outcome agrees with what was read."""
+    rng = np.random.default_rng(4)
+    n = 4
+    op = lambda m, *qs: wl.Op("gate", qs, np.asarray(m, complex)[None])
+    c, s = np.cos(theta / 2), np.sin(theta / 2)
+    u, cx = haar_unitary(rng, 2), wl.gate_matrix("CNOT")
+    ops = [op([[c, -s], [s, c]], 0), op(u, 1), op(cx, 1, 2), op(haar_unitary(rng, 2), 2), op(cx, 0, 3)]
+    if theta == 0:
+        ops = [op(u, 0), op(u, 1), op(cx, 0, 1), op(cx, 1, 3), op(cx, 1, 3), op(cx, 0, 1), op(u.conj().T, 1), op(u.conj().T, 0)]
+    want = wl.zero_state(n)
+    for o in ops:
+        oracle.apply_op(want, o)
+    want, tol = oracle.probabilities(want), 2.0 ** -22
+    if how == "batch":
+        b = q.Batch([wl.Circuit(n, ops)])
+        b.run()
+        assert np.abs(b.results()[0][0] - want).max() <= tol
+        return
+    d = q.Density(n)
+    if how == "fused":
+        d.set_mode(q.QCW_MODE_FUSED)
+        d.reset()
+    d.apply_packed(q.PackedOps(ops))
+    got = d.probabilities()
+    assert np.abs(got - want).max() <= tol
+    if got[0] >= 1e-12:
+        assert d.measure(0, 1) == (1, got[0])
+    else:
+        with pytest.raises(q.QcwError) as err:
+            d.measure(0, 1)
+        assert err.value.status == q.QCW_EZEROPROB
+    d.close()
