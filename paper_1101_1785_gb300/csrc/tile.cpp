@@ -52,10 +52,18 @@ static int tile_pos(const FPass &fp, int vbit)
 // (b00, b01, b10, b11) = (I + Z, X + D, X - D, I - Z); I, X, Z and i D are 2x the Pauli
 // coefficients tr(P b) of the 2x2 block.  Member e = 8 r_a + 4 r_b + 2 c_a + c_b keeps its bit
 // positions: Pauli index bits (2 r + c) per qubit.
-// Transfer-matrix entries below this are FP64 rounding residue of exact zeros (the entries of
-// a map of unit-norm operators are O(1)); they are stored as 0 so that, for instance, the trace
-// row of a trace-preserving map is exactly (2^-k, 0, ...).
+// Transfer-matrix entries below this, for a map of unit-norm operators, are FP64 rounding residue of
+// exact zeros; they are stored as 0 so that, for instance, the trace row of a trace-preserving map
+// is exactly (2^-k, 0, ...).  Any other map's are measured against its first entry, the largest of a
+// map sum_j K_j . K_j^dagger (2^-k for unit norm).
 constexpr double kTransferZero = 1e-14;
+
+static void clear_residue(double *R, int k)
+{
+    const double tiny = kTransferZero * R[0] * (1 << k);
+    for (int i = 0; i < 1 << (4 * k); i++)
+        if (std::abs(R[i]) < tiny) R[i] = 0.0;
+}
 
 static void pauli_fwd(c128 *x)
 {
@@ -119,8 +127,9 @@ void pauli_transfer(const std::vector<c128> &S, double R[16][16])
             c128 z = M[e][f] / 16.0;
             if (pauli_odd(e)) z *= c128(0, 1);
             if (pauli_odd(f)) z *= c128(0, -1);
-            R[e][f] = std::abs(z.real()) < kTransferZero ? 0.0 : z.real();
+            R[e][f] = z.real();
         }
+    clear_residue(R[0], 2);
 }
 
 // One qubit: members (b00, b01, b10, b11) -> (I, X, D, Z) by the same butterflies; the real
@@ -150,9 +159,10 @@ void pauli_transfer1(const c128 *S, double R[4][4])
             c128 z = sc[e] / 4.0;
             if (e == 2) z *= c128(0, 1);
             if (f == 2) z *= c128(0, -1);
-            R[e][f] = std::abs(z.real()) < kTransferZero ? 0.0 : z.real();
+            R[e][f] = z.real();
         }
     }
+    clear_residue(R[0], 1);
 }
 
 static void push_transfer1(const c128 *S, std::vector<float2> &out)

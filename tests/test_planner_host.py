@@ -485,3 +485,20 @@ def test_plain_transfer_form_reproduces_the_superoperator(shim, k):
         np.testing.assert_allclose(_pauli_apply_plain(R, x, k), Sd @ x, atol=1e-12)
         R32 = R.astype(np.float32)
         assert R32[0, 0] == np.float32(2.0 ** -k) and not R32[0, 1:].any()
+
+
+@pytest.mark.parametrize("k", [1, 2])
+@pytest.mark.parametrize("scale", [1e-12, 1e-8, 1e-3, 1e4])
+def test_transfer_form_of_small_and_large_operators(shim, k, scale):
+    """What counts as the residue of an exact zero is measured against the map's own size."""
+    rng = np.random.default_rng(7 + k)
+    P = ctypes.c_void_p
+    d = 1 << k
+    for S in (np.kron(u := haar_unitary(rng, d), u.conj()), _superop_kraus([0.8 * haar_unitary(rng, d), 0.5 * haar_unitary(rng, d)])):
+        S = np.ascontiguousarray(scale ** 2 * S, dtype=np.complex128)
+        R = np.zeros((4 ** k) ** 2)
+        shim.pauli_transfer_k(k, S.ctypes.data_as(P), R.ctypes.data_as(P))
+        R = R.reshape(4 ** k, 4 ** k)
+        x = rng.standard_normal(4 ** k) + 1j * rng.standard_normal(4 ** k)
+        np.testing.assert_allclose(_pauli_apply_plain(R, x, k), S @ x, atol=1e-12 * scale ** 2, rtol=0)
+        assert not R[0, 1:].any()
