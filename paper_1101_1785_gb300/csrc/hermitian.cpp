@@ -13,7 +13,7 @@ using cd = std::complex<double>;
 
 // Eigenvalues only: Householder reduction to a real tridiagonal matrix (Golub and Van Loan, "Matrix
 // Computations", Sec. 8.3: A <- A - v w^H - w v^H with w = p - (beta / 2) (p^H v) v, p = beta A v),
-// then implicit QR steps with Wilkinson's shift on it (Sec. 8.3.3, 8.3.4).  O(N^3) once where each sweep
+// then implicit QR steps with Wilkinson's shift on it (Sec. 8.3.5).  O(N^3) once where each sweep
 // of the Jacobi iteration below costs several times that: 64 x 64 took 6 ms with it.
 static void eigenvalues_only(const cd *A_in, int N, double *w)
 {
